@@ -160,9 +160,9 @@ typedef struct {
   int64_t np_launches;
   int64_t kernel_launches; /* all kernels this domain launched */
   int32_t lbm_block;   /* threads per block of the LBM step and of the */
-  int32_t np_block;    /* transport step, picked by the library's autotuner
-                          on the first solve (timing only: every block size
-                          computes the same bits); 0 before it ran */
+  int32_t np_block;    /* transport step, as chosen on the first solve and
+                          initialisation (timing only: every block size
+                          computes the same bits); 0 before */
   int32_t lbm_shape;   /* the launch shapes themselves (see */
   int32_t np_shape;    /* cdi_set_launch_shapes); -1 before they are chosen */
 } cdi_timing;
@@ -265,16 +265,16 @@ cdi_status cdi_set_implicit(cdi_domain *dom, double tol, int max_iter);
 
 /* Launch shapes of the two step kernels (the paper has no counterpart: it
  * states the method, not its launch configuration).  By default (-1) an autotuner
- * times every candidate shape of the LBM step (0-5) and of the transport
- * step (0-9) on the domain's first flow solve and first transport
- * initialisation and keeps the fastest; every shape computes the same bits
- * (the arithmetic of a lattice site or pore cell, and the per-warp account
- * slots, do not depend on the shape), so the choice changes speed only.
- * lbm_shape / np_shape in range fix the shape from the next step on; -1
- * returns the kernel to the autotuner (its cached choice, if any).  Shapes
- * are those of the FP32 kernels; FP64 maps the resident-grid shapes to plain
- * launches.  Out-of-range values fail with CDI_ERR_INVALID_ARG and change
- * nothing. */
+ * times every candidate shape of the LBM step (0-5) on the domain's first flow
+ * solve and keeps the fastest, and the transport step (0-9: 64, 128 or 256
+ * threads per block, 3-9 the default again) takes 128 threads; every shape
+ * computes the same bits (the arithmetic of a lattice site or pore cell, and
+ * the per-warp account slots, do not depend on the shape), so the choice
+ * changes speed only.  lbm_shape / np_shape in range fix the shape from the
+ * next step on; -1 returns the kernel to its default (the autotuner's cached
+ * choice, if any).  Shapes are those of the FP32 kernels; FP64 maps the
+ * resident-grid shapes to plain launches.  Out-of-range values fail with
+ * CDI_ERR_INVALID_ARG and change nothing. */
 cdi_status cdi_set_launch_shapes(cdi_domain *dom, int32_t lbm_shape, int32_t np_shape);
 
 /* Advance n_steps >= 0 transport steps (Eq. 3 with Eq. 6): explicit unless
@@ -305,7 +305,9 @@ typedef struct {
  * Needs a solved flow; blocks until done.  Replaces the domain's potential
  * and transport state (set them again before cdi_step_transport).  Device
  * memory for the members is taken from the domain's allocator for the call
- * only: about n_combos * (dim + 8) * 4 bytes per cell in FP32. */
+ * only: about n_combos * (3 dim + 2 n_species) * 4 bytes per pore cell in FP32
+ * (twice the concentrations' part with pair storage; where a face Peclet
+ * number reaches 1/2, (dim + 1) * n_species * 8 more). */
 cdi_status cdi_sweep_transport(cdi_domain *dom, const cdi_combo *combos, int n_combos,
                                const cdi_elec_params *p, const cdi_species *sp,
                                int n_species, double c0_molm3, double Ka_mps,
@@ -324,8 +326,8 @@ cdi_status cdi_sweep_transport(cdi_domain *dom, const cdi_combo *combos, int n_c
  *   doms: n_doms >= 1 distinct domains on the current device, all of the same
  *     dimension and precision, each with a solved flow.  doms[0] leads: its
  *     stream runs the batch and its allocator provides the members' device
- *     memory for the call only (about (dim + 8) * 4 bytes per pore cell per
- *     member in FP32, plus one potential per domain and applied_V).
+ *     memory for the call only (as cdi_sweep_transport's per pore cell and
+ *     member, plus one potential per domain and applied_V).
  *   gamma_out, cout_out: host, n_doms * n_combos * n_species doubles;
  *   dt_out: n_doms * n_combos doubles or NULL.
  * Blocks until done; replaces every domain's potential and transport state.

@@ -38,11 +38,22 @@ void *cdi_dev_alloc(cdi_domain *d, size_t bytes) {
   void *p = nullptr;
   if (d->has_alloc) {
     p = d->alloc.alloc(bytes, d->alloc.ctx);
+    if (p && ((uintptr_t)p & 15u)) {
+      // the kernels load 16-byte records: an allocator of looser alignment
+      // gives a larger block, of which the aligned part is used
+      d->alloc.free(p, bytes, d->alloc.ctx);
+      bytes += 16;
+      p = d->alloc.alloc(bytes, d->alloc.ctx);
+      if (!p) return nullptr;
+      void *q = (void *)(((uintptr_t)p + 15u) & ~(uintptr_t)15u);
+      d->blocks.push_back({q, bytes, p});
+      return q;
+    }
   } else if (cudaMallocAsync(&p, bytes, d->stream) != cudaSuccess) {
     (void)cudaGetLastError();
     p = nullptr;
   }
-  if (p) d->blocks.push_back({p, bytes});
+  if (p) d->blocks.push_back({p, bytes, p});
   return p;
 }
 
@@ -58,7 +69,7 @@ static void dev_free(cdi_domain *d, void *p, size_t bytes) {
 void cdi_dev_release(cdi_domain *d, void *p) {
   for (size_t i = 0; i < d->blocks.size(); i++) {
     if (d->blocks[i].p != p) continue;
-    dev_free(d, p, d->blocks[i].bytes);
+    dev_free(d, d->blocks[i].base, d->blocks[i].bytes);
     d->blocks.erase(d->blocks.begin() + (long)i);
     return;
   }
@@ -88,7 +99,7 @@ static void pinned_give(double *p) {
 
 static void free_all(cdi_domain *d) {
   if (d->stream) cudaStreamSynchronize(d->stream);
-  for (auto &b : d->blocks) dev_free(d, b.p, b.bytes);
+  for (auto &b : d->blocks) dev_free(d, b.base, b.bytes);
   d->blocks.clear();
   if (d->stream) cudaStreamSynchronize(d->stream);
   if (d->h_scal) pinned_give(d->h_scal);
@@ -312,12 +323,12 @@ cdi_status cdi_create_domain(const cdi_domain_desc *desc, const uint8_t *mask,
   d->d_u = A((size_t)D.dim * n_pore * T);
   d->d_psi = (double *)A(N * 8);
   d->d_phi = A((size_t)n_pore * 8);
-  d->d_C[0] = A((size_t)cdi::kMaxSpecies * n_pore * T);
-  d->d_C[1] = A((size_t)cdi::kMaxSpecies * n_pore * T);
-  if (d->cpair) {
-    d->d_Clo[0] = (float *)A((size_t)cdi::kMaxSpecies * n_pore * 4);
-    d->d_Clo[1] = (float *)A((size_t)cdi::kMaxSpecies * n_pore * 4);
-  }
+  const size_t c_bytes = (size_t)cdi::kMaxSpecies * n_pore * T * (d->cpair ? 2 : 1);
+  d->d_C[0] = A(c_bytes);
+  d->d_C[1] = A(c_bytes);
+  if (d->prec != CDI_FP64) d->d_fd = (float2 *)A((size_t)D.dim * n_pore * sizeof(float2));
+  d->d_latd = (short *)A((size_t)2 * (D.dim - 1) * n_pore * sizeof(short));
+  d->d_latb = (int *)A((size_t)2 * (D.dim - 1) * ((n_pore + 30) / 31) * sizeof(int));
   d->d_acc = (double *)A((size_t)3 * cdi::kMaxSpecies * d->np_accs * 8);
   d->d_part = (double *)A((size_t)16 * cdi::kRedBlocks * 8);
   d->d_counter = (unsigned int *)A(16 * sizeof(unsigned int));
@@ -349,11 +360,8 @@ cdi_status cdi_create_domain(const cdi_domain_desc *desc, const uint8_t *mask,
   chk(cudaMemsetAsync(d->d_u, 0, (size_t)D.dim * n_pore * T, d->stream), "memset");
   chk(cudaMemsetAsync(d->d_psi, 0, N * 8, d->stream), "memset");
   chk(cudaMemsetAsync(d->d_phi, 0, (size_t)n_pore * 8, d->stream), "memset");
-  chk(cudaMemsetAsync(d->d_C[0], 0, (size_t)cdi::kMaxSpecies * n_pore * T, d->stream), "memset");
-  chk(cudaMemsetAsync(d->d_C[1], 0, (size_t)cdi::kMaxSpecies * n_pore * T, d->stream), "memset");
-  for (int b = 0; b < 2 && d->cpair; b++)
-    chk(cudaMemsetAsync(d->d_Clo[b], 0, (size_t)cdi::kMaxSpecies * n_pore * 4, d->stream),
-        "memset");
+  chk(cudaMemsetAsync(d->d_C[0], 0, c_bytes, d->stream), "memset");
+  chk(cudaMemsetAsync(d->d_C[1], 0, c_bytes, d->stream), "memset");
   chk(cudaMemsetAsync(d->d_acc, 0, (size_t)3 * cdi::kMaxSpecies * d->np_accs * 8, d->stream),
       "memset");
   if (s == CDI_OK) s = cdi_flow_build_flags(d);
@@ -838,10 +846,7 @@ cdi_status cdi_query_column_means(cdi_domain *d, int species, double *out) {
 
 cdi_status cdi_copy_field(cdi_domain *d, int field, double *host, size_t count) {
   if (!d || !host) return cdi_fail(d, CDI_ERR_INVALID_ARG, "NULL argument");
-  const size_t T = d->prec == CDI_FP64 ? 8 : 4;
-  const void *src = nullptr;
-  const float *lo = nullptr;
-  int comps = 0;
+  int comps = 0, species = -1;
   double *tmp = d->d_cg;  // 4*N doubles of scratch outside a potential solve
   if (field == CDI_FIELD_U_LATTICE) {
     const size_t n = (size_t)d->dim * d->Nf;
@@ -859,20 +864,18 @@ cdi_status cdi_copy_field(cdi_domain *d, int field, double *host, size_t count) 
     return CDI_OK;
   } else if (field == CDI_FIELD_U) {
     comps = d->dim;
-    src = d->d_u;
   } else if (field >= CDI_FIELD_C && field < CDI_FIELD_C + cdi::kMaxSpecies) {
     int k = field - CDI_FIELD_C;
     if (!d->np_ready || k >= d->ns) return cdi_fail(d, CDI_ERR_STATE, "no such species state");
     comps = 1;
-    src = (const char *)d->d_C[d->cur] + (size_t)k * d->n_pore * T;
-    if (d->cpair) lo = d->d_Clo[d->cur] + (size_t)k * d->n_pore;
+    species = k;
   } else {
     return cdi_fail(d, CDI_ERR_INVALID_ARG, "unknown field");
   }
   // rank-ordered transport field -> lattice order (0 in solid cells)
   const size_t n = (size_t)comps * d->N;
   if (count != n) return cdi_fail(d, CDI_ERR_INVALID_ARG, "count mismatch");
-  cdi_status s = cdi_np_scatter(d, src, lo, comps, tmp);
+  cdi_status s = cdi_np_scatter(d, species, tmp);
   if (s != CDI_OK) return s;
   CDI_TRY(d, cudaMemcpyAsync(host, tmp, n * 8, cudaMemcpyDeviceToHost, d->stream), "copy field");
   CDI_TRY(d, cudaStreamSynchronize(d->stream), "copy field");

@@ -233,8 +233,9 @@ struct cdi_domain {
   bool has_alloc = false;
   std::string err;
   struct Block {
-    void *p;
+    void *p;       // what cdi_dev_alloc returned
     size_t bytes;
+    void *base;    // what the allocator returned
   };
   std::vector<Block> blocks;
 
@@ -273,9 +274,18 @@ struct cdi_domain {
   void *d_phi = nullptr;        // n_pore psi / V_T, 8 bytes a cell: double
                                 // (FP64) or a float2 (hi, lo) pair (FP32)
   bool cpair = false;           // concentrations stored as FP32 pairs (hi + lo)
-  float *d_Clo[2] = {nullptr, nullptr};  // their low words (pair storage only)
-  void *d_C[2] = {nullptr, nullptr};  // kMaxSpecies*n_pore concentrations,
-                                      // ping-pong, T
+  void *d_C[2] = {nullptr, nullptr};  // concentrations, ping-pong.  FP64: species
+                                // k of rank r at k * n_pore + r.  FP32: one record
+                                // per rank and species pair (2p, 2p + 1), the pairs
+                                // one after the other: c_2p[, c_2p+1][, their low
+                                // words] (see c_view); the layout follows ns
+  float2 *d_fd = nullptr;       // FP32: dim * n_pore face data (see k_np_faces)
+  float2 *d_bern = nullptr;     // FP32: Bernoulli pairs of the faces with |P| >= 1/2
+                                // (taken the first time there is one)
+  size_t bern_bytes = 0;
+  int np_mode = 0;              // which kernel the faces ask for (see np_warp31)
+  short *d_latd = nullptr;      // 2*(dim-1) 16-bit lateral differences per rank
+  int *d_latb = nullptr;        // and their bases per tile of 31 ranks
   double *d_acc = nullptr;      // 3*kMaxSpecies*np_accs per-warp sums (8 B each:
                                 // FP64, or an FP32 pair in FP32 modes)
   double *d_part = nullptr;     // reduction partials (8*kRedBlocks)
@@ -318,9 +328,9 @@ struct cdi_domain {
                                 // warps of 31 home cells)
   int np_accs = 0;              // account sets, one per warp (rounded up to a
                                 // multiple of 8: enough for any launch shape)
-  // block sizes of the step kernels, picked by the autotuners
+  // block sizes of the step kernels
   int lbm_block = 128, np_block = 128;
-  int np_variant = 1;           // transport launch shape (see tune_np)
+  int np_variant = 1;           // transport launch shape (see kNpVariantBlock)
   int lbm_variant = 1;          // LBM launch shape (see tune_lbm)
   bool lbm_tuned = false, np_tuned = false;
 
@@ -342,6 +352,35 @@ struct cdi_domain {
   cdi_timing timing{};
 };
 
+namespace cdi {
+
+// One species of a concentration buffer: hi word of rank r at p[r * stride],
+// its low word (pair storage; lo != 0) lo words further on.
+template <typename T> struct CView {
+  const T *p;
+  int stride, lo;
+  __device__ __forceinline__ double at(int r) const {
+    const T *q = p + (size_t)r * stride;
+    return (double)q[0] + (lo ? (double)q[lo] : 0.0);
+  }
+};
+template <typename T> struct CViews {
+  CView<T> v[kMaxSpecies];
+};
+template <typename T> inline CView<T> c_view(const cdi_domain *d, const void *C, int k) {
+  if (sizeof(T) == 8) return CView<T>{(const T *)C + (size_t)k * d->n_pore, 1, 0};
+  const int per = d->cpair ? 2 : 1, pair = k / 2, w = d->ns - 2 * pair >= 2 ? 2 : 1;
+  return CView<T>{(const T *)C + (size_t)pair * 2 * per * d->n_pore + (k & 1), w * per,
+                  d->cpair ? w : 0};
+}
+template <typename T> inline CViews<T> c_views(const cdi_domain *d, const void *C) {
+  CViews<T> v{};
+  for (int k = 0; k < d->ns; k++) v.v[k] = c_view<T>(d, C, k);
+  return v;
+}
+
+}  // namespace cdi
+
 // Scalar slots in d_scal / h_scal.
 enum {
   S_RES_NUM = 0, S_RES_DEN = 1, S_RES = 2,  // flow residual
@@ -362,7 +401,7 @@ enum {
 
 // Counter slots in d_counter.
 enum { C_RES = 0, C_ULAT = 1, C_CG1 = 2, C_CG2 = 3, C_DT = 4, C_OUT = 5, C_MASS = 6, C_ACC = 7,
-       C_GEOM = 8, C_IMP = 9, C_LINK = 10 };
+       C_GEOM = 8, C_IMP = 9, C_LINK = 10, C_FACE = 11 };
 
 enum { PH_FLOW = 0, PH_CHECK = 1, PH_PSI = 2, PH_NP = 3 };
 
@@ -404,8 +443,10 @@ cdi_status cdi_psi_solve(cdi_domain *d, double psi_s, double kdx2, const double 
 cdi_status cdi_psi_coupled(cdi_domain *d);
 cdi_status cdi_np_build_flags(cdi_domain *d);
 cdi_status cdi_np_build_compact(cdi_domain *d);
-cdi_status cdi_np_scatter(cdi_domain *d, const void *src, const float *lo, int comps,
-                          double *dst);
+cdi_status cdi_np_scatter(cdi_domain *d, int species, double *dst);
+cdi_status cdi_np_records_to_planes(cdi_domain *d, int b, float *planes);
+cdi_status cdi_np_planes_to_records(cdi_domain *d, const float *planes, int b);
+cdi_status cdi_np_faces(cdi_domain *d);
 cdi_status cdi_np_init(cdi_domain *d, double dt_s, double *dt_used);
 cdi_status cdi_np_dt(cdi_domain *d, double scale, double *dt_out);
 cdi_status cdi_np_geometry(cdi_domain *d, double *pores, double *faces, double *sum_ux);

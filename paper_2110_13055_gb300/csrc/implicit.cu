@@ -149,17 +149,14 @@ __device__ __forceinline__ double apply_scaled(const IGeo &g, const double *__re
 // dt b, r = rhs - M x, r0 = r, p = r; rho = r0.r, bb = rhs.rhs.
 template <typename T, int DIM>
 __global__ void __launch_bounds__(kRedThreads)
-    k_bi_start(IGeo g, const double *__restrict__ c, double dt, const T *__restrict__ Ck,
-               const float *__restrict__ Clk, double tol, double *__restrict__ x,
+    k_bi_start(IGeo g, const double *__restrict__ c, double dt, CView<T> Ck, double tol, double *__restrict__ x,
                double *__restrict__ rr, double *__restrict__ r0, double *__restrict__ p,
                double *__restrict__ part, unsigned int *counter, double *scal) {
   using C = ICoef<DIM>;
   __shared__ double sm[2 * 32];
   double v[2] = {0.0, 0.0};
   const size_t n = (size_t)g.n;
-  auto cval = [&](int q) {
-    return (double)Ck[q] + (Clk ? (double)Clk[q] : 0.0);
-  };
+  auto cval = [&](int q) { return Ck.at(q); };
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < g.n; r += gridDim.x * blockDim.x) {
     const double cP = cval(r);
     const double rhs = cP + dt * c[(size_t)C::B * n + r];
@@ -319,7 +316,7 @@ __global__ void k_bi_p(int n, double *__restrict__ p, const double *__restrict__
 // C^{n+1}, summed per warp of 32 ranks into the domain's per-warp accounts.
 template <typename T, int DIM>
 __global__ void k_bi_finish(IGeo g, const double *__restrict__ c, const double *__restrict__ x,
-                            T *__restrict__ Cout, float *__restrict__ Cout_l, int k,
+                            CView<T> Cout, int k,
                             typename std::conditional<std::is_same<T, float>::value, float2,
                                                       double>::type *__restrict__ acc,
                             int naccs) {
@@ -329,13 +326,10 @@ __global__ void k_bi_finish(IGeo g, const double *__restrict__ c, const double *
   double v[3] = {0.0, 0.0, 0.0};
   if (r < g.n) {
     const double xv = x[r];
-    if (std::is_same<T, float>::value) {
-      const float hi = (float)xv;
-      Cout[r] = (T)hi;
-      if (Cout_l) Cout_l[r] = (float)(xv - (double)hi);
-    } else {
-      Cout[r] = (T)xv;
-    }
+    T *o = const_cast<T *>(Cout.p) + (size_t)r * Cout.stride;
+    const T hi = (T)xv;
+    o[0] = hi;
+    if (Cout.lo) o[Cout.lo] = (T)(xv - (double)hi);
     v[0] = c[(size_t)C::GAM * n + r] * xv;
     v[1] = c[(size_t)C::BIN * n + r] - c[(size_t)C::AIN * n + r] * xv;
     v[2] = c[(size_t)C::AOUT * n + r] * xv;
@@ -403,11 +397,10 @@ cdi_status imp_step(cdi_domain *d) {
   using A = typename std::conditional<std::is_same<T, float>::value, float2, double>::type;
   for (int k = 0; k < d->ns; k++) {
     const double *c = d->d_icoef + (size_t)k * C::NC * nn;
-    const T *Ck = (const T *)d->d_C[in] + (size_t)k * nn;
-    const float *Clk = d->d_Clo[in] ? d->d_Clo[in] + (size_t)k * nn : nullptr;
+    const CView<T> Ck = c_view<T>(d, d->d_C[in], k);
     int iters = 0;
     k_bi_start<T, DIM><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        g, c, dt, Ck, Clk, d->imp_tol, x, rr, r0, p, d->d_part, d->d_counter + C_IMP,
+        g, c, dt, Ck, d->imp_tol, x, rr, r0, p, d->d_part, d->d_counter + C_IMP,
         d->d_iscal);
     d->timing.kernel_launches++;
     CDI_TRY(d, cudaMemcpyAsync(d->h_scal + S_IMP, d->d_iscal, B_N * sizeof(double),
@@ -444,10 +437,8 @@ cdi_status imp_step(cdi_domain *d) {
     if (!done)
       return cdi_fail(d, CDI_ERR_NOT_CONVERGED,
                       "implicit step: the linear solve did not reach tol within max_iter");
-    T *Co = (T *)d->d_C[1 - in] + (size_t)k * nn;
-    float *Col = d->d_Clo[1 - in] ? d->d_Clo[1 - in] + (size_t)k * nn : nullptr;
-    k_bi_finish<T, DIM><<<(n + 127) / 128, 128, 0, d->stream>>>(g, c, x, Co, Col, k, (A *)d->d_acc,
-                                                               d->np_accs);
+    k_bi_finish<T, DIM><<<(n + 127) / 128, 128, 0, d->stream>>>(
+        g, c, x, c_view<T>(d, d->d_C[1 - in], k), k, (A *)d->d_acc, d->np_accs);
     d->timing.kernel_launches++;
     CDI_TRY(d, cudaGetLastError(), "implicit finish");
   }

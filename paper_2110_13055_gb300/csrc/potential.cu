@@ -284,14 +284,13 @@ __global__ void k_cg_dir(long long N, double *__restrict__ p, const double *__re
 // src = coef * sum_k z_k C_k, coef = F dx^2 / (eps_r eps_0) (lattice order;
 // solid cells keep the 0 the caller cleared).
 template <typename T>
-__global__ void k_charge(int n, int ns, const int *__restrict__ cells, const T *__restrict__ C,
-                         const float *__restrict__ Cl, int4 z, double coef,
-                         double *__restrict__ src) {
+__global__ void k_charge(int n, int ns, const int *__restrict__ cells, CViews<T> C, int4 z,
+                         double coef, double *__restrict__ src) {
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
     const int zz[4] = {z.x, z.y, z.z, z.w};
     double q = 0.0;
     for (int k = 0; k < ns; k++)
-      q += zz[k] * ((double)C[(size_t)k * n + r] + (Cl ? (double)Cl[(size_t)k * n + r] : 0.0));
+      q += zz[k] * C.v[k].at(r);
     src[cells[r]] = coef * q;
   }
 }
@@ -443,12 +442,12 @@ cdi_status cdi_psi_coupled(cdi_domain *d) {
   const int4 z = make_int4(d->z[0], d->z[1], d->z[2], d->z[3]);
   if (d->prec == CDI_FP64)
     k_charge<double><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        (int)d->n_pore, d->ns, d->d_cell_list, (const double *)d->d_C[d->cur], nullptr, z, coef,
+        (int)d->n_pore, d->ns, d->d_cell_list, c_views<double>(d, d->d_C[d->cur]), z, coef,
         d->d_src);
   else
     k_charge<float><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        (int)d->n_pore, d->ns, d->d_cell_list, (const float *)d->d_C[d->cur], d->d_Clo[d->cur], z,
-        coef, d->d_src);
+        (int)d->n_pore, d->ns, d->d_cell_list, c_views<float>(d, d->d_C[d->cur]), z, coef,
+        d->d_src);
   d->timing.kernel_launches++;
   CDI_TRY(d, cudaGetLastError(), "charge");
   int it = 0;
@@ -456,5 +455,6 @@ cdi_status cdi_psi_coupled(cdi_domain *d) {
   cdi_status s = cdi_psi_solve(d, d->psi_s, 0.0, d->d_src, d->psi_tol, d->psi_max_iter, &it, &rel);
   if (s == CDI_ERR_NOT_CONVERGED)
     return cdi_fail(d, s, "coupled potential did not reach tol within max_iter");
-  return s;
+  if (s != CDI_OK) return s;
+  return cdi_np_faces(d);  // the step reads face data of the new potential
 }

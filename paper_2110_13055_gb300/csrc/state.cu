@@ -50,8 +50,11 @@ std::vector<Section> sections(cdi_domain *d, int c_buf) {
   s.push_back({d->d_u, (size_t)d->dim * d->n_pore * T});
   s.push_back({d->d_psi, (size_t)d->N * 8});
   s.push_back({d->d_phi, (size_t)d->n_pore * 8});
-  s.push_back({d->d_C[c_buf], (size_t)cdi::kMaxSpecies * d->n_pore * T});
-  if (d->cpair) s.push_back({d->d_Clo[c_buf], (size_t)cdi::kMaxSpecies * d->n_pore * 4});
+  // FP32 concentrations go through planes in the potential solver's scratch
+  // (kMaxSpecies hi words a rank, then kMaxSpecies lo words: at most 32 bytes
+  // a cell, what d_cg holds), so that the file does not follow the records
+  s.push_back({d->prec == CDI_FP64 ? d->d_C[c_buf] : (void *)d->d_cg,
+               (size_t)cdi::kMaxSpecies * d->n_pore * T * (d->cpair ? 2 : 1)});
   s.push_back({d->d_acc, (size_t)3 * cdi::kMaxSpecies * d->np_accs * 8});
   return s;
 }
@@ -100,6 +103,10 @@ cdi_status cdi_save_state(cdi_domain *d, void *host_buf, size_t *bytes) {
   char *out = static_cast<char *>(host_buf);
   std::memcpy(out, &h, sizeof(h));
   size_t off = sizeof(h);
+  if (d->prec != CDI_FP64) {
+    cdi_status rs = cdi_np_records_to_planes(d, d->cur, (float *)d->d_cg);
+    if (rs != CDI_OK) return rs;
+  }
   for (const Section &s : sections(d, d->cur)) {
     CDI_TRY(d, cudaMemcpyAsync(out + off, s.dev, s.bytes, cudaMemcpyDeviceToHost, d->stream),
             "save_state copy");
@@ -158,6 +165,12 @@ cdi_status cdi_load_state(cdi_domain *d, const void *host_buf, size_t bytes) {
   d->flow_steps = h.flow_steps; d->np_steps = h.np_steps;
   d->psi_s = h.psi_s; d->eps_r = h.eps_r; d->psi_tol = h.psi_tol;
   d->psi_max_iter = (int)h.psi_max_iter; d->couple_K = h.couple_K;
+  if (d->prec != CDI_FP64) {
+    cdi_status rs = cdi_np_planes_to_records(d, (const float *)d->d_cg, 0);
+    if (rs == CDI_OK) rs = cdi_np_faces(d);
+    if (rs != CDI_OK) return rs;
+    CDI_TRY(d, cudaStreamSynchronize(d->stream), "load_state");
+  }
   return CDI_OK;
 }
 

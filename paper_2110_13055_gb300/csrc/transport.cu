@@ -155,34 +155,17 @@ __device__ __noinline__ void bernoulli_pair_split(float adv, float z, float2 nb,
   Bm = neg ? Ba : Bma;
 }
 
-__device__ __forceinline__ float face_flux(float adv, float z, float dd, float2 nb, float2 pp,
-                                           float CP, float Cn) {
-  const float p = __fmaf_rn(-z, dd, adv);
-  if (fabsf(p) < 0.5f) {
-    const float p2 = __fmul_rn(p, p);
-    float E = __fmaf_rn(p2, 1.f / 30240.f, -1.f / 720.f);
-    E = __fmaf_rn(E, p2, 1.f / 12.f);
-    E = __fmaf_rn(E, p2, 1.f);
-    return __fmaf_rn(E, __fsub_rn(CP, Cn), __fmul_rn(__fmul_rn(0.5f, p), __fadd_rn(CP, Cn)));
-  }
-  float Bp, Bm;
-  bernoulli_pair_split(adv, z, nb, pp, Bp, Bm);
-  return r_fma(Bm, CP, -r_mul(Bp, Cn));
-}
-
 __device__ __forceinline__ double phi_diff(double nb, double pp) { return __dsub_rn(nb, pp); }
 __device__ __forceinline__ float phi_diff(float2 nb, float2 pp) {
   return __fadd_rn(__fsub_rn(nb.x, pp.x), __fsub_rn(nb.y, pp.y));
 }
 
-// Geometry of the compact transport layout handed to the step kernels.
+// Geometry of the compact transport layout handed to the FP64 step kernels.
 struct NPGeo {
   const uint2 *meta;   // per rank {flags | x << 16, row}
-  const NFlag *fl;     // per rank: its face flags alone (what the step reads)
-  const uint2 *words;  // per 32 cells of a row {first rank, pore bits}
   const int *lat;      // per lateral face f (y+, y-, z+, z-) and rank r, at
                        // (f - 2) * n + r: the pore neighbour's rank, or -1
-  int n, W, ny, nz, walls;
+  int n;
   int naccs;           // account sets (one per warp), the same for any launch shape
 };
 
@@ -194,20 +177,27 @@ struct NPGeo {
 // with its sign flipped (one shuffle).  Every x face is then evaluated once
 // instead of twice, and every lane of the warp takes the same path.
 constexpr int kHome = 31;
+// 16-bit lateral differences: a closed face, and one that does not fit.
+constexpr short kLatClosed = -32768, kLatWide = -32767;
 
-// The fields of one FP32 transport state as per-species / per-component
-// plane pointers: by value as kernel parameters (one launch, one state) or
-// in a member table (fused sweeps and batches), so that every access is a
-// base pointer plus a 32-bit rank.
+// The fields of one FP32 transport state, by value as kernel parameters (one
+// launch, one state) or in a member table (fused sweeps and batches).  The
+// concentrations of a species pair stand together, one record per rank
+// (c0, c1, and with pair storage their low words: 16 bytes), so a cell or a
+// neighbour is one load.
 struct NPFields {
-  const float *C[kMaxSpecies];   // concentrations read (hi words)
-  const float *Cl[kMaxSpecies];  // their low words (pair storage), else null
-  float *Co[kMaxSpecies];        // concentrations written
-  float *Col[kMaxSpecies];       // their low words
-  const float *u[3];             // velocity components
-  const int *lat[4];             // lateral neighbour ranks (y+, y-, z+, z-)
-  const float2 *phi;             // psi / V_T as (hi, lo)
+  const float *C[2];             // per species pair: records read
+  float *Co[2];                  // records written
+  const float2 *fd[3];           // per + face: face velocity, potential difference
+  const short *latd;             // lateral differences (y+, y-[, z+, z-]) per rank
+  const int *latb;               // their bases per tile of 31 ranks
+  const int *lat;                // full lateral ranks (kLatWide cells only)
+  const float *ux;               // x velocity (inlet cells only)
+  const float2 *phi;             // psi / V_T as (hi, lo) (|P| >= 1/2 and inlet only)
   const NFlag *fl;               // face flags
+  const float2 *bern;            // (B(P), B(-P)) of + face a, rank r, species k at
+                                 // (a * n + r) * ns + k, and of the feed face at
+                                 // a = dim; set where |P| >= 1/2
   float2 *acc;                   // per-warp accounts
 };
 __host__ __device__ constexpr long long np_warps(long long n) { return (n + kHome - 1) / kHome; }
@@ -365,46 +355,61 @@ __device__ __forceinline__ float2 pair_add(float2 t, float v) {
   return make_float2(s, __fadd_rn(t.y, e));
 }
 
-// The FP32 warp accounts of np_account, with the warp's adsorption slots
-// read ahead by lane 0 (np_account_read): a slot belongs to one warp tile, so
-// reading it before the tile's arithmetic gives the value acc_add would read
-// after it, and its latency no longer ends every tile.  (The inflow and
+// The FP32 warp accounts, two species at a time: lanes 0-15 carry species 2p
+// and lanes 16-31 species 2p + 1 after the first exchange, so the pair's sums
+// take 5 shuffles instead of 10 and end in lanes 0 and 16, which keep one
+// account slot each.  The sums are those of np_account's shuffle tree (every
+// addition has the same two operands), so the bits are too.  Each slot
+// belongs to one warp tile: it is read before the tile's arithmetic
+// (np_account_read), so its latency does not end the tile.  (The inflow and
 // outflow slots, touched by the few warps at the inlet and outlet, are read
-// at the end as before.)  The same sums and the same bits as np_account.
+// at the end.)
 template <int NS>
-__device__ __forceinline__ void np_account_read(float2 (&a)[NS], const float2 *acc, int wid,
-                                                int nw) {
-  if ((threadIdx.x & 31) != 0) return;
+__device__ __forceinline__ void np_account_read(float2 (&a)[(NS + 1) / 2], const float2 *acc,
+                                                int wid, int nw) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-  for (int k = 0; k < NS; k++) a[k] = acc[(size_t)(3 * k) * nw + wid];
+  for (int p = 0; p < (NS + 1) / 2; p++) {
+    const int k = 2 * p + (lane >> 4);
+    if ((lane & 15) == 0 && k < NS) a[p] = acc[(size_t)(3 * k) * nw + wid];
+  }
 }
+// v[p]: the lane's adsorbed fluxes of species (2p, 2p + 1).
 template <int NS>
-__device__ __forceinline__ void np_account_f32(float (&v)[3 * NS], bool io,
-                                               const float2 (&a)[NS], float2 *acc, int wid,
-                                               int nw) {
-  const bool any_io = __any_sync(0xffffffffu, io);
+__device__ __forceinline__ void np_account_f32(const float2 (&v)[(NS + 1) / 2],
+                                               const float2 (&a)[(NS + 1) / 2], float2 *acc,
+                                               int wid, int nw) {
+  const int lane = threadIdx.x & 31;
+  const bool hi = lane >= 16;
+#pragma unroll
+  for (int p = 0; p < (NS + 1) / 2; p++) {
+    const bool two = 2 * p + 1 < NS;
+    float own = v[p].x, other = v[p].x;
+    if (two) {
+      own = hi ? v[p].y : v[p].x;
+      other = hi ? v[p].x : v[p].y;
+    }
+    own = r_add(own, __shfl_xor_sync(0xffffffffu, other, 16));
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) own = r_add(own, __shfl_down_sync(0xffffffffu, own, o));
+    const int k = 2 * p + (hi ? 1 : 0);
+    if ((lane & 15) == 0 && k < NS) acc[(size_t)(3 * k) * nw + wid] = pair_add(a[p], own);
+  }
+}
+// The inflow (kind 1) and outflow (kind 2) sums of a warp with inlet or
+// outlet cells, as np_account forms them.
+template <int NS>
+__device__ __forceinline__ void np_account_io(float (&v)[2 * NS], float2 *acc, int wid, int nw) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-    for (int k = 0; k < NS; k++) v[k] = r_add(v[k], __shfl_down_sync(0xffffffffu, v[k], o));
-  if (any_io) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-      for (int k = NS; k < 3 * NS; k++)
-        v[k] = r_add(v[k], __shfl_down_sync(0xffffffffu, v[k], o));
-  }
-  if ((threadIdx.x & 31) == 0) {
+    for (int k = 0; k < 2 * NS; k++) v[k] = r_add(v[k], __shfl_down_sync(0xffffffffu, v[k], o));
+  if ((threadIdx.x & 31) == 0)
 #pragma unroll
     for (int k = 0; k < NS; k++) {
-      float2 *p = acc + (size_t)(3 * k) * nw + wid;
-      p[0] = pair_add(a[k], v[k]);
-      if (any_io) {
-        acc_add(p + nw, v[NS + k]);
-        acc_add(p + 2 * (size_t)nw, v[2 * NS + k]);
-      }
+      acc_add(acc + (size_t)(3 * k + 1) * nw + wid, v[k]);
+      acc_add(acc + (size_t)(3 * k + 2) * nw + wid, v[NS + k]);
     }
-  }
 }
 
 // Two species per packed FP32x2 operation (each component rounded exactly as
@@ -416,40 +421,89 @@ __device__ __forceinline__ float2 psub(float2 a, float2 b) { return __fadd2_rn(a
 __device__ __forceinline__ float2 pmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 pfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
-// Flux through one face for a pair of species (k0, k1): the same arithmetic,
-// species by species, as face_flux followed by the D/dx factor.  An odd
-// species count pads its last pair with a copy of the last species (k1 = k0).
-// Scalar flux of one species with pair-stored concentrations C + Cl: the
-// difference C_P - C_nb and the two Bernoulli products take the low words
-// along; everything else is face_flux.
-__device__ __forceinline__ float face_flux_lo(float adv, float z, float dd, float2 nb, float2 pp,
-                                              float CP, float Cn, float CPl, float Cnl) {
-  const float p = __fmaf_rn(-z, dd, adv);
+// Second species of pair p (a copy of the first when NS is odd).
+template <int NS> __device__ __forceinline__ constexpr int np_k1(int p) {
+  return 2 * p + 1 < NS ? 2 * p + 1 : 2 * p;
+}
+
+// The concentration record of rank r in a species-pair plane (two != 0: both
+// species of the pair; else a lone last species, copied into both halves).
+template <bool PAIR>
+__device__ __forceinline__ void rec_load(const float *__restrict__ base, bool two, int r,
+                                         float2 &c, float2 &l) {
+  if (PAIR && two) {
+    const float4 v = __ldg(reinterpret_cast<const float4 *>(base) + r);
+    c = make_float2(v.x, v.y);
+    l = make_float2(v.z, v.w);
+  } else if (two) {
+    c = __ldg(reinterpret_cast<const float2 *>(base) + r);
+    l = make_float2(0.f, 0.f);
+  } else if (PAIR) {
+    const float2 v = __ldg(reinterpret_cast<const float2 *>(base) + r);
+    c = bc(v.x);
+    l = bc(v.y);
+  } else {
+    c = bc(__ldg(base + r));
+    l = make_float2(0.f, 0.f);
+  }
+}
+template <bool PAIR>
+__device__ __forceinline__ void rec_store(float *__restrict__ base, bool two, int r, float2 c,
+                                          float2 l) {
+  if (PAIR && two)
+    reinterpret_cast<float4 *>(base)[r] = make_float4(c.x, c.y, l.x, l.y);
+  else if (two)
+    reinterpret_cast<float2 *>(base)[r] = c;
+  else if (PAIR)
+    reinterpret_cast<float2 *>(base)[r] = make_float2(c.x, l.x);
+  else
+    base[r] = c.x;
+}
+
+// Scalar flux of one species (pair-stored concentrations C + Cl with PAIR):
+// the two branches above, the Bernoulli pair supplied by bern(Bp, Bm) where |P| >= 1/2;
+// with PAIR the difference C_P - C_nb and the two products take the low words
+// along.
+template <bool PAIR, typename BF>
+__device__ __forceinline__ float face_flux_one(float p, BF bern, float CP, float Cn, float CPl,
+                                               float Cnl) {
   if (fabsf(p) < 0.5f) {
     const float p2 = __fmul_rn(p, p);
     float E = __fmaf_rn(p2, 1.f / 30240.f, -1.f / 720.f);
     E = __fmaf_rn(E, p2, 1.f / 12.f);
     E = __fmaf_rn(E, p2, 1.f);
-    const float dC = __fadd_rn(__fsub_rn(CP, Cn), __fsub_rn(CPl, Cnl));
+    float dC = __fsub_rn(CP, Cn);
+    if (PAIR) dC = __fadd_rn(dC, __fsub_rn(CPl, Cnl));
     return __fmaf_rn(E, dC, __fmul_rn(__fmul_rn(0.5f, p), __fadd_rn(CP, Cn)));
   }
   float Bp, Bm;
-  bernoulli_pair_split(adv, z, nb, pp, Bp, Bm);
-  return __fadd_rn(r_fma(Bm, CP, -r_mul(Bp, Cn)), r_fma(Bm, CPl, -r_mul(Bp, Cnl)));
+  bern(Bp, Bm);
+  const float J = r_fma(Bm, CP, -r_mul(Bp, Cn));
+  return PAIR ? __fadd_rn(J, r_fma(Bm, CPl, -r_mul(Bp, Cnl))) : J;
 }
 
-// Flux through one face for a pair of species (k0, k1): the same arithmetic,
-// species by species, as face_flux (face_flux_lo with PAIR) followed by the
-// D/dx factor.  An odd species count pads its last pair with a copy of the
-// last species (k1 = k0).
-template <bool PAIR>
-__device__ __forceinline__ float2 face_flux_pair(float uf, float dd, float2 phn, float2 phP,
-                                                 float2 CP, float2 Cn, float2 CPl, float2 Cnl,
-                                                 const NPConst<float> &c, int k0, int k1) {
-  const float2 adv = pmul(bc(uf), make_float2(c.dxD[k0], c.dxD[k1]));
-  const float2 p = pfma(make_float2(-c.zf[k0], -c.zf[k1]), bc(dd), adv);
+// Face Peclet numbers of a pair of species (k0, k1) from the face's velocity
+// and potential difference seen from the cell.
+__device__ __forceinline__ float2 face_peclet(float uf, float dd, const NPConst<float> &c, int k0,
+                                              int k1) {
+  return make_float2(__fmaf_rn(-c.zf[k0], dd, __fmul_rn(uf, c.dxD[k0])),
+                     __fmaf_rn(-c.zf[k1], dd, __fmul_rn(uf, c.dxD[k1])));
+}
+__device__ __forceinline__ bool big(float2 p) { return !(fabsf(p.x) < 0.5f && fabsf(p.y) < 0.5f); }
+
+// Flux through one face for a pair of species (k0, k1), times D/dx: for
+// |P| < 1/2 both species at once in packed arithmetic, otherwise species by
+// species (the same operations, each rounded the same way).  p: the face
+// Peclet numbers; bern(k, Bp, Bm) supplies species k's Bernoulli pair and is
+// asked only where |P| >= 1/2 (never with SMALL, whose caller knows that
+// |P| < 1/2 for both).  An odd species count pads its last pair with a copy
+// of the last species (k1 = k0).
+template <bool PAIR, bool SMALL, typename BF>
+__device__ __forceinline__ float2 face_flux_pair(float2 p, BF bern, float2 CP, float2 Cn,
+                                                 float2 CPl, float2 Cnl, const NPConst<float> &c,
+                                                 int k0, int k1) {
   float2 J;
-  if (fabsf(p.x) < 0.5f && fabsf(p.y) < 0.5f) {
+  if (SMALL || !big(p)) {
     const float2 p2 = pmul(p, p);
     float2 E = pfma(p2, bc(1.f / 30240.f), bc(-1.f / 720.f));
     E = pfma(E, p2, bc(1.f / 12.f));
@@ -457,12 +511,11 @@ __device__ __forceinline__ float2 face_flux_pair(float uf, float dd, float2 phn,
     float2 dC = psub(CP, Cn);
     if (PAIR) dC = padd(dC, psub(CPl, Cnl));
     J = pfma(E, dC, pmul(pmul(bc(0.5f), p), padd(CP, Cn)));
-  } else if (PAIR) {
-    J.x = face_flux_lo(adv.x, c.zf[k0], dd, phn, phP, CP.x, Cn.x, CPl.x, Cnl.x);
-    J.y = face_flux_lo(adv.y, c.zf[k1], dd, phn, phP, CP.y, Cn.y, CPl.y, Cnl.y);
   } else {
-    J.x = face_flux(adv.x, c.zf[k0], dd, phn, phP, CP.x, Cn.x);
-    J.y = face_flux(adv.y, c.zf[k1], dd, phn, phP, CP.y, Cn.y);
+    auto b0 = [&](float &Bp, float &Bm) { bern(k0, Bp, Bm); };
+    auto b1 = [&](float &Bp, float &Bm) { bern(k1, Bp, Bm); };
+    J.x = face_flux_one<PAIR>(p.x, b0, CP.x, Cn.x, CPl.x, Cnl.x);
+    J.y = face_flux_one<PAIR>(p.y, b1, CP.y, Cn.y, CPl.y, Cnl.y);
   }
   return pmul(make_float2(c.Ddx[k0], c.Ddx[k1]), J);
 }
@@ -474,18 +527,10 @@ __device__ __forceinline__ void ptwo_sum(float2 a, float2 b, float2 &s, float2 &
   e = padd(psub(a, psub(s, bp)), psub(b, bp));
 }
 
-// One explicit step of the home cells of warp w (FP32, NS species in
-// (NS + 1) / 2 packed pairs), with the per-warp accounts of Gamma, In and
-// Out.  PAIR: every concentration is an unevaluated pair hi + lo (the low
-// words in Cinl/Coutl), updated with the two-sum transformation, so rounding
-// does not build up over long runs; the fluxes take the low words into the
-// concentration differences.  All 32 lanes of the warp must call it.  Per
-// home cell the faces are summed in the order of np_cell (adsorption, +x,
-// -x, +y, -y, +z, -z), so without PAIR a cell whose faces all take the
-// |P| < 1/2 branch gets the bits np_cell gives.
-// The per-lane link data of warp w's tile: the lane's face flags and its
-// lateral neighbour ranks (-1 across a solid face or wall, or for the halo
-// lane).
+// The per-lane link data of warp w's tile: the lane's face flags (a lane
+// without a cell has a closed +x face) and its lateral neighbour ranks (-1
+// across a solid face or wall, or for the halo lane), decoded from the 16-bit
+// differences to the tile's bases.
 template <int DIM> struct NPLinks {
   unsigned f;
   int q[2 * DIM - 2];
@@ -497,277 +542,364 @@ __device__ __forceinline__ NPLinks<DIM> np_links(const NPFields &F, int n_cells,
   const bool valid = r >= 0 && r < n_cells;
   const bool home = valid && lane != 0;
   NPLinks<DIM> L;
-  L.f = valid ? (unsigned)F.fl[r] : 0u;
+  L.f = valid ? (unsigned)F.fl[r] : 1u << kFaceBit;
+  int base[2 * DIM - 2], d[2 * DIM - 2];
+  bool wide = false;
+  if constexpr (DIM == 3) {
+    const int4 b = reinterpret_cast<const int4 *>(F.latb)[w];
+    short4 v = make_short4(kLatClosed, kLatClosed, kLatClosed, kLatClosed);
+    if (home) v = reinterpret_cast<const short4 *>(F.latd)[r];
+    base[0] = b.x; base[1] = b.y; base[2] = b.z; base[3] = b.w;
+    d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
+  } else {
+    const int2 b = reinterpret_cast<const int2 *>(F.latb)[w];
+    short2 v = make_short2(kLatClosed, kLatClosed);
+    if (home) v = reinterpret_cast<const short2 *>(F.latd)[r];
+    base[0] = b.x; base[1] = b.y;
+    d[0] = v.x; d[1] = v.y;
+  }
 #pragma unroll
-  for (int j = 0; j < 2 * DIM - 2; j++) L.q[j] = home ? F.lat[j][r] : -1;
+  for (int j = 0; j < 2 * DIM - 2; j++) {
+    L.q[j] = d[j] == kLatClosed ? -1 : r + base[j] + d[j];
+    wide |= d[j] == kLatWide;
+  }
+  if (wide) {
+#pragma unroll
+    for (int j = 0; j < 2 * DIM - 2; j++) L.q[j] = F.lat[(size_t)j * n_cells + r];
+  }
   return L;
 }
 
-template <int DIM, int NS, bool PAIR>
-__device__ __forceinline__ void np_warp31(const NPFields &F, int n_cells, int naccs,
-                                          const NPConst<float> &c, int w) {
-  np_warp31<DIM, NS, PAIR>(F, n_cells, naccs, c, w, np_links<DIM>(F, n_cells, w));
-}
-
-// The values one lane of a warp tile works from: its cell's own fields, its
-// lateral neighbours' (the cell's own values across a closed face) and its +x
-// neighbour's (replaced by the cell's own unless that face is open and inside
-// the image).
+// What a lane works from: its cell's record, the records across its +x and
+// lateral faces (its own again across a closed face) and the face data seen
+// from the cell (0 across a closed face).
 template <int DIM, int NS> struct NPLane {
   static constexpr int NP = (NS + 1) / 2, NL = 2 * DIM - 2;
-  float2 CP[NP], CPl[NP], phP;
-  float uP[DIM];
-  float2 Cl[NL][NP], Cll[NL][NP], phl[NL];
-  float ul[NL];
-  float2 Cx[NP], Cxl[NP], phx;
-  float ux;
+  float2 C[NP], Cl[NP];
+  float2 Cx[NP], Cxl[NP], fx;
+  float2 Cn[NL][NP], Cnl[NL][NP], fn[NL];
 };
 
-// Second species of pair p (a copy of the first when NS is odd).
-template <int NS> __device__ __forceinline__ constexpr int np_k1(int p) {
-  return 2 * p + 1 < NS ? 2 * p + 1 : 2 * p;
-}
-
-// Lateral neighbours' values, read from the field arrays (own values are
-// already in V).
-template <int DIM, int NS, bool PAIR>
-__device__ __forceinline__ void np_load_lateral(const NPFields &F, const int *q,
-                                                NPLane<DIM, NS> &V) {
-  constexpr int NP = (NS + 1) / 2;
-#pragma unroll
-  for (int j = 0; j < 2 * DIM - 2; j++) {
-    const int fc = j + 2;
-    if (q[j] >= 0) {
-      const int Q = q[j];
-      V.ul[j] = F.u[fc >> 1][Q];
-      V.phl[j] = F.phi[Q];
-#pragma unroll
-      for (int p = 0; p < NP; p++) {
-        V.Cl[j][p] = make_float2(F.C[2 * p][Q], F.C[np_k1<NS>(p)][Q]);
-        V.Cll[j][p] = PAIR ? make_float2(F.Cl[2 * p][Q], F.Cl[np_k1<NS>(p)][Q])
-                           : make_float2(0.f, 0.f);
-      }
-    } else {
-      V.ul[j] = V.uP[fc >> 1];
-      V.phl[j] = V.phP;
-#pragma unroll
-      for (int p = 0; p < NP; p++) {
-        V.Cl[j][p] = V.CP[p];
-        V.Cll[j][p] = V.CPl[p];
-      }
-    }
-  }
-}
-
-// Own, lateral and +x values of warp w's tile, read from the field arrays:
-// the +x neighbour is the next lane's cell (np_finish_x, a shuffle), or for
-// lane 31 the next tile's first home cell (loaded here).
-template <int DIM, int NS, bool PAIR>
-__device__ __forceinline__ void np_issue_loads(const NPFields &F, int n_cells, int w,
-                                               unsigned f, const int *q, NPLane<DIM, NS> &V) {
-  constexpr int NP = (NS + 1) / 2;
-  const int lane = threadIdx.x & 31;
-  const int r = kHome * w + lane - 1;
-  const bool valid = r >= 0 && r < n_cells;
-  auto ldC = [&](const float *const *A, int Q, int p) {
-    return make_float2(A[2 * p][Q], A[np_k1<NS>(p)][Q]);
-  };
+// The update of warp w's tile from the values in V.  The +x face flux is
+// evaluated once per face and handed to the next lane as its -x flux; per
+// home cell the faces are summed in the order of np_cell (adsorption, +x, -x,
+// +y, -y, +z, -z).  SMALL: every face of the warp has |P| < 1/2, so the
+// arithmetic has no branch and its faces overlap.  EVAL: the Bernoulli pairs are not stored (no memory for
+// them) and are evaluated at every step.
+template <int DIM, int NS, bool PAIR, bool SMALL, bool EVAL>
+__device__ __forceinline__ void np_update(const NPFields &F, int n_cells, int naccs,
+                                          const NPConst<float> &c, int w, int r, bool home,
+                                          const NPLinks<DIM> &lk, const NPLane<DIM, NS> &V,
+                                          const float2 (&acc_pre)[(NS + 1) / 2]) {
+  constexpr int NF = 2 * DIM, NL = NF - 2, NP = (NS + 1) / 2;
+  const unsigned f = lk.f;
   const float2 z2 = make_float2(0.f, 0.f);
-#pragma unroll
-  for (int p = 0; p < NP; p++) V.CP[p] = V.CPl[p] = z2;
-#pragma unroll
-  for (int a = 0; a < DIM; a++) V.uP[a] = 0.f;
-  V.phP = z2;
-  if (valid) {
-#pragma unroll
-    for (int p = 0; p < NP; p++) {
-      V.CP[p] = ldC(F.C, r, p);
-      if (PAIR) V.CPl[p] = ldC(F.Cl, r, p);
+  const int rc = min(max(r, 0), n_cells - 1);
+  const bool xs = (f >> kFaceBit) & 1u, xe = (f >> kEdgeBit) & 1u;
+  const bool ms = (f >> (kFaceBit + 1)) & 1u, me = (f >> (kEdgeBit + 1)) & 1u;
+  float2 Jx[NP], Jm[NP];
+  // The Bernoulli pair of species k at + face a of rank own, or (flip) at the
+  // - face of the cell across it: the stored pair, with its two members
+  // exchanged there, or evaluated from the two potentials.
+  auto stored = [&](int a, int own, bool flip, float uf, float dd, int nb, int k, float &Bp,
+                    float &Bm) {
+    if (!EVAL) {
+      const float2 b = F.bern[((size_t)a * n_cells + own) * NS + k];
+      Bp = flip ? b.y : b.x;
+      Bm = flip ? b.x : b.y;
+    } else {
+      bernoulli_pair_split(__fmul_rn(uf, c.dxD[k]), c.zf[k], F.phi[nb], F.phi[rc], Bp, Bm);
     }
-#pragma unroll
-    for (int a = 0; a < DIM; a++) V.uP[a] = F.u[a][r];
-    V.phP = F.phi[r];
-  }
-  np_load_lateral<DIM, NS, PAIR>(F, q, V);
-  const bool xp = valid && !((f >> kFaceBit) & 1u) && !((f >> kEdgeBit) & 1u);
-  V.ux = 0.f;
-  V.phx = z2;
-#pragma unroll
-  for (int p = 0; p < NP; p++) V.Cx[p] = V.Cxl[p] = z2;
-  if (lane == 31 && xp) {  // rank r + 1 is the next warp's first home cell
-    V.ux = F.u[0][r + 1];
-    V.phx = F.phi[r + 1];
-#pragma unroll
-    for (int p = 0; p < NP; p++) {
-      V.Cx[p] = ldC(F.C, r + 1, p);
-      if (PAIR) V.Cxl[p] = ldC(F.Cl, r + 1, p);
-    }
-  }
-}
-
-// The +x neighbour's values of lanes 0-30: the next lane's own values.
-template <int DIM, int NS, bool PAIR>
-__device__ __forceinline__ void np_finish_x(NPLane<DIM, NS> &V) {
-  constexpr int NP = (NS + 1) / 2;
-  const bool take = (threadIdx.x & 31) != 31;
-  auto sh = [&](float v, float &dst) {
-    const float t = __shfl_down_sync(0xffffffffu, v, 1);
-    if (take) dst = t;
   };
-  sh(V.uP[0], V.ux);
-  sh(V.phP.x, V.phx.x);
-  sh(V.phP.y, V.phx.y);
 #pragma unroll
   for (int p = 0; p < NP; p++) {
-    sh(V.CP[p].x, V.Cx[p].x);
-    sh(V.CP[p].y, V.Cx[p].y);
-    if (PAIR) {
-      sh(V.CPl[p].x, V.Cxl[p].x);
-      sh(V.CPl[p].y, V.Cxl[p].y);
-    }
-  }
-}
-
-template <int DIM, int NS, bool PAIR>
-__device__ __forceinline__ void np_load_global(const NPFields &F, int n_cells, int w,
-                                               unsigned f, const int *q, NPLane<DIM, NS> &V) {
-  np_issue_loads<DIM, NS, PAIR>(F, n_cells, w, f, q, V);
-  np_finish_x<DIM, NS, PAIR>(V);
-}
-
-// The update of warp w's tile from the values in V: the +x face flux is
-// evaluated once per face and handed to the next lane as its -x flux; then
-// adsorption, the x faces and the lateral faces are summed in that order and
-// the new concentrations and the warp's accounts written.
-template <int DIM, int NS, bool PAIR>
-__device__ __forceinline__ void np_tile_update(const NPFields &F, int n_cells, int naccs,
-                                               const NPConst<float> &c, int w, unsigned f,
-                                               const int *q, NPLane<DIM, NS> &V) {
-  constexpr int NF = 2 * DIM;
-  constexpr int NP = (NS + 1) / 2;
-  const int lane = threadIdx.x & 31;
-  const int r = kHome * w + lane - 1;
-  const bool valid = r >= 0 && r < n_cells;
-  const bool home = valid && lane != 0;
-  const float2 z2 = make_float2(0.f, 0.f);
-  // the warp's adsorption account slots, read before the arithmetic
-  float2 acc_pre[NS];
-  np_account_read<NS>(acc_pre, F.acc, w, naccs);
-  // +x face: open and inside the image, else the outlet ghost copies the cell
-  const bool xs = (f >> kFaceBit) & 1u, xe = (f >> kEdgeBit) & 1u;
-  const bool xp = valid && !xs && !xe;
-  if (!xp) {
-    V.ux = V.uP[0];
-    V.phx = V.phP;
-#pragma unroll
-    for (int p = 0; p < NP; p++) {
-      V.Cx[p] = V.CP[p];
-      V.Cxl[p] = V.CPl[p];
-    }
-  }
-  float2 Jx[NP];
-  {
-    const float uf = (valid && !xs) ? r_mul(0.5f, r_add(V.uP[0], V.ux)) : 0.f;
-    const float dd = phi_diff(V.phx, V.phP);
-#pragma unroll
-    for (int p = 0; p < NP; p++)
-      Jx[p] = face_flux_pair<PAIR>(uf, dd, V.phx, V.phP, V.CP[p], V.Cx[p], V.CPl[p], V.Cxl[p], c,
-                                   2 * p, np_k1<NS>(p));
+    auto bern = [&](int k, float &Bp, float &Bm) {
+      stored(0, rc, false, V.fx.x, V.fx.y, xs || xe ? rc : rc + 1, k, Bp, Bm);
+    };
+    Jx[p] = face_flux_pair<PAIR, SMALL>(face_peclet(V.fx.x, V.fx.y, c, 2 * p, np_k1<NS>(p)), bern,
+                                        V.C[p], V.Cx[p], V.Cl[p], V.Cxl[p], c, 2 * p,
+                                        np_k1<NS>(p));
   }
   // -x face: the previous lane's +x face (pore neighbour), the feed ghost
   // (inlet), or closed (solid)
-  const bool ms = (f >> (kFaceBit + 1)) & 1u, me = (f >> (kEdgeBit + 1)) & 1u;
-  float2 Jm[NP];
 #pragma unroll
   for (int p = 0; p < NP; p++) {
     Jm[p].x = -__shfl_up_sync(0xffffffffu, Jx[p].x, 1);
-    Jm[p].y = -__shfl_up_sync(0xffffffffu, Jx[p].y, 1);
+    Jm[p].y = 2 * p + 1 < NS ? -__shfl_up_sync(0xffffffffu, Jx[p].y, 1) : Jm[p].x;
     if (ms) Jm[p] = z2;
   }
   if (home && me) {
-    const float uf = r_mul(-0.5f, r_add(V.uP[0], V.uP[0]));
-    const float dd = phi_diff(z2, V.phP);
+    const float uP = F.ux[r];
+    const float2 phP = F.phi[r];
+    const float uf = r_mul(-0.5f, r_add(uP, uP));
+    const float dd = phi_diff(z2, phP);
+    auto bern = [&](int k, float &Bp, float &Bm) {
+      if (!EVAL) {  // the feed faces' pairs stand behind those of the + faces
+        const float2 b = F.bern[((size_t)DIM * n_cells + r) * NS + k];
+        Bp = b.x;
+        Bm = b.y;
+      } else {
+        bernoulli_pair_split(__fmul_rn(uf, c.dxD[k]), c.zf[k], z2, phP, Bp, Bm);
+      }
+    };
 #pragma unroll
     for (int p = 0; p < NP; p++)
-      Jm[p] = face_flux_pair<PAIR>(uf, dd, z2, V.phP, V.CP[p], bc(c.c0), V.CPl[p], bc(c.c0lo), c,
-                                   2 * p, np_k1<NS>(p));
+      Jm[p] = face_flux_pair<PAIR, SMALL>(face_peclet(uf, dd, c, 2 * p, np_k1<NS>(p)), bern, V.C[p],
+                                          bc(c.c0), V.Cl[p], bc(c.c0lo), c, 2 * p,
+                                          np_k1<NS>(p));
   }
   // adsorption on the solid faces (Eq. 6), then the faces in order
-  float v[3 * NS];
-#pragma unroll
-  for (int j = 0; j < 3 * NS; j++) v[j] = 0.f;
+  float2 Ja[NP], sumJ[NP];
   const float ns_solid = (float)__popc(f & (((1u << NF) - 1u) << kFaceBit));
-  float2 sumJ[NP];
 #pragma unroll
   for (int p = 0; p < NP; p++) {
-    const float2 Ja =
-        pmul(pmul(bc(ns_solid), make_float2(c.Keff[2 * p], c.Keff[np_k1<NS>(p)])), V.CP[p]);
-    sumJ[p] = padd(padd(Ja, Jx[p]), Jm[p]);
-    if (home) {
-      v[2 * p] = r_add(0.f, Ja.x);
-      if (2 * p + 1 < NS) v[2 * p + 1] = r_add(0.f, Ja.y);
-      if (me) {
-        v[NS + 2 * p] = r_sub(0.f, Jm[p].x);
-        if (2 * p + 1 < NS) v[NS + 2 * p + 1] = r_sub(0.f, Jm[p].y);
-      }
-      if (xe) {
-        v[2 * NS + 2 * p] = r_add(0.f, Jx[p].x);
-        if (2 * p + 1 < NS) v[2 * NS + 2 * p + 1] = r_add(0.f, Jx[p].y);
-      }
-    }
+    Ja[p] = pmul(pmul(bc(ns_solid), make_float2(c.Keff[2 * p], c.Keff[np_k1<NS>(p)])), V.C[p]);
+    sumJ[p] = padd(padd(Ja[p], Jx[p]), Jm[p]);
   }
 #pragma unroll
-  for (int j = 0; j < NF - 2; j++) {
-    const int fc = j + 2;
-    const float half = (fc & 1) ? -0.5f : 0.5f;
-    const float uf = q[j] >= 0 ? r_mul(half, r_add(V.uP[fc >> 1], V.ul[j])) : 0.f;
-    const float dd = phi_diff(V.phl[j], V.phP);
+  for (int j = 0; j < NL; j++) {
+    const int q = lk.q[j] >= 0 ? lk.q[j] : rc;
+    auto bern = [&](int k, float &Bp, float &Bm) {
+      stored(1 + j / 2, (j & 1) ? q : rc, j & 1, V.fn[j].x, V.fn[j].y, q, k, Bp, Bm);
+    };
 #pragma unroll
     for (int p = 0; p < NP; p++)
-      sumJ[p] = padd(sumJ[p], face_flux_pair<PAIR>(uf, dd, V.phl[j], V.phP, V.CP[p], V.Cl[j][p],
-                                                   V.CPl[p], V.Cll[j][p], c, 2 * p,
-                                                   np_k1<NS>(p)));
+      sumJ[p] = padd(sumJ[p], face_flux_pair<PAIR, SMALL>(
+                                  face_peclet(V.fn[j].x, V.fn[j].y, c, 2 * p, np_k1<NS>(p)), bern,
+                                  V.C[p], V.Cn[j][p], V.Cl[p], V.Cnl[j][p], c, 2 * p,
+                                  np_k1<NS>(p)));
   }
   if (home) {
 #pragma unroll
     for (int p = 0; p < NP; p++) {
-      float2 Cn, Cnl;
+      float2 Cn, Cnl = z2;
       if (PAIR) {
         // (hi + lo) - dt/dx sum J by two-sum, renormalised
         float2 t, e;
-        ptwo_sum(V.CP[p], pmul(bc(-c.dtdx), sumJ[p]), t, e);
-        const float2 l = padd(V.CPl[p], e);
+        ptwo_sum(V.C[p], pmul(bc(-c.dtdx), sumJ[p]), t, e);
+        const float2 l = padd(V.Cl[p], e);
         Cn = padd(t, l);
         Cnl = psub(l, psub(Cn, t));
-        F.Col[2 * p][r] = Cnl.x;
-        if (2 * p + 1 < NS) F.Col[2 * p + 1][r] = Cnl.y;
       } else {
-        Cn = pfma(bc(-c.dtdx), sumJ[p], V.CP[p]);
+        Cn = pfma(bc(-c.dtdx), sumJ[p], V.C[p]);
       }
-      F.Co[2 * p][r] = Cn.x;
-      if (2 * p + 1 < NS) F.Co[2 * p + 1][r] = Cn.y;
+      rec_store<PAIR>(F.Co[p], 2 * p + 1 < NS, r, Cn, Cnl);
     }
   }
-  np_account_f32<NS>(v, home && (me || xe), acc_pre, F.acc, w, naccs);
+  if (!home) {
+#pragma unroll
+    for (int p = 0; p < NP; p++) Ja[p] = z2;
+  }
+  np_account_f32<NS>(Ja, acc_pre, F.acc, w, naccs);
+  if (__any_sync(0xffffffffu, home && (me || xe))) {
+    float v[2 * NS];
+#pragma unroll
+    for (int k = 0; k < NS; k++) {
+      v[k] = home && me ? r_sub(0.f, (k & 1) ? Jm[k / 2].y : Jm[k / 2].x) : 0.f;
+      v[NS + k] = home && xe ? r_add(0.f, (k & 1) ? Jx[k / 2].y : Jx[k / 2].x) : 0.f;
+    }
+    np_account_io<NS>(v, F.acc, w, naccs);
+  }
 }
 
+// Every load of warp w's tile.  All are unconditional: a closed face reads the
+// cell's own record, which costs an L1 hit instead of a branch and moves.
 template <int DIM, int NS, bool PAIR>
-__device__ __forceinline__ void np_warp31(const NPFields &F, int n_cells, int naccs,
-                                          const NPConst<float> &c, int w,
-                                          const NPLinks<DIM> &lk) {
-  NPLane<DIM, NS> V;
-  np_load_global<DIM, NS, PAIR>(F, n_cells, w, lk.f, lk.q, V);
-  np_tile_update<DIM, NS, PAIR>(F, n_cells, naccs, c, w, lk.f, lk.q, V);
+__device__ __forceinline__ void np_load(const NPFields &F, int n_cells, int naccs, int w, int r,
+                                        const NPLinks<DIM> &lk, NPLane<DIM, NS> &V,
+                                        float2 (&acc_pre)[(NS + 1) / 2]) {
+  constexpr int NL = 2 * DIM - 2, NP = (NS + 1) / 2;
+  const int rc = min(max(r, 0), n_cells - 1);
+  np_account_read<NS>(acc_pre, F.acc, w, naccs);
+  const bool xp = !(((lk.f >> kFaceBit) | (lk.f >> kEdgeBit)) & 1u);
+#pragma unroll
+  for (int p = 0; p < NP; p++) {
+    rec_load<PAIR>(F.C[p], 2 * p + 1 < NS, rc, V.C[p], V.Cl[p]);
+    rec_load<PAIR>(F.C[p], 2 * p + 1 < NS, xp ? rc + 1 : rc, V.Cx[p], V.Cxl[p]);
+  }
+  V.fx = __ldg(F.fd[0] + rc);
+#pragma unroll
+  for (int j = 0; j < NL; j++) {
+    const int q = lk.q[j] >= 0 ? lk.q[j] : rc;
+#pragma unroll
+    for (int p = 0; p < NP; p++)
+      rec_load<PAIR>(F.C[p], 2 * p + 1 < NS, q, V.Cn[j][p], V.Cnl[j][p]);
+    V.fn[j] = __ldg(F.fd[1 + j / 2] + ((j & 1) ? q : rc));
+  }
+#pragma unroll
+  for (int j = 1; j < NL; j += 2) {
+    // a - face is the + face of the neighbour across it, seen from the other
+    // side: velocity and potential difference change sign exactly (and are 0
+    // where it is closed)
+    const float s = lk.q[j] >= 0 ? -1.f : 0.f;
+    V.fn[j] = make_float2(__fmul_rn(s, V.fn[j].x), __fmul_rn(s, V.fn[j].y));
+  }
 }
 
-template <typename T, int DIM, int NS, bool PAIR>
+// One explicit step of the home cells of warp w (FP32, NS species in
+// (NS + 1) / 2 packed pairs), with the per-warp accounts of Gamma, In and
+// Out.  PAIR: every concentration is an unevaluated pair hi + lo, updated
+// with the two-sum transformation, so rounding does not build up over long
+// runs; the fluxes take the low words into the concentration differences.
+// All 32 lanes of the warp must call it.
+//
+// What bounds it is latency: a memory round trip for the link data, one for
+// the gathers, and the arithmetic's own chain.  So every load is issued
+// before any arithmetic, and the arithmetic of a launch whose faces all have
+// |P| < 1/2 (NP_SMALL; known when the face data is formed) has no branch: a
+// branch per face puts the faces' chains one after the other (172 instead of
+// 139 us a step on a 256^3 pack), and even one vote per warp between the two
+// costs the common one (150 to 172 us: the second path's registers).
+// Otherwise (NP_LARGE) a vote per warp chooses; NP_EVAL is NP_LARGE without
+// stored Bernoulli pairs.
+enum { NP_SMALL = 0, NP_LARGE = 1, NP_EVAL = 2 };
+template <int DIM, int NS, bool PAIR, int MODE>
+__device__ __forceinline__ void np_warp31(const NPFields &F, int n_cells, int naccs,
+                                          const NPConst<float> &c, int w) {
+  constexpr int NL = 2 * DIM - 2, NP = (NS + 1) / 2;
+  constexpr bool EVAL = MODE == NP_EVAL;
+  if (w >= (int)np_warps(n_cells)) return;  // whole warps
+  const int r = kHome * w + (int)(threadIdx.x & 31) - 1;
+  const bool valid = r >= 0 && r < n_cells, home = valid && (threadIdx.x & 31) != 0;
+  const NPLinks<DIM> lk = np_links<DIM>(F, n_cells, w);
+  NPLane<DIM, NS> V;
+  float2 acc_pre[NP];
+  np_load<DIM, NS, PAIR>(F, n_cells, naccs, w, r, lk, V, acc_pre);
+  if (MODE != NP_SMALL) {
+    bool large = false;
+#pragma unroll
+    for (int p = 0; p < NP; p++) {
+      large |= big(face_peclet(V.fx.x, V.fx.y, c, 2 * p, np_k1<NS>(p)));
+#pragma unroll
+      for (int j = 0; j < NL; j++)
+        large |= big(face_peclet(V.fn[j].x, V.fn[j].y, c, 2 * p, np_k1<NS>(p)));
+    }
+    if (valid && ((lk.f >> (kEdgeBit + 1)) & 1u)) {  // the feed face
+      const float uP = F.ux[r], uf = r_mul(-0.5f, r_add(uP, uP));
+      const float dd = phi_diff(make_float2(0.f, 0.f), F.phi[r]);
+#pragma unroll
+      for (int p = 0; p < NP; p++) large |= big(face_peclet(uf, dd, c, 2 * p, np_k1<NS>(p)));
+    }
+    if (__any_sync(0xffffffffu, large)) {
+      np_update<DIM, NS, PAIR, false, EVAL>(F, n_cells, naccs, c, w, r, home, lk, V, acc_pre);
+      return;
+    }
+  }
+  np_update<DIM, NS, PAIR, true, EVAL>(F, n_cells, naccs, c, w, r, home, lk, V, acc_pre);
+}
+
+// Rank across + face a of rank r (its own at the outlet), or -1 where closed.
+__device__ __forceinline__ int plus_face(unsigned f, const int *__restrict__ lat, int n, int a,
+                                         int r) {
+  if (a > 0) return lat[(size_t)(2 * a - 2) * n + r];
+  return (f >> kFaceBit) & 1u ? -1 : ((f >> kEdgeBit) & 1u ? r : r + 1);
+}
+
+// The face data of every + face, from the velocity and the potential: half
+// the sum of the two cells' velocity components (the cell's own twice at the
+// outlet) and the potential difference of the two (hi, lo) pairs, rounded
+// once each; 0 across a closed face.  The step reads these 8 bytes instead
+// of both cells' velocity and potential pair (12 bytes and three gathered
+// loads per lateral face) and skips the arithmetic on them; they stay the
+// same until the velocity or the potential changes.
+// *any_large is set to 1 when a face has |P| >= 1/2 for some species.
+template <int DIM>
+__global__ void k_np_faces(const NFlag *__restrict__ fl, const int *__restrict__ lat, int n,
+                           const float *__restrict__ u, const float2 *__restrict__ phi,
+                           NPConst<float> c, int ns, float2 *__restrict__ fd,
+                           int *__restrict__ any_large) {
+  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
+    const unsigned f = fl[r];
+    const float2 phP = phi[r];
+    bool large = false;
+    auto test = [&](float uf, float dd) {
+      for (int k = 0; k < ns; k++)
+        if (!(fabsf(__fmaf_rn(-c.zf[k], dd, __fmul_rn(uf, c.dxD[k]))) < 0.5f)) large = true;
+    };
+#pragma unroll
+    for (int a = 0; a < DIM; a++) {
+      const float uP = u[(size_t)a * n + r];
+      const int q = plus_face(f, lat, n, a, r);
+      float2 v = make_float2(0.f, 0.f);
+      if (q >= 0) {
+        v = make_float2(r_mul(0.5f, r_add(uP, u[(size_t)a * n + q])), phi_diff(phi[q], phP));
+        test(v.x, v.y);
+      }
+      fd[(size_t)a * n + r] = v;
+    }
+    if ((f >> (kEdgeBit + 1)) & 1u)
+      test(r_mul(-0.5f, r_add(u[r], u[r])), phi_diff(make_float2(0.f, 0.f), phP));
+    if (large) *any_large = 1;
+  }
+}
+
+// The Bernoulli pairs of the + faces and feed faces with |P| >= 1/2 (the
+// others' places are not read): the step's exponentials and divisions, done
+// once per velocity and potential instead of at every step.
+template <int DIM>
+__global__ void k_np_bern(const NFlag *__restrict__ fl, const int *__restrict__ lat, int n,
+                          const float *__restrict__ ux, const float2 *__restrict__ phi,
+                          const float2 *__restrict__ fd, NPConst<float> c, int ns,
+                          float2 *__restrict__ bern) {
+  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
+    const unsigned f = fl[r];
+    const float2 phP = phi[r];
+    auto put = [&](int a, float uf, float dd, float2 nb) {
+      for (int k = 0; k < ns; k++) {
+        const float adv = __fmul_rn(uf, c.dxD[k]);
+        if (fabsf(__fmaf_rn(-c.zf[k], dd, adv)) < 0.5f) continue;
+        float Bp, Bm;
+        bernoulli_pair_split(adv, c.zf[k], nb, phP, Bp, Bm);
+        bern[((size_t)a * n + r) * ns + k] = make_float2(Bp, Bm);
+      }
+    };
+    for (int a = 0; a < DIM; a++) {
+      const int q = plus_face(f, lat, n, a, r);
+      const float2 v = fd[(size_t)a * n + r];
+      if (q >= 0) put(a, v.x, v.y, phi[q]);
+    }
+    if ((f >> (kEdgeBit + 1)) & 1u) {
+      const float2 z2 = make_float2(0.f, 0.f);
+      put(DIM, r_mul(-0.5f, r_add(ux[r], ux[r])), phi_diff(z2, phP), z2);
+    }
+  }
+}
+
+// 16-bit lateral differences of the tiles of 31 ranks (one warp per tile, as
+// the step runs them): per face the tile's base is q - r of its first cell
+// with an open face, and each cell keeps (q - r) - base, kLatClosed across a
+// closed face, or kLatWide where it does not fit (the step then reads the
+// full table).
+template <int DIM>
+__global__ void k_lat_pack(const int *__restrict__ lat, int n, short *__restrict__ latd,
+                           int *__restrict__ latb) {
+  constexpr int NL = 2 * DIM - 2;
+  const int lane = threadIdx.x & 31;
+  const int nw = (int)np_warps(n), W = gridDim.x * (blockDim.x >> 5);
+  for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nw; w += W) {
+    const int r = kHome * w + lane - 1;
+    const bool home = lane != 0 && r < n;
+#pragma unroll
+    for (int j = 0; j < NL; j++) {
+      const int q = home ? lat[(size_t)j * n + r] : -1;
+      const unsigned open = __ballot_sync(0xffffffffu, q >= 0);
+      const int base = open ? __shfl_sync(0xffffffffu, q - r, __ffs(open) - 1) : 0;
+      const int d = q - r - base;
+      if (lane == 0) latb[(size_t)w * NL + j] = base;
+      if (home)
+        latd[(size_t)r * NL + j] =
+            (short)(q < 0 ? kLatClosed : (d < -32000 || d > 32000 ? kLatWide : d));
+    }
+  }
+}
+
+template <typename T, int DIM, int NS>
 __device__ __forceinline__ void np_step_body(const T *__restrict__ Cin, T *__restrict__ Cout,
-                                             const float *__restrict__ Cinl,
-                                             float *__restrict__ Coutl, const T *__restrict__ u,
+                                             const T *__restrict__ u,
                                              const typename PhiStore<T>::type *__restrict__ phi,
                                              const NPGeo &g, const NPConst<T> &c,
-                                             typename AccSlot<T>::type *__restrict__ acc) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+                                             typename AccSlot<T>::type *__restrict__ acc,
+                                             int r) {
   T v[3 * NS];
 #pragma unroll
   for (int j = 0; j < 3 * NS; j++) v[j] = T(0);
@@ -776,118 +908,89 @@ __device__ __forceinline__ void np_step_body(const T *__restrict__ Cin, T *__res
   np_account<T, NS>(v, io, acc, r >> 5, g.naccs);
 }
 
-// FP32 storage: warps of 31 home cells (np_warp31), fields by plane pointer.
-template <int DIM, int NS, int BS, bool PAIR>
-__global__ void __launch_bounds__(BS)
-    k_np_step32(NPFields F, int n, int naccs, NPConst<float> c) {
-  np_warp31<DIM, NS, PAIR>(F, n, naccs, c, (blockIdx.x * BS + threadIdx.x) >> 5);
-}
-
-template <int DIM, int NS, int BS, int MINT, bool PAIR>
-__global__ void __launch_bounds__(BS, MINT / BS)
-    k_np_step32_occ(NPFields F, int n, int naccs, NPConst<float> c) {
-  np_warp31<DIM, NS, PAIR>(F, n, naccs, c, (blockIdx.x * BS + threadIdx.x) >> 5);
-}
-
-// The same step with a resident grid: each warp walks tiles w, w + W, ...
-// (W the warps of the launch) and loads the next tile's link data while it
-// computes the current tile, so that load no longer adds a memory round trip
-// ahead of the neighbour loads.  Tiles and accounts are those of the other
-// launch shapes.  MINB > 0 caps the registers for MINB resident blocks per SM.
-template <int DIM, int NS, int BS, int MINB, bool PAIR>
-__global__ void __launch_bounds__(BS, MINB)
-    k_np_step32_pf(NPFields F, int n, int naccs, NPConst<float> c) {
-  const int nw = (int)np_warps(n);
-  const int W = gridDim.x * (BS / 32);
-  int w = (blockIdx.x * BS + threadIdx.x) >> 5;
-  if (w >= nw) return;  // whole warps leave together
-  NPLinks<DIM> cur = np_links<DIM>(F, n, w);
-  while (true) {
-    const int wn = w + W;
-    NPLinks<DIM> nxt;
-    if (wn < nw) nxt = np_links<DIM>(F, n, wn);
-    np_warp31<DIM, NS, PAIR>(F, n, naccs, c, w, cur);
-    if (wn >= nw) break;
-    w = wn;
-    cur = nxt;
+// Has the inputs of the tiles `ahead` of this block's fetched into L2 (one
+// thread, a bulk prefetch per array): the records across the high lateral
+// face (z+, or y+ in 2D: in rank order the first of a record's five reads;
+// the place is displaced as at this block's own tile, which is close enough
+// for a hint), the face data, the link data and the account slots.
+template <int DIM, int NS, int TILES, bool PAIR>
+__device__ __forceinline__ void np_prefetch(const NPFields &F, int n, int naccs, int w,
+                                            int ahead) {
+  constexpr int NL = 2 * DIM - 2, CELLS = TILES * kHome;
+  const int w0 = w + ahead;
+  if ((long long)(w0 + 2 * TILES) * kHome >= n) return;
+  // whole 16-byte units; at most 15 bytes to either side of the range, which
+  // the test above keeps inside the arrays
+  auto pre = [](const void *p, unsigned bytes) {
+    const unsigned long long at = (unsigned long long)p & ~15ull;
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(at), "r"((bytes + 15u) & ~15u)
+                 : "memory");
+  };
+  const size_t r0 = (size_t)w0 * kHome;
+  const long long z0 = (long long)r0 + F.latb[(size_t)w * NL + (DIM == 3 ? 2 : 0)];
+  if (z0 >= 0 && z0 + 2 * CELLS < n) {
+#pragma unroll
+    for (int p = 0; p < (NS + 1) / 2; p++) {
+      constexpr unsigned words = PAIR ? 2u : 1u;
+      const unsigned rec = (2 * p + 1 < NS ? 8u : 4u) * words;
+      pre((const char *)F.C[p] + (size_t)z0 * rec, CELLS * rec);
+    }
   }
+#pragma unroll
+  for (int a = 0; a < DIM; a++) pre(F.fd[a] + r0, CELLS * 8u);
+  pre(F.latd + r0 * NL, CELLS * NL * 2u);
+  pre(F.fl + r0, CELLS * 2u);
+  pre(F.latb + (size_t)w0 * NL, TILES * NL * 4u);
+#pragma unroll
+  for (int k = 0; k < NS; k++) pre(F.acc + (size_t)(3 * k) * naccs + w0, TILES * 8u);
 }
 
-// Blocks that fill every SM with the kernel at block size bs (once per
-// kernel; at most the blocks the work needs).
-template <typename K> int resident_grid(K kernel, int bs, long long units) {
-  static int blocks = 0;
-  if (blocks == 0) {
-    int dev = 0, sms = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, bs, 0);
-    (void)cudaGetLastError();
-    blocks = (per > 0 ? per : 1) * (sms > 0 ? sms : 1);
-  }
-  return (int)std::max<long long>(1, std::min<long long>(blocks, (units + bs - 1) / bs));
-}
-
-// BS threads per block, registers as the compiler sees fit.
-template <typename T, int DIM, int NS, int BS, bool PAIR>
+// FP32 storage: warps of 31 home cells (np_warp31); ahead > 0: np_prefetch.
+// 256^3 pack, pair concentrations: 235 us a step -> 139 us (1.6 -> 2.7 TB/s of
+// the method's 49 bytes a cell); 1024x512: 6.9 -> 5.8 us.
+template <int DIM, int NS, int BS, bool PAIR, int MODE>
 __global__ void __launch_bounds__(BS)
-    k_np_step(const T *__restrict__ Cin, T *__restrict__ Cout, const float *__restrict__ Cinl,
-              float *__restrict__ Coutl, const T *__restrict__ u,
+    k_np_step32(const __grid_constant__ NPFields F, int n, int naccs,
+                const __grid_constant__ NPConst<float> c, int ahead) {
+  const int w = (int)((blockIdx.x * BS + threadIdx.x) >> 5);
+  if (ahead > 0 && threadIdx.x == 0) np_prefetch<DIM, NS, BS / 32, PAIR>(F, n, naccs, w, ahead);
+  np_warp31<DIM, NS, PAIR, MODE>(F, n, naccs, c, w);
+}
+
+// FP64 storage, one thread per pore cell.
+template <typename T, int DIM, int NS, int BS>
+__global__ void __launch_bounds__(BS)
+    k_np_step(const T *__restrict__ Cin, T *__restrict__ Cout, const T *__restrict__ u,
               const typename PhiStore<T>::type *__restrict__ phi, NPGeo g, NPConst<T> c,
               typename AccSlot<T>::type *__restrict__ acc) {
-  np_step_body<T, DIM, NS, PAIR>(Cin, Cout, Cinl, Coutl, u, phi, g, c, acc);
-}
-
-// The same step with registers capped so that MINT threads share an SM (more
-// resident warps for the gathered loads, at the price of a few spilled
-// values).
-template <typename T, int DIM, int NS, int BS, int MINT, bool PAIR>
-__global__ void __launch_bounds__(BS, MINT / BS)
-    k_np_step_occ(const T *__restrict__ Cin, T *__restrict__ Cout, const float *__restrict__ Cinl,
-                  float *__restrict__ Coutl, const T *__restrict__ u,
-                  const typename PhiStore<T>::type *__restrict__ phi, NPGeo g, NPConst<T> c,
-                  typename AccSlot<T>::type *__restrict__ acc) {
-  np_step_body<T, DIM, NS, PAIR>(Cin, Cout, Cinl, Coutl, u, phi, g, c, acc);
+  np_step_body<T, DIM, NS>(Cin, Cout, u, phi, g, c, acc,
+                           (int)(blockIdx.x * blockDim.x + threadIdx.x));
 }
 
 // One member of a fused sweep: its own concentrations, velocity, potential,
 // constants (time step) and accounts.
 template <typename T> struct SweepMember {
   T *C[2];          // concentration buffers (ping-pong)
-  float *Cl[2];     // their low words (FP32 pair storage), else null
-  NPFields f[2];    // FP32: the fields as plane pointers, stepping from buffer 0 / 1
+  NPFields f[2];    // FP32: the fields of a step from buffer 0 / 1
   const T *u;
   const typename PhiStore<T>::type *phi;
   typename AccSlot<T>::type *acc;
   NPConst<T> c;
 };
 
-// All members of a sweep advance one step in one launch: each block runs the
-// same cells for every member in turn (the block -> cells map, the arithmetic
-// and the accounts of a member are those of k_np_step, so a member's result
-// equals a single run's bit for bit).
-template <typename T, int DIM, int NS, bool PAIR>
+// All members of a sweep advance one step in one launch: block (b, m) runs
+// the cells of block b for member m (the block -> cells map, the arithmetic
+// and the accounts of a member are those of a single run's launch, so a
+// member's result equals a single run's bit for bit).
+template <typename T, int DIM, int NS, bool PAIR, int MODE>
 __global__ void __launch_bounds__(kRowBlock)
-    k_np_sweep(const SweepMember<T> *__restrict__ members, int n_members, int in, NPGeo g) {
+    k_np_sweep(const SweepMember<T> *__restrict__ members, int in, NPGeo g) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if constexpr (std::is_same<T, float>::value) {
-    for (int m = 0; m < n_members; m++) {
-      const SweepMember<T> &mb = members[m];
-      np_warp31<DIM, NS, PAIR>(mb.f[in], g.n, g.naccs, mb.c, r >> 5);
-    }
-  } else {
-    const uint2 meta = r < g.n ? g.meta[r] : make_uint2(1u, 0u);
-    for (int m = 0; m < n_members; m++) {
-      const SweepMember<T> &mb = members[m];
-      T v[3 * NS];
-#pragma unroll
-      for (int j = 0; j < 3 * NS; j++) v[j] = T(0);
-      bool io = false;
-      if (r < g.n)
-        io = np_cell<T, DIM, NS>(mb.C[in], mb.C[1 - in], mb.u, mb.phi, g, meta, r, mb.c, v);
-      np_account<T, NS>(v, io, mb.acc, r >> 5, g.naccs);
-    }
-  }
+  const SweepMember<T> &mb = members[blockIdx.y];
+  if constexpr (std::is_same<T, float>::value)
+    np_warp31<DIM, NS, PAIR, MODE>(mb.f[in], g.n, g.naccs, mb.c, r >> 5);
+  else
+    np_step_body<T, DIM, NS>(mb.C[in], mb.C[1 - in], mb.u, mb.phi, g, mb.c, mb.acc, r);
 }
 
 // One member of a batch over several geometries: a sweep member plus its
@@ -904,7 +1007,7 @@ template <typename T> struct BatchMember {
 // local block b - block0: the same cells, arithmetic and accounts as block
 // b - block0 of the member's single-run launch, so each member equals its
 // single run bit for bit.
-template <typename T, int DIM, int NS, bool PAIR>
+template <typename T, int DIM, int NS, bool PAIR, int MODE>
 __global__ void __launch_bounds__(kRowBlock)
     k_np_batch(const BatchMember<T> *__restrict__ members, int n_members, int in) {
   int lo = 0, hi = n_members - 1;
@@ -916,18 +1019,11 @@ __global__ void __launch_bounds__(kRowBlock)
   const BatchMember<T> &mb = members[lo];
   const int b = (int)blockIdx.x - mb.block0;
   const int r = b * blockDim.x + threadIdx.x;
-  if constexpr (std::is_same<T, float>::value) {
-    np_warp31<DIM, NS, PAIR>(mb.s.f[in], mb.g.n, mb.g.naccs, mb.s.c, r >> 5);
-  } else {
-    T v[3 * NS];
-#pragma unroll
-    for (int j = 0; j < 3 * NS; j++) v[j] = T(0);
-    bool io = false;
-    if (r < mb.g.n)
-      io = np_cell<T, DIM, NS>(mb.s.C[in], mb.s.C[1 - in], mb.s.u, mb.s.phi, mb.g, mb.g.meta[r],
-                               r, mb.s.c, v);
-    np_account<T, NS>(v, io, mb.s.acc, r >> 5, mb.g.naccs);
-  }
+  if constexpr (std::is_same<T, float>::value)
+    np_warp31<DIM, NS, PAIR, MODE>(mb.s.f[in], mb.g.n, mb.g.naccs, mb.s.c, r >> 5);
+  else
+    np_step_body<T, DIM, NS>(mb.s.C[in], mb.s.C[1 - in], mb.s.u, mb.s.phi, mb.g, mb.s.c,
+                             mb.s.acc, r);
 }
 
 // Largest outflow rate over pore cells and species, in FP64 from the FP64
@@ -991,22 +1087,15 @@ __global__ void __launch_bounds__(kRedThreads)
   }
 }
 
+// The saturated start: every cell of species k at c0 (hi + lo).
 template <typename T>
-__global__ void k_np_init(T *__restrict__ C0, T *__restrict__ C1, float *__restrict__ L0,
-                          float *__restrict__ L1, int n, int ns, T c0, float c0lo) {
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
-#pragma unroll
-    for (int k = 0; k < kMaxSpecies; k++) {
-      const T v = k < ns ? c0 : T(0);
-      C0[(size_t)k * n + r] = v;
-      C1[(size_t)k * n + r] = v;
-      if (L0) {
-        const float l = k < ns ? c0lo : 0.f;
-        L0[(size_t)k * n + r] = l;
-        L1[(size_t)k * n + r] = l;
-      }
+__global__ void k_np_init(CViews<T> C, int n, int ns, T c0, T c0lo) {
+  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x)
+    for (int k = 0; k < ns; k++) {
+      T *p = const_cast<T *>(C.v[k].p) + (size_t)r * C.v[k].stride;
+      p[0] = c0;
+      if (C.v[k].lo) p[C.v[k].lo] = c0lo;
     }
-  }
 }
 
 // Dissolved amount, outlet sums (flux weighted and plain) per species.
@@ -1014,9 +1103,8 @@ __global__ void k_np_init(T *__restrict__ C0, T *__restrict__ C1, float *__restr
 // sum of C at the outlet, 13 pore cells in the outlet column.
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads)
-    k_np_sums(const uint2 *__restrict__ meta, const T *__restrict__ C,
-              const float *__restrict__ Cl, const T *__restrict__ u, int n, int ns,
-              double cell_vol, double *__restrict__ part, unsigned int *counter, double *scal) {
+    k_np_sums(const uint2 *__restrict__ meta, CViews<T> C, const T *__restrict__ u, int n,
+              int ns, double cell_vol, double *__restrict__ part, unsigned int *counter, double *scal) {
   constexpr int NV = 14;
   __shared__ double sm[NV * 32];
   double v[NV];
@@ -1028,7 +1116,7 @@ __global__ void __launch_bounds__(kRedThreads)
 #pragma unroll
     for (int k = 0; k < kMaxSpecies; k++) {
       if (k >= ns) break;
-      const double ck = (double)C[(size_t)k * n + r] + (Cl ? (double)Cl[(size_t)k * n + r] : 0.0);
+      const double ck = C.v[k].at(r);
       v[k] += ck;
       if (outlet) {
         v[4 + k] += ux * ck;
@@ -1121,8 +1209,8 @@ void acc_total(const cdi_domain *d, const void *acc, cudaStream_t st, double *sc
 // cells found through the row words).
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads)
-    k_colmeans(const uint2 *__restrict__ words, int W, const T *__restrict__ C,
-               const float *__restrict__ Cl, int rows, double *__restrict__ out) {
+    k_colmeans(const uint2 *__restrict__ words, int W, CView<T> C, int rows,
+               double *__restrict__ out) {
   __shared__ double sm[2 * 32];
   const int x = blockIdx.x;
   double v[2] = {0.0, 0.0};
@@ -1130,7 +1218,7 @@ __global__ void __launch_bounds__(kRedThreads)
     const uint2 t = words[(size_t)row * W + (x >> 5)];
     if (!((t.y >> (x & 31)) & 1u)) continue;
     const int r = t.x + __popc(t.y & ((1u << (x & 31)) - 1u));
-    v[0] += (double)C[r] + (Cl ? (double)Cl[r] : 0.0);
+    v[0] += C.at(r);
     v[1] += 1.0;
   }
   block_reduce<2>(v, sm, OpSum(), 0.0);
@@ -1190,17 +1278,37 @@ __global__ void k_words(const NFlag *__restrict__ fl, const int *__restrict__ ce
   }
 }
 
-// Compact (rank-ordered) field -> FP64 lattice field, 0 in solid cells:
-// dst[a * N + cells[r]] = src[a * n + r] for comps components.
+// Compact (rank-ordered) fields -> FP64 lattice fields, 0 in solid cells:
+// dst[a * N + cells[r]] = the value of component a at rank r.
 template <typename T>
-__global__ void k_scatter(const T *__restrict__ src, const float *__restrict__ lo, int comps,
-                          const int *__restrict__ cells, int n, long long N,
-                          double *__restrict__ dst) {
+__global__ void k_scatter(CViews<T> src, int comps, const int *__restrict__ cells, int n,
+                          long long N, double *__restrict__ dst) {
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
     const long long P = cells[r];
-    for (int a = 0; a < comps; a++)
-      dst[a * N + P] = (double)src[(size_t)a * n + r] + (lo ? (double)lo[(size_t)a * n + r] : 0.0);
+    for (int a = 0; a < comps; a++) dst[a * N + P] = src.v[a].at(r);
   }
+}
+
+// Species records <-> planes of kMaxSpecies hi words followed (pair storage)
+// by kMaxSpecies lo words, the order of a saved state; the planes of absent
+// species are 0.
+__global__ void k_records_to_planes(CViews<float> C, int n, int ns, float *__restrict__ hi,
+                                    float *__restrict__ lo) {
+  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x)
+    for (int k = 0; k < kMaxSpecies; k++) {
+      const float *p = k < ns ? C.v[k].p + (size_t)r * C.v[k].stride : nullptr;
+      hi[(size_t)k * n + r] = p ? p[0] : 0.f;
+      if (lo) lo[(size_t)k * n + r] = p ? p[C.v[k].lo] : 0.f;
+    }
+}
+__global__ void k_planes_to_records(CViews<float> C, int n, int ns, const float *__restrict__ hi,
+                                    const float *__restrict__ lo) {
+  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x)
+    for (int k = 0; k < ns; k++) {
+      float *p = const_cast<float *>(C.v[k].p) + (size_t)r * C.v[k].stride;
+      p[0] = hi[(size_t)k * n + r];
+      if (lo) p[C.v[k].lo] = lo[(size_t)k * n + r];
+    }
 }
 
 template <typename T> NPConst<T> make_const(const cdi_domain *d) {
@@ -1217,63 +1325,80 @@ template <typename T> NPConst<T> make_const(const cdi_domain *d) {
   return c;
 }
 
-// The FP32 fields of a transport state as plane pointers (stepping from
-// Cin/Cinl into Cout/Coutl).
-NPFields fields32(const cdi_domain *d, const void *Cin, const float *Cinl, void *Cout,
-                  float *Coutl, const void *u, const void *phi, void *acc) {
+// The FP32 fields of a transport state (stepping from Cin into Cout; fd the
+// face data of its velocity and potential).
+NPFields fields32(const cdi_domain *d, const void *Cin, void *Cout, const float2 *fd,
+                  const float2 *bern, const void *u, const void *phi, void *acc) {
   NPFields F{};
-  const size_t n = (size_t)d->n_pore;
-  for (int k = 0; k < kMaxSpecies; k++) {
-    F.C[k] = (const float *)Cin + (size_t)k * n;
-    F.Cl[k] = Cinl ? Cinl + (size_t)k * n : nullptr;
-    F.Co[k] = (float *)Cout + (size_t)k * n;
-    F.Col[k] = Coutl ? Coutl + (size_t)k * n : nullptr;
+  const size_t n = (size_t)d->n_pore, pair = 2 * n * (d->cpair ? 2 : 1);
+  for (int p = 0; p < 2; p++) {
+    F.C[p] = (const float *)Cin + p * pair;
+    F.Co[p] = (float *)Cout + p * pair;
   }
-  for (int a = 0; a < d->dim; a++) F.u[a] = (const float *)u + (size_t)a * n;
-  for (int j = 0; j < 2 * (d->dim - 1); j++) F.lat[j] = d->d_latnb + (size_t)j * n;
+  for (int a = 0; a < d->dim; a++) F.fd[a] = fd + (size_t)a * n;
+  F.latd = d->d_latd;
+  F.latb = d->d_latb;
+  F.lat = d->d_latnb;
+  F.ux = (const float *)u;
   F.phi = (const float2 *)phi;
   F.fl = d->d_cfl;
+  F.bern = bern;
   F.acc = (float2 *)acc;
   return F;
 }
 
-NPGeo make_geo(const cdi_domain *d) {
-  return NPGeo{d->d_cmeta, d->d_cfl, d->d_words, d->d_latnb, (int)d->n_pore, d->W, d->ny, d->nz,
-               d->walls, d->np_accs};
+// The face data of velocity u and potential phi (FP32 storage); *any_large
+// (device, cleared by the caller) tells whether a face has |P| >= 1/2.
+void launch_faces(const cdi_domain *d, cudaStream_t st, const void *u, const void *phi,
+                  float2 *fd, int *any_large) {
+  const int n = (int)d->n_pore, grid = std::min((n + 255) / 256, 16 * kRedBlocks);
+  const NPConst<float> c = make_const<float>(d);
+  auto *kern = d->dim == 2 ? k_np_faces<2> : k_np_faces<3>;
+  kern<<<grid, 256, 0, st>>>(d->d_cfl, d->d_latnb, n, (const float *)u, (const float2 *)phi, c,
+                             d->ns, fd, any_large);
+}
+void launch_bern(const cdi_domain *d, cudaStream_t st, const void *u, const void *phi,
+                 const float2 *fd, float2 *bern) {
+  const int n = (int)d->n_pore, grid = std::min((n + 255) / 256, 16 * kRedBlocks);
+  const NPConst<float> c = make_const<float>(d);
+  auto *kern = d->dim == 2 ? k_np_bern<2> : k_np_bern<3>;
+  kern<<<grid, 256, 0, st>>>(d->d_cfl, d->d_latnb, n, (const float *)u, (const float2 *)phi, fd, c,
+                             d->ns, bern);
+}
+size_t bern_bytes(const cdi_domain *d) {
+  return (size_t)(d->dim + 1) * d->n_pore * d->ns * sizeof(float2);
 }
 
-template <typename T, int DIM, int NS, int BS, int MINT, bool PAIR>
+NPGeo make_geo(const cdi_domain *d) {
+  return NPGeo{d->d_cmeta, d->d_latnb, (int)d->n_pore, d->np_accs};
+}
+
+// Tiles between a block and the ones whose inputs it has fetched into L2: one
+// to two waves of resident warps.  0 (no prefetch) where a step's whole
+// working set stays in L2 from one step to the next.
+int np_ahead_tiles(const cdi_domain *d) {
+  const size_t rec = (size_t)d->ns * (d->cpair ? 8 : 4);
+  const size_t step = (size_t)d->n_pore * (2 * rec + d->dim * 8 + 4 * (d->dim - 1) + 2);
+  return step > ((size_t)96 << 20) ? 8192 : 0;
+}
+
+template <typename T, int DIM, int NS, int BS, bool PAIR>
 void launch_step_bs(cdi_domain *d, cudaStream_t st, int in) {
   // FP64: one thread per pore rank; FP32: warps of 31 home cells (one
   // account set per warp either way)
   const long long units = std::is_same<T, float>::value ? np_warps(d->n_pore) * 32 : d->n_pore;
   const int grid = (int)((units + BS - 1) / BS);
-  const float *Cinl = PAIR ? d->d_Clo[in] : nullptr;
-  float *Coutl = PAIR ? d->d_Clo[1 - in] : nullptr;
   if constexpr (std::is_same<T, float>::value) {
-    const NPFields F = fields32(d, d->d_C[in], Cinl, d->d_C[1 - in], Coutl, d->d_u, d->d_phi,
-                                d->d_acc);
-    if constexpr (MINT < 0) {
-      // -1: registers as the compiler sees fit; -2: capped for 1024 threads
-      // per SM; -3: for 768
-      constexpr int MINB = MINT == -2 ? 1024 / BS : (MINT == -3 ? 768 / BS : 0);
-      auto *kern = k_np_step32_pf<DIM, NS, BS, MINB, PAIR>;
-      kern<<<resident_grid(kern, BS, units), BS, 0, st>>>(F, (int)d->n_pore, d->np_accs,
-                                                          make_const<float>(d));
-    } else if constexpr (MINT == 0)
-      k_np_step32<DIM, NS, BS, PAIR><<<grid, BS, 0, st>>>(F, (int)d->n_pore, d->np_accs,
-                                                          make_const<float>(d));
-    else
-      k_np_step32_occ<DIM, NS, BS, MINT, PAIR><<<grid, BS, 0, st>>>(F, (int)d->n_pore, d->np_accs,
-                                                                    make_const<float>(d));
-  } else if constexpr (MINT <= 0) {
-    k_np_step<T, DIM, NS, BS, PAIR><<<grid, BS, 0, st>>>(
-        (const T *)d->d_C[in], (T *)d->d_C[1 - in], Cinl, Coutl, (const T *)d->d_u,
-        (const typename PhiStore<T>::type *)d->d_phi, make_geo(d), make_const<T>(d),
-        (typename AccSlot<T>::type *)d->d_acc);
+    const NPFields F = fields32(d, d->d_C[in], d->d_C[1 - in], d->d_fd, d->d_bern, d->d_u,
+                                d->d_phi, d->d_acc);
+    auto *kern = d->np_mode == NP_SMALL   ? k_np_step32<DIM, NS, BS, PAIR, NP_SMALL>
+                 : d->np_mode == NP_LARGE ? k_np_step32<DIM, NS, BS, PAIR, NP_LARGE>
+                                          : k_np_step32<DIM, NS, BS, PAIR, NP_EVAL>;
+    kern<<<grid, BS, 0, st>>>(F, (int)d->n_pore, d->np_accs, make_const<float>(d),
+                              np_ahead_tiles(d));
   } else {
-    k_np_step_occ<T, DIM, NS, BS, MINT, PAIR><<<grid, BS, 0, st>>>(
-        (const T *)d->d_C[in], (T *)d->d_C[1 - in], Cinl, Coutl, (const T *)d->d_u,
+    k_np_step<T, DIM, NS, BS><<<grid, BS, 0, st>>>(
+        (const T *)d->d_C[in], (T *)d->d_C[1 - in], (const T *)d->d_u,
         (const typename PhiStore<T>::type *)d->d_phi, make_geo(d), make_const<T>(d),
         (typename AccSlot<T>::type *)d->d_acc);
   }
@@ -1281,17 +1406,10 @@ void launch_step_bs(cdi_domain *d, cudaStream_t st, int in) {
 
 template <typename T, int DIM, int NS, bool PAIR>
 void launch_step_t(cdi_domain *d, cudaStream_t st, int in) {
-  switch (d->np_variant) {
-    case 0: launch_step_bs<T, DIM, NS, 64, 0, PAIR>(d, st, in); break;
-    case 2: launch_step_bs<T, DIM, NS, 256, 0, PAIR>(d, st, in); break;
-    case 3: launch_step_bs<T, DIM, NS, 64, 1280, PAIR>(d, st, in); break;
-    case 4: launch_step_bs<T, DIM, NS, 128, 1280, PAIR>(d, st, in); break;
-    case 5: launch_step_bs<T, DIM, NS, 128, 1024, PAIR>(d, st, in); break;
-    case 6: launch_step_bs<T, DIM, NS, 256, 1024, PAIR>(d, st, in); break;
-    case 7: launch_step_bs<T, DIM, NS, 128, -1, PAIR>(d, st, in); break;
-    case 8: launch_step_bs<T, DIM, NS, 128, -2, PAIR>(d, st, in); break;
-    case 9: launch_step_bs<T, DIM, NS, 128, -3, PAIR>(d, st, in); break;
-    default: launch_step_bs<T, DIM, NS, 128, 0, PAIR>(d, st, in); break;
+  switch (d->np_block) {
+    case 64: launch_step_bs<T, DIM, NS, 64, PAIR>(d, st, in); break;
+    case 256: launch_step_bs<T, DIM, NS, 256, PAIR>(d, st, in); break;
+    default: launch_step_bs<T, DIM, NS, 128, PAIR>(d, st, in); break;
   }
 }
 
@@ -1320,62 +1438,15 @@ void launch_step(cdi_domain *d, cudaStream_t st, int in) {
 
 constexpr int kGraphSteps = 64;  // steps per captured transport graph (even)
 
-// Autotuner: times a few transport steps with each candidate launch shape
-// (64, 128 or 256 threads per block; for 64 and 128 also a variant compiled
-// for 1280 resident threads per SM, for 128 and 256 one for 1024, and FP32
-// resident grids that prefetch each warp's next link data, with registers as
-// the compiler sees fit or capped for 1024 or 768 threads per SM) on the
-// domain's stream and keeps the fastest.  Accounts are kept per warp of 32 ranks whatever the shape, and
-// the arithmetic of a thread does not depend on its register allocation, so
-// every choice computes the same bits.  Runs once per domain, before
-// cdi_np_init overwrites the concentrations and clears the accounts.
-constexpr int kNpVariantBlock[10] = {64, 128, 256, 64, 128, 128, 256, 128, 128, 128};
-cdi_status tune_np(cdi_domain *d) {
-  // variants 7-9 (resident grids with prefetch) are FP32 launch shapes; for
-  // FP64 they are plain launches of the same block size again
-  static const int cand[] = {0, 1, 2, 3, 4, 5, 6, 7, 8, 9};
-  const uint64_t key = cdi_tune_key(2, d->dim, d->prec, d->ns, d->n_pore, 0);
-  int known = 0;
-  if (cdi_tune_lookup(key, &known)) {
-    d->np_variant = known;
-    d->np_block = kNpVariantBlock[known];
-    d->np_tuned = true;
-    return CDI_OK;
-  }
-  cudaEvent_t a, b;
-  CDI_TRY(d, cudaEventCreate(&a), "tune event");
-  cudaError_t e = cudaEventCreate(&b);
-  if (e != cudaSuccess) {
-    cudaEventDestroy(a);
-    return cdi_cuda_fail(d, e, "tune event");
-  }
-  float best = 0.f;
-  int best_bs = 1;
-  for (int bs : cand) {
-    d->np_variant = bs;
-    launch_step(d, d->stream, 0);  // warm-up
-    e = cudaEventRecord(a, d->stream);
-    for (int k = 0; k < 8 && e == cudaSuccess; k++) launch_step(d, d->stream, k & 1);
-    if (e == cudaSuccess) e = cudaEventRecord(b, d->stream);
-    if (e == cudaSuccess) e = cudaEventSynchronize(b);
-    float ms = 0.f;
-    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, a, b);
-    if (e != cudaSuccess) break;
-    d->timing.kernel_launches += 9;
-    if (bs == cand[0] || ms < best) {
-      best = ms;
-      best_bs = bs;
-    }
-  }
-  cudaEventDestroy(a);
-  cudaEventDestroy(b);
-  d->np_variant = best_bs;
-  d->np_block = kNpVariantBlock[best_bs];
-  if (e != cudaSuccess) return cdi_cuda_fail(d, e, "tune transport step");
-  d->np_tuned = true;
-  cdi_tune_store(key, best_bs);
-  return CDI_OK;
-}
+// Launch shapes: 64, 128 or 256 threads per block (0-2); 3-9 name the default
+// again.  128 is taken unless a shape is fixed: it is the fastest or within
+// 4 % of it on every size measured (256^3: 155 / 139 / 154 us for 64 / 128 /
+// 256; 1024x512: 5.8 / 5.8 / 5.9; 96^3: 11.3 / 10.6 / 11.1), so no launch is
+// spent on timing candidates (FP64 storage: 64 threads, 16.5 / 17.7 / 30.2 us
+// on 128x64).  Accounts are kept per warp whatever the shape, so every choice
+// computes the same bits.
+constexpr int kNpDefaultShape = 1, kNpDefaultShape64 = 0;
+constexpr int kNpVariantBlock[10] = {64, 128, 256, 128, 128, 128, 128, 128, 128, 128};
 
 }  // namespace
 
@@ -1405,24 +1476,61 @@ cdi_status cdi_np_init(cdi_domain *d, double dt_s, double *dt_used) {
   }
   d->dt = dt;
   if (dt_used) *dt_used = dt;
+  cdi_status fs = cdi_np_faces(d);
+  if (fs != CDI_OK) return fs;
   if (!d->np_tuned) {
-    cdi_status s = tune_np(d);
-    if (s != CDI_OK) return s;
+    d->np_variant = d->prec == CDI_FP64 ? kNpDefaultShape64 : kNpDefaultShape;
+    d->np_block = kNpVariantBlock[d->np_variant];
+    d->np_tuned = true;
   }
   if (d->prec == CDI_FP64)
     k_np_init<double><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        (double *)d->d_C[0], (double *)d->d_C[1], nullptr, nullptr, (int)d->n_pore, d->ns, d->c0,
-        0.f);
+        c_views<double>(d, d->d_C[0]), (int)d->n_pore, d->ns, d->c0, 0.0);
   else
     k_np_init<float><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        (float *)d->d_C[0], (float *)d->d_C[1], d->d_Clo[0], d->d_Clo[1], (int)d->n_pore, d->ns,
-        (float)d->c0, (float)(d->c0 - (double)(float)d->c0));
+        c_views<float>(d, d->d_C[0]), (int)d->n_pore, d->ns, (float)d->c0,
+        (float)(d->c0 - (double)(float)d->c0));
   d->timing.kernel_launches++;
   CDI_TRY(d, cudaGetLastError(), "transport init");
   CDI_TRY(d, cudaMemsetAsync(d->d_acc, 0, (size_t)3 * kMaxSpecies * d->np_accs * 8, d->stream),
           "reset accumulators");
   d->cur = 0;
   d->np_steps = 0;
+  return CDI_OK;
+}
+
+// The face data of the domain's current velocity and potential (FP32 storage
+// only; after either, or the species, has changed), and the Bernoulli pairs
+// where some face needs them (their memory is taken the first time one does;
+// without it the step evaluates them itself).  Waits for the stream.
+cdi_status cdi_np_faces(cdi_domain *d) {
+  if (d->prec == CDI_FP64) return CDI_OK;
+  int *flag = (int *)(d->d_counter + C_FACE);
+  int large = 0;
+  CDI_TRY(d, cudaMemsetAsync(flag, 0, sizeof(int), d->stream), "face flag reset");
+  launch_faces(d, d->stream, d->d_u, d->d_phi, d->d_fd, flag);
+  d->timing.kernel_launches++;
+  CDI_TRY(d, cudaGetLastError(), "face data");
+  CDI_TRY(d, cudaMemcpyAsync(&large, flag, sizeof(int), cudaMemcpyDeviceToHost, d->stream),
+          "face flag");
+  CDI_TRY(d, cudaStreamSynchronize(d->stream), "face data");
+  d->np_mode = large ? NP_LARGE : NP_SMALL;
+  if (!large) return CDI_OK;
+  if (d->d_bern && d->bern_bytes < bern_bytes(d)) {
+    cdi_dev_release(d, d->d_bern);
+    d->d_bern = nullptr;
+  }
+  if (!d->d_bern) {
+    d->bern_bytes = bern_bytes(d);
+    d->d_bern = (float2 *)cdi_dev_alloc(d, d->bern_bytes);
+    if (!d->d_bern) {
+      d->np_mode = NP_EVAL;
+      return CDI_OK;
+    }
+  }
+  launch_bern(d, d->stream, d->d_u, d->d_phi, d->d_fd, d->d_bern);
+  d->timing.kernel_launches++;
+  CDI_TRY(d, cudaGetLastError(), "face data");
   return CDI_OK;
 }
 
@@ -1461,29 +1569,52 @@ cdi_status cdi_np_dt(cdi_domain *d, double scale, double *dt_out) {
 // ---------------------------------------------------------------------------
 namespace {
 
-template <typename T, int DIM, bool PAIR>
+template <typename T, int DIM, bool PAIR, int MODE>
 void launch_sweep_d(cdi_domain *d, cudaStream_t st, const void *members, int n, int in) {
   const SweepMember<T> *m = (const SweepMember<T> *)members;
   const NPGeo g = make_geo(d);
+  const dim3 grid(d->np_blocks, n);
   switch (d->ns) {
-    case 1: k_np_sweep<T, DIM, 1, PAIR><<<d->np_blocks, kRowBlock, 0, st>>>(m, n, in, g); break;
-    case 2: k_np_sweep<T, DIM, 2, PAIR><<<d->np_blocks, kRowBlock, 0, st>>>(m, n, in, g); break;
-    case 3: k_np_sweep<T, DIM, 3, PAIR><<<d->np_blocks, kRowBlock, 0, st>>>(m, n, in, g); break;
-    default: k_np_sweep<T, DIM, 4, PAIR><<<d->np_blocks, kRowBlock, 0, st>>>(m, n, in, g); break;
+    case 1: k_np_sweep<T, DIM, 1, PAIR, MODE><<<grid, kRowBlock, 0, st>>>(m, in, g); break;
+    case 2: k_np_sweep<T, DIM, 2, PAIR, MODE><<<grid, kRowBlock, 0, st>>>(m, in, g); break;
+    case 3: k_np_sweep<T, DIM, 3, PAIR, MODE><<<grid, kRowBlock, 0, st>>>(m, in, g); break;
+    default: k_np_sweep<T, DIM, 4, PAIR, MODE><<<grid, kRowBlock, 0, st>>>(m, in, g); break;
   }
 }
 
-void launch_sweep(cdi_domain *d, cudaStream_t st, const void *members, int n, int in) {
+template <int DIM, bool PAIR>
+void launch_sweep32(cdi_domain *d, cudaStream_t st, const void *members, int n, int in,
+                    int mode) {
+  if (mode == NP_SMALL) launch_sweep_d<float, DIM, PAIR, NP_SMALL>(d, st, members, n, in);
+  else if (mode == NP_LARGE) launch_sweep_d<float, DIM, PAIR, NP_LARGE>(d, st, members, n, in);
+  else launch_sweep_d<float, DIM, PAIR, NP_EVAL>(d, st, members, n, in);
+}
+
+void launch_sweep(cdi_domain *d, cudaStream_t st, const void *members, int n, int in, int mode) {
   if (d->prec == CDI_FP64) {
-    if (d->dim == 2) launch_sweep_d<double, 2, false>(d, st, members, n, in);
-    else launch_sweep_d<double, 3, false>(d, st, members, n, in);
+    if (d->dim == 2) launch_sweep_d<double, 2, false, NP_SMALL>(d, st, members, n, in);
+    else launch_sweep_d<double, 3, false, NP_SMALL>(d, st, members, n, in);
   } else if (d->cpair) {
-    if (d->dim == 2) launch_sweep_d<float, 2, true>(d, st, members, n, in);
-    else launch_sweep_d<float, 3, true>(d, st, members, n, in);
+    if (d->dim == 2) launch_sweep32<2, true>(d, st, members, n, in, mode);
+    else launch_sweep32<3, true>(d, st, members, n, in, mode);
   } else {
-    if (d->dim == 2) launch_sweep_d<float, 2, false>(d, st, members, n, in);
-    else launch_sweep_d<float, 3, false>(d, st, members, n, in);
+    if (d->dim == 2) launch_sweep32<2, false>(d, st, members, n, in, mode);
+    else launch_sweep32<3, false>(d, st, members, n, in, mode);
   }
+}
+
+// Face data of a member (its own arrays, named in its two field sets), and
+// its Bernoulli pairs where a face needs them (false: no memory for them).
+void member_faces(const cdi_domain *d, cudaStream_t st, NPFields (&f)[2], const void *u,
+                  int *count) {
+  launch_faces(d, st, u, f[0].phi, const_cast<float2 *>(f[0].fd[0]), count);
+}
+bool member_bern(const cdi_domain *d, cudaStream_t st, NPFields (&f)[2], const void *u,
+                 void *bern) {
+  if (!bern) return false;
+  launch_bern(d, st, u, f[0].phi, f[0].fd[0], (float2 *)bern);
+  f[0].bern = f[1].bern = (const float2 *)bern;
+  return true;
 }
 
 template <typename T>
@@ -1492,6 +1623,7 @@ cdi_status sweep_run(cdi_domain *d, int n, const double *scale, const int *group
                      double *gamma, double *cout) {
   const size_t TN = (size_t)d->n_pore * sizeof(T);
   const int ns = d->ns;
+  const bool f64 = d->prec == CDI_FP64;
   // per-member device memory: velocity, two concentration buffers, accounts
   std::vector<void *> blocks;
   auto take = [&](size_t bytes) {
@@ -1503,38 +1635,52 @@ cdi_status sweep_run(cdi_domain *d, int n, const double *scale, const int *group
   bool ok = true;
   for (int m = 0; m < n && ok; m++) {
     void *u = take((size_t)d->dim * TN);
-    void *c0 = take((size_t)kMaxSpecies * TN), *c1 = take((size_t)kMaxSpecies * TN);
+    const size_t CN = (size_t)ns * TN * (d->cpair ? 2 : 1);
+    void *c0 = take(CN), *c1 = take(CN);
     void *acc = take((size_t)3 * kMaxSpecies * d->np_accs * 8);
-    void *l0 = d->cpair ? take((size_t)kMaxSpecies * d->n_pore * 4) : nullptr;
-    void *l1 = d->cpair ? take((size_t)kMaxSpecies * d->n_pore * 4) : nullptr;
-    ok = u && c0 && c1 && acc && (!d->cpair || (l0 && l1));
+    float2 *fd = f64 ? nullptr : (float2 *)take((size_t)d->dim * d->n_pore * sizeof(float2));
+    ok = u && c0 && c1 && acc && (f64 || fd);
     if (!ok) break;
     d->dt = dts[m];
     hm[m].C[0] = (T *)c0;
     hm[m].C[1] = (T *)c1;
-    hm[m].Cl[0] = (float *)l0;
-    hm[m].Cl[1] = (float *)l1;
     for (int in = 0; in < 2; in++)
-      hm[m].f[in] = fields32(d, in ? c1 : c0, in ? (float *)l1 : (float *)l0, in ? c0 : c1,
-                             in ? (float *)l0 : (float *)l1, u, phi_groups[group[m]], acc);
+      hm[m].f[in] = fields32(d, in ? c1 : c0, in ? c0 : c1, fd, nullptr, u,
+                             phi_groups[group[m]], acc);
     hm[m].u = (const T *)u;
     hm[m].phi = (const typename PhiStore<T>::type *)phi_groups[group[m]];
     hm[m].acc = (typename AccSlot<T>::type *)acc;
     hm[m].c = make_const<T>(d);
   }
   void *dmem = ok ? take(sizeof(SweepMember<T>) * n) : nullptr;
+  int *count = dmem ? (int *)take(sizeof(int) * n) : nullptr;  // a face with |P| >= 1/2, per member
+  if (!count) dmem = nullptr;
   cdi_status s = CDI_OK;
   if (!ok || !dmem) s = cdi_fail(d, CDI_ERR_OOM, "sweep: device allocation failed");
+  if (s == CDI_OK && cudaMemsetAsync(count, 0, sizeof(int) * n, d->stream) != cudaSuccess)
+    s = cdi_fail(d, CDI_ERR_CUDA, "sweep: memset");
   for (int m = 0; m < n && s == CDI_OK; m++) {
     s = cdi_flow_scale_to(d, scale[m], (void *)hm[m].u);
     if (s != CDI_OK) break;
+    d->dt = dts[m];
+    if (!f64) member_faces(d, d->stream, hm[m].f, hm[m].u, count + m);
     k_np_init<T><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        hm[m].C[0], hm[m].C[1], hm[m].Cl[0], hm[m].Cl[1], (int)d->n_pore, ns, (T)d->c0,
-        (float)(d->c0 - (double)(T)d->c0));
-    d->timing.kernel_launches++;
+        c_views<T>(d, hm[m].C[0]), (int)d->n_pore, ns, (T)d->c0, (T)(d->c0 - (double)(T)d->c0));
+    d->timing.kernel_launches += f64 ? 1 : 2;
     if (cudaMemsetAsync(hm[m].acc, 0, (size_t)3 * kMaxSpecies * d->np_accs * 8, d->stream) !=
         cudaSuccess)
       s = cdi_fail(d, CDI_ERR_CUDA, "sweep: memset");
+  }
+  int mode = NP_SMALL;
+  if (s == CDI_OK && !f64) {
+    std::vector<int> large(n);
+    if (cudaMemcpyAsync(large.data(), count, sizeof(int) * n, cudaMemcpyDeviceToHost,
+                        d->stream) != cudaSuccess || cudaStreamSynchronize(d->stream) != cudaSuccess)
+      s = cdi_fail(d, CDI_ERR_CUDA, "sweep: face data");
+    for (int m = 0; m < n && s == CDI_OK; m++)
+      if (large[m])
+        mode = member_bern(d, d->stream, hm[m].f, hm[m].u, take(bern_bytes(d)))
+                   ? std::max<int>(mode, NP_LARGE) : NP_EVAL;
   }
   if (s == CDI_OK &&
       cudaMemcpyAsync(dmem, hm.data(), sizeof(SweepMember<T>) * n, cudaMemcpyHostToDevice,
@@ -1550,7 +1696,7 @@ cdi_status sweep_run(cdi_domain *d, int n, const double *scale, const int *group
       cudaGraph_t graph;
       cudaError_t e = cudaStreamBeginCapture(d->cap_stream, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
-        for (int k = 0; k < kGraphSteps; k++) launch_sweep(d, d->cap_stream, dmem, n, k & 1);
+        for (int k = 0; k < kGraphSteps; k++) launch_sweep(d, d->cap_stream, dmem, n, k & 1, mode);
         e = cudaStreamEndCapture(d->cap_stream, &graph);
       }
       if (e == cudaSuccess) {
@@ -1564,7 +1710,7 @@ cdi_status sweep_run(cdi_domain *d, int n, const double *scale, const int *group
         done += kGraphSteps;
       }
     }
-    for (; s == CDI_OK && done < n_steps; done++) launch_sweep(d, d->stream, dmem, n, (int)(done & 1));
+    for (; s == CDI_OK && done < n_steps; done++) launch_sweep(d, d->stream, dmem, n, (int)(done & 1), mode);
     cudaError_t e = cudaGetLastError();
     if (s == CDI_OK && e != cudaSuccess) s = cdi_cuda_fail(d, e, "sweep step");
     cdi_timing_end(d, ev, PH_NP, n_steps);
@@ -1576,7 +1722,7 @@ cdi_status sweep_run(cdi_domain *d, int n, const double *scale, const int *group
   const double vol = d->dim == 2 ? d->dx * d->dx : d->dx * d->dx * d->dx;
   for (int m = 0; m < n && s == CDI_OK; m++) {
     k_np_sums<T><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        d->d_cmeta, hm[m].C[cur], hm[m].Cl[cur], hm[m].u, (int)d->n_pore, ns, vol, d->d_part,
+        d->d_cmeta, c_views<T>(d, hm[m].C[cur]), hm[m].u, (int)d->n_pore, ns, vol, d->d_part,
         d->d_counter + C_MASS, d->d_scal);
     acc_total(d, hm[m].acc, d->stream, d->d_scal);
     d->timing.kernel_launches += 2;
@@ -1613,26 +1759,37 @@ cdi_status sweep_run(cdi_domain *d, int n, const double *scale, const int *group
 // ---------------------------------------------------------------------------
 namespace {
 
-template <typename T, int DIM, bool PAIR>
+template <typename T, int DIM, bool PAIR, int MODE>
 void launch_batch_d(cudaStream_t st, int ns, const void *members, int n, int blocks, int in) {
   const BatchMember<T> *m = (const BatchMember<T> *)members;
   switch (ns) {
-    case 1: k_np_batch<T, DIM, 1, PAIR><<<blocks, kRowBlock, 0, st>>>(m, n, in); break;
-    case 2: k_np_batch<T, DIM, 2, PAIR><<<blocks, kRowBlock, 0, st>>>(m, n, in); break;
-    case 3: k_np_batch<T, DIM, 3, PAIR><<<blocks, kRowBlock, 0, st>>>(m, n, in); break;
-    default: k_np_batch<T, DIM, 4, PAIR><<<blocks, kRowBlock, 0, st>>>(m, n, in); break;
+    case 1: k_np_batch<T, DIM, 1, PAIR, MODE><<<blocks, kRowBlock, 0, st>>>(m, n, in); break;
+    case 2: k_np_batch<T, DIM, 2, PAIR, MODE><<<blocks, kRowBlock, 0, st>>>(m, n, in); break;
+    case 3: k_np_batch<T, DIM, 3, PAIR, MODE><<<blocks, kRowBlock, 0, st>>>(m, n, in); break;
+    default: k_np_batch<T, DIM, 4, PAIR, MODE><<<blocks, kRowBlock, 0, st>>>(m, n, in); break;
   }
 }
 
-template <typename T>
+template <int DIM, bool PAIR>
+void launch_batch32(cudaStream_t st, int ns, const void *members, int n, int blocks, int in,
+                    int mode) {
+  if (mode == NP_SMALL) launch_batch_d<float, DIM, PAIR, NP_SMALL>(st, ns, members, n, blocks, in);
+  else if (mode == NP_LARGE) launch_batch_d<float, DIM, PAIR, NP_LARGE>(st, ns, members, n, blocks, in);
+  else launch_batch_d<float, DIM, PAIR, NP_EVAL>(st, ns, members, n, blocks, in);
+}
+
 void launch_batch(const cdi_domain *lead, cudaStream_t st, const void *members, int n,
-                  int blocks, int in) {
-  if (std::is_same<T, float>::value && lead->cpair) {
-    if (lead->dim == 2) launch_batch_d<T, 2, true>(st, lead->ns, members, n, blocks, in);
-    else launch_batch_d<T, 3, true>(st, lead->ns, members, n, blocks, in);
+                  int blocks, int in, int mode) {
+  const int ns = lead->ns;
+  if (lead->prec == CDI_FP64) {
+    if (lead->dim == 2) launch_batch_d<double, 2, false, NP_SMALL>(st, ns, members, n, blocks, in);
+    else launch_batch_d<double, 3, false, NP_SMALL>(st, ns, members, n, blocks, in);
+  } else if (lead->cpair) {
+    if (lead->dim == 2) launch_batch32<2, true>(st, ns, members, n, blocks, in, mode);
+    else launch_batch32<3, true>(st, ns, members, n, blocks, in, mode);
   } else {
-    if (lead->dim == 2) launch_batch_d<T, 2, false>(st, lead->ns, members, n, blocks, in);
-    else launch_batch_d<T, 3, false>(st, lead->ns, members, n, blocks, in);
+    if (lead->dim == 2) launch_batch32<2, false>(st, ns, members, n, blocks, in, mode);
+    else launch_batch32<3, false>(st, ns, members, n, blocks, in, mode);
   }
 }
 
@@ -1642,6 +1799,7 @@ cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, const do
                      double *gamma, double *cout) {
   cdi_domain *L = doms[0];  // the lead: its stream, allocator and scratch serve the batch
   const int n = n_doms * n_combos, ns = L->ns;
+  const bool f64 = L->prec == CDI_FP64;
   std::vector<void *> blocks;
   auto take = [&](size_t bytes) {
     void *p = cdi_dev_alloc(L, bytes);
@@ -1655,20 +1813,18 @@ cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, const do
     cdi_domain *d = doms[m / n_combos];
     const size_t TN = (size_t)d->n_pore * sizeof(T);
     void *u = take((size_t)d->dim * TN);
-    void *c0 = take((size_t)kMaxSpecies * TN), *c1 = take((size_t)kMaxSpecies * TN);
+    const size_t CN = (size_t)ns * TN * (d->cpair ? 2 : 1);
+    void *c0 = take(CN), *c1 = take(CN);
     void *acc = take((size_t)3 * kMaxSpecies * d->np_accs * 8);
-    void *l0 = d->cpair ? take((size_t)kMaxSpecies * d->n_pore * 4) : nullptr;
-    void *l1 = d->cpair ? take((size_t)kMaxSpecies * d->n_pore * 4) : nullptr;
-    ok = u && c0 && c1 && acc && (!d->cpair || (l0 && l1));
+    float2 *fd = f64 ? nullptr : (float2 *)take((size_t)d->dim * d->n_pore * sizeof(float2));
+    ok = u && c0 && c1 && acc && (f64 || fd);
     if (!ok) break;
     d->dt = dts[m];
     hm[m].s.C[0] = (T *)c0;
     hm[m].s.C[1] = (T *)c1;
-    hm[m].s.Cl[0] = (float *)l0;
-    hm[m].s.Cl[1] = (float *)l1;
     for (int in = 0; in < 2; in++)
-      hm[m].s.f[in] = fields32(d, in ? c1 : c0, in ? (float *)l1 : (float *)l0, in ? c0 : c1,
-                               in ? (float *)l0 : (float *)l1, u, phis[group[m]], acc);
+      hm[m].s.f[in] = fields32(d, in ? c1 : c0, in ? c0 : c1, fd, nullptr, u,
+                               phis[group[m]], acc);
     hm[m].s.u = (const T *)u;
     hm[m].s.phi = (const typename PhiStore<T>::type *)phis[group[m]];
     hm[m].s.acc = (typename AccSlot<T>::type *)acc;
@@ -1679,6 +1835,8 @@ cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, const do
     total_blocks += d->np_blocks;
   }
   void *dmem = ok ? take(sizeof(BatchMember<T>) * n) : nullptr;
+  int *count = dmem ? (int *)take(sizeof(int) * n) : nullptr;  // a face with |P| >= 1/2, per member
+  if (!count) dmem = nullptr;
   cdi_status s = CDI_OK;
   if (!ok || !dmem) s = cdi_fail(L, CDI_ERR_OOM, "batch: device allocation failed");
   // member velocities on their domains' streams (after the lead's stream
@@ -1691,15 +1849,31 @@ cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, const do
   for (int i = 0; i < n_doms && s == CDI_OK; i++)
     if (cudaStreamSynchronize(doms[i]->stream) != cudaSuccess)
       s = cdi_fail(L, CDI_ERR_CUDA, "batch: member setup");
+  if (s == CDI_OK && cudaMemsetAsync(count, 0, sizeof(int) * n, L->stream) != cudaSuccess)
+    s = cdi_fail(L, CDI_ERR_CUDA, "batch: memset");
   for (int m = 0; m < n && s == CDI_OK; m++) {
     const cdi_domain *d = doms[m / n_combos];
+    if (!f64) member_faces(d, L->stream, hm[m].s.f, hm[m].s.u, count + m);
     k_np_init<T><<<kRedBlocks, kRedThreads, 0, L->stream>>>(
-        hm[m].s.C[0], hm[m].s.C[1], hm[m].s.Cl[0], hm[m].s.Cl[1], (int)d->n_pore, ns, (T)d->c0,
-        (float)(d->c0 - (double)(T)d->c0));
-    L->timing.kernel_launches++;
+        c_views<T>(d, hm[m].s.C[0]), (int)d->n_pore, ns, (T)d->c0,
+        (T)(d->c0 - (double)(T)d->c0));
+    L->timing.kernel_launches += f64 ? 1 : 2;
     if (cudaMemsetAsync(hm[m].s.acc, 0, (size_t)3 * kMaxSpecies * d->np_accs * 8,
                         L->stream) != cudaSuccess)
       s = cdi_fail(L, CDI_ERR_CUDA, "batch: memset");
+  }
+  int mode = NP_SMALL;
+  if (s == CDI_OK && !f64) {
+    std::vector<int> large(n);
+    if (cudaMemcpyAsync(large.data(), count, sizeof(int) * n, cudaMemcpyDeviceToHost,
+                        L->stream) != cudaSuccess || cudaStreamSynchronize(L->stream) != cudaSuccess)
+      s = cdi_fail(L, CDI_ERR_CUDA, "batch: face data");
+    for (int m = 0; m < n && s == CDI_OK; m++) {
+      const cdi_domain *d = doms[m / n_combos];
+      if (large[m])
+        mode = member_bern(d, L->stream, hm[m].s.f, hm[m].s.u, take(bern_bytes(d)))
+                   ? std::max<int>(mode, NP_LARGE) : NP_EVAL;
+    }
   }
   if (s == CDI_OK &&
       cudaMemcpyAsync(dmem, hm.data(), sizeof(BatchMember<T>) * n, cudaMemcpyHostToDevice,
@@ -1715,7 +1889,7 @@ cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, const do
       cudaError_t e = cudaStreamBeginCapture(L->cap_stream, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
         for (int k = 0; k < kGraphSteps; k++)
-          launch_batch<T>(L, L->cap_stream, dmem, n, total_blocks, k & 1);
+          launch_batch(L, L->cap_stream, dmem, n, total_blocks, k & 1, mode);
         e = cudaStreamEndCapture(L->cap_stream, &graph);
       }
       if (e == cudaSuccess) {
@@ -1730,7 +1904,7 @@ cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, const do
       }
     }
     for (; s == CDI_OK && done < n_steps; done++)
-      launch_batch<T>(L, L->stream, dmem, n, total_blocks, (int)(done & 1));
+      launch_batch(L, L->stream, dmem, n, total_blocks, (int)(done & 1), mode);
     cudaError_t e = cudaGetLastError();
     if (s == CDI_OK && e != cudaSuccess) s = cdi_cuda_fail(L, e, "batch step");
     cdi_timing_end(L, ev, PH_NP, n_steps);
@@ -1743,7 +1917,7 @@ cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, const do
     const double area = d->dim == 2 ? d->dx : d->dx * d->dx;
     const double vol = d->dim == 2 ? d->dx * d->dx : d->dx * d->dx * d->dx;
     k_np_sums<T><<<kRedBlocks, kRedThreads, 0, L->stream>>>(
-        d->d_cmeta, hm[m].s.C[cur], hm[m].s.Cl[cur], hm[m].s.u, (int)d->n_pore, ns, vol,
+        d->d_cmeta, c_views<T>(d, hm[m].s.C[cur]), hm[m].s.u, (int)d->n_pore, ns, vol,
         L->d_part, L->d_counter + C_MASS, L->d_scal);
     acc_total(d, hm[m].s.acc, L->stream, L->d_scal);
     L->timing.kernel_launches += 2;
@@ -1871,11 +2045,11 @@ cdi_status cdi_np_reduce(cdi_domain *d) {
   const double vol = d->dim == 2 ? d->dx * d->dx : d->dx * d->dx * d->dx;
   if (d->prec == CDI_FP64)
     k_np_sums<double><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        d->d_cmeta, (const double *)d->d_C[d->cur], nullptr, (const double *)d->d_u,
+        d->d_cmeta, c_views<double>(d, d->d_C[d->cur]), (const double *)d->d_u,
         (int)d->n_pore, d->ns, vol, d->d_part, d->d_counter + C_MASS, d->d_scal);
   else
     k_np_sums<float><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        d->d_cmeta, (const float *)d->d_C[d->cur], d->d_Clo[d->cur], (const float *)d->d_u,
+        d->d_cmeta, c_views<float>(d, d->d_C[d->cur]), (const float *)d->d_u,
         (int)d->n_pore, d->ns, vol, d->d_part, d->d_counter + C_MASS, d->d_scal);
   acc_total(d, d->d_acc, d->stream, d->d_scal);
   d->timing.kernel_launches += 2;
@@ -1911,16 +2085,13 @@ cdi_status cdi_np_geometry(cdi_domain *d, double *pores, double *faces, double *
 }
 
 cdi_status cdi_np_column_means(cdi_domain *d, int k) {
-  const size_t T = d->prec == CDI_FP64 ? 8 : 4;
-  const void *C = (const char *)d->d_C[d->cur] + (size_t)k * d->n_pore * T;
-  const float *Cl = d->d_Clo[d->cur] ? d->d_Clo[d->cur] + (size_t)k * d->n_pore : nullptr;
   const int rows = d->ny * d->nz;
   if (d->prec == CDI_FP64)
-    k_colmeans<double><<<d->nx, kRedThreads, 0, d->stream>>>(d->d_words, d->W, (const double *)C,
-                                                             nullptr, rows, d->d_colout);
+    k_colmeans<double><<<d->nx, kRedThreads, 0, d->stream>>>(
+        d->d_words, d->W, c_view<double>(d, d->d_C[d->cur], k), rows, d->d_colout);
   else
-    k_colmeans<float><<<d->nx, kRedThreads, 0, d->stream>>>(d->d_words, d->W, (const float *)C,
-                                                            Cl, rows, d->d_colout);
+    k_colmeans<float><<<d->nx, kRedThreads, 0, d->stream>>>(
+        d->d_words, d->W, c_view<float>(d, d->d_C[d->cur], k), rows, d->d_colout);
   d->timing.kernel_launches++;
   CDI_TRY(d, cudaGetLastError(), "column means");
   return CDI_OK;
@@ -1937,23 +2108,55 @@ cdi_status cdi_np_build_compact(cdi_domain *d) {
                                                      n_words, d->d_words);
   k_lat_nbr<<<kRedBlocks, kRedThreads, 0, d->stream>>>(d->d_cmeta, d->d_words, n, d->W, d->ny,
                                                        d->nz, d->walls, 2 * d->dim, d->d_latnb);
-  d->timing.kernel_launches += 3;
+  if (d->dim == 2)
+    k_lat_pack<2><<<kRedBlocks, kRedThreads, 0, d->stream>>>(d->d_latnb, n, d->d_latd, d->d_latb);
+  else
+    k_lat_pack<3><<<kRedBlocks, kRedThreads, 0, d->stream>>>(d->d_latnb, n, d->d_latd, d->d_latb);
+  d->timing.kernel_launches += 4;
   CDI_TRY(d, cudaGetLastError(), "compact layout");
   return CDI_OK;
 }
 
-// comps rank-ordered components of the domain's precision -> FP64 lattice
-// fields (dst: comps * N doubles, 0 in solid cells).
-cdi_status cdi_np_scatter(cdi_domain *d, const void *src, const float *lo, int comps,
-                          double *dst) {
+// Rank-ordered fields of the domain's precision (species k of the current
+// concentrations, or with species < 0 the dim velocity components) -> FP64
+// lattice fields (dst: N doubles each, 0 in solid cells).
+template <typename T> static void scatter(cdi_domain *d, int species, double *dst) {
+  CViews<T> v{};
+  int comps = 1;
+  if (species >= 0) {
+    v.v[0] = c_view<T>(d, d->d_C[d->cur], species);
+  } else {
+    comps = d->dim;
+    for (int a = 0; a < comps; a++)
+      v.v[a] = CView<T>{(const T *)d->d_u + (size_t)a * d->n_pore, 1, 0};
+  }
+  k_scatter<T><<<kRedBlocks, kRedThreads, 0, d->stream>>>(v, comps, d->d_cell_list,
+                                                          (int)d->n_pore, d->N, dst);
+}
+cdi_status cdi_np_scatter(cdi_domain *d, int species, double *dst) {
+  const int comps = species >= 0 ? 1 : d->dim;
   CDI_TRY(d, cudaMemsetAsync(dst, 0, (size_t)comps * d->N * 8, d->stream), "scatter reset");
-  if (d->prec == CDI_FP64)
-    k_scatter<double><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        (const double *)src, nullptr, comps, d->d_cell_list, (int)d->n_pore, d->N, dst);
-  else
-    k_scatter<float><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        (const float *)src, lo, comps, d->d_cell_list, (int)d->n_pore, d->N, dst);
+  if (d->prec == CDI_FP64) scatter<double>(d, species, dst);
+  else scatter<float>(d, species, dst);
   d->timing.kernel_launches++;
   CDI_TRY(d, cudaGetLastError(), "scatter");
+  return CDI_OK;
+}
+
+// FP32 concentrations of buffer b as the planes of a saved state, and back.
+cdi_status cdi_np_records_to_planes(cdi_domain *d, int b, float *planes) {
+  const size_t np = (size_t)kMaxSpecies * d->n_pore;
+  k_records_to_planes<<<kRedBlocks, kRedThreads, 0, d->stream>>>(
+      c_views<float>(d, d->d_C[b]), (int)d->n_pore, d->ns, planes, d->cpair ? planes + np : nullptr);
+  d->timing.kernel_launches++;
+  CDI_TRY(d, cudaGetLastError(), "state planes");
+  return CDI_OK;
+}
+cdi_status cdi_np_planes_to_records(cdi_domain *d, const float *planes, int b) {
+  const size_t np = (size_t)kMaxSpecies * d->n_pore;
+  k_planes_to_records<<<kRedBlocks, kRedThreads, 0, d->stream>>>(
+      c_views<float>(d, d->d_C[b]), (int)d->n_pore, d->ns, planes, d->cpair ? planes + np : nullptr);
+  d->timing.kernel_launches++;
+  CDI_TRY(d, cudaGetLastError(), "state planes");
   return CDI_OK;
 }
