@@ -280,8 +280,9 @@ struct cdi_domain {
                                 // one after the other: c_2p[, c_2p+1][, their low
                                 // words] (see c_view); the layout follows ns
   float2 *d_fd = nullptr;       // FP32: dim * n_pore face data (see k_np_faces)
-  float2 *d_bern = nullptr;     // FP32: Bernoulli pairs of the faces with |P| >= 1/2
-                                // (taken the first time there is one)
+  void *d_bern = nullptr;       // FP32: Bernoulli pairs of the faces with |P| >= 1/2
+                                // (taken the first time there is one); FP64: face
+                                // coefficients (taken by the first transport state)
   size_t bern_bytes = 0;
   int np_mode = 0;              // which kernel the faces ask for (see np_warp31)
   short *d_latd = nullptr;      // 2*(dim-1) 16-bit lateral differences per rank

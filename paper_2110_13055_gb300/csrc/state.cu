@@ -165,8 +165,9 @@ cdi_status cdi_load_state(cdi_domain *d, const void *host_buf, size_t bytes) {
   d->flow_steps = h.flow_steps; d->np_steps = h.np_steps;
   d->psi_s = h.psi_s; d->eps_r = h.eps_r; d->psi_tol = h.psi_tol;
   d->psi_max_iter = (int)h.psi_max_iter; d->couple_K = h.couple_K;
-  if (d->prec != CDI_FP64) {
-    cdi_status rs = cdi_np_planes_to_records(d, (const float *)d->d_cg, 0);
+  if (d->np_ready) {
+    cdi_status rs = CDI_OK;
+    if (d->prec != CDI_FP64) rs = cdi_np_planes_to_records(d, (const float *)d->d_cg, 0);
     if (rs == CDI_OK) rs = cdi_np_faces(d);
     if (rs != CDI_OK) return rs;
     CDI_TRY(d, cudaStreamSynchronize(d->stream), "load_state");

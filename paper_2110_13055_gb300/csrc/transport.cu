@@ -110,15 +110,9 @@ __device__ __forceinline__ int lateral_row(unsigned f, int fc, int row, int ny, 
   return row + (edge ? -s * (ext - 1) * step : s * step);
 }
 
-// Face flux divided by D/dx, J' = B(-P) C_P - B(P) C_nb, for the face Peclet
-// number P = adv - z (phi_nb - phi_P); dd is phi_nb - phi_P.
-__device__ __forceinline__ double face_flux(double adv, double z, double dd, double, double,
-                                            double CP, double Cn) {
-  double Bp, Bm;
-  bernoulli_pair(r_fma(-z, dd, adv), Bp, Bm);
-  return r_fma(Bm, CP, -r_mul(Bp, Cn));
-}
-
+// Face flux divided by D/dx: J' = B(-P) C_P - B(P) C_nb, for the face Peclet
+// number P = adv - z (phi_nb - phi_P).
+//
 // FP32: phi and P are carried as unevaluated pairs (hi + lo) where it
 // matters: an exponent |P| rounded to FP32 costs a relative error of about
 // |P| * 6e-8 in each Boltzmann factor exp(P), which accumulates across an
@@ -162,7 +156,7 @@ __device__ __forceinline__ float phi_diff(float2 nb, float2 pp) {
 
 // Geometry of the compact transport layout handed to the FP64 step kernels.
 struct NPGeo {
-  const uint2 *meta;   // per rank {flags | x << 16, row}
+  const NFlag *fl;     // per rank: its face flags
   const int *lat;      // per lateral face f (y+, y-, z+, z-) and rank r, at
                        // (f - 2) * n + r: the pore neighbour's rank, or -1
   int n;
@@ -202,91 +196,70 @@ struct NPFields {
 };
 __host__ __device__ constexpr long long np_warps(long long n) { return (n + kHome - 1) / kHome; }
 
-// One explicit step of the pore cell of rank r for NS species: writes the
-// new concentrations and adds the cell's adsorbed (v[k]), inflow (v[NS+k])
-// and outflow (v[2NS+k]) fluxes.  Returns whether the cell has an inlet or
-// outlet face.
+// FP64 storage: one explicit step of species k at the pore cell of rank r.
+// Writes the new concentration and returns the cell's adsorbed, inflow and
+// outflow fluxes in v (io: it has an inlet or outlet face).  One thread per
+// cell and species: the arithmetic is a chain of FP64 operations at a rate of
+// 2 a clock and SM, so more, shorter threads are what hides it.
 //
-// A face that does not lead to a pore cell reads the cell's own values: the
-// outlet ghost copies the cell (J = u_x C_P), the inlet ghost then takes
-// C = c0 and phi = 0, and a solid or wall face gets u_f = 0, for which the
-// flux expression is exactly 0 (C_nb = C_P, dphi = 0); the adsorption flux of
-// the n_s solid faces, n_s K_eff C_P, is added once per cell.
-template <typename T, int DIM, int NS>
-__device__ __forceinline__ bool np_cell(const T *__restrict__ Cin, T *__restrict__ Cout,
-                                        const T *__restrict__ u,
-                                        const typename PhiStore<T>::type *__restrict__ phi,
-                                        const NPGeo &g, uint2 meta, int r, const NPConst<T> &c,
-                                        T (&v)[3 * NS]) {
-  using PT = typename PhiStore<T>::type;
+// The outlet ghost copies the cell (J = u_x C_P), the feed ghost has C = c0
+// and phi = 0, a closed face has no flux, and the adsorption flux of the n_s
+// solid faces, n_s K_eff C_P, is added once per cell.
+//
+// co: the stored face coefficients ((D/dx) B(P), (D/dx) B(-P)) of + face a at
+// co[a * n + r], and of the feed face at a = DIM (k_np_coef64); a - face is
+// the + face of the cell across it with the two exchanged.  They take the
+// exponentials and divisions (about 60 FP64 operations a face) out of the
+// step: 128x64 image, two species: 16.4 -> 4.0 us a step.  co null (no memory
+// for them): every face is evaluated from the velocity and the potential.
+template <int DIM>
+__device__ __forceinline__ bool np_cell(const double *__restrict__ Cin, double *__restrict__ Cout,
+                                        const double2 *__restrict__ co,
+                                        const double *__restrict__ u,
+                                        const double *__restrict__ phi, const NPGeo &g,
+                                        unsigned f, int r, const NPConst<double> &c, int k,
+                                        double (&v)[3]) {
   constexpr int NF = 2 * DIM;
-  const unsigned f = meta.x & 0xffffu;
   const size_t n = (size_t)g.n;
-  // neighbour ranks first (x neighbours are the adjacent ranks, lateral ones
-  // come from the table)
-  int Q[NF];
-  bool open[NF];
-#pragma unroll
-  for (int fc = 0; fc < NF; fc++) {
-    const bool solid = (f >> (kFaceBit + fc)) & 1u;
-    const bool edge = (f >> (kEdgeBit + fc)) & 1u;
-    if (fc < 2) {
-      open[fc] = !solid;
-      Q[fc] = (solid || edge) ? r : r + ((fc & 1) ? -1 : 1);
-    } else {
-      // the lateral neighbour's rank, found once at set-up from the row words
-      const int q = g.lat[(size_t)(fc - 2) * n + r];
-      open[fc] = q >= 0;
-      Q[fc] = q >= 0 ? q : r;
-    }
-  }
-  // every load before any arithmetic (memory-level parallelism)
-  T CP[NS], Cn[NF][NS], uP[DIM], un[NF];
-  PT phn[NF];
-#pragma unroll
-  for (int k = 0; k < NS; k++) CP[k] = Cin[k * n + r];
-#pragma unroll
-  for (int a = 0; a < DIM; a++) uP[a] = u[a * n + r];
-  const PT phP = phi[r];
-#pragma unroll
-  for (int fc = 0; fc < NF; fc++) {
-    un[fc] = u[(fc >> 1) * n + Q[fc]];
-    phn[fc] = phi[Q[fc]];
-#pragma unroll
-    for (int k = 0; k < NS; k++) Cn[fc][k] = Cin[k * n + Q[fc]];
-  }
-  // the feed ghost across the inlet face (face 1 at x = 0)
   const bool inlet = (f >> (kEdgeBit + 1)) & 1u, outlet = (f >> kEdgeBit) & 1u;
-  if (inlet) {
-    phn[1] = PhiStore<T>::zero();
+  int q[NF];  // rank across the face (own rank at the inlet and outlet), -1 closed
+  q[0] = (f >> kFaceBit) & 1u ? -1 : (outlet ? r : r + 1);
+  q[1] = (f >> (kFaceBit + 1)) & 1u ? -1 : (inlet ? r : r - 1);
 #pragma unroll
-    for (int k = 0; k < NS; k++) Cn[1][k] = c.c0;
-  }
-  // adsorption on the solid faces (Eq. 6)
-  const T ns_solid = (T)__popc(f & (((1u << NF) - 1u) << kFaceBit));
-  T sumJ[NS];
-#pragma unroll
-  for (int k = 0; k < NS; k++) {
-    const T Ja = r_mul(r_mul(ns_solid, c.Keff[k]), CP[k]);
-    sumJ[k] = Ja;
-    v[k] = r_add(v[k], Ja);
-  }
+  for (int fc = 2; fc < NF; fc++) q[fc] = g.lat[(size_t)(fc - 2) * n + r];
+  const double CP = Cin[r];
+  double Cn[NF], Bp[NF], Bm[NF];
 #pragma unroll
   for (int fc = 0; fc < NF; fc++) {
-    const T half = (fc & 1) ? T(-0.5) : T(0.5);
-    const T uf = open[fc] ? r_mul(half, r_add(uP[fc >> 1], un[fc])) : T(0);
-    const T dd = phi_diff(phn[fc], phP);
-#pragma unroll
-    for (int k = 0; k < NS; k++) {
-      const T J = r_mul(c.Ddx[k], face_flux(r_mul(uf, c.dxD[k]), c.zf[k], dd, phn[fc], phP,
-                                            CP[k], Cn[fc][k]));
-      sumJ[k] = r_add(sumJ[k], J);
-      if (fc == 1 && inlet) v[NS + k] = r_sub(v[NS + k], J);
-      if (fc == 0 && outlet) v[2 * NS + k] = r_add(v[2 * NS + k], J);
+    Cn[fc] = Bp[fc] = Bm[fc] = 0.0;
+    if (q[fc] < 0) continue;
+    Cn[fc] = Cin[q[fc]];
+    if (co) {
+      const bool feed = fc == 1 && inlet, flip = (fc & 1) && !feed;
+      const double2 b = co[feed ? DIM * n + r : (fc >> 1) * n + (flip ? q[fc] : r)];
+      Bp[fc] = flip ? b.y : b.x;
+      Bm[fc] = flip ? b.x : b.y;
+    } else {
+      const double *ua = u + (fc >> 1) * n;
+      const double uf = r_mul((fc & 1) ? -0.5 : 0.5, r_add(ua[r], ua[q[fc]]));
+      const double dd = phi_diff(fc == 1 && inlet ? 0.0 : phi[q[fc]], phi[r]);
+      bernoulli_pair(r_fma(-c.zf[k], dd, r_mul(uf, c.dxD[k])), Bp[fc], Bm[fc]);
+      Bp[fc] = r_mul(c.Ddx[k], Bp[fc]);
+      Bm[fc] = r_mul(c.Ddx[k], Bm[fc]);
     }
   }
+  if (inlet) Cn[1] = c.c0;
+  const double ns_solid = (double)__popc(f & (((1u << NF) - 1u) << kFaceBit));
+  v[0] = r_mul(r_mul(ns_solid, c.Keff[k]), CP);
+  double sumJ = v[0];
 #pragma unroll
-  for (int k = 0; k < NS; k++) Cout[k * n + r] = r_fma(-c.dtdx, sumJ[k], CP[k]);
+  for (int fc = 0; fc < NF; fc++) {
+    const double J = r_fma(Bm[fc], CP, -r_mul(Bp[fc], Cn[fc]));
+    sumJ = r_add(sumJ, J);
+    if (fc == 1 && inlet) v[1] = -J;
+    if (fc == 0 && outlet) v[2] = J;
+  }
+  Cout[r] = r_fma(-c.dtdx, sumJ, CP);
   return inlet || outlet;
 }
 
@@ -311,37 +284,28 @@ __device__ __forceinline__ void acc_add(float2 *a, float v) {
 __device__ __forceinline__ double acc_value(double a) { return a; }
 __device__ __forceinline__ double acc_value(float2 a) { return (double)a.x + (double)a.y; }
 
-// Warp sums of v in T, added by lane 0 to the warp's own accounts
-// acc[(3*k + kind) * nw + wid], kind 0 Gamma, 1 In, 2 Out (one thread per
-// pore cell, so the warp -> cells map is fixed and the totals are
-// deterministic).  A warp without inlet or outlet cells skips the In/Out sums
-// (its values are 0).  No block barrier: each warp retires on its own.  All
-// 32 lanes of the warp must call it.
-template <typename T, int NS>
-__device__ __forceinline__ void np_account(T (&v)[3 * NS], bool io,
-                                           typename AccSlot<T>::type *__restrict__ acc,
+// Warp sums of one species' fluxes v (FP64), added by lane 0 to the warp's own
+// accounts acc[kind * nw + wid], kind 0 Gamma, 1 In, 2 Out (a fixed warp ->
+// cells map, so the totals are deterministic).  A warp without inlet or
+// outlet cells skips the In/Out sums (its values are 0).  All 32 lanes of the
+// warp must call it.
+__device__ __forceinline__ void np_account(double (&v)[3], bool io, double *__restrict__ acc,
                                            int wid, int nw) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-    for (int k = 0; k < NS; k++) v[k] = r_add(v[k], __shfl_down_sync(0xffffffffu, v[k], o));
   const bool any_io = __any_sync(0xffffffffu, io);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v[0] = r_add(v[0], __shfl_down_sync(0xffffffffu, v[0], o));
   if (any_io) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-      for (int k = NS; k < 3 * NS; k++)
-        v[k] = r_add(v[k], __shfl_down_sync(0xffffffffu, v[k], o));
+      for (int j = 1; j < 3; j++) v[j] = r_add(v[j], __shfl_down_sync(0xffffffffu, v[j], o));
   }
   if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-    for (int k = 0; k < NS; k++) {
-      typename AccSlot<T>::type *a = acc + (size_t)(3 * k) * nw + wid;
-      acc_add(a, v[k]);
-      if (any_io) {
-        acc_add(a + nw, v[NS + k]);
-        acc_add(a + 2 * (size_t)nw, v[2 * NS + k]);
-      }
+    double *a = acc + wid;
+    acc_add(a, v[0]);
+    if (any_io) {
+      acc_add(a + nw, v[1]);
+      acc_add(a + 2 * (size_t)nw, v[2]);
     }
   }
 }
@@ -582,8 +546,8 @@ template <int DIM, int NS> struct NPLane {
 
 // The update of warp w's tile from the values in V.  The +x face flux is
 // evaluated once per face and handed to the next lane as its -x flux; per
-// home cell the faces are summed in the order of np_cell (adsorption, +x, -x,
-// +y, -y, +z, -z).  SMALL: every face of the warp has |P| < 1/2, so the
+// home cell the faces are summed in the order adsorption, +x, -x, +y,
+// -y, +z, -z.  SMALL: every face of the warp has |P| < 1/2, so the
 // arithmetic has no branch and its faces overlap.  EVAL: the Bernoulli pairs are not stored (no memory for
 // them) and are evaluated at every step.
 template <int DIM, int NS, bool PAIR, bool SMALL, bool EVAL>
@@ -893,19 +857,49 @@ __global__ void k_lat_pack(const int *__restrict__ lat, int n, short *__restrict
   }
 }
 
-template <typename T, int DIM, int NS>
-__device__ __forceinline__ void np_step_body(const T *__restrict__ Cin, T *__restrict__ Cout,
-                                             const T *__restrict__ u,
-                                             const typename PhiStore<T>::type *__restrict__ phi,
-                                             const NPGeo &g, const NPConst<T> &c,
-                                             typename AccSlot<T>::type *__restrict__ acc,
-                                             int r) {
-  T v[3 * NS];
+// The face coefficients of np_cell: species k's at co[k * (DIM + 1) * n + ...].
+template <int DIM>
+__global__ void k_np_coef64(const NFlag *__restrict__ fl, const int *__restrict__ lat, int n,
+                            const double *__restrict__ u, const double *__restrict__ phi,
+                            NPConst<double> c, int ns, double2 *__restrict__ co) {
+  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
+    const unsigned f = fl[r];
+    const double phP = phi[r];
+    auto put = [&](int a, double uf, double dd) {
+      for (int k = 0; k < ns; k++) {
+        double Bp, Bm;
+        bernoulli_pair(r_fma(-c.zf[k], dd, r_mul(uf, c.dxD[k])), Bp, Bm);
+        co[((size_t)k * (DIM + 1) + a) * n + r] =
+            make_double2(r_mul(c.Ddx[k], Bp), r_mul(c.Ddx[k], Bm));
+      }
+    };
 #pragma unroll
-  for (int j = 0; j < 3 * NS; j++) v[j] = T(0);
+    for (int a = 0; a < DIM; a++) {
+      const double uP = u[(size_t)a * n + r];
+      const int q = plus_face(f, lat, n, a, r);
+      if (q >= 0) put(a, r_mul(0.5, r_add(uP, u[(size_t)a * n + q])), phi_diff(phi[q], phP));
+    }
+    if ((f >> (kEdgeBit + 1)) & 1u) put(DIM, r_mul(-0.5, r_add(u[r], u[r])), phi_diff(0.0, phP));
+  }
+}
+
+// One FP64 step of species k at rank r (of all 32 ranks of its warp) and its
+// account.
+template <int DIM>
+__device__ __forceinline__ void np_step_body(const double *__restrict__ Cin,
+                                             double *__restrict__ Cout,
+                                             const double *__restrict__ u,
+                                             const double *__restrict__ phi,
+                                             const double2 *__restrict__ co, const NPGeo &g,
+                                             const NPConst<double> &c, double *__restrict__ acc,
+                                             int r, int k) {
+  const size_t n = (size_t)g.n;
+  double v[3] = {0.0, 0.0, 0.0};
   bool io = false;
-  if (r < g.n) io = np_cell<T, DIM, NS>(Cin, Cout, u, phi, g, g.meta[r], r, c, v);
-  np_account<T, NS>(v, io, acc, r >> 5, g.naccs);
+  if (r < g.n)
+    io = np_cell<DIM>(Cin + k * n, Cout + k * n, co ? co + (size_t)k * (DIM + 1) * n : nullptr, u,
+                      phi, g, g.fl[r], r, c, k, v);
+  np_account(v, io, acc + (size_t)(3 * k) * g.naccs, r >> 5, g.naccs);
 }
 
 // Has the inputs of the tiles `ahead` of this block's fetched into L2 (one
@@ -957,14 +951,15 @@ __global__ void __launch_bounds__(BS)
   np_warp31<DIM, NS, PAIR, MODE>(F, n, naccs, c, w);
 }
 
-// FP64 storage, one thread per pore cell.
-template <typename T, int DIM, int NS, int BS>
+// FP64 storage, one thread per pore cell and species (blockIdx.y).
+template <int DIM, int BS>
 __global__ void __launch_bounds__(BS)
-    k_np_step(const T *__restrict__ Cin, T *__restrict__ Cout, const T *__restrict__ u,
-              const typename PhiStore<T>::type *__restrict__ phi, NPGeo g, NPConst<T> c,
-              typename AccSlot<T>::type *__restrict__ acc) {
-  np_step_body<T, DIM, NS>(Cin, Cout, u, phi, g, c, acc,
-                           (int)(blockIdx.x * blockDim.x + threadIdx.x));
+    k_np_step(const double *__restrict__ Cin, double *__restrict__ Cout,
+              const double *__restrict__ u, const double *__restrict__ phi,
+              const double2 *__restrict__ co, NPGeo g, NPConst<double> c,
+              double *__restrict__ acc) {
+  np_step_body<DIM>(Cin, Cout, u, phi, co, g, c, acc, (int)(blockIdx.x * BS + threadIdx.x),
+                    (int)blockIdx.y);
 }
 
 // One member of a fused sweep: its own concentrations, velocity, potential,
@@ -974,6 +969,7 @@ template <typename T> struct SweepMember {
   NPFields f[2];    // FP32: the fields of a step from buffer 0 / 1
   const T *u;
   const typename PhiStore<T>::type *phi;
+  const double2 *co;  // FP64: face coefficients (null: evaluated at every step)
   typename AccSlot<T>::type *acc;
   NPConst<T> c;
 };
@@ -990,7 +986,8 @@ __global__ void __launch_bounds__(kRowBlock)
   if constexpr (std::is_same<T, float>::value)
     np_warp31<DIM, NS, PAIR, MODE>(mb.f[in], g.n, g.naccs, mb.c, r >> 5);
   else
-    np_step_body<T, DIM, NS>(mb.C[in], mb.C[1 - in], mb.u, mb.phi, g, mb.c, mb.acc, r);
+    for (int k = 0; k < NS; k++)
+      np_step_body<DIM>(mb.C[in], mb.C[1 - in], mb.u, mb.phi, mb.co, g, mb.c, mb.acc, r, k);
 }
 
 // One member of a batch over several geometries: a sweep member plus its
@@ -1022,8 +1019,9 @@ __global__ void __launch_bounds__(kRowBlock)
   if constexpr (std::is_same<T, float>::value)
     np_warp31<DIM, NS, PAIR, MODE>(mb.s.f[in], mb.g.n, mb.g.naccs, mb.s.c, r >> 5);
   else
-    np_step_body<T, DIM, NS>(mb.s.C[in], mb.s.C[1 - in], mb.s.u, mb.s.phi, mb.g, mb.s.c,
-                             mb.s.acc, r);
+    for (int k = 0; k < NS; k++)
+      np_step_body<DIM>(mb.s.C[in], mb.s.C[1 - in], mb.s.u, mb.s.phi, mb.s.co, mb.g, mb.s.c,
+                        mb.s.acc, r, k);
 }
 
 // Largest outflow rate over pore cells and species, in FP64 from the FP64
@@ -1365,12 +1363,21 @@ void launch_bern(const cdi_domain *d, cudaStream_t st, const void *u, const void
   kern<<<grid, 256, 0, st>>>(d->d_cfl, d->d_latnb, n, (const float *)u, (const float2 *)phi, fd, c,
                              d->ns, bern);
 }
+void launch_coef64(const cdi_domain *d, cudaStream_t st, const void *u, const void *phi,
+                   void *co) {
+  const int n = (int)d->n_pore, grid = std::min((n + 127) / 128, 16 * kRedBlocks);
+  auto *kern = d->dim == 2 ? k_np_coef64<2> : k_np_coef64<3>;
+  kern<<<grid, 128, 0, st>>>(d->d_cfl, d->d_latnb, n, (const double *)u, (const double *)phi,
+                             make_const<double>(d), d->ns, (double2 *)co);
+}
+// Bytes of the stored Bernoulli pairs (FP32) or face coefficients (FP64).
 size_t bern_bytes(const cdi_domain *d) {
-  return (size_t)(d->dim + 1) * d->n_pore * d->ns * sizeof(float2);
+  return (size_t)(d->dim + 1) * d->n_pore * d->ns *
+         (d->prec == CDI_FP64 ? sizeof(double2) : sizeof(float2));
 }
 
 NPGeo make_geo(const cdi_domain *d) {
-  return NPGeo{d->d_cmeta, d->d_latnb, (int)d->n_pore, d->np_accs};
+  return NPGeo{d->d_cfl, d->d_latnb, (int)d->n_pore, d->np_accs};
 }
 
 // Tiles between a block and the ones whose inputs it has fetched into L2: one
@@ -1389,7 +1396,7 @@ void launch_step_bs(cdi_domain *d, cudaStream_t st, int in) {
   const long long units = std::is_same<T, float>::value ? np_warps(d->n_pore) * 32 : d->n_pore;
   const int grid = (int)((units + BS - 1) / BS);
   if constexpr (std::is_same<T, float>::value) {
-    const NPFields F = fields32(d, d->d_C[in], d->d_C[1 - in], d->d_fd, d->d_bern, d->d_u,
+    const NPFields F = fields32(d, d->d_C[in], d->d_C[1 - in], d->d_fd, (const float2 *)d->d_bern, d->d_u,
                                 d->d_phi, d->d_acc);
     auto *kern = d->np_mode == NP_SMALL   ? k_np_step32<DIM, NS, BS, PAIR, NP_SMALL>
                  : d->np_mode == NP_LARGE ? k_np_step32<DIM, NS, BS, PAIR, NP_LARGE>
@@ -1397,10 +1404,10 @@ void launch_step_bs(cdi_domain *d, cudaStream_t st, int in) {
     kern<<<grid, BS, 0, st>>>(F, (int)d->n_pore, d->np_accs, make_const<float>(d),
                               np_ahead_tiles(d));
   } else {
-    k_np_step<T, DIM, NS, BS><<<grid, BS, 0, st>>>(
-        (const T *)d->d_C[in], (T *)d->d_C[1 - in], (const T *)d->d_u,
-        (const typename PhiStore<T>::type *)d->d_phi, make_geo(d), make_const<T>(d),
-        (typename AccSlot<T>::type *)d->d_acc);
+    k_np_step<DIM, BS><<<dim3(grid, NS), BS, 0, st>>>(
+        (const double *)d->d_C[in], (double *)d->d_C[1 - in], (const double *)d->d_u,
+        (const double *)d->d_phi, d->np_mode == NP_EVAL ? nullptr : (const double2 *)d->d_bern,
+        make_geo(d), make_const<double>(d), d->d_acc);
   }
 }
 
@@ -1442,10 +1449,9 @@ constexpr int kGraphSteps = 64;  // steps per captured transport graph (even)
 // again.  128 is taken unless a shape is fixed: it is the fastest or within
 // 4 % of it on every size measured (256^3: 155 / 139 / 154 us for 64 / 128 /
 // 256; 1024x512: 5.8 / 5.8 / 5.9; 96^3: 11.3 / 10.6 / 11.1), so no launch is
-// spent on timing candidates (FP64 storage: 64 threads, 16.5 / 17.7 / 30.2 us
-// on 128x64).  Accounts are kept per warp whatever the shape, so every choice
-// computes the same bits.
-constexpr int kNpDefaultShape = 1, kNpDefaultShape64 = 0;
+// spent on timing candidates (FP64, 128x64: 4.0 / 4.0 / 4.9).  Accounts are
+// kept per warp whatever the shape, so every choice computes the same bits.
+constexpr int kNpDefaultShape = 1;
 constexpr int kNpVariantBlock[10] = {64, 128, 256, 128, 128, 128, 128, 128, 128, 128};
 
 }  // namespace
@@ -1479,7 +1485,7 @@ cdi_status cdi_np_init(cdi_domain *d, double dt_s, double *dt_used) {
   cdi_status fs = cdi_np_faces(d);
   if (fs != CDI_OK) return fs;
   if (!d->np_tuned) {
-    d->np_variant = d->prec == CDI_FP64 ? kNpDefaultShape64 : kNpDefaultShape;
+    d->np_variant = kNpDefaultShape;
     d->np_block = kNpVariantBlock[d->np_variant];
     d->np_tuned = true;
   }
@@ -1499,12 +1505,34 @@ cdi_status cdi_np_init(cdi_domain *d, double dt_s, double *dt_used) {
   return CDI_OK;
 }
 
-// The face data of the domain's current velocity and potential (FP32 storage
-// only; after either, or the species, has changed), and the Bernoulli pairs
-// where some face needs them (their memory is taken the first time one does;
-// without it the step evaluates them itself).  Waits for the stream.
+// Memory for the domain's Bernoulli pairs or face coefficients (kept for its
+// life); false when there is none.
+static bool take_bern(cdi_domain *d) {
+  if (d->d_bern && d->bern_bytes < bern_bytes(d)) {
+    cdi_dev_release(d, d->d_bern);
+    d->d_bern = nullptr;
+  }
+  if (!d->d_bern) {
+    d->bern_bytes = bern_bytes(d);
+    d->d_bern = cdi_dev_alloc(d, d->bern_bytes);
+  }
+  return d->d_bern != nullptr;
+}
+
+// What the step keeps of the domain's current velocity and potential (after
+// either, or the species, has changed).  FP64: the face coefficients.  FP32:
+// the face data, and the Bernoulli pairs where some face needs them (their
+// memory is taken the first time one does; waits for the stream).  Without
+// memory for them the step evaluates every face itself.
 cdi_status cdi_np_faces(cdi_domain *d) {
-  if (d->prec == CDI_FP64) return CDI_OK;
+  if (d->prec == CDI_FP64) {
+    d->np_mode = take_bern(d) ? NP_SMALL : NP_EVAL;
+    if (d->np_mode == NP_EVAL) return CDI_OK;
+    launch_coef64(d, d->stream, d->d_u, d->d_phi, d->d_bern);
+    d->timing.kernel_launches++;
+    CDI_TRY(d, cudaGetLastError(), "face coefficients");
+    return CDI_OK;
+  }
   int *flag = (int *)(d->d_counter + C_FACE);
   int large = 0;
   CDI_TRY(d, cudaMemsetAsync(flag, 0, sizeof(int), d->stream), "face flag reset");
@@ -1514,21 +1542,9 @@ cdi_status cdi_np_faces(cdi_domain *d) {
   CDI_TRY(d, cudaMemcpyAsync(&large, flag, sizeof(int), cudaMemcpyDeviceToHost, d->stream),
           "face flag");
   CDI_TRY(d, cudaStreamSynchronize(d->stream), "face data");
-  d->np_mode = large ? NP_LARGE : NP_SMALL;
-  if (!large) return CDI_OK;
-  if (d->d_bern && d->bern_bytes < bern_bytes(d)) {
-    cdi_dev_release(d, d->d_bern);
-    d->d_bern = nullptr;
-  }
-  if (!d->d_bern) {
-    d->bern_bytes = bern_bytes(d);
-    d->d_bern = (float2 *)cdi_dev_alloc(d, d->bern_bytes);
-    if (!d->d_bern) {
-      d->np_mode = NP_EVAL;
-      return CDI_OK;
-    }
-  }
-  launch_bern(d, d->stream, d->d_u, d->d_phi, d->d_fd, d->d_bern);
+  d->np_mode = large ? (take_bern(d) ? NP_LARGE : NP_EVAL) : NP_SMALL;
+  if (d->np_mode != NP_LARGE) return CDI_OK;
+  launch_bern(d, d->stream, d->d_u, d->d_phi, d->d_fd, (float2 *)d->d_bern);
   d->timing.kernel_launches++;
   CDI_TRY(d, cudaGetLastError(), "face data");
   return CDI_OK;
@@ -1662,11 +1678,16 @@ cdi_status sweep_run(cdi_domain *d, int n, const double *scale, const int *group
   for (int m = 0; m < n && s == CDI_OK; m++) {
     s = cdi_flow_scale_to(d, scale[m], (void *)hm[m].u);
     if (s != CDI_OK) break;
-    d->dt = dts[m];
-    if (!f64) member_faces(d, d->stream, hm[m].f, hm[m].u, count + m);
+    if (f64) {
+      void *co = take(bern_bytes(d));
+      if (co) launch_coef64(d, d->stream, hm[m].u, hm[m].phi, co);
+      hm[m].co = (const double2 *)co;
+    } else {
+      member_faces(d, d->stream, hm[m].f, hm[m].u, count + m);
+    }
     k_np_init<T><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
         c_views<T>(d, hm[m].C[0]), (int)d->n_pore, ns, (T)d->c0, (T)(d->c0 - (double)(T)d->c0));
-    d->timing.kernel_launches += f64 ? 1 : 2;
+    d->timing.kernel_launches += 2;
     if (cudaMemsetAsync(hm[m].acc, 0, (size_t)3 * kMaxSpecies * d->np_accs * 8, d->stream) !=
         cudaSuccess)
       s = cdi_fail(d, CDI_ERR_CUDA, "sweep: memset");
@@ -1853,11 +1874,17 @@ cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, const do
     s = cdi_fail(L, CDI_ERR_CUDA, "batch: memset");
   for (int m = 0; m < n && s == CDI_OK; m++) {
     const cdi_domain *d = doms[m / n_combos];
-    if (!f64) member_faces(d, L->stream, hm[m].s.f, hm[m].s.u, count + m);
+    if (f64) {
+      void *co = take(bern_bytes(d));
+      if (co) launch_coef64(d, L->stream, hm[m].s.u, hm[m].s.phi, co);
+      hm[m].s.co = (const double2 *)co;
+    } else {
+      member_faces(d, L->stream, hm[m].s.f, hm[m].s.u, count + m);
+    }
     k_np_init<T><<<kRedBlocks, kRedThreads, 0, L->stream>>>(
         c_views<T>(d, hm[m].s.C[0]), (int)d->n_pore, ns, (T)d->c0,
         (T)(d->c0 - (double)(T)d->c0));
-    L->timing.kernel_launches += f64 ? 1 : 2;
+    L->timing.kernel_launches += 2;
     if (cudaMemsetAsync(hm[m].s.acc, 0, (size_t)3 * kMaxSpecies * d->np_accs * 8,
                         L->stream) != cudaSuccess)
       s = cdi_fail(L, CDI_ERR_CUDA, "batch: memset");

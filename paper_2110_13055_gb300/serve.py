@@ -77,9 +77,9 @@ def footprint_bytes(mask: np.ndarray, precision: int, mirror: bool = True) -> in
     links = (4 + (4 if dim == 2 else 8)) * n_fp + n_off * 4 * ((n_fp + 31) // 32)
     flow = (Q * Tpop * n_fp + links + (Q - 1) * 4 * n_ovf
             + Nf * (2 if dim == 2 else 4) + dim * Nf * 8)
-    # with the lateral differences and, in FP32 storage, the face data and the
-    # Bernoulli pairs a resolved double layer needs (two species)
-    faces = 0 if precision == cdi.FP64 else dim * 8 + (dim + 1) * 16
+    # with the lateral differences and, for two species, the face coefficients
+    # (FP64) or the face data and the Bernoulli pairs a resolved double layer needs
+    faces = (dim + 1) * 32 if precision == cdi.FP64 else dim * 8 + (dim + 1) * 16
     transport = (n_pore * (4 + 8 + 2 + 2 * (dim - 1) * (4 + 2 + 1) + dim * T + 8 + 2 * 4 * Tc
                            + faces)
                  + rows * ((nx + 31) // 32) * 8)
