@@ -1,6 +1,7 @@
 // C ABI of the CDI library: domain lifecycle, argument checking, errors,
 // device memory, event timing, field copies and queries.  The numerical work
 // lives in flow.cu, potential.cu and transport.cu.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -73,6 +74,20 @@ void cdi_dev_release(cdi_domain *d, void *p) {
     d->blocks.erase(d->blocks.begin() + (long)i);
     return;
   }
+}
+
+int cdi::grid_shape(const void *kernel, long long n, int *threads) {
+  int dev = 0, sms = 0, per = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (sms < 1) return 0;
+  const long long each = ((n + sms - 1) / sms + 31) / 32 * 32;
+  const int t = (int)std::max(32ll, std::min((long long)cdi::kGridThreads, each));
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, t, 0);
+  (void)cudaGetLastError();
+  *threads = t;
+  if (per < 1) return 0;
+  return (int)std::max<long long>(1, std::min<long long>(std::min(sms, cdi::kRedBlocks), (n + t - 1) / t));
 }
 
 // Pinned host blocks for the device scalars, recycled across domains

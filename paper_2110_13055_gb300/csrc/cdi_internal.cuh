@@ -156,6 +156,104 @@ __device__ __forceinline__ void combine_partials(const double *partials, int nbl
   block_reduce<NV>(v, smem, op, identity);
 }
 
+// ---------------------------------------------------------------------------
+// Iterative solvers as one cooperative launch: one block an SM, every vector
+// pass a grid-stride loop, the passes separated by grid barriers that carry
+// the dot products.
+//
+// A warp's shuffle tree costs five FP64 instructions a value on a part with 2
+// FP64 lanes an SM; here 128 threads add a block's values through shared
+// memory first (51 warp instructions for 1024 threads instead of 165).
+// ---------------------------------------------------------------------------
+constexpr int kGridThreads = 1024;
+constexpr long long kBarrierPolls = 1ll << 26;  // tens of seconds
+constexpr int kGridSums = 2 * kMaxSpecies;      // dot products of a phase, at most
+
+struct GridBarrier {
+  unsigned *counter;  // arrivals since the launch (0 before it)
+  double *part;       // 2 * kGridSums * gridDim.x partials
+  unsigned target;
+  int parity;         // which half of part this phase writes: a block may be
+                      // reading the last phase's half still
+};
+
+// Block sums of v into slots [at, at + NV) of this phase's partials.
+// blockDim.x is a multiple of 32; sm holds NV * blockDim.x values.
+template <int NV>
+__device__ __forceinline__ void grid_partial(const GridBarrier &b, const double (&v)[NV],
+                                             double *sm, int at) {
+  const int t = threadIdx.x, T = blockDim.x, W = T < 128 ? T : 128;
+#pragma unroll
+  for (int k = 0; k < NV; k++) sm[k * T + t] = v[k];
+  __syncthreads();
+  if (t < W) {
+    double s[NV];
+#pragma unroll
+    for (int k = 0; k < NV; k++) {
+      s[k] = sm[k * T + t];
+      for (int j = t + W; j < T; j += W) s[k] += sm[k * T + j];
+    }
+    warp_reduce<NV>(s, OpSum());
+    __syncwarp();
+    if ((t & 31) == 0)
+#pragma unroll
+      for (int k = 0; k < NV; k++) sm[k * T + t] = s[k];
+  }
+  __syncthreads();
+  if (t < NV) {
+    double s = sm[t * T];
+    for (int w = 32; w < W; w += 32) s += sm[t * T + w];
+    __stcg(b.part + ((size_t)b.parity * kGridSums + at + t) * gridDim.x + blockIdx.x, s);
+  }
+  __syncthreads();  // sm is free again
+}
+
+// Barrier over the grid (whose blocks are all resident: a cooperative launch),
+// then the sums of this phase's nv partials in tot[0 .. nv), the same bits in
+// every block.  False in every thread of a block whose wait ran into its
+// limit: the block must return (the others then run into theirs).
+__device__ __forceinline__ bool grid_totals(GridBarrier &b, double *tot, int nv) {
+  const int t = threadIdx.x;
+  b.target += gridDim.x;
+  int ok = 1;
+  __syncthreads();
+  if (t < 32) {
+    if (t == 0) {
+      __threadfence();  // the block's writes, partials included, before its arrival
+      atomicAdd(b.counter, 1u);
+      ok = 0;
+      for (long long i = 0; i < kBarrierPolls; i++) {
+        unsigned c;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(b.counter) : "memory");
+        if ((int)(c - b.target) >= 0) {
+          ok = 1;
+          break;
+        }
+      }
+      __threadfence();
+    }
+    __syncwarp();
+    for (int k = 0; k < nv; k++) {
+      const double *p = b.part + ((size_t)b.parity * kGridSums + k) * gridDim.x;
+      double s = 0.0;
+      for (int i = t; i < (int)gridDim.x; i += 32) s += __ldcg(p + i);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+      if (t == 0) tot[k] = s;
+    }
+  }
+  b.parity ^= 1;
+  return __syncthreads_and(ok);
+}
+__device__ __forceinline__ void grid_give_up(double *flag) {
+  if (threadIdx.x == 0) *flag = 1.0;
+}
+
+// Blocks and threads of a cooperative launch over n items: one block an SM,
+// as few threads as cover the items (few items are spread over all SMs, whose
+// FP64 units are the bound).  0 if not even one block fits.
+int grid_shape(const void *kernel, long long n, int *threads);
+
 // psi / V_T as stored for the transport kernel: FP64, or an unevaluated
 // FP32 pair hi + lo (so that face differences keep FP64-like accuracy while
 // the arithmetic stays on the FP32 units).
@@ -319,7 +417,8 @@ struct cdi_domain {
   int64_t imp_iters = 0;        // linear iterations so far
   double imp_last_rel = 0.0;    // last relative residual
   double *d_icoef = nullptr;    // operator coefficients of every species (FP64)
-  double *d_iwork = nullptr;    // 7 * n_pore FP64 work vectors
+  double *d_iwork = nullptr;    // imp_sets * 6 * n_pore FP64 work vectors
+  int imp_sets = 0;             // species whose vectors d_iwork holds
   double *d_iscal = nullptr;    // the solver's device scalars (16)
   double *d_src = nullptr;      // N charge terms of Eq. 4 (coupled mode only)
   int cur = 0;                  // which of d_C holds the current state

@@ -7,9 +7,9 @@
 // half-cell Robin closure at solid faces, the feed ghost at the inlet, the
 // copying ghost at the outlet).  The operator is assembled once per
 // transport state in FP64 (a diagonal, one coefficient per face and the
-// inlet source, by pore rank); the solve is matrix-free, Jacobi-
-// preconditioned BiCGStab in FP64 with every scalar on the device and
-// fixed-order block reductions, so a run is deterministic.  The adsorbed,
+// account coefficients, by pore rank); the solve is matrix-free, Jacobi-
+// preconditioned BiCGStab in FP64, all of it in one cooperative launch with
+// fixed-order sums, so a run is deterministic.  The adsorbed,
 // inflow and outflow accounts take the fluxes at C^{n+1}, so the mass balance
 // closes as in the explicit scheme.  The step is unconditionally stable and
 // positivity-preserving (I + dt A is an M-matrix), so dt may exceed the
@@ -24,20 +24,27 @@ using namespace cdi;
 
 namespace {
 
-// Scalar slots of the solver (d_iscal).
-enum { B_RHO = 0, B_ALPHA, B_OMEGA, B_BETA, B_BB, B_REL, B_DONE, B_TOL, B_IT, B_R0V, B_N };
+// Scalar slots of the solver (d_iscal): per species of a launch its last
+// relative residual and iterations, then the launch's verdict (0: every
+// species converged) and the barrier's (0: no barrier ran into its limit).
+enum { B_REL = 0, B_IT = kMaxSpecies, B_FAIL = 2 * kMaxSpecies, B_BAR, B_N };
 
-// Coefficients of species k, component j at ((k * NC) + j) * n + r:
-// j = 0 diagonal of A, 1..2 dim its face coefficients (face j - 1: +x, -x,
-// +y, -y, +z, -z; 0 across a closed face), then the inlet source b, and the
-// account coefficients: ain = (D/dx) B(-P_in), bin = (D/dx) B(P_in) c0 (the
-// inflow is bin - ain C_P), aout = (D/dx) (B(-P_out) - B(P_out)) (outflow
-// aout C_P), gam = n_solid K_eff (adsorption gam C_P).
+// The solver works on y = K x, K = 1 + dt A_PP (Jacobi preconditioning from
+// the right), so that an iteration has neither divisions nor the diagonal:
+// M y = y_P + sum_f off_f y_nb with off_f = dt a_f / K_nb formed once per
+// operator.  At 2 FP64 operations a clock and SM the arithmetic bounds an
+// iteration; a division is worth about ten multiply-adds.
+//
+// Coefficients of species k, component j at ((k * NC) + j) * n + r: K, off of
+// the faces (+x, -x, +y, -y, +z, -z; exactly 0 across a closed face), and
+// the account coefficients ain = (D/dx) B(-P_in), bin = (D/dx) B(P_in) c0
+// (the inflow is bin - ain C_P), aout = (D/dx) (B(-P_out) - B(P_out))
+// (outflow aout C_P).
 template <int DIM> struct ICoef {
   static constexpr int NF = 2 * DIM;
-  static constexpr int DIAG = 0, FACE = 1, B = 1 + NF, AIN = 2 + NF, BIN = 3 + NF,
-                       AOUT = 4 + NF, GAM = 5 + NF, NC = 6 + NF;
+  static constexpr int K = 0, FACE = 1, AIN = 1 + NF, BIN = 2 + NF, AOUT = 3 + NF, NC = 4 + NF;
 };
+constexpr int kImpVecs = 6;  // y, r, r0, p, v, t per species
 
 struct IGeo {
   const NFlag *fl;   // per rank face flags
@@ -75,7 +82,7 @@ template <typename T, int DIM>
 __global__ void k_imp_coef(IGeo g, const T *__restrict__ u,
                            const typename PhiStore<T>::type *__restrict__ phi, int ns,
                            PerSpecies dxD, PerSpecies Ddx, PerSpecies Keff, PerSpecies zf,
-                           double inv_dx, double c0, double *__restrict__ co) {
+                           double inv_dx, double c0, double dt, double *__restrict__ co) {
   using C = ICoef<DIM>;
   const double *dxDk = dxD.v, *Ddxk = Ddx.v, *Kk = Keff.v, *zk = zf.v;
   const size_t n = (size_t)g.n;
@@ -84,14 +91,13 @@ __global__ void k_imp_coef(IGeo g, const T *__restrict__ u,
     const double phP = phi_of(phi[r]);
     for (int k = 0; k < ns; k++) {
       double *c = co + (size_t)k * C::NC * n;
-      double diag = 0.0, b = 0.0, ain = 0.0, bin = 0.0, aout = 0.0, gam = 0.0;
+      double diag = 0.0, ain = 0.0, bin = 0.0, aout = 0.0;
       for (int fc = 0; fc < C::NF; fc++) {
         int q;
         const int kind = ikind(g, f, fc, r, q);
         double off = 0.0;
         if (kind == K_SOLID) {
           diag += Kk[k] * inv_dx;
-          gam += Kk[k];
         } else if (kind != K_WALL) {
           const int a = fc >> 1;
           const double uP = (double)u[(size_t)a * n + r];
@@ -106,7 +112,6 @@ __global__ void k_imp_coef(IGeo g, const T *__restrict__ u,
             off = -Ddxk[k] * inv_dx * Bp;
           } else if (kind == K_INLET) {
             diag += Ddxk[k] * inv_dx * Bm;
-            b += Ddxk[k] * inv_dx * Bp * c0;
             ain = Ddxk[k] * Bm;
             bin = Ddxk[k] * Bp * c0;
           } else {
@@ -116,221 +121,248 @@ __global__ void k_imp_coef(IGeo g, const T *__restrict__ u,
         }
         c[(size_t)(C::FACE + fc) * n + r] = off;
       }
-      c[(size_t)C::DIAG * n + r] = diag;
-      c[(size_t)C::B * n + r] = b;
+      c[(size_t)C::K * n + r] = 1.0 + dt * diag;
       c[(size_t)C::AIN * n + r] = ain;
       c[(size_t)C::BIN * n + r] = bin;
       c[(size_t)C::AOUT * n + r] = aout;
-      c[(size_t)C::GAM * n + r] = gam;
     }
   }
 }
 
-// (I + dt A) (x / K) at rank r, K = 1 + dt A_PP the Jacobi preconditioner;
-// xv(q) supplies x at rank q.
-template <int DIM, typename X>
-__device__ __forceinline__ double apply_scaled(const IGeo &g, const double *__restrict__ c,
-                                               double dt, int r, X xv) {
+// off_f = dt a_f / K_nb, once every K stands.
+template <int DIM>
+__global__ void k_imp_scale(IGeo g, int ns, double dt, double *__restrict__ co) {
   using C = ICoef<DIM>;
   const size_t n = (size_t)g.n;
-  const unsigned f = g.fl[r];
-  double acc = xv(r);  // K x / K
-  for (int fc = 0; fc < C::NF; fc++) {
-    const double off = c[(size_t)(C::FACE + fc) * n + r];
-    if (off == 0.0) continue;
-    int q;
-    ikind(g, f, fc, r, q);
-    acc += dt * off * (xv(q) / (1.0 + dt * c[(size_t)C::DIAG * n + q]));
-  }
-  return acc;
-}
-
-// Start of a step for one species: x = C^n (the first guess), rhs = C^n +
-// dt b, r = rhs - M x, r0 = r, p = r; rho = r0.r, bb = rhs.rhs.
-template <typename T, int DIM>
-__global__ void __launch_bounds__(kRedThreads)
-    k_bi_start(IGeo g, const double *__restrict__ c, double dt, CView<T> Ck, double tol, double *__restrict__ x,
-               double *__restrict__ rr, double *__restrict__ r0, double *__restrict__ p,
-               double *__restrict__ part, unsigned int *counter, double *scal) {
-  using C = ICoef<DIM>;
-  __shared__ double sm[2 * 32];
-  double v[2] = {0.0, 0.0};
-  const size_t n = (size_t)g.n;
-  auto cval = [&](int q) { return Ck.at(q); };
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < g.n; r += gridDim.x * blockDim.x) {
-    const double cP = cval(r);
-    const double rhs = cP + dt * c[(size_t)C::B * n + r];
-    // M x with x = C: (1 + dt A_PP) C_P + dt sum off C_nb
     const unsigned f = g.fl[r];
-    double Mx = (1.0 + dt * c[(size_t)C::DIAG * n + r]) * cP;
     for (int fc = 0; fc < C::NF; fc++) {
-      const double off = c[(size_t)(C::FACE + fc) * n + r];
-      if (off == 0.0) continue;
       int q;
-      ikind(g, f, fc, r, q);
-      Mx += dt * off * cval(q);
-    }
-    const double res = rhs - Mx;
-    x[r] = cP;
-    rr[r] = res;
-    r0[r] = res;
-    p[r] = res;
-    v[0] += res * res;
-    v[1] += rhs * rhs;
-  }
-  block_reduce<2>(v, sm, OpSum(), 0.0);
-  if (threadIdx.x == 0) {
-    part[blockIdx.x] = v[0];
-    part[gridDim.x + blockIdx.x] = v[1];
-  }
-  if (last_block(counter, gridDim.x)) {
-    combine_partials<2>(part, gridDim.x, v, sm, OpSum(), 0.0);
-    if (threadIdx.x == 0) {
-      scal[B_RHO] = v[0];
-      scal[B_BB] = v[1];
-      scal[B_TOL] = tol;
-      scal[B_IT] = 0.0;
-      const double rel = v[1] > 0.0 ? sqrt(v[0] / v[1]) : 0.0;
-      scal[B_REL] = rel;
-      scal[B_DONE] = (rel < tol || v[0] == 0.0) ? 1.0 : 0.0;
-      *counter = 0;
+      if (ikind(g, f, fc, r, q) != K_PORE) continue;
+      for (int k = 0; k < ns; k++) {
+        double *c = co + (size_t)k * C::NC * n;
+        double *o = c + (size_t)(C::FACE + fc) * n + r;
+        *o = dt * *o / c[(size_t)C::K * n + q];
+      }
     }
   }
 }
 
-// v = M (p / K); alpha = rho / (r0 . v).
-template <int DIM>
-__global__ void __launch_bounds__(kRedThreads)
-    k_bi_v(IGeo g, const double *__restrict__ c, double dt, const double *__restrict__ p,
-           const double *__restrict__ r0, double *__restrict__ vv, double *__restrict__ part,
-           unsigned int *counter, double *scal) {
-  if (scal[B_DONE] != 0.0) return;
-  __shared__ double sm[32];
-  double v[1] = {0.0};
-  auto pv = [&](int q) { return p[q]; };
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < g.n; r += gridDim.x * blockDim.x) {
-    const double y = apply_scaled<DIM>(g, c, dt, r, pv);
-    vv[r] = y;
-    v[0] += r0[r] * y;
+// The neighbours of rank r across its open faces: fn(q, off) in face order.
+// A closed face has off exactly +0 (an integer test: an FP64 comparison would
+// take the FP64 pipe); its q is not formed.
+template <int DIM, typename F>
+__device__ __forceinline__ void open_faces(const int *__restrict__ lat,
+                                           const double *__restrict__ off, size_t n, int r, F fn) {
+  double o[2 * DIM];
+  int q[2 * DIM];
+#pragma unroll
+  for (int f = 0; f < 2 * DIM; f++) {
+    o[f] = off[(size_t)f * n + r];
+    q[f] = f < 2 ? r + (f == 0 ? 1 : -1) : lat[(size_t)(f - 2) * n + r];
   }
-  block_reduce<1>(v, sm, OpSum(), 0.0);
-  if (threadIdx.x == 0) part[blockIdx.x] = v[0];
-  if (last_block(counter, gridDim.x)) {
-    combine_partials<1>(part, gridDim.x, v, sm, OpSum(), 0.0);
-    if (threadIdx.x == 0) {
-      scal[B_R0V] = v[0];
-      scal[B_ALPHA] = v[0] != 0.0 ? scal[B_RHO] / v[0] : 0.0;
-      *counter = 0;
-    }
-  }
+#pragma unroll
+  for (int f = 0; f < 2 * DIM; f++)
+    if (__double_as_longlong(o[f]) != 0) fn(q[f], o[f]);
 }
 
-// s = r - alpha v (stored over r), t = M (s / K); omega = (t . s) / (t . t).
-// The neighbours' s are formed on the fly from their r and v.
-template <int DIM>
-__global__ void __launch_bounds__(kRedThreads)
-    k_bi_t(IGeo g, const double *__restrict__ c, double dt, const double *__restrict__ rr,
-           const double *__restrict__ vv, double *__restrict__ s, double *__restrict__ t,
-           double *__restrict__ part, unsigned int *counter, double *scal) {
-  if (scal[B_DONE] != 0.0) return;
-  __shared__ double sm[2 * 32];
-  const double alpha = scal[B_ALPHA];
-  double v[2] = {0.0, 0.0};
-  auto sv = [&](int q) { return rr[q] - alpha * vv[q]; };
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < g.n; r += gridDim.x * blockDim.x) {
-    const double sP = sv(r);
-    const double y = apply_scaled<DIM>(g, c, dt, r, sv);
-    s[r] = sP;
-    t[r] = y;
-    v[0] += y * sP;
-    v[1] += y * y;
-  }
-  block_reduce<2>(v, sm, OpSum(), 0.0);
-  if (threadIdx.x == 0) {
-    part[blockIdx.x] = v[0];
-    part[gridDim.x + blockIdx.x] = v[1];
-  }
-  if (last_block(counter, gridDim.x)) {
-    combine_partials<2>(part, gridDim.x, v, sm, OpSum(), 0.0);
-    if (threadIdx.x == 0) {
-      scal[B_OMEGA] = v[1] != 0.0 ? v[0] / v[1] : 0.0;
-      *counter = 0;
-    }
-  }
-}
+template <typename T> struct BiArgs {
+  const double *co;   // coefficients of the launch's first species
+  const int *lat;
+  int n, ns, max_iter;
+  double dt_dx, tol;  // dt / dx
+  CViews<T> C;        // C^n of the launch's species
+  double *w;          // kImpVecs vectors per species
+  double *part, *scal;
+  unsigned *counter;
+};
 
-// x += (alpha p + omega s) / K, r = s - omega t; rho' = r0 . r, beta =
-// (rho' / rho)(alpha / omega); convergence on ||r|| / ||rhs||.
-template <int DIM>
-__global__ void __launch_bounds__(kRedThreads)
-    k_bi_x(IGeo g, const double *__restrict__ c, double dt, double *__restrict__ x,
-           double *__restrict__ rr, const double *__restrict__ r0, const double *__restrict__ p,
-           const double *__restrict__ s, const double *__restrict__ t,
-           double *__restrict__ part, unsigned int *counter, double *scal) {
+// One backward Euler step's linear solves, all species of the launch side by
+// side: Jacobi-preconditioned BiCGStab from the first guess C^n, the
+// iterations and their dot products in one cooperative launch.
+//
+// What bounds it: FP64 arithmetic (31 operations a cell, species and
+// iteration in 3D), then the four grid barriers of an iteration.  Before, an
+// iteration was four launches a species, divided by K of every neighbour in
+// both products and summed by five FP64 shuffle rounds a warp: 80^3, two
+// species, 6 steps of 40 explicit ones 40.5 -> 12.5 ms.  The neighbours'
+// s = r - alpha v are formed on the fly: a pass of their own would cost
+// another barrier.
+template <typename T, int DIM>
+__global__ void __launch_bounds__(kGridThreads) k_bi_solve(BiArgs<T> a) {
   using C = ICoef<DIM>;
-  if (scal[B_DONE] != 0.0) return;
-  __shared__ double sm[2 * 32];
-  const double alpha = scal[B_ALPHA], omega = scal[B_OMEGA];
-  double v[2] = {0.0, 0.0};
-  const size_t n = (size_t)g.n;
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < g.n; r += gridDim.x * blockDim.x) {
-    const double K = 1.0 + dt * c[(size_t)C::DIAG * n + r];
-    x[r] += (alpha * p[r] + omega * s[r]) / K;
-    const double rv = s[r] - omega * t[r];
-    rr[r] = rv;
-    v[0] += r0[r] * rv;
-    v[1] += rv * rv;
+  __shared__ double sm[2 * kGridThreads];
+  __shared__ double tot[2 * kMaxSpecies];
+  __shared__ double rho[kMaxSpecies], alpha[kMaxSpecies], omega[kMaxSpecies], beta[kMaxSpecies],
+      bb[kMaxSpecies], rel[kMaxSpecies];
+  __shared__ int it[kMaxSpecies], done[kMaxSpecies];
+  const size_t n = (size_t)a.n;
+  const int first = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+  GridBarrier bar{a.counter, a.part, 0u, 0};
+
+  for (int k = 0; k < a.ns; k++) {
+    const double *c = a.co + (size_t)k * C::NC * n;
+    double *y = a.w + (size_t)k * kImpVecs * n, *rr = y + n, *r0 = rr + n, *p = r0 + n;
+    const CView<T> Ck = a.C.v[k];
+    double v[2] = {0.0, 0.0};
+    for (int r = first; r < a.n; r += stride) {
+      const double cP = Ck.at(r), yP = c[(size_t)C::K * n + r] * cP;
+      const double rhs = cP + a.dt_dx * c[(size_t)C::BIN * n + r];
+      double My = yP;
+      open_faces<DIM>(a.lat, c + (size_t)C::FACE * n, n, r,
+                      [&](int q, double o) { My += o * (c[(size_t)C::K * n + q] * Ck.at(q)); });
+      const double res = rhs - My;
+      y[r] = yP;
+      rr[r] = res;
+      r0[r] = res;
+      p[r] = res;
+      v[0] += res * res;
+      v[1] += rhs * rhs;
+    }
+    grid_partial<2>(bar, v, sm, 2 * k);
   }
-  block_reduce<2>(v, sm, OpSum(), 0.0);
-  if (threadIdx.x == 0) {
-    part[blockIdx.x] = v[0];
-    part[gridDim.x + blockIdx.x] = v[1];
+  if (!grid_totals(bar, tot, 2 * a.ns)) return grid_give_up(a.scal + B_BAR);
+  if (threadIdx.x < a.ns) {
+    const int k = threadIdx.x;
+    rho[k] = tot[2 * k];
+    bb[k] = tot[2 * k + 1];
+    rel[k] = bb[k] > 0.0 ? sqrt(rho[k] / bb[k]) : 0.0;
+    it[k] = 0;
+    done[k] = rel[k] < a.tol || rho[k] == 0.0;
   }
-  if (last_block(counter, gridDim.x)) {
-    combine_partials<2>(part, gridDim.x, v, sm, OpSum(), 0.0);
-    if (threadIdx.x == 0) {
-      const double rho = scal[B_RHO];
-      scal[B_BETA] = (rho != 0.0 && omega != 0.0) ? (v[0] / rho) * (alpha / omega) : 0.0;
-      scal[B_RHO] = v[0];
-      const double rel = scal[B_BB] > 0.0 ? sqrt(v[1] / scal[B_BB]) : 0.0;
-      scal[B_REL] = rel;
-      scal[B_IT] += 1.0;
-      // converged, or broken down (no new direction): the host restarts or stops
-      if (rel < scal[B_TOL] || v[0] == 0.0 || omega == 0.0) scal[B_DONE] = 1.0;
-      *counter = 0;
+  __syncthreads();
+
+  for (int step = 0; step < a.max_iter; step++) {
+    bool all = true;
+    for (int k = 0; k < a.ns; k++) all = all && done[k];
+    if (all) break;
+
+    // v = M p; alpha = rho / (r0 . v)
+    for (int k = 0; k < a.ns; k++) {
+      double v[1] = {0.0};
+      if (!done[k]) {
+        const double *off = a.co + ((size_t)k * C::NC + C::FACE) * n;
+        double *y = a.w + (size_t)k * kImpVecs * n;
+        const double *r0 = y + 2 * n, *p = y + 3 * n;
+        double *vv = y + 4 * n;
+        for (int r = first; r < a.n; r += stride) {
+          double m = p[r];
+          open_faces<DIM>(a.lat, off, n, r, [&](int q, double o) { m += o * p[q]; });
+          vv[r] = m;
+          v[0] += r0[r] * m;
+        }
+      }
+      grid_partial<1>(bar, v, sm, k);
+    }
+    if (!grid_totals(bar, tot, a.ns)) return grid_give_up(a.scal + B_BAR);
+    if (threadIdx.x < a.ns && !done[threadIdx.x])
+      alpha[threadIdx.x] = tot[threadIdx.x] != 0.0 ? rho[threadIdx.x] / tot[threadIdx.x] : 0.0;
+    __syncthreads();
+
+    // s = r - alpha v, t = M s; omega = (t . s) / (t . t)
+    for (int k = 0; k < a.ns; k++) {
+      double v[2] = {0.0, 0.0};
+      if (!done[k]) {
+        const double *off = a.co + ((size_t)k * C::NC + C::FACE) * n;
+        double *y = a.w + (size_t)k * kImpVecs * n;
+        const double *rr = y + n, *vv = y + 4 * n;
+        double *t = y + 5 * n;
+        const double al = alpha[k];
+        for (int r = first; r < a.n; r += stride) {
+          const double sP = rr[r] - al * vv[r];
+          double m = sP;
+          open_faces<DIM>(a.lat, off, n, r,
+                          [&](int q, double o) { m += o * (rr[q] - al * vv[q]); });
+          t[r] = m;
+          v[0] += m * sP;
+          v[1] += m * m;
+        }
+      }
+      grid_partial<2>(bar, v, sm, 2 * k);
+    }
+    if (!grid_totals(bar, tot, 2 * a.ns)) return grid_give_up(a.scal + B_BAR);
+    if (threadIdx.x < a.ns && !done[threadIdx.x]) {
+      const int k = threadIdx.x;
+      omega[k] = tot[2 * k + 1] != 0.0 ? tot[2 * k] / tot[2 * k + 1] : 0.0;
+    }
+    __syncthreads();
+
+    // y += alpha p + omega s, r = s - omega t; rho' = r0 . r
+    for (int k = 0; k < a.ns; k++) {
+      double v[2] = {0.0, 0.0};
+      if (!done[k]) {
+        double *y = a.w + (size_t)k * kImpVecs * n, *rr = y + n;
+        const double *r0 = y + 2 * n, *p = y + 3 * n, *vv = y + 4 * n, *t = y + 5 * n;
+        const double al = alpha[k], om = omega[k];
+        for (int r = first; r < a.n; r += stride) {
+          const double sP = rr[r] - al * vv[r];
+          y[r] += al * p[r] + om * sP;
+          const double rv = sP - om * t[r];
+          rr[r] = rv;
+          v[0] += r0[r] * rv;
+          v[1] += rv * rv;
+        }
+      }
+      grid_partial<2>(bar, v, sm, 2 * k);
+    }
+    if (!grid_totals(bar, tot, 2 * a.ns)) return grid_give_up(a.scal + B_BAR);
+    if (threadIdx.x < a.ns && !done[threadIdx.x]) {
+      const int k = threadIdx.x;
+      const double r1 = tot[2 * k];
+      beta[k] = (rho[k] != 0.0 && omega[k] != 0.0) ? (r1 / rho[k]) * (alpha[k] / omega[k]) : 0.0;
+      rho[k] = r1;
+      rel[k] = bb[k] > 0.0 ? sqrt(tot[2 * k + 1] / bb[k]) : 0.0;
+      it[k]++;
+      // converged, or broken down (no new direction)
+      if (rel[k] < a.tol || r1 == 0.0 || omega[k] == 0.0) done[k] = 1;
+    }
+    __syncthreads();
+
+    // p = r + beta (p - omega v)
+    for (int k = 0; k < a.ns; k++) {
+      if (done[k]) continue;
+      double *y = a.w + (size_t)k * kImpVecs * n;
+      const double *rr = y + n, *vv = y + 4 * n;
+      double *p = y + 3 * n;
+      const double be = beta[k], om = omega[k];
+      for (int r = first; r < a.n; r += stride) p[r] = rr[r] + be * (p[r] - om * vv[r]);
+    }
+    if (!grid_totals(bar, tot, 0)) return grid_give_up(a.scal + B_BAR);
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    for (int k = 0; k < a.ns; k++) {
+      a.scal[B_REL + k] = rel[k];
+      a.scal[B_IT + k] = it[k];
+      if (!(rel[k] < a.tol)) a.scal[B_FAIL] = 1.0;
     }
   }
 }
 
-// p = r + beta (p - omega v).
-__global__ void k_bi_p(int n, double *__restrict__ p, const double *__restrict__ rr,
-                       const double *__restrict__ vv, const double *__restrict__ scal) {
-  if (scal[B_DONE] != 0.0) return;
-  const double beta = scal[B_BETA], omega = scal[B_OMEGA];
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x)
-    p[r] = rr[r] + beta * (p[r] - omega * vv[r]);
-}
-
-// C^{n+1} = x into the storage type (an FP32 pair splits into hi + lo), and
-// the accounts of the step: the adsorbed, inflow and outflow fluxes at
+// C^{n+1} = y / K into the storage type (an FP32 pair splits into hi + lo),
+// unless a solve of the step failed (the step is then not taken), and the
+// accounts of the step: the adsorbed, inflow and outflow fluxes at
 // C^{n+1}, summed per warp of 32 ranks into the domain's per-warp accounts.
 template <typename T, int DIM>
-__global__ void k_bi_finish(IGeo g, const double *__restrict__ c, const double *__restrict__ x,
-                            CView<T> Cout, int k,
+__global__ void k_bi_finish(IGeo g, const double *__restrict__ c, const double *__restrict__ y,
+                            const double *__restrict__ scal, double Keff, CView<T> Cout, int k,
                             typename std::conditional<std::is_same<T, float>::value, float2,
                                                       double>::type *__restrict__ acc,
                             int naccs) {
   using C = ICoef<DIM>;
+  if (scal[B_FAIL] != 0.0 || scal[B_BAR] != 0.0) return;
   const size_t n = (size_t)g.n;
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   double v[3] = {0.0, 0.0, 0.0};
   if (r < g.n) {
-    const double xv = x[r];
+    const double xv = y[r] / c[(size_t)C::K * n + r];
     T *o = const_cast<T *>(Cout.p) + (size_t)r * Cout.stride;
     const T hi = (T)xv;
     o[0] = hi;
     if (Cout.lo) o[Cout.lo] = (T)(xv - (double)hi);
-    v[0] = c[(size_t)C::GAM * n + r] * xv;
+    const unsigned f = g.fl[r];
+    int solids = 0, q;
+    for (int fc = 0; fc < C::NF; fc++) solids += ikind(g, f, fc, r, q) == K_SOLID;
+    v[0] = solids * Keff * xv;
     v[1] = c[(size_t)C::BIN * n + r] - c[(size_t)C::AIN * n + r] * xv;
     v[2] = c[(size_t)C::AOUT * n + r] * xv;
   }
@@ -377,70 +409,74 @@ cdi_status imp_coefs(cdi_domain *d) {
   }
   k_imp_coef<T, DIM><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
       make_igeo(d), (const T *)d->d_u, (const typename PhiStore<T>::type *)d->d_phi, d->ns,
-      dxD, Ddx, Keff, zf, 1.0 / d->dx, d->c0, d->d_icoef);
-  d->timing.kernel_launches++;
+      dxD, Ddx, Keff, zf, 1.0 / d->dx, d->c0, d->dt, d->d_icoef);
+  k_imp_scale<DIM><<<kRedBlocks, kRedThreads, 0, d->stream>>>(make_igeo(d), d->ns, d->dt,
+                                                              d->d_icoef);
+  d->timing.kernel_launches += 2;
   CDI_TRY(d, cudaGetLastError(), "implicit operator");
   d->imp_stale = false;
   return CDI_OK;
 }
 
+// One step: the species solved side by side in one launch where their vectors
+// could be had, else one after the other in one set of vectors.
 template <typename T, int DIM>
 cdi_status imp_step(cdi_domain *d) {
   using C = ICoef<DIM>;
+  using A = typename std::conditional<std::is_same<T, float>::value, float2, double>::type;
   const int n = (int)d->n_pore;
   const size_t nn = (size_t)n;
-  double *x = d->d_iwork, *rr = x + nn, *r0 = x + 2 * nn, *p = x + 3 * nn, *vv = x + 4 * nn,
-         *s = x + 5 * nn, *t = x + 6 * nn;
   const IGeo g = make_igeo(d);
-  const double dt = d->dt;
   const int in = d->cur;
-  using A = typename std::conditional<std::is_same<T, float>::value, float2, double>::type;
-  for (int k = 0; k < d->ns; k++) {
-    const double *c = d->d_icoef + (size_t)k * C::NC * nn;
-    const CView<T> Ck = c_view<T>(d, d->d_C[in], k);
-    int iters = 0;
-    k_bi_start<T, DIM><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        g, c, dt, Ck, d->imp_tol, x, rr, r0, p, d->d_part, d->d_counter + C_IMP,
-        d->d_iscal);
-    d->timing.kernel_launches++;
+  const int side = std::min(d->ns, d->imp_sets);
+  int threads = 0;
+  const int blocks = grid_shape((const void *)k_bi_solve<T, DIM>, n, &threads);
+  if (blocks == 0) return cdi_fail(d, CDI_ERR_CUDA, "implicit step: no resident block");
+  CDI_TRY(d, cudaMemsetAsync(d->d_iscal, 0, B_N * sizeof(double), d->stream), "implicit scalars");
+  for (int k0 = 0; k0 < d->ns; k0 += side) {
+    BiArgs<T> a;
+    a.co = d->d_icoef + (size_t)k0 * C::NC * nn;
+    a.lat = d->d_latnb;
+    a.n = n;
+    a.ns = std::min(side, d->ns - k0);
+    a.max_iter = d->imp_max_iter;
+    a.dt_dx = d->dt / d->dx;
+    a.tol = d->imp_tol;
+    for (int k = 0; k < a.ns; k++) a.C.v[k] = c_view<T>(d, d->d_C[in], k0 + k);
+    a.w = d->d_iwork;
+    a.part = d->d_part;
+    a.scal = d->d_iscal;
+    a.counter = d->d_counter + C_IMP;
+    CDI_TRY(d, cudaMemsetAsync(a.counter, 0, sizeof(unsigned), d->stream), "implicit barrier");
+    void *args[] = {&a};
+    CDI_TRY(d, cudaLaunchCooperativeKernel((const void *)k_bi_solve<T, DIM>, dim3(blocks),
+                                           dim3(threads), args, 0, d->stream),
+            "implicit solve");
+    for (int k = 0; k < a.ns; k++) {
+      const double Dk = d->D[k0 + k];
+      const double Keff = d->Ka / (1.0 + d->Ka * d->dx / (2.0 * Dk));
+      k_bi_finish<T, DIM><<<(n + 127) / 128, 128, 0, d->stream>>>(
+          g, a.co + (size_t)k * C::NC * nn, a.w + (size_t)k * kImpVecs * nn, d->d_iscal, Keff,
+          c_view<T>(d, d->d_C[1 - in], k0 + k), k0 + k, (A *)d->d_acc, d->np_accs);
+    }
+    d->timing.kernel_launches += 1 + a.ns;
+    CDI_TRY(d, cudaGetLastError(), "implicit step");
     CDI_TRY(d, cudaMemcpyAsync(d->h_scal + S_IMP, d->d_iscal, B_N * sizeof(double),
                                cudaMemcpyDeviceToHost, d->stream),
-            "implicit start");
-    CDI_TRY(d, cudaStreamSynchronize(d->stream), "implicit start");
-    int chunk = 4;
-    while (d->h_scal[S_IMP + B_DONE] == 0.0 && iters < d->imp_max_iter) {
-      const int m = std::min(chunk, d->imp_max_iter - iters);
-      for (int j = 0; j < m; j++) {
-        k_bi_v<DIM><<<kRedBlocks, kRedThreads, 0, d->stream>>>(g, c, dt, p, r0, vv, d->d_part,
-                                                                 d->d_counter + C_IMP,
-                                                                 d->d_iscal);
-        k_bi_t<DIM><<<kRedBlocks, kRedThreads, 0, d->stream>>>(g, c, dt, rr, vv, s, t,
-                                                                 d->d_part,
-                                                                 d->d_counter + C_IMP,
-                                                                 d->d_iscal);
-        k_bi_x<DIM><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-            g, c, dt, x, rr, r0, p, s, t, d->d_part, d->d_counter + C_IMP, d->d_iscal);
-        k_bi_p<<<kRedBlocks, kRedThreads, 0, d->stream>>>(n, p, rr, vv, d->d_iscal);
-      }
-      d->timing.kernel_launches += 4 * m;
-      iters += m;
-      CDI_TRY(d, cudaGetLastError(), "implicit iteration");
-      CDI_TRY(d, cudaMemcpyAsync(d->h_scal + S_IMP, d->d_iscal, B_N * sizeof(double),
-                                 cudaMemcpyDeviceToHost, d->stream),
-              "implicit poll");
-      CDI_TRY(d, cudaStreamSynchronize(d->stream), "implicit poll");
-      chunk = std::min(chunk * 2, 64);
+            "implicit result");
+    CDI_TRY(d, cudaStreamSynchronize(d->stream), "implicit step");
+    const double *h = d->h_scal + S_IMP;
+    if (h[B_BAR] != 0.0) {
+      // blocks may have left at different points
+      return cdi_fail(d, CDI_ERR_CUDA, "implicit step: a grid barrier ran into its limit");
     }
-    const bool done = d->h_scal[S_IMP + B_REL] < d->imp_tol;
-    d->imp_iters += iters;
-    d->imp_last_rel = d->h_scal[S_IMP + B_REL];
-    if (!done)
+    for (int k = 0; k < a.ns; k++) {
+      d->imp_iters += (int64_t)h[B_IT + k];
+      d->imp_last_rel = h[B_REL + k];
+    }
+    if (h[B_FAIL] != 0.0)
       return cdi_fail(d, CDI_ERR_NOT_CONVERGED,
                       "implicit step: the linear solve did not reach tol within max_iter");
-    k_bi_finish<T, DIM><<<(n + 127) / 128, 128, 0, d->stream>>>(
-        g, c, x, c_view<T>(d, d->d_C[1 - in], k), k, (A *)d->d_acc, d->np_accs);
-    d->timing.kernel_launches++;
-    CDI_TRY(d, cudaGetLastError(), "implicit finish");
   }
   d->cur = 1 - in;
   return CDI_OK;
@@ -451,6 +487,14 @@ cdi_status imp_steps(cdi_domain *d, int64_t n) {
   if (d->imp_stale) {
     cdi_status s = imp_coefs<T, DIM>(d);
     if (s != CDI_OK) return s;
+  }
+  if (d->imp_sets < d->ns) {  // vectors for all species at once, where memory allows
+    double *w = (double *)cdi_dev_alloc(d, (size_t)d->ns * kImpVecs * d->n_pore * 8);
+    if (w) {
+      cdi_dev_release(d, d->d_iwork);
+      d->d_iwork = w;
+      d->imp_sets = d->ns;
+    }
   }
   cudaEvent_t ev;
   cdi_timing_begin(d, &ev);
@@ -469,12 +513,14 @@ cdi_status imp_steps(cdi_domain *d, int64_t n) {
 }  // namespace
 
 // Work memory of the implicit scheme (allocated on first use, kept for the
-// domain's life): the operator of every species and seven FP64 vectors.
+// domain's life): the operator of every species and the vectors of one (the
+// first step takes those of the others).
 cdi_status cdi_imp_prepare(cdi_domain *d) {
   const int NC = d->dim == 2 ? ICoef<2>::NC : ICoef<3>::NC;
   if (!d->d_icoef) {
     d->d_icoef = (double *)cdi_dev_alloc(d, (size_t)kMaxSpecies * NC * d->n_pore * 8);
-    d->d_iwork = (double *)cdi_dev_alloc(d, (size_t)7 * d->n_pore * 8);
+    d->d_iwork = (double *)cdi_dev_alloc(d, (size_t)kImpVecs * d->n_pore * 8);
+    d->imp_sets = 1;
     d->d_iscal = (double *)cdi_dev_alloc(d, 16 * 8);
     if (!d->d_icoef || !d->d_iwork || !d->d_iscal)
       return cdi_fail(d, CDI_ERR_OOM, "implicit scheme: device memory");
