@@ -1,5 +1,5 @@
 // Frozen electric potential (Eq. 4-5 with the Dirichlet surface value of
-// Sec. 2) by Jacobi-preconditioned conjugate gradients in FP64.
+// Sec. 2) by Jacobi-preconditioned conjugate gradients, accurate to FP64.
 //
 // For a pore cell P the discrete equation is
 //   sum_f T_f (psi_nb - psi_P) - kdx2 psi_P = 0,
@@ -8,8 +8,10 @@
 // kdx2 = (dx / lambda_D)^2 screens the field (Debye-Hueckel linearisation of
 // Eq. 4-5; 0 gives Laplace).  With the coupling of Eq. 3-5 on, the right-hand
 // side also carries the charge term dx^2 rho_e / (eps_r eps_0) of every pore
-// cell (Eq. 5 from the current concentrations).  All CG scalars stay on the
-// device; the host only polls the convergence flag every few iterations.
+// cell (Eq. 5 from the current concentrations).  The linear modes run as FP32
+// corrections of an FP64 residual (k_psi_refine); the nonlinear mode, and what
+// the corrections cannot solve, as an FP64 iteration whose scalars stay on the
+// device, its convergence flag polled every few iterations.
 #include <cmath>
 
 #include "cdi_internal.cuh"
@@ -280,6 +282,200 @@ __global__ void k_cg_dir(long long N, double *__restrict__ p, const double *__re
     p[P] = zq[P] + beta * p[P];
 }
 
+// ---------------------------------------------------------------------------
+// The linear potential by iterative refinement: the residual b - A x and the
+// sums x += d in FP64, the corrections A d = r by the same Jacobi-PCG in FP32
+// to a relative 1e-4, repeated until the FP64 residual itself (not a
+// recurrence of it) is below tol.  One cooperative launch, vectors by pore
+// rank.
+//
+// Why: at 2 FP64 operations a clock and SM an FP64 iteration is bound by its
+// arithmetic (14 operations a cell and a division), and as three launches over
+// the whole lattice with 64-bit coordinate divisions it took far longer; an
+// FP32 iteration moves 64 bytes a cell, out of L2 up to 128^3.  The direction
+// update is folded into the product (a neighbour's new p from its z and old
+// p), which leaves two grid barriers an iteration.
+// ---------------------------------------------------------------------------
+struct PsiArgs {
+  const NFlag *fl;    // per rank face flags
+  const int *lat;     // lateral neighbour ranks
+  const int *cells;
+  const double *src;  // lattice order, or null
+  int n, walls, max_iter;
+  double kdx2, psi_s, tol;
+  double *x;          // rank order
+  float *f;           // 6 n: p (two buffers), z, r, d, q
+  uint16_t *meta;     // n: see psi_meta
+  double *psi;        // lattice order, zero at solid cells
+  double *part, *scal;
+  unsigned *counter;
+};
+
+// Open (pore) faces of a pore cell in bits 8.., the integer part of its
+// diagonal (1 a pore or inlet face, 2 a solid one) below.
+template <int DIM> __device__ __forceinline__ unsigned psi_meta(unsigned f, int walls, int &solids) {
+  unsigned t = 0, open = 0;
+  solids = 0;
+#pragma unroll
+  for (int fc = 0; fc < 2 * DIM; fc++) {
+    const bool solid = (f >> (kFaceBit + fc)) & 1u, edge = (f >> (kEdgeBit + fc)) & 1u;
+    if (fc == 1 && edge) {
+      t += 1;                                          // inlet feed
+    } else if (edge && (fc == 0 || (fc > 1 && walls))) {
+    } else if (solid) {                                // no flux above
+      t += 2;
+      solids++;
+    } else {
+      t += 1;
+      open |= 1u << fc;
+    }
+  }
+  return t | open << 8;
+}
+
+template <int DIM, typename F>
+__device__ __forceinline__ void psi_faces(const int *__restrict__ lat, unsigned m, int n, int r,
+                                          F fn) {
+  int q[2 * DIM];
+#pragma unroll
+  for (int f = 0; f < 2 * DIM; f++)
+    q[f] = f < 2 ? r + (f == 0 ? 1 : -1) : lat[(size_t)(f - 2) * n + r];
+#pragma unroll
+  for (int f = 0; f < 2 * DIM; f++)
+    if ((m >> (8 + f)) & 1u) fn(q[f]);
+}
+
+// s + c += v (the rounding errors of s gathered in c).
+__device__ __forceinline__ void sum_acc(float v, float &s, float &c) {
+  const float t = __fadd_rn(s, v), b = __fsub_rn(t, s);
+  c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b)));
+  s = t;
+}
+
+template <int DIM> __global__ void __launch_bounds__(kGridThreads) k_psi_refine(PsiArgs a) {
+  __shared__ double sm[2 * kGridThreads];
+  __shared__ double tot[kGridSums];
+  __shared__ float dia[16], idia[16];
+  const int first = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+  const size_t n = (size_t)a.n;
+  float *p0 = a.f, *p1 = a.f + n, *z = a.f + 2 * n, *rr = a.f + 3 * n, *d = a.f + 4 * n,
+        *q = a.f + 5 * n;
+  GridBarrier bar{a.counter, a.part, 0u, 0};
+  if (threadIdx.x < 16) {
+    const double v = a.kdx2 + threadIdx.x;
+    dia[threadIdx.x] = (float)v;
+    idia[threadIdx.x] = v > 0.0 ? (float)(1.0 / v) : 0.f;
+  }
+  double v[2] = {0.0, 0.0};
+  for (int r = first; r < a.n; r += stride) {
+    int solids;
+    a.meta[r] = (uint16_t)psi_meta<DIM>(a.fl[r], a.walls, solids);
+    const double b = 2.0 * solids * a.psi_s + (a.src ? a.src[a.cells[r]] : 0.0);
+    a.x[r] = 0.0;
+    v[0] += b * b;
+  }
+  {
+    const double w[1] = {v[0]};
+    grid_partial<1>(bar, w, sm, 0);
+  }
+  if (!grid_totals(bar, tot, 1)) return grid_give_up(a.scal + S_CG_ALPHA);
+  const double bb = tot[0];
+  double rel = bb > 0.0 ? 1.0 : 0.0, scale = bb > 0.0 ? sqrt(a.n / bb) : 1.0;
+  int it = 0;
+  bool done = bb == 0.0;
+
+  for (int cycle = 0; !done; cycle++) {
+    // r = b - A x, its FP32 image scaled to a mean square of about 1
+    v[0] = 0.0;
+    float zs = 0.f, zc = 0.f;
+    for (int r = first; r < a.n; r += stride) {
+      const unsigned m = a.meta[r];
+      int solids;
+      psi_meta<DIM>(a.fl[r], a.walls, solids);
+      double res = 2.0 * solids * a.psi_s + (a.src ? a.src[a.cells[r]] : 0.0);
+      if (cycle > 0) {
+        psi_faces<DIM>(a.lat, m, a.n, r, [&](int k) { res += a.x[k]; });
+        res -= (a.kdx2 + (m & 255u)) * a.x[r];
+      }
+      v[0] += res * res;
+      const float rv = (float)(res * scale), zv = rv * idia[m & 255u];
+      rr[r] = rv;
+      z[r] = zv;
+      d[r] = 0.f;
+      p0[r] = 0.f;
+      sum_acc(rv * zv, zs, zc);
+    }
+    v[1] = (double)zs + (double)zc;
+    grid_partial<2>(bar, v, sm, 0);
+    if (!grid_totals(bar, tot, 2)) return grid_give_up(a.scal + S_CG_ALPHA);
+    const double rr64 = tot[0], old = rel;
+    double rz = tot[1];
+    rel = sqrt(rr64 / bb);
+    if (rel < a.tol || rr64 == 0.0) {
+      done = true;
+      break;
+    }
+    if (it >= a.max_iter || (cycle > 0 && !(rel < 0.5 * old))) break;
+
+    const double eta = fmin(fmax(0.3 * a.tol / rel, 1e-4), 0.1);
+    const double target = eta * eta * (rr64 * scale * scale);
+    double rr32 = 0.0;
+    float beta = 0.f;
+    while (it < a.max_iter) {
+      // p = z + beta p, q = A p; p . q
+      float s = 0.f, c = 0.f;
+      for (int r = first; r < a.n; r += stride) {
+        const unsigned m = a.meta[r];
+        const float pv = fmaf(beta, p0[r], z[r]);
+        float off = 0.f;
+        psi_faces<DIM>(a.lat, m, a.n, r, [&](int k) { off += fmaf(beta, p0[k], z[k]); });
+        const float qv = fmaf(dia[m & 255u], pv, -off);
+        p1[r] = pv;
+        q[r] = qv;
+        sum_acc(pv * qv, s, c);
+      }
+      {
+        const double w[1] = {(double)s + (double)c};
+        grid_partial<1>(bar, w, sm, 0);
+      }
+      if (!grid_totals(bar, tot, 1)) return grid_give_up(a.scal + S_CG_ALPHA);
+      const double pq = tot[0];
+      const float alpha = pq != 0.0 ? (float)(rz / pq) : 0.f;
+      // d += alpha p, r -= alpha q, z = r / diag; r . z and r . r
+      float zs = 0.f, zc = 0.f, rs = 0.f, rc = 0.f;
+      for (int r = first; r < a.n; r += stride) {
+        const float rv = fmaf(-alpha, q[r], rr[r]), zv = rv * idia[a.meta[r] & 255u];
+        d[r] = fmaf(alpha, p1[r], d[r]);
+        rr[r] = rv;
+        z[r] = zv;
+        sum_acc(rv * zv, zs, zc);
+        sum_acc(rv * rv, rs, rc);
+      }
+      const double w[2] = {(double)zs + (double)zc, (double)rs + (double)rc};
+      grid_partial<2>(bar, w, sm, 0);
+      if (!grid_totals(bar, tot, 2)) return grid_give_up(a.scal + S_CG_ALPHA);
+      beta = rz != 0.0 ? (float)(tot[0] / rz) : 0.f;
+      rz = tot[0];
+      rr32 = tot[1];
+      float *t = p0;
+      p0 = p1;
+      p1 = t;
+      it++;
+      if (!(rr32 > target)) break;  // (a NaN also ends it: the cycle's test sees that)
+    }
+    // x += d
+    for (int r = first; r < a.n; r += stride) a.x[r] += (double)d[r] / scale;
+    if (!grid_totals(bar, tot, 0)) return grid_give_up(a.scal + S_CG_ALPHA);
+    if (rr32 > 0.0 && rr32 < 1e30) scale *= sqrt(a.n / rr32);
+  }
+  for (int r = first; r < a.n; r += stride) a.psi[a.cells[r]] = a.x[r];
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    a.scal[S_CG_REL] = rel;
+    a.scal[S_CG_DONE] = done ? 1.0 : 0.0;
+    a.scal[S_CG_IT] = it;
+  }
+}
+
 // The charge term of Eq. 4 at every pore cell from Eq. 5:
 // src = coef * sum_k z_k C_k, coef = F dx^2 / (eps_r eps_0) (lattice order;
 // solid cells keep the 0 the caller cleared).
@@ -341,19 +537,72 @@ static cdi_status cg_iterate(cdi_domain *d, const Geo &g, double *r, double *p, 
 static cdi_status finish_potential(cdi_domain *d, cudaEvent_t ev, bool done, int *iters,
                                    double *relres);
 
+// The refinement above; *done says whether it reached tol.  Where it does not
+// (max_iter ran out first, tol below what an FP64 residual can show, or a
+// system too ill-conditioned for FP32 corrections) the caller starts over
+// with the FP64 iteration, whose own residual is a recurrence.
+static cdi_status psi_refine(cdi_domain *d, double psi_s, double kdx2, const double *src,
+                             double tol, int max_iter, bool *done) {
+  *done = false;
+  const void *kern = d->dim == 2 ? (const void *)k_psi_refine<2> : (const void *)k_psi_refine<3>;
+  const int n = (int)d->n_pore;
+  int threads = 0;
+  const int blocks = n > 0 ? grid_shape(kern, n, &threads) : 0;
+  if (blocks == 0) return CDI_OK;
+  PsiArgs a;
+  a.fl = d->d_cfl;
+  a.lat = d->d_latnb;
+  a.cells = d->d_cell_list;
+  a.src = src;
+  a.n = n;
+  a.walls = d->walls;
+  a.max_iter = max_iter;
+  a.kdx2 = kdx2;
+  a.psi_s = psi_s;
+  a.tol = tol;
+  a.x = (double *)d->d_phi;  // 8 bytes a rank; phi is formed again after the solve
+  a.f = (float *)d->d_cg;    // 26 of its 32 bytes a cell
+  a.meta = (uint16_t *)(a.f + 6 * (size_t)n);
+  a.psi = d->d_psi;
+  a.part = d->d_part;
+  a.scal = d->d_scal;
+  a.counter = d->d_counter + C_CG1;
+  CDI_TRY(d, cudaMemsetAsync(d->d_psi, 0, (size_t)d->N * 8, d->stream), "potential reset");
+  CDI_TRY(d, cudaMemsetAsync(a.counter, 0, sizeof(unsigned), d->stream), "potential barrier");
+  CDI_TRY(d, cudaMemsetAsync(d->d_scal + S_CG_ALPHA, 0, sizeof(double), d->stream),
+          "potential barrier");
+  void *args[] = {&a};
+  CDI_TRY(d, cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3(threads), args, 0, d->stream),
+          "potential solve");
+  d->timing.kernel_launches++;
+  CDI_TRY(d, cudaMemcpyAsync(d->h_scal + S_CG_ALPHA, d->d_scal + S_CG_ALPHA, 8 * sizeof(double),
+                             cudaMemcpyDeviceToHost, d->stream),
+          "potential result");
+  // the barrier's arrivals leave the slot that other kernels expect at 0
+  CDI_TRY(d, cudaMemsetAsync(a.counter, 0, sizeof(unsigned), d->stream), "potential barrier");
+  CDI_TRY(d, cudaStreamSynchronize(d->stream), "potential");
+  if (d->h_scal[S_CG_ALPHA] != 0.0)
+    return cdi_fail(d, CDI_ERR_CUDA, "potential solve: a grid barrier ran into its limit");
+  *done = d->h_scal[S_CG_DONE] != 0.0;
+  return CDI_OK;
+}
+
 cdi_status cdi_psi_solve(cdi_domain *d, double psi_s, double kdx2, const double *src,
                          double tol, int max_iter, int *iters, double *relres) {
   Geo g{d->nx, d->ny, d->nz, d->dim, d->walls, d->N};
   double *r = d->d_cg, *p = d->d_cg + d->N, *q = d->d_cg + 2 * d->N, *dg = d->d_cg + 3 * d->N;
   cudaEvent_t ev;
   cdi_timing_begin(d, &ev);
+  bool done = false;
+  cdi_status cs = psi_refine(d, psi_s, kdx2, src, tol, max_iter, &done);
+  if (cs != CDI_OK) return cs;
+  if (done) return finish_potential(d, ev, done, iters, relres);
   k_cg_setup<<<kRedBlocks, kRedThreads, 0, d->stream>>>(g, d->d_nflags, kdx2, psi_s, src, tol,
                                                          d->d_psi, r, p, dg, d->d_part,
                                                          d->d_counter + C_CG1, d->d_scal);
   d->timing.kernel_launches++;
   CDI_TRY(d, cudaGetLastError(), "cg setup");
-  bool done = false;
-  cdi_status cs = cg_iterate(d, g, r, p, q, dg, max_iter, &done);
+  cs = cg_iterate(d, g, r, p, q, dg, max_iter, &done);
   if (cs != CDI_OK) return cs;
   return finish_potential(d, ev, done, iters, relres);
 }
