@@ -442,17 +442,16 @@ __global__ void k_links_ovf(const typename FlowFlag<DIM>::type *__restrict__ fl,
 // (more resident blocks per SM: the step is latency-bound on its scattered
 // loads, so occupancy matters more than a few spare registers; the bound is
 // chosen per variant so that nothing spills)
+// (lbm_collide: FP32 and BF16 storage; gi the values read.)
 template <typename S, int DIM, bool ODD, typename PL>
-__device__ __forceinline__ void lbm_body_nb(const PL &g, const int (&nb)[Lat<DIM>::Q], int k0,
+__device__ __forceinline__ void lbm_collide(const PL &g, const int (&nb)[Lat<DIM>::Q], int k0,
+                                            const typename Arith<S>::type (&gi)[Lat<DIM>::Q],
                                             typename Arith<S>::type omega,
                                             typename Arith<S>::type fx_half,
                                             typename Arith<S>::type fsrc) {
   using T = typename Arith<S>::type;
   using L = Lat<DIM>;
   constexpr int Q = L::Q;
-  T gi[Q];
-#pragma unroll
-  for (int i = 0; i < Q; i++) gi[i] = widen(*slot_ptr<DIM, ODD, true>(g, nb, k0, i));
   T drho = T(0), jx = fx_half, jy = T(0), jz = T(0);
 #pragma unroll
   for (int i = 0; i < Q; i++) {
@@ -489,6 +488,89 @@ __device__ __forceinline__ void lbm_body_nb(const PL &g, const int (&nb)[Lat<DIM
   }
   const T go0 = kClose ? (T)__fadd_rn(__fsub_rn(ms, ss), __fsub_rn(mc, sc)) : post(0);
   *slot_ptr<DIM, ODD, false>(g, nb, k0, 0) = narrow<S>(go0);
+}
+
+// The FP64 collision by opposite pairs (i, o): with s = g_i + g_o and d = g_i -
+// g_o, drho = g_0 + sum s and j = F/2 + sum e d, and both post-collision values
+// are (1 - omega) g + (A_w +- E), A_w = omega w drho by weight class, E = e.(3
+// omega w j + w (1 - 1/(2 tau)) 3 F) with its components formed once per
+// class.  With tau = 1 the first term is zero and left out.  At 2 FP64
+// operations a clock and SM the arithmetic is what bounds a small image:
+// D2Q9 34 operations a site (43 with tau != 1) instead of about 75 term by
+// term; 128x64 image 4.9 -> 3.4 us a step.  (FP32 storage keeps the terms of
+// lbm_collide: there the rounded class constants cost accuracy, 2.5e-7 -> 1.1e-6
+// of the velocity in 600 steps on a 256^3 pack.)
+template <int DIM, bool ODD, typename PL>
+__device__ __forceinline__ void lbm_collide_f64(const PL &g, const int (&nb)[Lat<DIM>::Q], int k0,
+                                                const double (&gi)[Lat<DIM>::Q], double omega,
+                                                double fx_half, double fsrc) {
+  using L = Lat<DIM>;
+  constexpr int H = L::H;
+  double drho = gi[0], j[3] = {fx_half, 0.0, 0.0};
+#pragma unroll
+  for (int i = 1; i <= H; i++) {
+    const double d = r_sub(gi[i], gi[i + H]);
+    drho = r_add(drho, r_add(gi[i], gi[i + H]));
+    const int e[3] = {L::ex(i), L::ey(i), L::ez(i)};
+#pragma unroll
+    for (int a = 0; a < DIM; a++) {
+      if (e[a] > 0) j[a] = r_add(j[a], d);
+      if (e[a] < 0) j[a] = r_sub(j[a], d);
+    }
+  }
+  constexpr double wa = L::w(1), wd = L::w(H);
+  auto collide = [&](auto tau1) {
+    constexpr bool T1 = decltype(tau1)::value;
+    auto scaled = [&](double w) { return T1 ? w : r_mul(omega, w); };
+    const double om1 = T1 ? 0.0 : r_sub(1.0, omega);
+    const double A0 = r_mul(scaled(L::w(0)), drho), Aa = r_mul(scaled(wa), drho),
+                 Ad = r_mul(scaled(wd), drho);
+    double Ja[DIM], Jd[DIM];
+#pragma unroll
+    for (int a = 0; a < DIM; a++) {
+      Ja[a] = r_mul(scaled(3.0 * wa), j[a]);
+      Jd[a] = r_mul(scaled(3.0 * wd), j[a]);
+    }
+    Ja[0] = r_fma(wa, fsrc, Ja[0]);
+    Jd[0] = r_fma(wd, fsrc, Jd[0]);
+    auto out = [&](int i, double eq) {
+      *slot_ptr<DIM, ODD, false>(g, nb, k0, i) = T1 ? eq : r_fma(om1, gi[i], eq);
+    };
+#pragma unroll
+    for (int i = 1; i <= H; i++) {
+      const int e[3] = {L::ex(i), L::ey(i), L::ez(i)};
+      const bool axis = e[0] * e[0] + e[1] * e[1] + e[2] * e[2] == 1;
+      double E = 0.0;
+      bool some = false;
+#pragma unroll
+      for (int a = 0; a < DIM; a++) {
+        if (e[a] == 0) continue;
+        const double c = axis ? Ja[a] : Jd[a];
+        E = some ? (e[a] > 0 ? r_add(E, c) : r_sub(E, c)) : (e[a] > 0 ? c : -c);
+        some = true;
+      }
+      out(i, r_add(axis ? Aa : Ad, E));
+      out(i + H, r_sub(axis ? Aa : Ad, E));
+    }
+    out(0, A0);
+  };
+  // (an integer test: an FP64 comparison would take the FP64 pipe)
+  if (__double_as_longlong(omega) == __double_as_longlong(1.0)) collide(std::true_type());
+  else collide(std::false_type());
+}
+
+template <typename S, int DIM, bool ODD, typename PL>
+__device__ __forceinline__ void lbm_body_nb(const PL &g, const int (&nb)[Lat<DIM>::Q], int k0,
+                                            typename Arith<S>::type omega,
+                                            typename Arith<S>::type fx_half,
+                                            typename Arith<S>::type fsrc) {
+  typename Arith<S>::type gi[Lat<DIM>::Q];
+#pragma unroll
+  for (int i = 0; i < Lat<DIM>::Q; i++) gi[i] = widen(*slot_ptr<DIM, ODD, true>(g, nb, k0, i));
+  if constexpr (std::is_same<S, double>::value)
+    lbm_collide_f64<DIM, ODD>(g, nb, k0, gi, omega, fx_half, fsrc);
+  else
+    lbm_collide<S, DIM, ODD>(g, nb, k0, gi, omega, fx_half, fsrc);
 }
 
 template <typename S, int DIM, bool ODD, typename PL>
@@ -885,14 +967,16 @@ void step_pair_bs(cdi_domain *d, cudaStream_t st, double tau, double force) {
       if constexpr (MI == 0)
         k_lbm_step_split<DIM, false, T1, BS><<<grid, BS, 0, st>>>(gh, gl, lk, n, c);
       else
-        k_lbm_step_split_occ<DIM, false, T1, BS, MI><<<grid, BS, 0, st>>>(gh, gl, lk, n, c);
+        k_lbm_step_split_occ<DIM, false, T1, BS, MI><<<grid, BS, 0, st>>>(gh, gl, lk,
+                   n, c);
       if constexpr (MINT < 0) {
         auto *kern = k_lbm_split_odd_pf<DIM, T1, BS>;
         kern<<<resident_grid(kern, BS, n), BS, 0, st>>>(gh, gl, lk, n, c);
       } else if constexpr (MI == 0) {
         k_lbm_step_split<DIM, true, T1, BS><<<grid, BS, 0, st>>>(gh, gl, lk, n, c);
       } else {
-        k_lbm_step_split_occ<DIM, true, T1, BS, MI><<<grid, BS, 0, st>>>(gh, gl, lk, n, c);
+        k_lbm_step_split_occ<DIM, true, T1, BS, MI><<<grid, BS, 0, st>>>(gh, gl, lk,
+                   n, c);
       }
     };
     if (tau == 1.0) pair(std::true_type());
@@ -905,7 +989,8 @@ void step_pair_bs(cdi_domain *d, cudaStream_t st, double tau, double force) {
     k_lbm_step<T, DIM, false, BS, MI><<<grid, BS, 0, st>>>(g, lk, n, omega, fxh, fsrc);
     if constexpr (MINT < 0) {
       auto *kern = k_lbm_odd_pf<T, DIM, BS>;
-      kern<<<resident_grid(kern, BS, n), BS, 0, st>>>(g, lk, n, omega, fxh, fsrc);
+      kern<<<resident_grid(kern, BS, n), BS, 0, st>>>(g, lk, n, omega, fxh,
+                 fsrc);
     } else {
       k_lbm_step<T, DIM, true, BS, MI><<<grid, BS, 0, st>>>(g, lk, n, omega, fxh, fsrc);
     }
@@ -1146,15 +1231,11 @@ cdi_status flow_batch(cdi_domain *const *doms, int n_doms, const cdi_flow_params
     for (int k = 0; k < K / 2; k++) {
       const bool t1 = M == M_SPLIT && tau == 1.0;
       if (t1) {
-        k_lbm_batch<S, DIM, false, M, true><<<blocks, kLbmBatchBlock, 0, L->cap_stream>>>(
-            dtab, nm, omega, fxh, fsrc, c);
-        k_lbm_batch<S, DIM, true, M, true><<<blocks, kLbmBatchBlock, 0, L->cap_stream>>>(
-            dtab, nm, omega, fxh, fsrc, c);
+        k_lbm_batch<S, DIM, false, M, true><<<blocks, kLbmBatchBlock, 0, L->cap_stream>>>(dtab, nm, omega, fxh, fsrc, c);
+        k_lbm_batch<S, DIM, true, M, true><<<blocks, kLbmBatchBlock, 0, L->cap_stream>>>(dtab, nm, omega, fxh, fsrc, c);
       } else {
-        k_lbm_batch<S, DIM, false, M, false><<<blocks, kLbmBatchBlock, 0, L->cap_stream>>>(
-            dtab, nm, omega, fxh, fsrc, c);
-        k_lbm_batch<S, DIM, true, M, false><<<blocks, kLbmBatchBlock, 0, L->cap_stream>>>(
-            dtab, nm, omega, fxh, fsrc, c);
+        k_lbm_batch<S, DIM, false, M, false><<<blocks, kLbmBatchBlock, 0, L->cap_stream>>>(dtab, nm, omega, fxh, fsrc, c);
+        k_lbm_batch<S, DIM, true, M, false><<<blocks, kLbmBatchBlock, 0, L->cap_stream>>>(dtab, nm, omega, fxh, fsrc, c);
       }
     }
     cudaError_t e = cudaStreamEndCapture(L->cap_stream, &graph);
