@@ -435,6 +435,10 @@ __global__ void k_links_ovf(const typename FlowFlag<DIM>::type *__restrict__ fl,
   }
 }
 
+// The steps of a solve follow one another by programmatic dependent launch: a
+// step's blocks come up and read their link data (which no step writes) while
+// the step before it ends, and wait there for its populations.  The next
+// launch is allowed only behind that wait, so at most two steps overlap.
 // One full lattice Boltzmann step (stream + collide) at every pore site,
 // FP64, FP32 or BF16 storage (S), arithmetic in T = Arith<S>.  Collision (Eq. 8) with the Stokes-linear
 // equilibrium g_eq_i = w_i (drho + 3 e_i.j), j = sum e_i g_i + F/2, and the
@@ -580,6 +584,8 @@ __device__ __forceinline__ void lbm_body(const PL &g, const LinkGeo &lg, int n, 
                                          typename Arith<S>::type fsrc) {
   int nb[Lat<DIM>::Q];
   load_links<DIM, ODD>(lg, k0, n, nb);
+  pdl_wait();
+  pdl_launch();
   lbm_body_nb<S, DIM, ODD>(g, nb, k0, omega, fx_half, fsrc);
 }
 
@@ -596,6 +602,8 @@ __global__ void __launch_bounds__(BS, sizeof(S) == 8 ? 1 : (DIM == 2 ? 8 : 6) * 
   int k = blockIdx.x * BS + threadIdx.x;
   if (k >= n) return;
   LinkData<DIM> cur = load_link_data<DIM>(lg, k, n);
+  pdl_wait();
+  pdl_launch();
   while (true) {
     const int kn = k + stride;
     LinkData<DIM> nxt;
@@ -709,6 +717,8 @@ __device__ __forceinline__ void lbm_split_body(const PL &gh, const PL &gl, const
                                                int n, int k0, const SplitConst &c) {
   int nb[Lat<DIM>::Q];
   load_links<DIM, ODD>(lg, k0, n, nb);
+  pdl_wait();
+  pdl_launch();
   lbm_split_body_nb<DIM, ODD, TAU1>(gh, gl, nb, k0, c);
 }
 
@@ -722,6 +732,8 @@ __global__ void __launch_bounds__(BS)
   int k = blockIdx.x * BS + threadIdx.x;
   if (k >= n) return;
   LinkData<DIM> cur = load_link_data<DIM>(lg, k, n);
+  pdl_wait();
+  pdl_launch();
   while (true) {
     const int kn = k + stride;
     LinkData<DIM> nxt;
@@ -965,17 +977,17 @@ void step_pair_bs(cdi_domain *d, cudaStream_t st, double tau, double force) {
     auto pair = [&](auto tau1) {
       constexpr bool T1 = decltype(tau1)::value;
       if constexpr (MI == 0)
-        k_lbm_step_split<DIM, false, T1, BS><<<grid, BS, 0, st>>>(gh, gl, lk, n, c);
+        launch_pdl(k_lbm_step_split<DIM, false, T1, BS>, grid, BS, st, true, gh, gl, lk, n, c);
       else
-        k_lbm_step_split_occ<DIM, false, T1, BS, MI><<<grid, BS, 0, st>>>(gh, gl, lk,
+        launch_pdl(k_lbm_step_split_occ<DIM, false, T1, BS, MI>, grid, BS, st, true, gh, gl, lk,
                    n, c);
       if constexpr (MINT < 0) {
         auto *kern = k_lbm_split_odd_pf<DIM, T1, BS>;
-        kern<<<resident_grid(kern, BS, n), BS, 0, st>>>(gh, gl, lk, n, c);
+        launch_pdl(kern, resident_grid(kern, BS, n), BS, st, true, gh, gl, lk, n, c);
       } else if constexpr (MI == 0) {
-        k_lbm_step_split<DIM, true, T1, BS><<<grid, BS, 0, st>>>(gh, gl, lk, n, c);
+        launch_pdl(k_lbm_step_split<DIM, true, T1, BS>, grid, BS, st, true, gh, gl, lk, n, c);
       } else {
-        k_lbm_step_split_occ<DIM, true, T1, BS, MI><<<grid, BS, 0, st>>>(gh, gl, lk,
+        launch_pdl(k_lbm_step_split_occ<DIM, true, T1, BS, MI>, grid, BS, st, true, gh, gl, lk,
                    n, c);
       }
     };
@@ -986,13 +998,13 @@ void step_pair_bs(cdi_domain *d, cudaStream_t st, double tau, double force) {
     const A omega = A(1.0 / tau), fxh = A(0.5 * force);
     const A fsrc = A((1.0 - 0.5 / tau) * 3.0 * force);
     const Planes<T, Q> g = make_planes<T, Q>((T *)d->d_g, n);
-    k_lbm_step<T, DIM, false, BS, MI><<<grid, BS, 0, st>>>(g, lk, n, omega, fxh, fsrc);
+    launch_pdl(k_lbm_step<T, DIM, false, BS, MI>, grid, BS, st, true, g, lk, n, omega, fxh, fsrc);
     if constexpr (MINT < 0) {
       auto *kern = k_lbm_odd_pf<T, DIM, BS>;
-      kern<<<resident_grid(kern, BS, n), BS, 0, st>>>(g, lk, n, omega, fxh,
+      launch_pdl(kern, resident_grid(kern, BS, n), BS, st, true, g, lk, n, omega, fxh,
                  fsrc);
     } else {
-      k_lbm_step<T, DIM, true, BS, MI><<<grid, BS, 0, st>>>(g, lk, n, omega, fxh, fsrc);
+      launch_pdl(k_lbm_step<T, DIM, true, BS, MI>, grid, BS, st, true, g, lk, n, omega, fxh, fsrc);
     }
   }
 }
@@ -1231,11 +1243,15 @@ cdi_status flow_batch(cdi_domain *const *doms, int n_doms, const cdi_flow_params
     for (int k = 0; k < K / 2; k++) {
       const bool t1 = M == M_SPLIT && tau == 1.0;
       if (t1) {
-        k_lbm_batch<S, DIM, false, M, true><<<blocks, kLbmBatchBlock, 0, L->cap_stream>>>(dtab, nm, omega, fxh, fsrc, c);
-        k_lbm_batch<S, DIM, true, M, true><<<blocks, kLbmBatchBlock, 0, L->cap_stream>>>(dtab, nm, omega, fxh, fsrc, c);
+        launch_pdl(k_lbm_batch<S, DIM, false, M, true>, blocks, kLbmBatchBlock, L->cap_stream, k > 0,
+                   dtab, nm, omega, fxh, fsrc, c);
+        launch_pdl(k_lbm_batch<S, DIM, true, M, true>, blocks, kLbmBatchBlock, L->cap_stream, k > 0,
+                   dtab, nm, omega, fxh, fsrc, c);
       } else {
-        k_lbm_batch<S, DIM, false, M, false><<<blocks, kLbmBatchBlock, 0, L->cap_stream>>>(dtab, nm, omega, fxh, fsrc, c);
-        k_lbm_batch<S, DIM, true, M, false><<<blocks, kLbmBatchBlock, 0, L->cap_stream>>>(dtab, nm, omega, fxh, fsrc, c);
+        launch_pdl(k_lbm_batch<S, DIM, false, M, false>, blocks, kLbmBatchBlock, L->cap_stream, k > 0,
+                   dtab, nm, omega, fxh, fsrc, c);
+        launch_pdl(k_lbm_batch<S, DIM, true, M, false>, blocks, kLbmBatchBlock, L->cap_stream, k > 0,
+                   dtab, nm, omega, fxh, fsrc, c);
       }
     }
     cudaError_t e = cudaStreamEndCapture(L->cap_stream, &graph);

@@ -171,6 +171,7 @@ struct NPGeo {
 // with its sign flipped (one shuffle).  Every x face is then evaluated once
 // instead of twice, and every lane of the warp takes the same path.
 constexpr int kHome = 31;
+
 // 16-bit lateral differences: a closed face, and one that does not fit.
 constexpr short kLatClosed = -32768, kLatWide = -32767;
 
@@ -212,8 +213,8 @@ __host__ __device__ constexpr long long np_warps(long long n) { return (n + kHom
 // exponentials and divisions (about 60 FP64 operations a face) out of the
 // step: 128x64 image, two species: 16.4 -> 4.0 us a step.  co null (no memory
 // for them): every face is evaluated from the velocity and the potential.
-template <int DIM>
-__device__ __forceinline__ bool np_cell(const double *__restrict__ Cin, double *__restrict__ Cout,
+template <int DIM, bool EARLY>
+__device__ __forceinline__ bool np_cell(const double *Cin, double *Cout,
                                         const double2 *__restrict__ co,
                                         const double *__restrict__ u,
                                         const double *__restrict__ phi, const NPGeo &g,
@@ -227,13 +228,11 @@ __device__ __forceinline__ bool np_cell(const double *__restrict__ Cin, double *
   q[1] = (f >> (kFaceBit + 1)) & 1u ? -1 : (inlet ? r : r - 1);
 #pragma unroll
   for (int fc = 2; fc < NF; fc++) q[fc] = g.lat[(size_t)(fc - 2) * n + r];
-  const double CP = Cin[r];
   double Cn[NF], Bp[NF], Bm[NF];
 #pragma unroll
   for (int fc = 0; fc < NF; fc++) {
-    Cn[fc] = Bp[fc] = Bm[fc] = 0.0;
+    Bp[fc] = Bm[fc] = 0.0;
     if (q[fc] < 0) continue;
-    Cn[fc] = Cin[q[fc]];
     if (co) {
       const bool feed = fc == 1 && inlet, flip = (fc & 1) && !feed;
       const double2 b = co[feed ? DIM * n + r : (fc >> 1) * n + (flip ? q[fc] : r)];
@@ -248,6 +247,13 @@ __device__ __forceinline__ bool np_cell(const double *__restrict__ Cin, double *
       Bm[fc] = r_mul(c.Ddx[k], Bm[fc]);
     }
   }
+  if (EARLY) {
+    pdl_wait();  // the step before has written C
+    pdl_launch();
+  }
+  const double CP = Cin[r];
+#pragma unroll
+  for (int fc = 0; fc < NF; fc++) Cn[fc] = q[fc] < 0 ? 0.0 : Cin[q[fc]];
   if (inlet) Cn[1] = c.c0;
   const double ns_solid = (double)__popc(f & (((1u << NF) - 1u) << kFaceBit));
   v[0] = r_mul(r_mul(ns_solid, c.Keff[k]), CP);
@@ -392,22 +398,28 @@ template <int NS> __device__ __forceinline__ constexpr int np_k1(int p) {
 
 // The concentration record of rank r in a species-pair plane (two != 0: both
 // species of the pair; else a lone last species, copied into both halves).
-template <bool PAIR>
-__device__ __forceinline__ void rec_load(const float *__restrict__ base, bool two, int r,
-                                         float2 &c, float2 &l) {
+// Read through the non-coherent path, except behind a wait (EARLY: see
+// pdl_wait).
+template <bool EARLY, typename V> __device__ __forceinline__ V rec_get(const V *p) {
+  if constexpr (EARLY) return *p;
+  else return __ldg(p);
+}
+template <bool PAIR, bool EARLY>
+__device__ __forceinline__ void rec_load(const float *base, bool two, int r, float2 &c,
+                                         float2 &l) {
   if (PAIR && two) {
-    const float4 v = __ldg(reinterpret_cast<const float4 *>(base) + r);
+    const float4 v = rec_get<EARLY>(reinterpret_cast<const float4 *>(base) + r);
     c = make_float2(v.x, v.y);
     l = make_float2(v.z, v.w);
   } else if (two) {
-    c = __ldg(reinterpret_cast<const float2 *>(base) + r);
+    c = rec_get<EARLY>(reinterpret_cast<const float2 *>(base) + r);
     l = make_float2(0.f, 0.f);
   } else if (PAIR) {
-    const float2 v = __ldg(reinterpret_cast<const float2 *>(base) + r);
+    const float2 v = rec_get<EARLY>(reinterpret_cast<const float2 *>(base) + r);
     c = bc(v.x);
     l = bc(v.y);
   } else {
-    c = bc(__ldg(base + r));
+    c = bc(rec_get<EARLY>(base + r));
     l = make_float2(0.f, 0.f);
   }
 }
@@ -666,29 +678,40 @@ __device__ __forceinline__ void np_update(const NPFields &F, int n_cells, int na
   }
 }
 
-// Every load of warp w's tile.  All are unconditional: a closed face reads the
-// cell's own record, which costs an L1 hit instead of a branch and moves.
-template <int DIM, int NS, bool PAIR>
+// Every load of warp w's tile, the face data (which no step writes) before
+// the wait for the step before.  All are unconditional: a closed face reads
+// the cell's own record, which costs an L1 hit instead of a branch and moves.
+template <int DIM, int NS, bool PAIR, bool EARLY>
 __device__ __forceinline__ void np_load(const NPFields &F, int n_cells, int naccs, int w, int r,
                                         const NPLinks<DIM> &lk, NPLane<DIM, NS> &V,
                                         float2 (&acc_pre)[(NS + 1) / 2]) {
   constexpr int NL = 2 * DIM - 2, NP = (NS + 1) / 2;
   const int rc = min(max(r, 0), n_cells - 1);
-  np_account_read<NS>(acc_pre, F.acc, w, naccs);
   const bool xp = !(((lk.f >> kFaceBit) | (lk.f >> kEdgeBit)) & 1u);
+  int q[NL];
+#pragma unroll
+  for (int j = 0; j < NL; j++) q[j] = lk.q[j] >= 0 ? lk.q[j] : rc;
+  auto face = [&](int j) { V.fn[j] = __ldg(F.fd[1 + j / 2] + ((j & 1) ? q[j] : rc)); };
+  if (EARLY) {
+    V.fx = __ldg(F.fd[0] + rc);
+#pragma unroll
+    for (int j = 0; j < NL; j++) face(j);
+    pdl_wait();
+    pdl_launch();
+  }
+  np_account_read<NS>(acc_pre, F.acc, w, naccs);
 #pragma unroll
   for (int p = 0; p < NP; p++) {
-    rec_load<PAIR>(F.C[p], 2 * p + 1 < NS, rc, V.C[p], V.Cl[p]);
-    rec_load<PAIR>(F.C[p], 2 * p + 1 < NS, xp ? rc + 1 : rc, V.Cx[p], V.Cxl[p]);
+    rec_load<PAIR, EARLY>(F.C[p], 2 * p + 1 < NS, rc, V.C[p], V.Cl[p]);
+    rec_load<PAIR, EARLY>(F.C[p], 2 * p + 1 < NS, xp ? rc + 1 : rc, V.Cx[p], V.Cxl[p]);
   }
-  V.fx = __ldg(F.fd[0] + rc);
+  if (!EARLY) V.fx = __ldg(F.fd[0] + rc);
 #pragma unroll
   for (int j = 0; j < NL; j++) {
-    const int q = lk.q[j] >= 0 ? lk.q[j] : rc;
 #pragma unroll
     for (int p = 0; p < NP; p++)
-      rec_load<PAIR>(F.C[p], 2 * p + 1 < NS, q, V.Cn[j][p], V.Cnl[j][p]);
-    V.fn[j] = __ldg(F.fd[1 + j / 2] + ((j & 1) ? q : rc));
+      rec_load<PAIR, EARLY>(F.C[p], 2 * p + 1 < NS, q[j], V.Cn[j][p], V.Cnl[j][p]);
+    if (!EARLY) face(j);
   }
 #pragma unroll
   for (int j = 1; j < NL; j += 2) {
@@ -717,7 +740,7 @@ __device__ __forceinline__ void np_load(const NPFields &F, int n_cells, int nacc
 // Otherwise (NP_LARGE) a vote per warp chooses; NP_EVAL is NP_LARGE without
 // stored Bernoulli pairs.
 enum { NP_SMALL = 0, NP_LARGE = 1, NP_EVAL = 2 };
-template <int DIM, int NS, bool PAIR, int MODE>
+template <int DIM, int NS, bool PAIR, int MODE, bool EARLY>
 __device__ __forceinline__ void np_warp31(const NPFields &F, int n_cells, int naccs,
                                           const NPConst<float> &c, int w) {
   constexpr int NL = 2 * DIM - 2, NP = (NS + 1) / 2;
@@ -728,7 +751,7 @@ __device__ __forceinline__ void np_warp31(const NPFields &F, int n_cells, int na
   const NPLinks<DIM> lk = np_links<DIM>(F, n_cells, w);
   NPLane<DIM, NS> V;
   float2 acc_pre[NP];
-  np_load<DIM, NS, PAIR>(F, n_cells, naccs, w, r, lk, V, acc_pre);
+  np_load<DIM, NS, PAIR, EARLY>(F, n_cells, naccs, w, r, lk, V, acc_pre);
   if (MODE != NP_SMALL) {
     bool large = false;
 #pragma unroll
@@ -885,20 +908,19 @@ __global__ void k_np_coef64(const NFlag *__restrict__ fl, const int *__restrict_
 
 // One FP64 step of species k at rank r (of all 32 ranks of its warp) and its
 // account.
-template <int DIM>
-__device__ __forceinline__ void np_step_body(const double *__restrict__ Cin,
-                                             double *__restrict__ Cout,
+template <int DIM, bool EARLY>
+__device__ __forceinline__ void np_step_body(const double *Cin, double *Cout,
                                              const double *__restrict__ u,
                                              const double *__restrict__ phi,
                                              const double2 *__restrict__ co, const NPGeo &g,
-                                             const NPConst<double> &c, double *__restrict__ acc,
-                                             int r, int k) {
+                                             const NPConst<double> &c, double *acc, int r, int k) {
   const size_t n = (size_t)g.n;
   double v[3] = {0.0, 0.0, 0.0};
   bool io = false;
   if (r < g.n)
-    io = np_cell<DIM>(Cin + k * n, Cout + k * n, co ? co + (size_t)k * (DIM + 1) * n : nullptr, u,
+    io = np_cell<DIM, EARLY>(Cin + k * n, Cout + k * n, co ? co + (size_t)k * (DIM + 1) * n : nullptr, u,
                       phi, g, g.fl[r], r, c, k, v);
+  if (EARLY) pdl_wait();  // (a warp without cells has not waited yet)
   np_account(v, io, acc + (size_t)(3 * k) * g.naccs, r >> 5, g.naccs);
 }
 
@@ -948,17 +970,17 @@ __global__ void __launch_bounds__(BS)
                 const __grid_constant__ NPConst<float> c, int ahead) {
   const int w = (int)((blockIdx.x * BS + threadIdx.x) >> 5);
   if (ahead > 0 && threadIdx.x == 0) np_prefetch<DIM, NS, BS / 32, PAIR>(F, n, naccs, w, ahead);
-  np_warp31<DIM, NS, PAIR, MODE>(F, n, naccs, c, w);
+  np_warp31<DIM, NS, PAIR, MODE, true>(F, n, naccs, c, w);
 }
 
 // FP64 storage, one thread per pore cell and species (blockIdx.y).
 template <int DIM, int BS>
 __global__ void __launch_bounds__(BS)
-    k_np_step(const double *__restrict__ Cin, double *__restrict__ Cout,
+    k_np_step(const double *Cin, double *Cout,
               const double *__restrict__ u, const double *__restrict__ phi,
               const double2 *__restrict__ co, NPGeo g, NPConst<double> c,
-              double *__restrict__ acc) {
-  np_step_body<DIM>(Cin, Cout, u, phi, co, g, c, acc, (int)(blockIdx.x * BS + threadIdx.x),
+              double *acc) {
+  np_step_body<DIM, true>(Cin, Cout, u, phi, co, g, c, acc, (int)(blockIdx.x * BS + threadIdx.x),
                     (int)blockIdx.y);
 }
 
@@ -974,6 +996,9 @@ template <typename T> struct SweepMember {
   NPConst<T> c;
 };
 
+// (Sweep and batch steps follow one another in full order, EARLY = false: over
+// their many waves the gap between launches is a small share of a step.)
+//
 // All members of a sweep advance one step in one launch: block (b, m) runs
 // the cells of block b for member m (the block -> cells map, the arithmetic
 // and the accounts of a member are those of a single run's launch, so a
@@ -984,10 +1009,10 @@ __global__ void __launch_bounds__(kRowBlock)
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   const SweepMember<T> &mb = members[blockIdx.y];
   if constexpr (std::is_same<T, float>::value)
-    np_warp31<DIM, NS, PAIR, MODE>(mb.f[in], g.n, g.naccs, mb.c, r >> 5);
+    np_warp31<DIM, NS, PAIR, MODE, false>(mb.f[in], g.n, g.naccs, mb.c, r >> 5);
   else
     for (int k = 0; k < NS; k++)
-      np_step_body<DIM>(mb.C[in], mb.C[1 - in], mb.u, mb.phi, mb.co, g, mb.c, mb.acc, r, k);
+      np_step_body<DIM, false>(mb.C[in], mb.C[1 - in], mb.u, mb.phi, mb.co, g, mb.c, mb.acc, r, k);
 }
 
 // One member of a batch over several geometries: a sweep member plus its
@@ -1017,10 +1042,10 @@ __global__ void __launch_bounds__(kRowBlock)
   const int b = (int)blockIdx.x - mb.block0;
   const int r = b * blockDim.x + threadIdx.x;
   if constexpr (std::is_same<T, float>::value)
-    np_warp31<DIM, NS, PAIR, MODE>(mb.s.f[in], mb.g.n, mb.g.naccs, mb.s.c, r >> 5);
+    np_warp31<DIM, NS, PAIR, MODE, false>(mb.s.f[in], mb.g.n, mb.g.naccs, mb.s.c, r >> 5);
   else
     for (int k = 0; k < NS; k++)
-      np_step_body<DIM>(mb.s.C[in], mb.s.C[1 - in], mb.s.u, mb.s.phi, mb.s.co, mb.g, mb.s.c,
+      np_step_body<DIM, false>(mb.s.C[in], mb.s.C[1 - in], mb.s.u, mb.s.phi, mb.s.co, mb.g, mb.s.c,
                         mb.s.acc, r, k);
 }
 
@@ -1389,8 +1414,11 @@ int np_ahead_tiles(const cdi_domain *d) {
   return step > ((size_t)96 << 20) ? 8192 : 0;
 }
 
+// dep: the launch before this one in the stream is a step too, so this one may
+// start early (launch_pdl).  Behind anything else a step starts in full order:
+// it reads face data and member tables ahead of its wait.
 template <typename T, int DIM, int NS, int BS, bool PAIR>
-void launch_step_bs(cdi_domain *d, cudaStream_t st, int in) {
+void launch_step_bs(cdi_domain *d, cudaStream_t st, int in, bool dep) {
   // FP64: one thread per pore rank; FP32: warps of 31 home cells (one
   // account set per warp either way)
   const long long units = std::is_same<T, float>::value ? np_warps(d->n_pore) * 32 : d->n_pore;
@@ -1401,45 +1429,45 @@ void launch_step_bs(cdi_domain *d, cudaStream_t st, int in) {
     auto *kern = d->np_mode == NP_SMALL   ? k_np_step32<DIM, NS, BS, PAIR, NP_SMALL>
                  : d->np_mode == NP_LARGE ? k_np_step32<DIM, NS, BS, PAIR, NP_LARGE>
                                           : k_np_step32<DIM, NS, BS, PAIR, NP_EVAL>;
-    kern<<<grid, BS, 0, st>>>(F, (int)d->n_pore, d->np_accs, make_const<float>(d),
-                              np_ahead_tiles(d));
+    launch_pdl(kern, grid, BS, st, dep, F, (int)d->n_pore, d->np_accs, make_const<float>(d),
+               np_ahead_tiles(d));
   } else {
-    k_np_step<DIM, BS><<<dim3(grid, NS), BS, 0, st>>>(
-        (const double *)d->d_C[in], (double *)d->d_C[1 - in], (const double *)d->d_u,
-        (const double *)d->d_phi, d->np_mode == NP_EVAL ? nullptr : (const double2 *)d->d_bern,
-        make_geo(d), make_const<double>(d), d->d_acc);
+    launch_pdl(k_np_step<DIM, BS>, dim3(grid, NS), BS, st, dep, (const double *)d->d_C[in],
+               (double *)d->d_C[1 - in], (const double *)d->d_u, (const double *)d->d_phi,
+               d->np_mode == NP_EVAL ? nullptr : (const double2 *)d->d_bern, make_geo(d),
+               make_const<double>(d), d->d_acc);
   }
 }
 
 template <typename T, int DIM, int NS, bool PAIR>
-void launch_step_t(cdi_domain *d, cudaStream_t st, int in) {
+void launch_step_t(cdi_domain *d, cudaStream_t st, int in, bool dep) {
   switch (d->np_block) {
-    case 64: launch_step_bs<T, DIM, NS, 64, PAIR>(d, st, in); break;
-    case 256: launch_step_bs<T, DIM, NS, 256, PAIR>(d, st, in); break;
-    default: launch_step_bs<T, DIM, NS, 128, PAIR>(d, st, in); break;
+    case 64: launch_step_bs<T, DIM, NS, 64, PAIR>(d, st, in, dep); break;
+    case 256: launch_step_bs<T, DIM, NS, 256, PAIR>(d, st, in, dep); break;
+    default: launch_step_bs<T, DIM, NS, 128, PAIR>(d, st, in, dep); break;
   }
 }
 
 template <typename T, int DIM, bool PAIR>
-void launch_step_d(cdi_domain *d, cudaStream_t st, int in) {
+void launch_step_d(cdi_domain *d, cudaStream_t st, int in, bool dep) {
   switch (d->ns) {
-    case 1: launch_step_t<T, DIM, 1, PAIR>(d, st, in); break;
-    case 2: launch_step_t<T, DIM, 2, PAIR>(d, st, in); break;
-    case 3: launch_step_t<T, DIM, 3, PAIR>(d, st, in); break;
-    default: launch_step_t<T, DIM, 4, PAIR>(d, st, in); break;
+    case 1: launch_step_t<T, DIM, 1, PAIR>(d, st, in, dep); break;
+    case 2: launch_step_t<T, DIM, 2, PAIR>(d, st, in, dep); break;
+    case 3: launch_step_t<T, DIM, 3, PAIR>(d, st, in, dep); break;
+    default: launch_step_t<T, DIM, 4, PAIR>(d, st, in, dep); break;
   }
 }
 
-void launch_step(cdi_domain *d, cudaStream_t st, int in) {
+void launch_step(cdi_domain *d, cudaStream_t st, int in, bool dep) {
   if (d->prec == CDI_FP64) {
-    if (d->dim == 2) launch_step_d<double, 2, false>(d, st, in);
-    else launch_step_d<double, 3, false>(d, st, in);
+    if (d->dim == 2) launch_step_d<double, 2, false>(d, st, in, dep);
+    else launch_step_d<double, 3, false>(d, st, in, dep);
   } else if (d->cpair) {
-    if (d->dim == 2) launch_step_d<float, 2, true>(d, st, in);
-    else launch_step_d<float, 3, true>(d, st, in);
+    if (d->dim == 2) launch_step_d<float, 2, true>(d, st, in, dep);
+    else launch_step_d<float, 3, true>(d, st, in, dep);
   } else {
-    if (d->dim == 2) launch_step_d<float, 2, false>(d, st, in);
-    else launch_step_d<float, 3, false>(d, st, in);
+    if (d->dim == 2) launch_step_d<float, 2, false>(d, st, in, dep);
+    else launch_step_d<float, 3, false>(d, st, in, dep);
   }
 }
 
@@ -2015,7 +2043,7 @@ static cdi_status np_steps_coupled(cdi_domain *d, int64_t n) {
     cudaEvent_t ev;
     cdi_timing_begin(d, &ev);
     for (int64_t k = 0; k < block; k++) {
-      launch_step(d, d->stream, d->cur);
+      launch_step(d, d->stream, d->cur, k > 0);
       d->cur = 1 - d->cur;
     }
     CDI_TRY(d, cudaGetLastError(), "transport step");
@@ -2035,7 +2063,7 @@ cdi_status cdi_np_steps(cdi_domain *d, int64_t n) {
   cdi_timing_begin(d, &ev);
   int64_t left = n;
   if (d->cur == 1) {
-    launch_step(d, d->stream, 1);
+    launch_step(d, d->stream, 1, false);
     d->cur = 0;
     left--;
   }
@@ -2044,7 +2072,7 @@ cdi_status cdi_np_steps(cdi_domain *d, int64_t n) {
       cudaGraph_t graph;
       CDI_TRY(d, cudaStreamBeginCapture(d->cap_stream, cudaStreamCaptureModeThreadLocal),
               "begin capture");
-      for (int k = 0; k < kGraphSteps; k++) launch_step(d, d->cap_stream, k & 1);
+      for (int k = 0; k < kGraphSteps; k++) launch_step(d, d->cap_stream, k & 1, k > 0);
       cudaError_t e = cudaStreamEndCapture(d->cap_stream, &graph);
       CDI_TRY(d, e, "end capture");
       e = cudaGraphInstantiate(&d->np_graph, graph, 0);
@@ -2056,10 +2084,9 @@ cdi_status cdi_np_steps(cdi_domain *d, int64_t n) {
       left -= kGraphSteps;
     }
   }
-  while (left > 0) {
-    launch_step(d, d->stream, d->cur);
+  for (bool dep = false; left > 0; left--, dep = true) {
+    launch_step(d, d->stream, d->cur, dep);
     d->cur = 1 - d->cur;
-    left--;
   }
   CDI_TRY(d, cudaGetLastError(), "transport step");
   cdi_timing_end(d, ev, PH_NP, n);
