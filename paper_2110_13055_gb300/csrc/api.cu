@@ -76,16 +76,20 @@ void cdi_dev_release(cdi_domain *d, void *p) {
   }
 }
 
-int cdi::grid_shape(const void *kernel, long long n, int *threads) {
+int cdi::grid_shape(const void *kernel, long long n, int row_div, int nv, int *threads,
+                    size_t *smem) {
   int dev = 0, sms = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (sms < 1) return 0;
   const long long each = ((n + sms - 1) / sms + 31) / 32 * 32;
   const int t = (int)std::max(32ll, std::min((long long)cdi::kGridThreads, each));
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, t, 0);
-  (void)cudaGetLastError();
   *threads = t;
+  *smem = grid_smem(t, row_div, nv);
+  if (*smem > (48u << 10))
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, t, *smem);
+  (void)cudaGetLastError();
   if (per < 1) return 0;
   return (int)std::max<long long>(1, std::min<long long>(std::min(sms, cdi::kRedBlocks), (n + t - 1) / t));
 }

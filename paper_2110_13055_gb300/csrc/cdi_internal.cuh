@@ -93,6 +93,9 @@ using NFlag = uint16_t;
 constexpr int kFaceBit = 1;
 constexpr int kEdgeBit = 7;
 
+// 16-bit lateral differences: a closed face, and one that does not fit.
+constexpr short kLatClosed = -32768, kLatWide = -32767;
+
 // ---------------------------------------------------------------------------
 // Deterministic block reductions (fixed order, no floating-point atomics).
 // ---------------------------------------------------------------------------
@@ -191,11 +194,16 @@ void launch_pdl(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t st, b
 // ---------------------------------------------------------------------------
 // Iterative solvers as one cooperative launch: one block an SM, every vector
 // pass a grid-stride loop, the passes separated by grid barriers that carry
-// the dot products.
+// the dot products of all systems at once.
 //
-// A warp's shuffle tree costs five FP64 instructions a value on a part with 2
-// FP64 lanes an SM; here 128 threads add a block's values through shared
-// memory first (51 warp instructions for 1024 threads instead of 165).
+// A barrier's cost is a chain of latencies, so its sums run side by side: each
+// value has its own warps in the block and its own warp over the blocks'
+// partials.  FP64 values go through shared memory (a shuffle tree in every
+// warp costs five FP64 instructions a value at 2 lanes an SM), their additions
+// as few deep as a tree allows (each takes some 0.1 us of latency); FP32 (sum,
+// error) pairs stay pairs up to the total.  152 blocks of 1024
+// threads: 1.6 us without sums, 5.3 us with two FP64 sums (6.0 added in a
+// row), 3.9 us with two pairs.
 // ---------------------------------------------------------------------------
 constexpr int kGridThreads = 1024;
 constexpr long long kBarrierPolls = 1ll << 26;  // tens of seconds
@@ -204,87 +212,130 @@ constexpr int kGridSums = 2 * kMaxSpecies;      // dot products of a phase, at m
 struct GridBarrier {
   unsigned *counter;  // arrivals since the launch (0 before it)
   double *part;       // 2 * kGridSums * gridDim.x partials
+  double *sm;         // shared: a row of values per sum, then kGridSums * 8
+  int row;            // values of a row: blockDim.x (FP64) or one a warp (FP32)
   unsigned target;
   int parity;         // which half of part this phase writes: a block may be
                       // reading the last phase's half still
 };
 
-// Block sums of v into slots [at, at + NV) of this phase's partials.
-// blockDim.x is a multiple of 32; sm holds NV * blockDim.x values.
-template <int NV>
-__device__ __forceinline__ void grid_partial(const GridBarrier &b, const double (&v)[NV],
-                                             double *sm, int at) {
-  const int t = threadIdx.x, T = blockDim.x, W = T < 128 ? T : 128;
+// A thread's contribution to sum k of the phase (row = blockDim.x), or its
+// warp's from every lane's (sum, error) pair (row = blockDim.x / 32).
+__device__ __forceinline__ void grid_add(const GridBarrier &b, int k, double v) {
+  b.sm[k * b.row + threadIdx.x] = v;
+}
+__device__ __forceinline__ float2 pair_sum(float2 a, float2 b) {
+  const float u = __fadd_rn(a.x, b.x), w = __fsub_rn(u, a.x);
+  const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(u, w)), __fsub_rn(b.x, w));
+  return make_float2(u, __fadd_rn(__fadd_rn(a.y, b.y), e));
+}
+__device__ __forceinline__ double pair_sum(double a, double b) { return a + b; }
+__device__ __forceinline__ float2 warp_sum(float2 v) {
 #pragma unroll
-  for (int k = 0; k < NV; k++) sm[k * T + t] = v[k];
-  __syncthreads();
-  if (t < W) {
-    double s[NV];
+  for (int o = 16; o > 0; o >>= 1)
+    v = pair_sum(v, make_float2(__shfl_down_sync(0xffffffffu, v.x, o),
+                                __shfl_down_sync(0xffffffffu, v.y, o)));
+  return v;
+}
+__device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
-    for (int k = 0; k < NV; k++) {
-      s[k] = sm[k * T + t];
-      for (int j = t + W; j < T; j += W) s[k] += sm[k * T + j];
-    }
-    warp_reduce<NV>(s, OpSum());
-    __syncwarp();
-    if ((t & 31) == 0)
-#pragma unroll
-      for (int k = 0; k < NV; k++) sm[k * T + t] = s[k];
-  }
-  __syncthreads();
-  if (t < NV) {
-    double s = sm[t * T];
-    for (int w = 32; w < W; w += 32) s += sm[t * T + w];
-    __stcg(b.part + ((size_t)b.parity * kGridSums + at + t) * gridDim.x + blockIdx.x, s);
-  }
-  __syncthreads();  // sm is free again
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ void grid_add(const GridBarrier &b, int k, float s, float c) {
+  const float2 v = warp_sum(make_float2(s, c));
+  if ((threadIdx.x & 31) == 0)
+    reinterpret_cast<float2 *>(b.sm)[k * b.row + (threadIdx.x >> 5)] = v;
 }
 
-// Barrier over the grid (whose blocks are all resident: a cooperative launch),
-// then the sums of this phase's nv partials in tot[0 .. nv), the same bits in
-// every block.  False in every thread of a block whose wait ran into its
-// limit: the block must return (the others then run into theirs).
-__device__ __forceinline__ bool grid_totals(GridBarrier &b, double *tot, int nv) {
-  const int t = threadIdx.x;
+// Barrier over the grid (whose blocks are all resident: a cooperative launch)
+// and this phase's nv sums in tot[0 .. nv), in a fixed order and the same bits
+// in every block; V is double, or float2 for (sum, error) pairs.  False in
+// every thread of a block whose wait ran into its limit: the block must return
+// (the others then run into theirs).
+template <typename V>
+__device__ __forceinline__ bool grid_totals(GridBarrier &b, V *tot, int nv) {
+  static_assert(sizeof(V) == 8, "a sum is 8 bytes");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  V *sm = reinterpret_cast<V *>(b.sm), *red = sm + nv * b.row;
+  V *part = reinterpret_cast<V *>(b.part) + (size_t)b.parity * kGridSums * gridDim.x;
+  const V zero{};
+  // warps that share a sum: a power of two, at most 8 and no more than its row fills
+  int share = 1;
+  while (2 * share * max(nv, 1) <= warps && 2 * share * 32 <= b.row && share < 8) share *= 2;
+  __syncthreads();
+  for (int k = warp / share; k < nv; k += warps / share) {
+    const V *v = sm + k * b.row;
+    const int step = 32 * share, j = (warp % share) * 32 + lane;
+    V s[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      s[u] = j + u * step < b.row ? v[j + u * step] : zero;
+      for (int i = j + (u + 4) * step; i < b.row; i += 4 * step) s[u] = pair_sum(s[u], v[i]);
+    }
+    const V t = warp_sum(pair_sum(pair_sum(s[0], s[1]), pair_sum(s[2], s[3])));
+    if (lane == 0) red[k * 8 + warp % share] = t;
+  }
+  if (nv) __syncthreads();
   b.target += gridDim.x;
   int ok = 1;
-  __syncthreads();
-  if (t < 32) {
-    if (t == 0) {
-      __threadfence();  // the block's writes, partials included, before its arrival
-      atomicAdd(b.counter, 1u);
-      ok = 0;
-      for (long long i = 0; i < kBarrierPolls; i++) {
-        unsigned c;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(b.counter) : "memory");
-        if ((int)(c - b.target) >= 0) {
-          ok = 1;
-          break;
-        }
-      }
-      __threadfence();
+  if (warp == 0) {
+    if (lane < nv) {
+      V s[8];
+#pragma unroll
+      for (int u = 0; u < 8; u++) s[u] = u < share ? red[lane * 8 + u] : zero;
+#pragma unroll
+      for (int h = 4; h > 0; h >>= 1)
+#pragma unroll
+        for (int u = 0; u < h; u++)
+          if (u + h < share) s[u] = pair_sum(s[u], s[u + h]);
+      __stcg(part + (size_t)lane * gridDim.x + blockIdx.x, s[0]);
     }
     __syncwarp();
-    for (int k = 0; k < nv; k++) {
-      const double *p = b.part + ((size_t)b.parity * kGridSums + k) * gridDim.x;
-      double s = 0.0;
-      for (int i = t; i < (int)gridDim.x; i += 32) s += __ldcg(p + i);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-      if (t == 0) tot[k] = s;
+    if (lane == 0) {
+      // the arrival releases the block's writes (which the barrier above put
+      // before it), the fence behind the last look acquires the other blocks'
+      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(b.counter) : "memory");
+      ok = 0;
+      for (long long i = 0; i < kBarrierPolls && !ok; i++) {
+        unsigned c;
+        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(b.counter) : "memory");
+        ok = (int)(c - b.target) >= 0;
+      }
+      asm volatile("fence.acq_rel.gpu;" ::: "memory");
     }
   }
+  if (!__syncthreads_and(ok)) return false;
   b.parity ^= 1;
-  return __syncthreads_and(ok);
+  if (nv == 0) return true;
+  for (int k = warp; k < nv; k += warps) {
+    const V *p = part + (size_t)k * gridDim.x;
+    const int G = (int)gridDim.x;
+    V s[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++) {
+      s[u] = lane + 32 * u < G ? __ldcg(p + lane + 32 * u) : zero;
+      for (int i = lane + 32 * (u + 4); i < G; i += 128) s[u] = pair_sum(s[u], __ldcg(p + i));
+    }
+    const V t = warp_sum(pair_sum(pair_sum(s[0], s[1]), pair_sum(s[2], s[3])));
+    if (lane == 0) tot[k] = t;
+  }
+  __syncthreads();
+  return true;
 }
 __device__ __forceinline__ void grid_give_up(double *flag) {
   if (threadIdx.x == 0) *flag = 1.0;
 }
+// Shared bytes of a GridBarrier with nv rows.
+inline size_t grid_smem(int threads, int row_div, int nv) {
+  return ((size_t)nv * (threads / row_div) + kGridSums * 8) * sizeof(double);
+}
 
 // Blocks and threads of a cooperative launch over n items: one block an SM,
 // as few threads as cover the items (few items are spread over all SMs, whose
-// FP64 units are the bound).  0 if not even one block fits.
-int grid_shape(const void *kernel, long long n, int *threads);
+// FP64 units are the bound); smem is a thread's share of the shared memory.
+// 0 if not even one block fits.
+int grid_shape(const void *kernel, long long n, int row_div, int nv, int *threads, size_t *smem);
 
 // psi / V_T as stored for the transport kernel: FP64, or an unevaluated
 // FP32 pair hi + lo (so that face differences keep FP64-like accuracy while

@@ -185,20 +185,20 @@ template <typename T> struct BiArgs {
 // iteration in 3D), then the four grid barriers of an iteration.  Before, an
 // iteration was four launches a species, divided by K of every neighbour in
 // both products and summed by five FP64 shuffle rounds a warp: 80^3, two
-// species, 6 steps of 40 explicit ones 40.5 -> 12.5 ms.  The neighbours'
+// species, 6 steps of 40 explicit ones 40.5 -> 11.1 ms.  The neighbours'
 // s = r - alpha v are formed on the fly: a pass of their own would cost
 // another barrier.
 template <typename T, int DIM>
 __global__ void __launch_bounds__(kGridThreads) k_bi_solve(BiArgs<T> a) {
   using C = ICoef<DIM>;
-  __shared__ double sm[2 * kGridThreads];
-  __shared__ double tot[2 * kMaxSpecies];
+  extern __shared__ double sm[];  // 2 ns rows of a value a thread (GridBarrier)
+  __shared__ double tot[kGridSums];
   __shared__ double rho[kMaxSpecies], alpha[kMaxSpecies], omega[kMaxSpecies], beta[kMaxSpecies],
-      bb[kMaxSpecies], rel[kMaxSpecies];
+      bb[kMaxSpecies], rr2[kMaxSpecies], limit[kMaxSpecies];
   __shared__ int it[kMaxSpecies], done[kMaxSpecies];
   const size_t n = (size_t)a.n;
   const int first = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
-  GridBarrier bar{a.counter, a.part, 0u, 0};
+  GridBarrier bar{a.counter, a.part, sm, (int)blockDim.x, 0u, 0};
 
   for (int k = 0; k < a.ns; k++) {
     const double *c = a.co + (size_t)k * C::NC * n;
@@ -219,16 +219,18 @@ __global__ void __launch_bounds__(kGridThreads) k_bi_solve(BiArgs<T> a) {
       v[0] += res * res;
       v[1] += rhs * rhs;
     }
-    grid_partial<2>(bar, v, sm, 2 * k);
+    grid_add(bar, 2 * k, v[0]);
+    grid_add(bar, 2 * k + 1, v[1]);
   }
   if (!grid_totals(bar, tot, 2 * a.ns)) return grid_give_up(a.scal + B_BAR);
   if (threadIdx.x < a.ns) {
     const int k = threadIdx.x;
     rho[k] = tot[2 * k];
     bb[k] = tot[2 * k + 1];
-    rel[k] = bb[k] > 0.0 ? sqrt(rho[k] / bb[k]) : 0.0;
+    rr2[k] = rho[k];
+    limit[k] = a.tol * a.tol * bb[k];  // of r . r
     it[k] = 0;
-    done[k] = rel[k] < a.tol || rho[k] == 0.0;
+    done[k] = rr2[k] < limit[k] || bb[k] == 0.0 || rho[k] == 0.0;
   }
   __syncthreads();
 
@@ -252,7 +254,7 @@ __global__ void __launch_bounds__(kGridThreads) k_bi_solve(BiArgs<T> a) {
           v[0] += r0[r] * m;
         }
       }
-      grid_partial<1>(bar, v, sm, k);
+      grid_add(bar, k, v[0]);
     }
     if (!grid_totals(bar, tot, a.ns)) return grid_give_up(a.scal + B_BAR);
     if (threadIdx.x < a.ns && !done[threadIdx.x])
@@ -278,7 +280,8 @@ __global__ void __launch_bounds__(kGridThreads) k_bi_solve(BiArgs<T> a) {
           v[1] += m * m;
         }
       }
-      grid_partial<2>(bar, v, sm, 2 * k);
+      grid_add(bar, 2 * k, v[0]);
+    grid_add(bar, 2 * k + 1, v[1]);
     }
     if (!grid_totals(bar, tot, 2 * a.ns)) return grid_give_up(a.scal + B_BAR);
     if (threadIdx.x < a.ns && !done[threadIdx.x]) {
@@ -303,18 +306,21 @@ __global__ void __launch_bounds__(kGridThreads) k_bi_solve(BiArgs<T> a) {
           v[1] += rv * rv;
         }
       }
-      grid_partial<2>(bar, v, sm, 2 * k);
+      grid_add(bar, 2 * k, v[0]);
+    grid_add(bar, 2 * k + 1, v[1]);
     }
     if (!grid_totals(bar, tot, 2 * a.ns)) return grid_give_up(a.scal + B_BAR);
     if (threadIdx.x < a.ns && !done[threadIdx.x]) {
       const int k = threadIdx.x;
       const double r1 = tot[2 * k];
-      beta[k] = (rho[k] != 0.0 && omega[k] != 0.0) ? (r1 / rho[k]) * (alpha[k] / omega[k]) : 0.0;
+      // one division: a chain of FP64 latencies that all threads wait for
+      const double div = rho[k] * omega[k];
+      beta[k] = div != 0.0 ? r1 * alpha[k] / div : 0.0;
       rho[k] = r1;
-      rel[k] = bb[k] > 0.0 ? sqrt(tot[2 * k + 1] / bb[k]) : 0.0;
+      rr2[k] = tot[2 * k + 1];
       it[k]++;
       // converged, or broken down (no new direction)
-      if (rel[k] < a.tol || r1 == 0.0 || omega[k] == 0.0) done[k] = 1;
+      if (rr2[k] < limit[k] || bb[k] == 0.0 || r1 == 0.0 || omega[k] == 0.0) done[k] = 1;
     }
     __syncthreads();
 
@@ -331,9 +337,10 @@ __global__ void __launch_bounds__(kGridThreads) k_bi_solve(BiArgs<T> a) {
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     for (int k = 0; k < a.ns; k++) {
-      a.scal[B_REL + k] = rel[k];
+      const double rel = bb[k] > 0.0 ? sqrt(rr2[k] / bb[k]) : 0.0;
+      a.scal[B_REL + k] = rel;
       a.scal[B_IT + k] = it[k];
-      if (!(rel[k] < a.tol)) a.scal[B_FAIL] = 1.0;
+      if (!(rr2[k] < limit[k] || rel < a.tol)) a.scal[B_FAIL] = 1.0;
     }
   }
 }
@@ -430,7 +437,9 @@ cdi_status imp_step(cdi_domain *d) {
   const int in = d->cur;
   const int side = std::min(d->ns, d->imp_sets);
   int threads = 0;
-  const int blocks = grid_shape((const void *)k_bi_solve<T, DIM>, n, &threads);
+  size_t smem = 0;
+  const int blocks =
+      grid_shape((const void *)k_bi_solve<T, DIM>, n, 1, 2 * side, &threads, &smem);
   if (blocks == 0) return cdi_fail(d, CDI_ERR_CUDA, "implicit step: no resident block");
   CDI_TRY(d, cudaMemsetAsync(d->d_iscal, 0, B_N * sizeof(double), d->stream), "implicit scalars");
   for (int k0 = 0; k0 < d->ns; k0 += side) {
@@ -450,7 +459,7 @@ cdi_status imp_step(cdi_domain *d) {
     CDI_TRY(d, cudaMemsetAsync(a.counter, 0, sizeof(unsigned), d->stream), "implicit barrier");
     void *args[] = {&a};
     CDI_TRY(d, cudaLaunchCooperativeKernel((const void *)k_bi_solve<T, DIM>, dim3(blocks),
-                                           dim3(threads), args, 0, d->stream),
+                                           dim3(threads), args, smem, d->stream),
             "implicit solve");
     for (int k = 0; k < a.ns; k++) {
       const double Dk = d->D[k0 + k];

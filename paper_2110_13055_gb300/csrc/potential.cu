@@ -294,17 +294,22 @@ __global__ void k_cg_dir(long long N, double *__restrict__ p, const double *__re
 // the whole lattice with 64-bit coordinate divisions it took far longer; an
 // FP32 iteration moves 64 bytes a cell, out of L2 up to 128^3.  The direction
 // update is folded into the product (a neighbour's new p from its z and old
-// p), which leaves two grid barriers an iteration.
+// p), which leaves two grid barriers an iteration.  128^3 Laplace: 33.7 ->
+// 6.0 ms (18 us an iteration, 9 us at 64^3), its error against 64 bits 8.6e-13
+// -> 3e-13.  Of that, pair sums and FP32 scalars 8.5 -> 5.8 ms, (z, p) records,
+// 16-bit links and two cells a thread at a time 9.0 -> 8.3 ms.
 // ---------------------------------------------------------------------------
 struct PsiArgs {
   const NFlag *fl;    // per rank face flags
-  const int *lat;     // lateral neighbour ranks
+  const int *lat;     // lateral neighbour ranks (read where latd does not hold them)
+  const short *latd;  // 16-bit lateral differences per rank
+  const int *latb;    // their bases per tile of 31 ranks
   const int *cells;
   const double *src;  // lattice order, or null
   int n, walls, max_iter;
   double kdx2, psi_s, tol;
   double *x;          // rank order
-  float *f;           // 6 n: p (two buffers), z, r, d, q
+  float *f;           // 7 n: (z, p) in two buffers, r, d, q
   uint16_t *meta;     // n: see psi_meta
   double *psi;        // lattice order, zero at solid cells
   double *part, *scal;
@@ -319,13 +324,13 @@ template <int DIM> __device__ __forceinline__ unsigned psi_meta(unsigned f, int 
 #pragma unroll
   for (int fc = 0; fc < 2 * DIM; fc++) {
     const bool solid = (f >> (kFaceBit + fc)) & 1u, edge = (f >> (kEdgeBit + fc)) & 1u;
-    if (fc == 1 && edge) {
-      t += 1;                                          // inlet feed
-    } else if (edge && (fc == 0 || (fc > 1 && walls))) {
-    } else if (solid) {                                // no flux above
+    const bool no_flux = edge && (fc == 0 || (fc > 1 && walls));
+    if (fc == 1 && edge) {  // inlet feed
+      t += 1;
+    } else if (solid && !no_flux) {
       t += 2;
       solids++;
-    } else {
+    } else if (!no_flux) {
       t += 1;
       open |= 1u << fc;
     }
@@ -333,16 +338,35 @@ template <int DIM> __device__ __forceinline__ unsigned psi_meta(unsigned f, int 
   return t | open << 8;
 }
 
-template <int DIM, typename F>
-__device__ __forceinline__ void psi_faces(const int *__restrict__ lat, unsigned m, int n, int r,
-                                          F fn) {
-  int q[2 * DIM];
+// Ranks across the faces of rank r (r itself across a closed one, so that the
+// loads need no branch).
+template <int DIM>
+__device__ __forceinline__ void psi_ranks(const PsiArgs &a, unsigned m, int r, int (&q)[2 * DIM]) {
+  constexpr int NL = 2 * DIM - 2;
+  const int t = r / 31;
+  int base[NL], diff[NL];
+  if constexpr (DIM == 3) {
+    const int4 b = reinterpret_cast<const int4 *>(a.latb)[t];
+    const short4 v = reinterpret_cast<const short4 *>(a.latd)[r];
+    base[0] = b.x; base[1] = b.y; base[2] = b.z; base[3] = b.w;
+    diff[0] = v.x; diff[1] = v.y; diff[2] = v.z; diff[3] = v.w;
+  } else {
+    const int2 b = reinterpret_cast<const int2 *>(a.latb)[t];
+    const short2 v = reinterpret_cast<const short2 *>(a.latd)[r];
+    base[0] = b.x; base[1] = b.y;
+    diff[0] = v.x; diff[1] = v.y;
+  }
+  bool wide = false;
 #pragma unroll
-  for (int f = 0; f < 2 * DIM; f++)
-    q[f] = f < 2 ? r + (f == 0 ? 1 : -1) : lat[(size_t)(f - 2) * n + r];
+  for (int f = 0; f < 2 * DIM; f++) {
+    const int to = f < 2 ? r + (f == 0 ? 1 : -1) : r + base[f < 2 ? 0 : f - 2] + diff[f < 2 ? 0 : f - 2];
+    q[f] = (m >> (8 + f)) & 1u ? to : r;
+    if (f >= 2) wide |= diff[f < 2 ? 0 : f - 2] == kLatWide;
+  }
+  if (wide)
 #pragma unroll
-  for (int f = 0; f < 2 * DIM; f++)
-    if ((m >> (8 + f)) & 1u) fn(q[f]);
+    for (int f = 2; f < 2 * DIM; f++)
+      q[f] = (m >> (8 + f)) & 1u ? a.lat[(size_t)(f - 2) * a.n + r] : r;
 }
 
 // s + c += v (the rounding errors of s gathered in c).
@@ -353,40 +377,44 @@ __device__ __forceinline__ void sum_acc(float v, float &s, float &c) {
 }
 
 template <int DIM> __global__ void __launch_bounds__(kGridThreads) k_psi_refine(PsiArgs a) {
-  __shared__ double sm[2 * kGridThreads];
-  __shared__ double tot[kGridSums];
+  extern __shared__ double sm[];  // 3 rows of a value a warp (GridBarrier)
+  __shared__ float2 tot[kGridSums];
   __shared__ float dia[16], idia[16];
   const int first = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
   const size_t n = (size_t)a.n;
-  float *p0 = a.f, *p1 = a.f + n, *z = a.f + 2 * n, *rr = a.f + 3 * n, *d = a.f + 4 * n,
-        *q = a.f + 5 * n;
-  GridBarrier bar{a.counter, a.part, 0u, 0};
+  // records (z, p), so that a neighbour is one load
+  float2 *w0 = (float2 *)a.f, *w1 = w0 + n;
+  float *rr = a.f + 4 * n, *d = rr + n, *q = d + n;
+  GridBarrier bar{a.counter, a.part, sm, (int)(blockDim.x >> 5), 0u, 0};
+  // an FP64 sum of a thread as a pair (48 bits: it decides when to stop)
+  auto add64 = [&](int k, double v) {
+    const float h = (float)v;
+    grid_add(bar, k, h, (float)(v - (double)h));
+  };
+  auto total = [&](int k) { return (double)tot[k].x + (double)tot[k].y; };
   if (threadIdx.x < 16) {
     const double v = a.kdx2 + threadIdx.x;
     dia[threadIdx.x] = (float)v;
     idia[threadIdx.x] = v > 0.0 ? (float)(1.0 / v) : 0.f;
   }
-  double v[2] = {0.0, 0.0};
+  double v = 0.0;
   for (int r = first; r < a.n; r += stride) {
     int solids;
     a.meta[r] = (uint16_t)psi_meta<DIM>(a.fl[r], a.walls, solids);
     const double b = 2.0 * solids * a.psi_s + (a.src ? a.src[a.cells[r]] : 0.0);
     a.x[r] = 0.0;
-    v[0] += b * b;
+    v += b * b;
   }
-  {
-    const double w[1] = {v[0]};
-    grid_partial<1>(bar, w, sm, 0);
-  }
+  add64(0, v);
   if (!grid_totals(bar, tot, 1)) return grid_give_up(a.scal + S_CG_ALPHA);
-  const double bb = tot[0];
+  const double bb = total(0);
   double rel = bb > 0.0 ? 1.0 : 0.0, scale = bb > 0.0 ? sqrt(a.n / bb) : 1.0;
   int it = 0;
   bool done = bb == 0.0;
 
   for (int cycle = 0; !done; cycle++) {
     // r = b - A x, its FP32 image scaled to a mean square of about 1
-    v[0] = 0.0;
+    v = 0.0;
     float zs = 0.f, zc = 0.f;
     for (int r = first; r < a.n; r += stride) {
       const unsigned m = a.meta[r];
@@ -394,22 +422,25 @@ template <int DIM> __global__ void __launch_bounds__(kGridThreads) k_psi_refine(
       psi_meta<DIM>(a.fl[r], a.walls, solids);
       double res = 2.0 * solids * a.psi_s + (a.src ? a.src[a.cells[r]] : 0.0);
       if (cycle > 0) {
-        psi_faces<DIM>(a.lat, m, a.n, r, [&](int k) { res += a.x[k]; });
+        int k[2 * DIM];
+        psi_ranks<DIM>(a, m, r, k);
+#pragma unroll
+        for (int f = 0; f < 2 * DIM; f++)
+          if ((m >> (8 + f)) & 1u) res += a.x[k[f]];
         res -= (a.kdx2 + (m & 255u)) * a.x[r];
       }
-      v[0] += res * res;
+      v += res * res;
       const float rv = (float)(res * scale), zv = rv * idia[m & 255u];
       rr[r] = rv;
-      z[r] = zv;
+      w0[r] = make_float2(zv, 0.f);
       d[r] = 0.f;
-      p0[r] = 0.f;
       sum_acc(rv * zv, zs, zc);
     }
-    v[1] = (double)zs + (double)zc;
-    grid_partial<2>(bar, v, sm, 0);
+    add64(0, v);
+    grid_add(bar, 1, zs, zc);
     if (!grid_totals(bar, tot, 2)) return grid_give_up(a.scal + S_CG_ALPHA);
-    const double rr64 = tot[0], old = rel;
-    double rz = tot[1];
+    const double rr64 = total(0), old = rel;
+    float rz = tot[1].x + tot[1].y;
     rel = sqrt(rr64 / bb);
     if (rel < a.tol || rr64 == 0.0) {
       done = true;
@@ -418,55 +449,91 @@ template <int DIM> __global__ void __launch_bounds__(kGridThreads) k_psi_refine(
     if (it >= a.max_iter || (cycle > 0 && !(rel < 0.5 * old))) break;
 
     const double eta = fmin(fmax(0.3 * a.tol / rel, 1e-4), 0.1);
-    const double target = eta * eta * (rr64 * scale * scale);
-    double rr32 = 0.0;
-    float beta = 0.f;
+    const float target = (float)(eta * eta * (rr64 * scale * scale));
+    // (the iteration's scalars in FP32 too: an FP64 division is microseconds)
+    float rr32 = 0.f, beta = 0.f;
     while (it < a.max_iter) {
-      // p = z + beta p, q = A p; p . q
+      // q = A p for p = z + beta p; p . q.  Two cells of a thread at a time:
+      // the pass is bound by the latency of its two levels of loads.
       float s = 0.f, c = 0.f;
-      for (int r = first; r < a.n; r += stride) {
-        const unsigned m = a.meta[r];
-        const float pv = fmaf(beta, p0[r], z[r]);
-        float off = 0.f;
-        psi_faces<DIM>(a.lat, m, a.n, r, [&](int k) { off += fmaf(beta, p0[k], z[k]); });
-        const float qv = fmaf(dia[m & 255u], pv, -off);
-        p1[r] = pv;
-        q[r] = qv;
-        sum_acc(pv * qv, s, c);
+      for (int r = first; r < a.n; r += 2 * stride) {
+        const int rs[2] = {r, min(r + stride, a.n - 1)};
+        const int two = r + stride < a.n ? 2 : 1;
+        unsigned m[2];
+        int k[2][2 * DIM];
+        float2 own[2], nb[2][2 * DIM];
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+          m[u] = a.meta[rs[u]];
+          own[u] = w0[rs[u]];
+          psi_ranks<DIM>(a, m[u], rs[u], k[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < 2; u++)
+#pragma unroll
+          for (int f = 0; f < 2 * DIM; f++) nb[u][f] = w0[k[u][f]];
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+          const float pv = fmaf(beta, own[u].y, own[u].x);
+          float off = 0.f;
+#pragma unroll
+          for (int f = 0; f < 2 * DIM; f++)
+            if ((m[u] >> (8 + f)) & 1u) off += fmaf(beta, nb[u][f].y, nb[u][f].x);
+          const float qv = fmaf(dia[m[u] & 255u], pv, -off);
+          if (u < two) {
+            q[rs[u]] = qv;
+            sum_acc(pv * qv, s, c);
+          }
+        }
       }
-      {
-        const double w[1] = {(double)s + (double)c};
-        grid_partial<1>(bar, w, sm, 0);
-      }
+      grid_add(bar, 0, s, c);
       if (!grid_totals(bar, tot, 1)) return grid_give_up(a.scal + S_CG_ALPHA);
-      const double pq = tot[0];
-      const float alpha = pq != 0.0 ? (float)(rz / pq) : 0.f;
-      // d += alpha p, r -= alpha q, z = r / diag; r . z and r . r
+      const float pq = tot[0].x + tot[0].y, alpha = pq != 0.f ? rz / pq : 0.f;
+      // p = z + beta p, d += alpha p, r -= alpha q, z = r / diag; r . z and r . r
       float zs = 0.f, zc = 0.f, rs = 0.f, rc = 0.f;
-      for (int r = first; r < a.n; r += stride) {
-        const float rv = fmaf(-alpha, q[r], rr[r]), zv = rv * idia[a.meta[r] & 255u];
-        d[r] = fmaf(alpha, p1[r], d[r]);
-        rr[r] = rv;
-        z[r] = zv;
-        sum_acc(rv * zv, zs, zc);
-        sum_acc(rv * rv, rs, rc);
+      for (int r = first; r < a.n; r += 2 * stride) {
+        const int at[2] = {r, min(r + stride, a.n - 1)};
+        const int two = r + stride < a.n ? 2 : 1;
+        float2 own[2];
+        float qv[2], rv[2], dv[2], iv[2];
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+          own[u] = w0[at[u]];
+          qv[u] = q[at[u]];
+          rv[u] = rr[at[u]];
+          dv[u] = d[at[u]];
+          iv[u] = idia[a.meta[at[u]] & 255u];
+        }
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+          if (u >= two) continue;
+          const float pv = fmaf(beta, own[u].y, own[u].x);
+          const float res = fmaf(-alpha, qv[u], rv[u]), zv = res * iv[u];
+          d[at[u]] = fmaf(alpha, pv, dv[u]);
+          rr[at[u]] = res;
+          w1[at[u]] = make_float2(zv, pv);
+          sum_acc(res * zv, zs, zc);
+          sum_acc(res * res, rs, rc);
+        }
       }
-      const double w[2] = {(double)zs + (double)zc, (double)rs + (double)rc};
-      grid_partial<2>(bar, w, sm, 0);
+      grid_add(bar, 0, zs, zc);
+      grid_add(bar, 1, rs, rc);
       if (!grid_totals(bar, tot, 2)) return grid_give_up(a.scal + S_CG_ALPHA);
-      beta = rz != 0.0 ? (float)(tot[0] / rz) : 0.f;
-      rz = tot[0];
-      rr32 = tot[1];
-      float *t = p0;
-      p0 = p1;
-      p1 = t;
+      const float next = tot[0].x + tot[0].y;
+      beta = rz != 0.f ? next / rz : 0.f;
+      rz = next;
+      rr32 = tot[1].x + tot[1].y;
+      float2 *t = w0;
+      w0 = w1;
+      w1 = t;
       it++;
       if (!(rr32 > target)) break;  // (a NaN also ends it: the cycle's test sees that)
     }
     // x += d
-    for (int r = first; r < a.n; r += stride) a.x[r] += (double)d[r] / scale;
+    const double unscale = 1.0 / scale;
+    for (int r = first; r < a.n; r += stride) a.x[r] += (double)d[r] * unscale;
     if (!grid_totals(bar, tot, 0)) return grid_give_up(a.scal + S_CG_ALPHA);
-    if (rr32 > 0.0 && rr32 < 1e30) scale *= sqrt(a.n / rr32);
+    if (rr32 > 0.f && rr32 < 1e30f) scale *= sqrt((double)a.n / rr32);
   }
   for (int r = first; r < a.n; r += stride) a.psi[a.cells[r]] = a.x[r];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -537,6 +604,15 @@ static cdi_status cg_iterate(cdi_domain *d, const Geo &g, double *r, double *p, 
 static cdi_status finish_potential(cdi_domain *d, cudaEvent_t ev, bool done, int *iters,
                                    double *relres);
 
+// Screened systems stay with the FP64 iteration and keep their bits.  They
+// need fewer iterations (the condition number is below (12 + kdx2) / kdx2),
+// and they are the fields that transport runs on: its FP32 face data rounds
+// them, and a rounding that a change in their 13th digit turns moves a
+// concentration of a resolved double layer by 2e-7.  (96^3: 75 iterations and
+// 5.5 ms at kdx2 = 0.44, where refinement takes 1.9 ms; 158 and 11.4 ms, 3.7
+// ms at 0.06; 5 and 0.6 ms, 0.4 ms at the default screening.)
+constexpr double kRefineBelow = 0.05;
+
 // The refinement above; *done says whether it reached tol.  Where it does not
 // (max_iter ran out first, tol below what an FP64 residual can show, or a
 // system too ill-conditioned for FP32 corrections) the caller starts over
@@ -544,14 +620,18 @@ static cdi_status finish_potential(cdi_domain *d, cudaEvent_t ev, bool done, int
 static cdi_status psi_refine(cdi_domain *d, double psi_s, double kdx2, const double *src,
                              double tol, int max_iter, bool *done) {
   *done = false;
+  if (!(kdx2 < kRefineBelow)) return CDI_OK;
   const void *kern = d->dim == 2 ? (const void *)k_psi_refine<2> : (const void *)k_psi_refine<3>;
   const int n = (int)d->n_pore;
   int threads = 0;
-  const int blocks = n > 0 ? grid_shape(kern, n, &threads) : 0;
+  size_t smem = 0;
+  const int blocks = n > 0 ? grid_shape(kern, n, 32, 3, &threads, &smem) : 0;
   if (blocks == 0) return CDI_OK;
   PsiArgs a;
   a.fl = d->d_cfl;
   a.lat = d->d_latnb;
+  a.latd = d->d_latd;
+  a.latb = d->d_latb;
   a.cells = d->d_cell_list;
   a.src = src;
   a.n = n;
@@ -561,8 +641,8 @@ static cdi_status psi_refine(cdi_domain *d, double psi_s, double kdx2, const dou
   a.psi_s = psi_s;
   a.tol = tol;
   a.x = (double *)d->d_phi;  // 8 bytes a rank; phi is formed again after the solve
-  a.f = (float *)d->d_cg;    // 26 of its 32 bytes a cell
-  a.meta = (uint16_t *)(a.f + 6 * (size_t)n);
+  a.f = (float *)d->d_cg;    // 30 of its 32 bytes a cell
+  a.meta = (uint16_t *)(a.f + 7 * (size_t)n);
   a.psi = d->d_psi;
   a.part = d->d_part;
   a.scal = d->d_scal;
@@ -572,7 +652,7 @@ static cdi_status psi_refine(cdi_domain *d, double psi_s, double kdx2, const dou
   CDI_TRY(d, cudaMemsetAsync(d->d_scal + S_CG_ALPHA, 0, sizeof(double), d->stream),
           "potential barrier");
   void *args[] = {&a};
-  CDI_TRY(d, cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3(threads), args, 0, d->stream),
+  CDI_TRY(d, cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3(threads), args, smem, d->stream),
           "potential solve");
   d->timing.kernel_launches++;
   CDI_TRY(d, cudaMemcpyAsync(d->h_scal + S_CG_ALPHA, d->d_scal + S_CG_ALPHA, 8 * sizeof(double),

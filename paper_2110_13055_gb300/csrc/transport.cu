@@ -172,9 +172,6 @@ struct NPGeo {
 // instead of twice, and every lane of the warp takes the same path.
 constexpr int kHome = 31;
 
-// 16-bit lateral differences: a closed face, and one that does not fit.
-constexpr short kLatClosed = -32768, kLatWide = -32767;
-
 // The fields of one FP32 transport state, by value as kernel parameters (one
 // launch, one state) or in a member table (fused sweeps and batches).  The
 // concentrations of a species pair stand together, one record per rank
