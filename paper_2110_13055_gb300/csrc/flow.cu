@@ -443,9 +443,11 @@ __global__ void k_links_ovf(const typename FlowFlag<DIM>::type *__restrict__ fl,
 // FP64, FP32 or BF16 storage (S), arithmetic in T = Arith<S>.  Collision (Eq. 8) with the Stokes-linear
 // equilibrium g_eq_i = w_i (drho + 3 e_i.j), j = sum e_i g_i + F/2, and the
 // force source (1 - 1/(2 tau)) 3 w_i e_i.F; omega = 1/tau.
-// (more resident blocks per SM: the step is latency-bound on its scattered
-// loads, so occupancy matters more than a few spare registers; the bound is
-// chosen per variant so that nothing spills)
+// What bounds it on a large image is L2: even and odd step both move 11.7 TB/s
+// of 32-byte sectors, the odd one 1.46 times as many (its gathers and scatters
+// of 32 consecutive ranks break where a grain ends a row), in 1.43 times the
+// time; 256^3 pack 440 us a launch on average.  Registers are bounded per
+// variant so that enough blocks are resident and nothing spills.
 // (lbm_collide: FP32 and BF16 storage; gi the values read.)
 template <typename S, int DIM, bool ODD, typename PL>
 __device__ __forceinline__ void lbm_collide(const PL &g, const int (&nb)[Lat<DIM>::Q], int k0,
