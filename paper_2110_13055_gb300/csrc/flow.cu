@@ -439,6 +439,7 @@ __global__ void k_links_ovf(const typename FlowFlag<DIM>::type *__restrict__ fl,
 // step's blocks come up and read their link data (which no step writes) while
 // the step before it ends, and wait there for its populations.  The next
 // launch is allowed only behind that wait, so at most two steps overlap.
+//
 // One full lattice Boltzmann step (stream + collide) at every pore site,
 // FP64, FP32 or BF16 storage (S), arithmetic in T = Arith<S>.  Collision (Eq. 8) with the Stokes-linear
 // equilibrium g_eq_i = w_i (drho + 3 e_i.j), j = sum e_i g_i + F/2, and the
