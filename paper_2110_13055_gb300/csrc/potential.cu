@@ -379,6 +379,7 @@ __device__ __forceinline__ void sum_acc(float v, float &s, float &c) {
 template <int DIM> __global__ void __launch_bounds__(kGridThreads) k_psi_refine(PsiArgs a) {
   extern __shared__ double sm[];  // 3 rows of a value a warp (GridBarrier)
   __shared__ float2 tot[kGridSums];
+  __shared__ double tot64[2];
   __shared__ float dia[16], idia[16];
   const int first = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
   const size_t n = (size_t)a.n;
@@ -386,12 +387,12 @@ template <int DIM> __global__ void __launch_bounds__(kGridThreads) k_psi_refine(
   float2 *w0 = (float2 *)a.f, *w1 = w0 + n;
   float *rr = a.f + 4 * n, *d = rr + n, *q = d + n;
   GridBarrier bar{a.counter, a.part, sm, (int)(blockDim.x >> 5), 0u, 0};
-  // an FP64 sum of a thread as a pair (48 bits: it decides when to stop)
+  // the norms, once a cycle, stay FP64: they decide when to stop, and squares
+  // of a small potential's residuals leave FP32's range
   auto add64 = [&](int k, double v) {
-    const float h = (float)v;
-    grid_add(bar, k, h, (float)(v - (double)h));
+    v = warp_sum(v);
+    if ((threadIdx.x & 31) == 0) sm[k * bar.row + (threadIdx.x >> 5)] = v;
   };
-  auto total = [&](int k) { return (double)tot[k].x + (double)tot[k].y; };
   if (threadIdx.x < 16) {
     const double v = a.kdx2 + threadIdx.x;
     dia[threadIdx.x] = (float)v;
@@ -406,8 +407,8 @@ template <int DIM> __global__ void __launch_bounds__(kGridThreads) k_psi_refine(
     v += b * b;
   }
   add64(0, v);
-  if (!grid_totals(bar, tot, 1)) return grid_give_up(a.scal + S_CG_ALPHA);
-  const double bb = total(0);
+  if (!grid_totals(bar, tot64, 1)) return grid_give_up(a.scal + S_CG_ALPHA);
+  const double bb = tot64[0];
   double rel = bb > 0.0 ? 1.0 : 0.0, scale = bb > 0.0 ? sqrt(a.n / bb) : 1.0;
   int it = 0;
   bool done = bb == 0.0;
@@ -437,10 +438,10 @@ template <int DIM> __global__ void __launch_bounds__(kGridThreads) k_psi_refine(
       sum_acc(rv * zv, zs, zc);
     }
     add64(0, v);
-    grid_add(bar, 1, zs, zc);
-    if (!grid_totals(bar, tot, 2)) return grid_give_up(a.scal + S_CG_ALPHA);
-    const double rr64 = total(0), old = rel;
-    float rz = tot[1].x + tot[1].y;
+    add64(1, (double)zs + (double)zc);
+    if (!grid_totals(bar, tot64, 2)) return grid_give_up(a.scal + S_CG_ALPHA);
+    const double rr64 = tot64[0], old = rel;
+    float rz = (float)tot64[1];
     rel = sqrt(rr64 / bb);
     if (rel < a.tol || rr64 == 0.0) {
       done = true;

@@ -93,3 +93,21 @@ def test_implicit_solver_shapes(shape, Z, D):
     np.testing.assert_allclose(G, Go, rtol=1e-9)
     np.testing.assert_allclose(I, Io, rtol=1e-9, atol=1e-9 * np.abs(Io).max())
     np.testing.assert_allclose(Ou, Oo, rtol=1e-9, atol=1e-9 * np.abs(Io).max())
+
+
+@pytest.mark.parametrize("shift", [-90, -45, 80])
+@pytest.mark.parametrize("mode,lam", [("laplace", 0.0), ("debye", 1e-6)])
+@pytest.mark.parametrize("shape", [(61, 83), (18, 21, 25)], ids=str)
+def test_potential_of_any_size(shape, mode, lam, shift):
+    """Eq. 4 is linear: a surface potential 2^shift times as large has the
+    same relative field and residual, also where its square leaves FP32's
+    range.  Both residuals are below 1e-13, at condition numbers below 1.2e3."""
+    m = image(shape)
+    with cdi.Domain(m) as d:
+        d.solve_flow(tol=0.0, max_steps=0, U_target=0.0)
+        it, _ = d.set_potential(0.75, lambda_D=lam, mode=mode, tol=1e-13)
+        a = d.psi()
+        it2, res = d.set_potential(0.75 * 2.0 ** shift, lambda_D=lam, mode=mode, tol=1e-13)
+        b = d.psi() * 2.0 ** -shift
+    assert it2 == it and 0.0 < res < 1e-13
+    assert rel(b, a) < 2.4e-10
