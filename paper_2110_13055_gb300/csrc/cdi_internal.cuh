@@ -466,6 +466,8 @@ struct cdi_domain {
                                 // coefficients (taken by the first transport state)
   size_t bern_bytes = 0;
   int np_mode = 0;              // which kernel the faces ask for (see np_warp31)
+  bool faces_stale = true;      // d_fd, d_bern and np_mode are not those of the
+                                // current potential (explicit steps form them again)
   short *d_latd = nullptr;      // 2*(dim-1) 16-bit lateral differences per rank
   int *d_latb = nullptr;        // and their bases per tile of 31 ranks
   double *d_acc = nullptr;      // 3*kMaxSpecies*np_accs per-warp sums (8 B each:

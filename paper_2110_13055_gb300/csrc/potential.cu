@@ -782,9 +782,11 @@ cdi_status cdi_psi_coupled(cdi_domain *d) {
   CDI_TRY(d, cudaGetLastError(), "charge");
   int it = 0;
   double rel = 0.0;
+  // converged or not, the solve replaces the potential that both schemes'
+  // face coefficients were formed from
+  d->faces_stale = d->imp_stale = true;
   cdi_status s = cdi_psi_solve(d, d->psi_s, 0.0, d->d_src, d->psi_tol, d->psi_max_iter, &it, &rel);
   if (s == CDI_ERR_NOT_CONVERGED)
     return cdi_fail(d, s, "coupled potential did not reach tol within max_iter");
-  if (s != CDI_OK) return s;
-  return cdi_np_faces(d);  // the step reads face data of the new potential
+  return s;
 }

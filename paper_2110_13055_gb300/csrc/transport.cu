@@ -1499,7 +1499,7 @@ cdi_status cdi_np_build_flags(cdi_domain *d) {
 cdi_status cdi_np_init(cdi_domain *d, double dt_s, double *dt_used) {
   if (d->np_graph) cudaGraphExecDestroy(d->np_graph);
   d->np_graph = nullptr;
-  d->imp_stale = true;  // the implicit operator follows u, phi and the species
+  d->imp_stale = d->faces_stale = true;  // they follow u, phi and the species
   double dt = dt_s;
   if (dt <= 0.0) {
     cdi_status s = cdi_np_dt(d, d->h_scal[S_SCALE], &dt);
@@ -1549,7 +1549,7 @@ static bool take_bern(cdi_domain *d) {
 // the face data, and the Bernoulli pairs where some face needs them (their
 // memory is taken the first time one does; waits for the stream).  Without
 // memory for them the step evaluates every face itself.
-cdi_status cdi_np_faces(cdi_domain *d) {
+static cdi_status form_faces(cdi_domain *d) {
   if (d->prec == CDI_FP64) {
     d->np_mode = take_bern(d) ? NP_SMALL : NP_EVAL;
     if (d->np_mode == NP_EVAL) return CDI_OK;
@@ -1573,6 +1573,14 @@ cdi_status cdi_np_faces(cdi_domain *d) {
   d->timing.kernel_launches++;
   CDI_TRY(d, cudaGetLastError(), "face data");
   return CDI_OK;
+}
+cdi_status cdi_np_faces(cdi_domain *d) {
+  // captured steps hold the mode and the memory of the faces before
+  if (d->np_graph) cudaGraphExecDestroy(d->np_graph);
+  d->np_graph = nullptr;
+  const cdi_status s = form_faces(d);
+  d->faces_stale = s != CDI_OK;
+  return s;
 }
 
 // Explicit time step for the current potential (d_psi) and the solved flow
@@ -2024,18 +2032,19 @@ static cdi_status np_steps_coupled(cdi_domain *d, int64_t n) {
   const int64_t K = d->couple_K;
   while (n > 0) {
     if (d->np_steps % K == 0) {
-      if (d->np_graph) cudaGraphExecDestroy(d->np_graph);
-      d->np_graph = nullptr;
       cdi_status s = cdi_psi_coupled(d);
       if (s != CDI_OK) return s;
     }
     const int64_t block = std::min<int64_t>(n, K - d->np_steps % K);
     if (d->imp_tol > 0.0) {  // implicit steps in the re-solved potential
-      d->imp_stale = true;
       cdi_status s = cdi_imp_steps(d, block);
       if (s != CDI_OK) return s;
       n -= block;
       continue;
+    }
+    if (d->faces_stale) {
+      cdi_status s = cdi_np_faces(d);
+      if (s != CDI_OK) return s;
     }
     cudaEvent_t ev;
     cdi_timing_begin(d, &ev);
@@ -2056,6 +2065,10 @@ cdi_status cdi_np_steps(cdi_domain *d, int64_t n) {
   if (n == 0) return CDI_OK;
   if (d->couple_K > 0) return np_steps_coupled(d, n);
   if (d->imp_tol > 0.0) return cdi_imp_steps(d, n);
+  if (d->faces_stale) {
+    cdi_status s = cdi_np_faces(d);
+    if (s != CDI_OK) return s;
+  }
   cudaEvent_t ev;
   cdi_timing_begin(d, &ev);
   int64_t left = n;
