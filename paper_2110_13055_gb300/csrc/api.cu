@@ -86,10 +86,15 @@ int cdi::grid_shape(const void *kernel, long long n, int row_div, int nv, int *t
   const int t = (int)std::max(32ll, std::min((long long)cdi::kGridThreads, each));
   *threads = t;
   *smem = grid_smem(t, row_div, nv);
-  if (*smem > (48u << 10))
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, t, *smem);
-  (void)cudaGetLastError();
+  // The limit is the kernel's, for the whole process: always the largest size
+  // that any shape asks for, so that another thread's call never lowers it
+  // between this one and its launch.
+  const size_t most = grid_smem(cdi::kGridThreads, row_div, cdi::kGridSums);
+  if ((most > (48u << 10) &&
+       cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) !=
+           cudaSuccess) ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, t, *smem) != cudaSuccess)
+    (void)cudaGetLastError();
   if (per < 1) return 0;
   return (int)std::max<long long>(1, std::min<long long>(std::min(sms, cdi::kRedBlocks), (n + t - 1) / t));
 }

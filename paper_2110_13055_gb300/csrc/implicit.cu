@@ -425,22 +425,23 @@ cdi_status imp_coefs(cdi_domain *d) {
   return CDI_OK;
 }
 
+// The solver's launch: the same for every step of a call.
+struct BiShape {
+  int side, blocks, threads;  // species side by side, and the grid
+  size_t smem;
+};
+
 // One step: the species solved side by side in one launch where their vectors
 // could be had, else one after the other in one set of vectors.
 template <typename T, int DIM>
-cdi_status imp_step(cdi_domain *d) {
+cdi_status imp_step(cdi_domain *d, const BiShape &shape) {
   using C = ICoef<DIM>;
   using A = typename std::conditional<std::is_same<T, float>::value, float2, double>::type;
   const int n = (int)d->n_pore;
   const size_t nn = (size_t)n;
   const IGeo g = make_igeo(d);
   const int in = d->cur;
-  const int side = std::min(d->ns, d->imp_sets);
-  int threads = 0;
-  size_t smem = 0;
-  const int blocks =
-      grid_shape((const void *)k_bi_solve<T, DIM>, n, 1, 2 * side, &threads, &smem);
-  if (blocks == 0) return cdi_fail(d, CDI_ERR_CUDA, "implicit step: no resident block");
+  const int side = shape.side;
   CDI_TRY(d, cudaMemsetAsync(d->d_iscal, 0, B_N * sizeof(double), d->stream), "implicit scalars");
   for (int k0 = 0; k0 < d->ns; k0 += side) {
     BiArgs<T> a;
@@ -458,8 +459,8 @@ cdi_status imp_step(cdi_domain *d) {
     a.counter = d->d_counter + C_IMP;
     CDI_TRY(d, cudaMemsetAsync(a.counter, 0, sizeof(unsigned), d->stream), "implicit barrier");
     void *args[] = {&a};
-    CDI_TRY(d, cudaLaunchCooperativeKernel((const void *)k_bi_solve<T, DIM>, dim3(blocks),
-                                           dim3(threads), args, smem, d->stream),
+    CDI_TRY(d, cudaLaunchCooperativeKernel((const void *)k_bi_solve<T, DIM>, dim3(shape.blocks),
+                                           dim3(shape.threads), args, shape.smem, d->stream),
             "implicit solve");
     for (int k = 0; k < a.ns; k++) {
       const double Dk = d->D[k0 + k];
@@ -505,10 +506,15 @@ cdi_status imp_steps(cdi_domain *d, int64_t n) {
       d->imp_sets = d->ns;
     }
   }
+  BiShape shape;
+  shape.side = std::min(d->ns, d->imp_sets);
+  shape.blocks = grid_shape((const void *)k_bi_solve<T, DIM>, d->n_pore, 1, 2 * shape.side,
+                            &shape.threads, &shape.smem);
+  if (shape.blocks == 0) return cdi_fail(d, CDI_ERR_CUDA, "implicit step: no resident block");
   cudaEvent_t ev;
   cdi_timing_begin(d, &ev);
   for (int64_t i = 0; i < n; i++) {
-    cdi_status s = imp_step<T, DIM>(d);
+    cdi_status s = imp_step<T, DIM>(d, shape);
     if (s != CDI_OK) {
       cdi_timing_end(d, ev, PH_NP, i);
       return s;
