@@ -259,8 +259,8 @@ cdi_status cdi_set_coupling(cdi_domain *dom, int64_t every_steps);
  * tol <= 0 returns to the explicit scheme.  With cdi_set_coupling the
  * potential is still re-solved before every block of K steps.  Sweeps and
  * batches always step explicitly.  cdi_step_transport waits for the stream
- * after every step.  Device memory: 4 (8 or 10) + 6 FP64 values per pore
- * cell, taken on the first call, and 6 a species where the first step finds
+ * after every step.  Device memory: 4 (8 or 10) + 5 FP64 values per pore
+ * cell, taken on the first call, and 5 a species where the first step finds
  * them (the species are then solved side by side). */
 cdi_status cdi_set_implicit(cdi_domain *dom, double tol, int max_iter);
 

@@ -476,7 +476,8 @@ struct cdi_domain {
   unsigned int *d_counter = nullptr;  // last-block counters (8 slots)
   double *d_scal = nullptr;     // device scalars (S_COUNT)
   double *h_scal = nullptr;     // pinned host copy of the scalars (S_COUNT)
-  double *d_cg = nullptr;       // 4*N CG work vectors (r, p, q, diag)
+  double *d_cg = nullptr;       // 4*N CG work vectors (r, p, q, diag), scratch of
+                                // other calls between solves
   double *d_colout = nullptr;   // nx column means
 
   // state
@@ -502,7 +503,7 @@ struct cdi_domain {
   int64_t imp_iters = 0;        // linear iterations so far
   double imp_last_rel = 0.0;    // last relative residual
   double *d_icoef = nullptr;    // operator coefficients of every species (FP64)
-  double *d_iwork = nullptr;    // imp_sets * 6 * n_pore FP64 work vectors
+  double *d_iwork = nullptr;    // imp_sets * 5 * n_pore FP64 work vectors
   int imp_sets = 0;             // species whose vectors d_iwork holds
   double *d_iscal = nullptr;    // the solver's device scalars (16)
   double *d_src = nullptr;      // N charge terms of Eq. 4 (coupled mode only)

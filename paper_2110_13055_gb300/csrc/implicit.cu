@@ -44,7 +44,7 @@ template <int DIM> struct ICoef {
   static constexpr int NF = 2 * DIM;
   static constexpr int K = 0, FACE = 1, AIN = 1 + NF, BIN = 2 + NF, AOUT = 3 + NF, NC = 4 + NF;
 };
-constexpr int kImpVecs = 6;  // y, r, r0, p, v, t per species
+constexpr int kImpVecs = 5;  // r, r0, p, v, t per species
 
 struct IGeo {
   const NFlag *fl;   // per rank face flags
@@ -172,6 +172,7 @@ template <typename T> struct BiArgs {
   int n, ns, max_iter;
   double dt_dx, tol;  // dt / dx
   CViews<T> C;        // C^n of the launch's species
+  double *y;          // a vector per species, the solution
   double *w;          // kImpVecs vectors per species
   double *part, *scal;
   unsigned *counter;
@@ -202,7 +203,8 @@ __global__ void __launch_bounds__(kGridThreads) k_bi_solve(BiArgs<T> a) {
 
   for (int k = 0; k < a.ns; k++) {
     const double *c = a.co + (size_t)k * C::NC * n;
-    double *y = a.w + (size_t)k * kImpVecs * n, *rr = y + n, *r0 = rr + n, *p = r0 + n;
+    double *y = a.y + (size_t)k * n;
+    double *rr = a.w + (size_t)k * kImpVecs * n, *r0 = rr + n, *p = r0 + n;
     const CView<T> Ck = a.C.v[k];
     double v[2] = {0.0, 0.0};
     for (int r = first; r < a.n; r += stride) {
@@ -244,9 +246,8 @@ __global__ void __launch_bounds__(kGridThreads) k_bi_solve(BiArgs<T> a) {
       double v[1] = {0.0};
       if (!done[k]) {
         const double *off = a.co + ((size_t)k * C::NC + C::FACE) * n;
-        double *y = a.w + (size_t)k * kImpVecs * n;
-        const double *r0 = y + 2 * n, *p = y + 3 * n;
-        double *vv = y + 4 * n;
+        double *rr = a.w + (size_t)k * kImpVecs * n, *vv = rr + 3 * n;
+        const double *r0 = rr + n, *p = rr + 2 * n;
         for (int r = first; r < a.n; r += stride) {
           double m = p[r];
           open_faces<DIM>(a.lat, off, n, r, [&](int q, double o) { m += o * p[q]; });
@@ -266,9 +267,8 @@ __global__ void __launch_bounds__(kGridThreads) k_bi_solve(BiArgs<T> a) {
       double v[2] = {0.0, 0.0};
       if (!done[k]) {
         const double *off = a.co + ((size_t)k * C::NC + C::FACE) * n;
-        double *y = a.w + (size_t)k * kImpVecs * n;
-        const double *rr = y + n, *vv = y + 4 * n;
-        double *t = y + 5 * n;
+        double *t = a.w + ((size_t)k * kImpVecs + 4) * n;
+        const double *rr = t - 4 * n, *vv = t - n;
         const double al = alpha[k];
         for (int r = first; r < a.n; r += stride) {
           const double sP = rr[r] - al * vv[r];
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(kGridThreads) k_bi_solve(BiArgs<T> a) {
         }
       }
       grid_add(bar, 2 * k, v[0]);
-    grid_add(bar, 2 * k + 1, v[1]);
+      grid_add(bar, 2 * k + 1, v[1]);
     }
     if (!grid_totals(bar, tot, 2 * a.ns)) return grid_give_up(a.scal + B_BAR);
     if (threadIdx.x < a.ns && !done[threadIdx.x]) {
@@ -294,8 +294,8 @@ __global__ void __launch_bounds__(kGridThreads) k_bi_solve(BiArgs<T> a) {
     for (int k = 0; k < a.ns; k++) {
       double v[2] = {0.0, 0.0};
       if (!done[k]) {
-        double *y = a.w + (size_t)k * kImpVecs * n, *rr = y + n;
-        const double *r0 = y + 2 * n, *p = y + 3 * n, *vv = y + 4 * n, *t = y + 5 * n;
+        double *y = a.y + (size_t)k * n, *rr = a.w + (size_t)k * kImpVecs * n;
+        const double *r0 = rr + n, *p = rr + 2 * n, *vv = rr + 3 * n, *t = rr + 4 * n;
         const double al = alpha[k], om = omega[k];
         for (int r = first; r < a.n; r += stride) {
           const double sP = rr[r] - al * vv[r];
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(kGridThreads) k_bi_solve(BiArgs<T> a) {
         }
       }
       grid_add(bar, 2 * k, v[0]);
-    grid_add(bar, 2 * k + 1, v[1]);
+      grid_add(bar, 2 * k + 1, v[1]);
     }
     if (!grid_totals(bar, tot, 2 * a.ns)) return grid_give_up(a.scal + B_BAR);
     if (threadIdx.x < a.ns && !done[threadIdx.x]) {
@@ -327,9 +327,8 @@ __global__ void __launch_bounds__(kGridThreads) k_bi_solve(BiArgs<T> a) {
     // p = r + beta (p - omega v)
     for (int k = 0; k < a.ns; k++) {
       if (done[k]) continue;
-      double *y = a.w + (size_t)k * kImpVecs * n;
-      const double *rr = y + n, *vv = y + 4 * n;
-      double *p = y + 3 * n;
+      double *p = a.w + ((size_t)k * kImpVecs + 2) * n;
+      const double *rr = p - 2 * n, *vv = p + n;
       const double be = beta[k], om = omega[k];
       for (int r = first; r < a.n; r += stride) p[r] = rr[r] + be * (p[r] - om * vv[r]);
     }
@@ -432,7 +431,9 @@ struct BiShape {
 };
 
 // One step: the species solved side by side in one launch where their vectors
-// could be had, else one after the other in one set of vectors.
+// could be had, else one after the other in one set of vectors.  The solutions
+// stand in the potential solver's scratch (kMaxSpecies doubles a cell) and are
+// taken into the state and the accounts once every species has converged.
 template <typename T, int DIM>
 cdi_status imp_step(cdi_domain *d, const BiShape &shape) {
   using C = ICoef<DIM>;
@@ -453,6 +454,7 @@ cdi_status imp_step(cdi_domain *d, const BiShape &shape) {
     a.dt_dx = d->dt / d->dx;
     a.tol = d->imp_tol;
     for (int k = 0; k < a.ns; k++) a.C.v[k] = c_view<T>(d, d->d_C[in], k0 + k);
+    a.y = d->d_cg + (size_t)k0 * nn;
     a.w = d->d_iwork;
     a.part = d->d_part;
     a.scal = d->d_iscal;
@@ -462,14 +464,15 @@ cdi_status imp_step(cdi_domain *d, const BiShape &shape) {
     CDI_TRY(d, cudaLaunchCooperativeKernel((const void *)k_bi_solve<T, DIM>, dim3(shape.blocks),
                                            dim3(shape.threads), args, shape.smem, d->stream),
             "implicit solve");
-    for (int k = 0; k < a.ns; k++) {
-      const double Dk = d->D[k0 + k];
-      const double Keff = d->Ka / (1.0 + d->Ka * d->dx / (2.0 * Dk));
+    d->timing.kernel_launches++;
+    const bool last = k0 + side >= d->ns;
+    for (int k = 0; last && k < d->ns; k++) {
+      const double Keff = d->Ka / (1.0 + d->Ka * d->dx / (2.0 * d->D[k]));
       k_bi_finish<T, DIM><<<(n + 127) / 128, 128, 0, d->stream>>>(
-          g, a.co + (size_t)k * C::NC * nn, a.w + (size_t)k * kImpVecs * nn, d->d_iscal, Keff,
-          c_view<T>(d, d->d_C[1 - in], k0 + k), k0 + k, (A *)d->d_acc, d->np_accs);
+          g, d->d_icoef + (size_t)k * C::NC * nn, d->d_cg + (size_t)k * nn, d->d_iscal, Keff,
+          c_view<T>(d, d->d_C[1 - in], k), k, (A *)d->d_acc, d->np_accs);
+      d->timing.kernel_launches++;
     }
-    d->timing.kernel_launches += 1 + a.ns;
     CDI_TRY(d, cudaGetLastError(), "implicit step");
     CDI_TRY(d, cudaMemcpyAsync(d->h_scal + S_IMP, d->d_iscal, B_N * sizeof(double),
                                cudaMemcpyDeviceToHost, d->stream),
