@@ -535,13 +535,18 @@ cdi_status imp_steps(cdi_domain *d, int64_t n) {
 // first step takes those of the others).
 cdi_status cdi_imp_prepare(cdi_domain *d) {
   const int NC = d->dim == 2 ? ICoef<2>::NC : ICoef<3>::NC;
-  if (!d->d_icoef) {
-    d->d_icoef = (double *)cdi_dev_alloc(d, (size_t)kMaxSpecies * NC * d->n_pore * 8);
-    d->d_iwork = (double *)cdi_dev_alloc(d, (size_t)kImpVecs * d->n_pore * 8);
-    d->imp_sets = 1;
-    d->d_iscal = (double *)cdi_dev_alloc(d, 16 * 8);
-    if (!d->d_icoef || !d->d_iwork || !d->d_iscal)
+  if (!d->d_icoef) {  // all of it, or nothing
+    void *p[3] = {cdi_dev_alloc(d, (size_t)kMaxSpecies * NC * d->n_pore * 8),
+                  cdi_dev_alloc(d, (size_t)kImpVecs * d->n_pore * 8), cdi_dev_alloc(d, 16 * 8)};
+    if (!p[0] || !p[1] || !p[2]) {
+      for (void *q : p)
+        if (q) cdi_dev_release(d, q);
       return cdi_fail(d, CDI_ERR_OOM, "implicit scheme: device memory");
+    }
+    d->d_icoef = (double *)p[0];
+    d->d_iwork = (double *)p[1];
+    d->d_iscal = (double *)p[2];
+    d->imp_sets = 1;
     CDI_TRY(d, cudaMemsetAsync(d->d_iscal, 0, 16 * 8, d->stream), "implicit scalars");
   }
   d->imp_stale = true;

@@ -83,3 +83,31 @@ def test_implicit_species_after_one_another(prec):
     for one_set, limit in ((True, 500), (False, 3), (True, 3)):
         for x, y in zip(run(one_set, limit), ref):
             assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("fail_at", [1, 2, 3])
+def test_implicit_memory_all_or_nothing(fail_at):
+    """Every call that cannot have the implicit scheme's memory fails and keeps
+    none of it; the first that can, works."""
+    m = pack()
+
+    def run(tries):
+        a = Allocator()
+        with cdi.Domain(m, torch_resources=a) as d:
+            d.solve_flow(tol=0.0, max_steps=0, U_target=0.0)
+            d.set_potential(0.3, lambda_D=1.5e-7, tol=1e-12)
+            d.init_transport(Z, D, c0=10.0, Ka=1e-6)
+            before = a.total()
+            for _ in range(tries):
+                calls = []
+                a.refuse = lambda nbytes: calls.append(nbytes) or len(calls) >= fail_at
+                with pytest.raises(cdi.CDIError) as e:
+                    d.set_implicit(1e-10, 500)
+                assert e.value.status == 2
+                assert a.total() == before
+            a.refuse = lambda nbytes: False
+            d.set_implicit(1e-10, 500)
+            d.step(2)
+            return d.C()
+
+    assert np.array_equal(run(2), run(0))
