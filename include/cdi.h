@@ -225,7 +225,11 @@ cdi_status cdi_set_potential(cdi_domain *dom, double applied_V,
  * solid face.  dt_s > 0 fixes the time step; dt_s == 0 takes
  * 0.9 / (largest outflow rate of any cell and species), which keeps the
  * explicit update positive.  Needs a solved flow (or U_target 0 and no flow
- * solve: then u = 0) and a potential.  Resets Gamma/In/Out to zero. */
+ * solve: then u = 0) and a potential.  Resets Gamma/In/Out to zero.
+ * Device memory: explicit steps keep (dim + 1) * n_species * 16 bytes of face
+ * coefficients per pore cell in FP64, half of it in FP32 where a face Peclet
+ * number reaches 1/2; without it they compute the same bits more slowly, and
+ * a later call on the domain that needs memory gets it back first. */
 cdi_status cdi_init_transport(cdi_domain *dom, const cdi_species *sp,
                               int n_species, double c0_molm3, double Ka_mps,
                               double dt_s, double *dt_used);

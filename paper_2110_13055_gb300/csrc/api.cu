@@ -76,6 +76,33 @@ void cdi_dev_release(cdi_domain *d, void *p) {
   }
 }
 
+// Memory that a call cannot do without: what the domain holds only to be
+// faster is given back for it.
+void *cdi_dev_need(cdi_domain *d, size_t bytes) {
+  void *p = cdi_dev_alloc(d, bytes);
+  return p || !cdi_give_back(d) ? p : cdi_dev_alloc(d, bytes);
+}
+
+// The steps' stored coefficients and the vectors of implicit species beyond
+// one set (both taken again, where there is memory, by the next step that uses
+// them).  False where there was nothing to give.
+bool cdi_give_back(cdi_domain *d) {
+  if (!d->d_bern && d->imp_sets < 2) return false;
+  cudaStreamSynchronize(d->stream);
+  if (d->np_graph) cudaGraphExecDestroy(d->np_graph);
+  d->np_graph = nullptr;
+  if (d->d_bern) cdi_dev_release(d, d->d_bern);
+  d->d_bern = nullptr;
+  d->faces_stale = true;
+  if (d->imp_sets > 1) {
+    cdi_dev_release(d, d->d_iwork);
+    d->d_iwork = nullptr;
+    d->imp_sets = 0;
+  }
+  cudaStreamSynchronize(d->stream);  // (stream-ordered frees: available to other streams too)
+  return true;
+}
+
 int cdi::grid_shape(const void *kernel, long long n, int row_div, int nv, int *threads,
                     size_t *smem) {
   int dev = 0, sms = 0, per = 0;
@@ -543,7 +570,7 @@ cdi_status cdi_set_implicit(cdi_domain *d, double tol, int max_iter) {
   if (!std::isfinite(tol)) return cdi_fail(d, CDI_ERR_INVALID_ARG, "non-finite tolerance");
   if (tol <= 0.0) {
     d->imp_tol = 0.0;
-    return CDI_OK;
+    return d->np_ready && d->faces_stale ? cdi_np_faces(d) : CDI_OK;
   }
   if (max_iter < 1) return cdi_fail(d, CDI_ERR_INVALID_ARG, "max_iter must be >= 1");
   cdi_status s = cdi_imp_prepare(d);
@@ -583,7 +610,7 @@ cdi_status cdi_set_coupling(cdi_domain *d, int64_t every_steps) {
   if (every_steps > 0 && !d->psi_done)
     return cdi_fail(d, CDI_ERR_STATE, "set the potential first (its parameters are reused)");
   if (every_steps > 0 && !d->d_src) {
-    d->d_src = (double *)cdi_dev_alloc(d, (size_t)d->N * 8);
+    d->d_src = (double *)cdi_dev_need(d, (size_t)d->N * 8);
     if (!d->d_src) return cdi_fail(d, CDI_ERR_OOM, "coupling: charge buffer");
   }
   d->couple_K = every_steps;
@@ -680,7 +707,8 @@ cdi_status prepare_sweep(cdi_domain *d, cdi_domain *owner, const cdi_combo *comb
   for (size_t g = 0; g < gv.size() && s == CDI_OK; g++) {
     s = cdi_set_potential(d, gv[g], ep, nullptr, nullptr);
     if (s != CDI_OK) break;
-    void *ph = cdi_dev_alloc(owner, (size_t)d->n_pore * 8);
+    void *ph = cdi_dev_need(owner, (size_t)d->n_pore * 8);
+    if (!ph && cdi_give_back(d)) ph = cdi_dev_alloc(owner, (size_t)d->n_pore * 8);
     if (!ph) {
       s = cdi_fail(d, CDI_ERR_OOM, "sweep: potential buffer");
       break;

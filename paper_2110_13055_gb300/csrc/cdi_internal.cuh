@@ -463,7 +463,8 @@ struct cdi_domain {
   float2 *d_fd = nullptr;       // FP32: dim * n_pore face data (see k_np_faces)
   void *d_bern = nullptr;       // FP32: Bernoulli pairs of the faces with |P| >= 1/2
                                 // (taken the first time there is one); FP64: face
-                                // coefficients (taken by the first transport state)
+                                // coefficients (taken for the first explicit steps);
+                                // done without where memory is short
   size_t bern_bytes = 0;
   int np_mode = 0;              // which kernel the faces ask for (see np_warp31)
   bool faces_stale = true;      // d_fd, d_bern and np_mode are not those of the
@@ -595,6 +596,8 @@ enum { PH_FLOW = 0, PH_CHECK = 1, PH_PSI = 2, PH_NP = 3 };
 cdi_status cdi_fail(cdi_domain *d, cdi_status s, const std::string &msg);
 cdi_status cdi_cuda_fail(cdi_domain *d, cudaError_t e, const char *what);
 void *cdi_dev_alloc(cdi_domain *d, size_t bytes);
+void *cdi_dev_need(cdi_domain *d, size_t bytes);
+bool cdi_give_back(cdi_domain *d);
 void cdi_timing_begin(cdi_domain *d, cudaEvent_t *a);
 void cdi_timing_end(cdi_domain *d, cudaEvent_t a, int phase, int64_t launches);
 cudaError_t cdi_timing_resolve(cdi_domain *d);

@@ -1188,7 +1188,7 @@ cdi_status flow_batch(cdi_domain *const *doms, int n_doms, const cdi_flow_params
   const SplitConst c{host_pair(1.0 / tau), host_pair(1.0 - 1.0 / tau), host_pair(0.5 * force),
                      host_pair(fs * Lat<DIM>::w(1)),
                      host_pair(fs * (DIM == 2 ? Lat<2>::w(3) : Lat<3>::w(4)))};
-  LbmMember<S> *dtab = (LbmMember<S> *)cdi_dev_alloc(L, sizeof(LbmMember<S>) * n_doms);
+  LbmMember<S> *dtab = (LbmMember<S> *)cdi_dev_need(L, sizeof(LbmMember<S>) * n_doms);
   if (!dtab) return cdi_fail(L, CDI_ERR_OOM, "flow batch: member table");
   std::vector<LbmMember<S>> tab;
   std::vector<int> active(n_doms);

@@ -501,14 +501,18 @@ cdi_status imp_steps(cdi_domain *d, int64_t n) {
     cdi_status s = imp_coefs<T, DIM>(d);
     if (s != CDI_OK) return s;
   }
-  if (d->imp_sets < d->ns) {  // vectors for all species at once, where memory allows
-    double *w = (double *)cdi_dev_alloc(d, (size_t)d->ns * kImpVecs * d->n_pore * 8);
-    if (w) {
-      cdi_dev_release(d, d->d_iwork);
-      d->d_iwork = w;
-      d->imp_sets = d->ns;
-    }
+  // vectors for all species at once, where memory allows (the one set of
+  // cdi_imp_prepare may have been given back)
+  for (int sets : {d->ns, 1}) {
+    if (d->imp_sets >= sets) continue;
+    double *w = (double *)(sets > 1 ? cdi_dev_alloc : cdi_dev_need)(
+        d, (size_t)sets * kImpVecs * d->n_pore * 8);
+    if (!w) continue;
+    cdi_dev_release(d, d->d_iwork);
+    d->d_iwork = w;
+    d->imp_sets = sets;
   }
+  if (d->imp_sets < 1) return cdi_fail(d, CDI_ERR_OOM, "implicit scheme: device memory");
   BiShape shape;
   shape.side = std::min(d->ns, d->imp_sets);
   shape.blocks = grid_shape((const void *)k_bi_solve<T, DIM>, d->n_pore, 1, 2 * shape.side,
@@ -536,8 +540,8 @@ cdi_status imp_steps(cdi_domain *d, int64_t n) {
 cdi_status cdi_imp_prepare(cdi_domain *d) {
   const int NC = d->dim == 2 ? ICoef<2>::NC : ICoef<3>::NC;
   if (!d->d_icoef) {  // all of it, or nothing
-    void *p[3] = {cdi_dev_alloc(d, (size_t)kMaxSpecies * NC * d->n_pore * 8),
-                  cdi_dev_alloc(d, (size_t)kImpVecs * d->n_pore * 8), cdi_dev_alloc(d, 16 * 8)};
+    void *p[3] = {cdi_dev_need(d, (size_t)kMaxSpecies * NC * d->n_pore * 8),
+                  cdi_dev_need(d, (size_t)kImpVecs * d->n_pore * 8), cdi_dev_need(d, 16 * 8)};
     if (!p[0] || !p[1] || !p[2]) {
       for (void *q : p)
         if (q) cdi_dev_release(d, q);

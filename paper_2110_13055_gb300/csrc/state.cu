@@ -135,7 +135,7 @@ cdi_status cdi_load_state(cdi_domain *d, const void *host_buf, size_t bytes) {
   if (bytes != state_bytes(d))
     return cdi_fail(d, CDI_ERR_INVALID_ARG, "load_state: size does not match the domain");
   if (h.couple_K > 0 && !d->d_src) {
-    d->d_src = (double *)cdi_dev_alloc(d, (size_t)d->N * 8);
+    d->d_src = (double *)cdi_dev_need(d, (size_t)d->N * 8);
     if (!d->d_src) return cdi_fail(d, CDI_ERR_OOM, "load_state: charge buffer");
   }
   // the loaded concentrations go to buffer 0; any captured graph is stale
@@ -168,7 +168,7 @@ cdi_status cdi_load_state(cdi_domain *d, const void *host_buf, size_t bytes) {
   if (d->np_ready) {
     cdi_status rs = CDI_OK;
     if (d->prec != CDI_FP64) rs = cdi_np_planes_to_records(d, (const float *)d->d_cg, 0);
-    if (rs == CDI_OK) rs = cdi_np_faces(d);
+    if (rs == CDI_OK && !(d->imp_tol > 0.0)) rs = cdi_np_faces(d);
     if (rs != CDI_OK) return rs;
     CDI_TRY(d, cudaStreamSynchronize(d->stream), "load_state");
   }

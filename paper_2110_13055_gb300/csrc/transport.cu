@@ -1507,8 +1507,10 @@ cdi_status cdi_np_init(cdi_domain *d, double dt_s, double *dt_used) {
   }
   d->dt = dt;
   if (dt_used) *dt_used = dt;
-  cdi_status fs = cdi_np_faces(d);
-  if (fs != CDI_OK) return fs;
+  if (!(d->imp_tol > 0.0)) {  // (implicit steps do not read them)
+    cdi_status fs = cdi_np_faces(d);
+    if (fs != CDI_OK) return fs;
+  }
   if (!d->np_tuned) {
     d->np_variant = kNpDefaultShape;
     d->np_block = kNpVariantBlock[d->np_variant];
@@ -1534,6 +1536,7 @@ cdi_status cdi_np_init(cdi_domain *d, double dt_s, double *dt_used) {
 // life); false when there is none.
 static bool take_bern(cdi_domain *d) {
   if (d->d_bern && d->bern_bytes < bern_bytes(d)) {
+    cudaStreamSynchronize(d->stream);  // steps in flight read it
     cdi_dev_release(d, d->d_bern);
     d->d_bern = nullptr;
   }
@@ -1675,8 +1678,8 @@ cdi_status sweep_run(cdi_domain *d, int n, const double *scale, const int *group
   const bool f64 = d->prec == CDI_FP64;
   // per-member device memory: velocity, two concentration buffers, accounts
   std::vector<void *> blocks;
-  auto take = [&](size_t bytes) {
-    void *p = cdi_dev_alloc(d, bytes);
+  auto take = [&](size_t bytes, bool need = true) {
+    void *p = need ? cdi_dev_need(d, bytes) : cdi_dev_alloc(d, bytes);
     if (p) blocks.push_back(p);
     return p;
   };
@@ -1712,7 +1715,7 @@ cdi_status sweep_run(cdi_domain *d, int n, const double *scale, const int *group
     s = cdi_flow_scale_to(d, scale[m], (void *)hm[m].u);
     if (s != CDI_OK) break;
     if (f64) {
-      void *co = take(bern_bytes(d));
+      void *co = take(bern_bytes(d), false);
       if (co) launch_coef64(d, d->stream, hm[m].u, hm[m].phi, co);
       hm[m].co = (const double2 *)co;
     } else {
@@ -1733,7 +1736,7 @@ cdi_status sweep_run(cdi_domain *d, int n, const double *scale, const int *group
       s = cdi_fail(d, CDI_ERR_CUDA, "sweep: face data");
     for (int m = 0; m < n && s == CDI_OK; m++)
       if (large[m])
-        mode = member_bern(d, d->stream, hm[m].f, hm[m].u, take(bern_bytes(d)))
+        mode = member_bern(d, d->stream, hm[m].f, hm[m].u, take(bern_bytes(d), false))
                    ? std::max<int>(mode, NP_LARGE) : NP_EVAL;
   }
   if (s == CDI_OK &&
@@ -1855,8 +1858,10 @@ cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, const do
   const int n = n_doms * n_combos, ns = L->ns;
   const bool f64 = L->prec == CDI_FP64;
   std::vector<void *> blocks;
-  auto take = [&](size_t bytes) {
+  auto take = [&](size_t bytes, bool need = true) {
     void *p = cdi_dev_alloc(L, bytes);
+    for (int i = 0; i < n_doms && !p && need; i++)
+      if (cdi_give_back(doms[i])) p = cdi_dev_alloc(L, bytes);
     if (p) blocks.push_back(p);
     return p;
   };
@@ -1908,7 +1913,7 @@ cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, const do
   for (int m = 0; m < n && s == CDI_OK; m++) {
     const cdi_domain *d = doms[m / n_combos];
     if (f64) {
-      void *co = take(bern_bytes(d));
+      void *co = take(bern_bytes(d), false);
       if (co) launch_coef64(d, L->stream, hm[m].s.u, hm[m].s.phi, co);
       hm[m].s.co = (const double2 *)co;
     } else {
@@ -1931,7 +1936,7 @@ cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, const do
     for (int m = 0; m < n && s == CDI_OK; m++) {
       const cdi_domain *d = doms[m / n_combos];
       if (large[m])
-        mode = member_bern(d, L->stream, hm[m].s.f, hm[m].s.u, take(bern_bytes(d)))
+        mode = member_bern(d, L->stream, hm[m].s.f, hm[m].s.u, take(bern_bytes(d), false))
                    ? std::max<int>(mode, NP_LARGE) : NP_EVAL;
     }
   }
