@@ -1691,6 +1691,7 @@ cdi_status sweep_run(cdi_domain *d, int n, const double *scale, const int *group
     void *c0 = take(CN), *c1 = take(CN);
     void *acc = take((size_t)3 * kMaxSpecies * d->np_accs * 8);
     float2 *fd = f64 ? nullptr : (float2 *)take((size_t)d->dim * d->n_pore * sizeof(float2));
+    if (!fd && m == 0) fd = d->d_fd;  // the domain's own state is replaced
     ok = u && c0 && c1 && acc && (f64 || fd);
     if (!ok) break;
     d->dt = dts[m];
@@ -1851,11 +1852,11 @@ void launch_batch(const cdi_domain *lead, cudaStream_t st, const void *members, 
 }
 
 template <typename T>
-cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, const double *scale,
-                     const int *group, void *const *phis, const double *dts, int64_t n_steps,
+cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, int m0, int n,
+                     const double *scale, const int *group, void *const *phis, const double *dts, int64_t n_steps,
                      double *gamma, double *cout) {
   cdi_domain *L = doms[0];  // the lead: its stream, allocator and scratch serve the batch
-  const int n = n_doms * n_combos, ns = L->ns;
+  const int ns = L->ns;
   const bool f64 = L->prec == CDI_FP64;
   std::vector<void *> blocks;
   auto take = [&](size_t bytes, bool need = true) {
@@ -1869,13 +1870,14 @@ cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, const do
   bool ok = true;
   int total_blocks = 0;
   for (int m = 0; m < n && ok; m++) {
-    cdi_domain *d = doms[m / n_combos];
+    cdi_domain *d = doms[(m0 + m) / n_combos];
     const size_t TN = (size_t)d->n_pore * sizeof(T);
     void *u = take((size_t)d->dim * TN);
     const size_t CN = (size_t)ns * TN * (d->cpair ? 2 : 1);
     void *c0 = take(CN), *c1 = take(CN);
     void *acc = take((size_t)3 * kMaxSpecies * d->np_accs * 8);
     float2 *fd = f64 ? nullptr : (float2 *)take((size_t)d->dim * d->n_pore * sizeof(float2));
+    if (!fd && (m == 0 || d != doms[(m0 + m - 1) / n_combos])) fd = d->d_fd;
     ok = u && c0 && c1 && acc && (f64 || fd);
     if (!ok) break;
     d->dt = dts[m];
@@ -1904,14 +1906,14 @@ cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, const do
   if (s == CDI_OK && cudaStreamSynchronize(L->stream) != cudaSuccess)
     s = cdi_fail(L, CDI_ERR_CUDA, "batch: member memory");
   for (int m = 0; m < n && s == CDI_OK; m++)
-    s = cdi_flow_scale_to(doms[m / n_combos], scale[m], (void *)hm[m].s.u);
+    s = cdi_flow_scale_to(doms[(m0 + m) / n_combos], scale[m], (void *)hm[m].s.u);
   for (int i = 0; i < n_doms && s == CDI_OK; i++)
     if (cudaStreamSynchronize(doms[i]->stream) != cudaSuccess)
       s = cdi_fail(L, CDI_ERR_CUDA, "batch: member setup");
   if (s == CDI_OK && cudaMemsetAsync(count, 0, sizeof(int) * n, L->stream) != cudaSuccess)
     s = cdi_fail(L, CDI_ERR_CUDA, "batch: memset");
   for (int m = 0; m < n && s == CDI_OK; m++) {
-    const cdi_domain *d = doms[m / n_combos];
+    const cdi_domain *d = doms[(m0 + m) / n_combos];
     if (f64) {
       void *co = take(bern_bytes(d), false);
       if (co) launch_coef64(d, L->stream, hm[m].s.u, hm[m].s.phi, co);
@@ -1934,7 +1936,7 @@ cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, const do
                         L->stream) != cudaSuccess || cudaStreamSynchronize(L->stream) != cudaSuccess)
       s = cdi_fail(L, CDI_ERR_CUDA, "batch: face data");
     for (int m = 0; m < n && s == CDI_OK; m++) {
-      const cdi_domain *d = doms[m / n_combos];
+      const cdi_domain *d = doms[(m0 + m) / n_combos];
       if (large[m])
         mode = member_bern(d, L->stream, hm[m].s.f, hm[m].s.u, take(bern_bytes(d), false))
                    ? std::max<int>(mode, NP_LARGE) : NP_EVAL;
@@ -1978,7 +1980,7 @@ cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, const do
   // outputs per member, through the same reductions as a single run
   const int cur = (int)(n_steps & 1);
   for (int m = 0; m < n && s == CDI_OK; m++) {
-    const cdi_domain *d = doms[m / n_combos];
+    const cdi_domain *d = doms[(m0 + m) / n_combos];
     const double area = d->dim == 2 ? d->dx : d->dx * d->dx;
     const double vol = d->dim == 2 ? d->dx * d->dx : d->dx * d->dx * d->dx;
     k_np_sums<T><<<kRedBlocks, kRedThreads, 0, L->stream>>>(
@@ -2013,21 +2015,34 @@ cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, const do
 
 }  // namespace
 
+// Members [m, m + n) by run(m, n), in halves where their memory cannot be had
+// at once (members are independent: the same bits).
+template <typename R> static cdi_status in_parts(int m, int n, const R &run) {
+  cdi_status s = run(m, n);
+  if (s != CDI_ERR_OOM || n < 2) return s;
+  s = in_parts(m, n / 2, run);
+  return s == CDI_OK ? in_parts(m + n / 2, n - n / 2, run) : s;
+}
+
 cdi_status cdi_np_batch(cdi_domain *const *doms, int n_doms, int n_combos, const double *scale,
                         const int *group, void *const *phis, const double *dts, int64_t n_steps,
                         double *gamma, double *cout) {
-  if (doms[0]->prec == CDI_FP64)
-    return batch_run<double>(doms, n_doms, n_combos, scale, group, phis, dts, n_steps, gamma,
-                             cout);
-  return batch_run<float>(doms, n_doms, n_combos, scale, group, phis, dts, n_steps, gamma, cout);
+  const int ns = doms[0]->ns;
+  return in_parts(0, n_doms * n_combos, [&](int m, int n) {
+    auto *run = doms[0]->prec == CDI_FP64 ? batch_run<double> : batch_run<float>;
+    return run(doms, n_doms, n_combos, m, n, scale + m, group + m, phis, dts + m, n_steps,
+               gamma + (size_t)m * ns, cout + (size_t)m * ns);
+  });
 }
 
-cdi_status cdi_np_sweep(cdi_domain *d, int n, const double *scale, const int *group,
+cdi_status cdi_np_sweep(cdi_domain *d, int n_members, const double *scale, const int *group,
                         void *const *phi_groups, const double *dts, int64_t n_steps,
                         double *gamma, double *cout) {
-  if (d->prec == CDI_FP64)
-    return sweep_run<double>(d, n, scale, group, phi_groups, dts, n_steps, gamma, cout);
-  return sweep_run<float>(d, n, scale, group, phi_groups, dts, n_steps, gamma, cout);
+  return in_parts(0, n_members, [&](int m, int n) {
+    auto *run = d->prec == CDI_FP64 ? sweep_run<double> : sweep_run<float>;
+    return run(d, n, scale + m, group + m, phi_groups, dts + m, n_steps,
+               gamma + (size_t)m * d->ns, cout + (size_t)m * d->ns);
+  });
 }
 
 // Coupled stepping (Eq. 3-5): before every block of couple_K steps (counted

@@ -208,3 +208,47 @@ def test_stored_coefficients_give_way(prec):
         d.init_transport(Z, D, c0=1e-3, Ka=1e-6)
         d.step(2)
         assert not any(named(b) for b in a.live.values())
+
+
+@pytest.mark.parametrize("prec", [cdi.FP64, cdi.FP32, cdi.FP32_CPAIR])
+def test_sweep_members_in_parts(prec):
+    """Five members in the memory of two: in parts, with the same bits.  Less
+    than one member needs: an error, and nothing kept.  (A member: velocity,
+    two concentration buffers and accounts; its face data may be the domain's.)"""
+    m = pack((9, 13, 35))
+    n, w = int((m == 0).sum()), 8 if prec == cdi.FP64 else 4
+    words = 2 if prec == cdi.FP32_CPAIR else 1
+    member = sum(-(-b // 256) * 256 for b in (
+        3 * w * n, 2 * w * words * n, 2 * w * words * n, 3 * 4 * 8 * (((n + 30) // 31 + 7) // 8 * 8)))
+    combos = [(1e-2, 0.3), (1e-3, 0.3), (1e-3, 0.0), (0.0, 0.3), (2e-3, 0.3)]
+    p = cdi.cdi_elec_params(298.15, 78.5, 10.0, 1.5e-7, 0, 1e-12, 100000)
+
+    def run(members):
+        a = Allocator()
+        with cdi.Domain(m, precision=prec, torch_resources=a) as d, \
+                cdi.Domain(m[:, :, ::-1].copy(), precision=prec) as other:
+            for x in (d, other):
+                x.solve_flow(tol=0.0, max_steps=200, U_target=1e-2)
+            before = a.total()
+            out = []
+            for phis, call in ((2, lambda: cdi.sweep_transport(d.handle, combos, p, Z, D, 10.0,
+                                                               1e-6, 70)),
+                               (4, lambda: cdi.sweep_batch([d.handle, other.handle], combos, p, Z,
+                                                           D, 10.0, 1e-6, 70))):
+                # the potentials, two small tables, and the members
+                cap = before + phis * (-(-8 * n // 256) * 256) + 4096 + int(members * member)
+                a.refuse = lambda nbytes: a.total() + nbytes > cap
+                if members < 1:
+                    with pytest.raises(cdi.CDIError) as e:
+                        call()
+                    assert e.value.status == 2
+                else:
+                    out += list(call())
+                assert a.total() == before and (a.refused > 0) == (members < 1000)
+            return out
+
+    ref = run(1000)
+    for members in (1, 2):
+        for x, y in zip(run(members), ref):
+            assert np.array_equal(x, y)
+    assert run(0.5) == []
