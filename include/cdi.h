@@ -65,8 +65,12 @@ typedef enum {
 
 typedef enum {
   CDI_FP64 = 0,      /* populations, velocity, potential, concentrations in FP64 */
-  CDI_FP32 = 1,      /* the same fields stored and updated in FP32; reductions,
-                        the potential solve and all accumulators stay FP64 */
+  CDI_FP32 = 1,      /* the same fields stored and updated in FP32.  In every
+                        precision the potential is FP64, solved to an FP64
+                        residual (its corrections may be FP32, see
+                        cdi_set_potential), and reductions are FP64; the
+                        transport accounts are FP64, or FP32 pairs (48 bits)
+                        in FP32 storage */
   CDI_FP32_SPLIT = 2, /* as CDI_FP32, but every population and every
                          concentration is an unevaluated pair of FP32 words
                          (hi + lo) updated with error-free FP32
@@ -132,7 +136,8 @@ typedef struct {
                           (mode 2: of the nonlinear equation against the
                           surface terms; each linear solve runs to tol / 10) */
   int max_iter;        /* conjugate-gradient iterations (mode 2: per Newton
-                          step, at most 200 steps) */
+                          step, at most 200 steps; the linear modes may run
+                          as many FP32 iterations before, see below) */
 } cdi_elec_params;
 
 typedef struct {
@@ -215,7 +220,11 @@ cdi_status cdi_set_velocity(cdi_domain *dom, double U_target_mps);
 /* Solve the potential with surface value psi_s = -applied_V on every solid
  * face (Eq. 4 with the Dirichlet condition of Sec. 2), psi = 0 in the inlet
  * feed, no flux through the outlet and lateral walls.  Invalidates an
- * initialised transport state.  iters_out / relres_out may be NULL. */
+ * initialised transport state.  The linear modes with dx / lambda_D below
+ * 0.22 are solved by FP32 corrections of an FP64 residual; where these do not
+ * reach tol within max_iter iterations, and for all other fields, by an FP64
+ * iteration.  iters_out / relres_out (of the solve that gave the field) may be
+ * NULL. */
 cdi_status cdi_set_potential(cdi_domain *dom, double applied_V,
                              const cdi_elec_params *p, int *iters_out,
                              double *relres_out);

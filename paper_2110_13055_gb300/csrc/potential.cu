@@ -617,7 +617,9 @@ constexpr double kRefineBelow = 0.05;
 // The refinement above; *done says whether it reached tol.  Where it does not
 // (max_iter ran out first, tol below what an FP64 residual can show, or a
 // system too ill-conditioned for FP32 corrections) the caller starts over
-// with the FP64 iteration, whose own residual is a recurrence.
+// with the FP64 iteration, whose own residual is a recurrence.  That one gets
+// all of max_iter again, since corrections may take more iterations than it
+// does; the figures returned are its own, the timing counts both.
 static cdi_status psi_refine(cdi_domain *d, double psi_s, double kdx2, const double *src,
                              double tol, int max_iter, bool *done) {
   *done = false;
@@ -665,6 +667,7 @@ static cdi_status psi_refine(cdi_domain *d, double psi_s, double kdx2, const dou
   if (d->h_scal[S_CG_ALPHA] != 0.0)
     return cdi_fail(d, CDI_ERR_CUDA, "potential solve: a grid barrier ran into its limit");
   *done = d->h_scal[S_CG_DONE] != 0.0;
+  if (!*done) d->timing.psi_iters += (int64_t)d->h_scal[S_CG_IT];
   return CDI_OK;
 }
 
@@ -676,7 +679,10 @@ cdi_status cdi_psi_solve(cdi_domain *d, double psi_s, double kdx2, const double 
   cdi_timing_begin(d, &ev);
   bool done = false;
   cdi_status cs = psi_refine(d, psi_s, kdx2, src, tol, max_iter, &done);
-  if (cs != CDI_OK) return cs;
+  if (cs != CDI_OK) {
+    cdi_timing_end(d, ev, PH_PSI, 0);
+    return cs;
+  }
   if (done) return finish_potential(d, ev, done, iters, relres);
   k_cg_setup<<<kRedBlocks, kRedThreads, 0, d->stream>>>(g, d->d_nflags, kdx2, psi_s, src, tol,
                                                          d->d_psi, r, p, dg, d->d_part,

@@ -111,3 +111,25 @@ def test_potential_of_any_size(shape, mode, lam, shift):
         b = d.psi() * 2.0 ** -shift
     assert it2 == it and 0.0 < res < 1e-13
     assert rel(b, a) < 2.4e-10
+
+
+def test_iterations_counted():
+    """The timing counts the iterations of every solve; the call returns those
+    of the solve that gave the field."""
+    m = image((61, 83))
+
+    def counted(**kw):
+        d.timing(reset=True)
+        it = d.set_potential(0.7, lambda_D=1e-6, **kw)[0]
+        return it, d.timing()["psi_iters"]
+
+    with cdi.Domain(m) as d:
+        d.solve_flow(tol=0.0, max_steps=0, U_target=0.0)
+        it, n = counted(tol=1e-13)
+        assert n == it
+        it, n = counted(tol=1e-18)       # begun again by the FP64 iteration
+        assert n > it > 0
+        d.timing(reset=True)
+        with pytest.raises(cdi.CDIError):
+            d.set_potential(0.7, lambda_D=1e-6, tol=1e-13, max_iter=2)
+        assert d.timing()["psi_iters"] == 4
