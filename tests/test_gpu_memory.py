@@ -252,3 +252,41 @@ def test_sweep_members_in_parts(prec):
         for x, y in zip(run(members), ref):
             assert np.array_equal(x, y)
     assert run(0.5) == []
+
+
+@pytest.mark.parametrize("prec", [cdi.FP64, cdi.FP32_CPAIR])
+def test_allocator_of_looser_alignment(prec):
+    """Blocks that start on 8 bytes only: the same bits as on 256."""
+    m = pack((9, 13, 35))
+
+    class Loose(Allocator):
+        def __init__(self):
+            import torch
+            self.live = {}
+
+            def _alloc(nbytes, ctx):
+                p = torch.cuda.caching_allocator_alloc(int(nbytes) + 8, 0) + 8
+                self.live[p] = nbytes
+                return p
+
+            def _free(ptr, nbytes, ctx):
+                assert self.live.pop(ptr) == nbytes
+                torch.cuda.caching_allocator_delete(ptr - 8)
+
+            self._a, self._f = cdi.ALLOC_FN(_alloc), cdi.FREE_FN(_free)
+            self.allocator = cdi.cdi_allocator(self._a, self._f, None)
+
+    def run(a):
+        with cdi.Domain(m, precision=prec, torch_resources=a) as d:
+            d.solve_flow(tol=0.0, max_steps=200, U_target=1e-2)
+            d.set_potential(0.3, mode="laplace", tol=1e-12)
+            d.init_transport((1, -1, 2), (1.33e-9, 2.03e-9, 0.7e-9), c0=1e-3, Ka=1e-6)
+            d.step(70)
+            d.set_implicit(1e-10, 500)
+            d.step(2)
+            out = [d.C(), *d.mass_balance()]
+        assert not a.live
+        return out
+
+    for x, y in zip(run(Loose()), run(Allocator())):
+        assert np.array_equal(x, y)

@@ -133,3 +133,18 @@ def test_iterations_counted():
         with pytest.raises(cdi.CDIError):
             d.set_potential(0.7, lambda_D=1e-6, tol=1e-13, max_iter=2)
         assert d.timing()["psi_iters"] == 4
+
+
+@pytest.mark.parametrize("walls", [False, True])
+def test_potential_lateral_differences_beyond_16_bits(walls):
+    """Cells whose z neighbours lie more than 32,000 ranks apart (the refinement
+    then reads their full ranks); at the bar of test_potential_solver_shapes."""
+    m = np.zeros((3, 190, 256), np.uint8)
+    m[1, 2:185, :] = 1
+    ref, _, _ = O.psi(m, -0.7, dx=1e-7, c_bulk=10.0, mode="laplace", tol=1e-14,
+                      lateral_walls=walls)
+    with cdi.Domain(m, lateral_walls=walls) as d:
+        d.solve_flow(tol=0.0, max_steps=0, U_target=0.0)
+        d.set_potential(0.7, c_bulk=10.0, mode="laplace", tol=1e-13)
+        ps = d.psi()
+    assert rel(ps, ref) < 1e-10

@@ -55,3 +55,15 @@ def test_lateral_differences_beyond_16_bits():
     c, g, _ = advance(m, cdi.FP32_CPAIR, 2, 0.0, 6, dt=dt)
     assert rel(c, C) < 1e-6
     assert np.all(np.abs(g - G) < 1e-6 * np.abs(G).sum())
+
+
+@pytest.mark.parametrize("prec", [cdi.FP32, cdi.FP32_CPAIR])
+@pytest.mark.parametrize("ns", [2, 3])
+def test_steps_of_a_state_larger_than_l2(ns, prec):
+    """1.8 million pore cells: the step asks for its inputs ahead (one and two
+    species pairs).  Four steps; the bars of test_species_records_and_faces."""
+    m = inputs.grain_pack((120, 125, 171), 0.7, 8.0, 14.0, seed=3)[0]
+    C, G, dt = advance(m, cdi.FP64, ns, 0.0, 4)
+    c, g, _ = advance(m, prec, ns, 0.0, 4, dt=dt)
+    assert rel(c, C) < 1e-4
+    assert np.all(np.abs(g - G) < 1e-6 * np.abs(G).sum() + 1e-5 * np.abs(G))
