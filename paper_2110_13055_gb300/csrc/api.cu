@@ -347,12 +347,9 @@ cdi_status cdi_create_domain(const cdi_domain_desc *desc, const uint8_t *mask,
     return p;
   };
   d->d_mask = (uint8_t *)A(N);
-  d->d_fflags = A(Nf * fflag);
   d->d_nflags = (cdi::NFlag *)A(N * sizeof(cdi::NFlag));
   d->d_flow_list = (int *)A((size_t)d->n_flow_pore * sizeof(int));
   d->d_cell_list = (int *)A((size_t)n_pore * sizeof(int));
-  int *list_work = (int *)A(cdi_lists_work_ints(Nf) * sizeof(int));
-  int *rank_work = (int *)A((size_t)Nf * sizeof(int));
   // populations stored by pore rank: Q * n_flow_pore values
   const size_t nq = (size_t)Q * d->n_flow_pore;
   const size_t Tpop = d->prec == CDI_FP64 ? 8 : d->prec == CDI_BF16_POP ? 2 : 4;
@@ -367,7 +364,6 @@ cdi_status cdi_create_domain(const cdi_domain_desc *desc, const uint8_t *mask,
   // transport fields by pore rank
   d->W = (D.nx + 31) / 32;
   const size_t n_words = (size_t)D.ny * D.nz * d->W;
-  d->d_cmeta = (uint2 *)A((size_t)n_pore * sizeof(uint2));
   d->d_cfl = (cdi::NFlag *)A((size_t)n_pore * sizeof(cdi::NFlag));
   d->d_words = (uint2 *)A(n_words * sizeof(uint2));
   d->d_latnb = (int *)A((size_t)2 * (D.dim - 1) * n_pore * sizeof(int));
@@ -384,7 +380,11 @@ cdi_status cdi_create_domain(const cdi_domain_desc *desc, const uint8_t *mask,
   d->d_part = (double *)A((size_t)16 * cdi::kRedBlocks * 8);
   d->d_counter = (unsigned int *)A(16 * sizeof(unsigned int));
   d->d_scal = (double *)A(S_COUNT * 8);
-  d->d_cg = (double *)A((size_t)4 * N * 8);
+  // the flow flags, ranks and lists that only this call needs stand in the
+  // potential solver's scratch
+  const size_t ff_bytes = ((size_t)Nf * fflag + 15) & ~size_t(15);
+  const size_t work_bytes = ff_bytes + ((size_t)Nf + cdi_lists_work_ints(Nf)) * sizeof(int);
+  d->d_cg = (double *)A(std::max<size_t>((size_t)4 * N * 8, work_bytes));
   d->d_colout = (double *)A((size_t)D.nx * 8);
   if (!ok) {
     free_all(d);
@@ -415,16 +415,14 @@ cdi_status cdi_create_domain(const cdi_domain_desc *desc, const uint8_t *mask,
   chk(cudaMemsetAsync(d->d_C[1], 0, c_bytes, d->stream), "memset");
   chk(cudaMemsetAsync(d->d_acc, 0, (size_t)3 * cdi::kMaxSpecies * d->np_accs * 8, d->stream),
       "memset");
-  if (s == CDI_OK) s = cdi_flow_build_flags(d);
+  void *fflags = d->d_cg;
+  int *rank_work = (int *)((char *)fflags + ff_bytes), *list_work = rank_work + Nf;
+  if (s == CDI_OK) s = cdi_flow_build_flags(d, fflags);
   if (s == CDI_OK) s = cdi_np_build_flags(d);
-  if (s == CDI_OK) s = cdi_build_lists(d, list_work);
+  if (s == CDI_OK) s = cdi_build_lists(d, fflags, list_work);
   if (s == CDI_OK) s = cdi_np_build_compact(d);
-  if (s == CDI_OK) s = cdi_flow_build_links(d, rank_work);
+  if (s == CDI_OK) s = cdi_flow_build_links(d, fflags, rank_work);
   if (s == CDI_OK) chk(cudaStreamSynchronize(d->stream), "create domain");
-  if (s == CDI_OK) {  // the work arrays are needed at create time only
-    cdi_dev_release(d, rank_work);
-    cdi_dev_release(d, list_work);
-  }
   if (s != CDI_OK) {
     g_create_error = d->err;
     free_all(d);

@@ -422,7 +422,6 @@ struct cdi_domain {
 
   // device buffers
   uint8_t *d_mask = nullptr;    // N
-  void *d_fflags = nullptr;     // Nf flow flags
   cdi::NFlag *d_nflags = nullptr;  // N face flags
   int *d_flow_list = nullptr;   // pore sites of the flow grid, ascending
   long long n_flow_pore = 0;
@@ -439,8 +438,7 @@ struct cdi_domain {
   int n_lovf = 0;
   int *d_cell_list = nullptr;   // pore cells of the transport grid, ascending:
                                 // entry r is the lattice cell of pore rank r
-  uint2 *d_cmeta = nullptr;     // n_pore: {face flags | x << 16, row = z*ny + y}
-  cdi::NFlag *d_cfl = nullptr;  // n_pore: face flags alone (read by the FP32 step)
+  cdi::NFlag *d_cfl = nullptr;  // n_pore: face flags
   uint2 *d_words = nullptr;     // ny*nz*W: per 32 cells of a row {rank of the
                                 // first pore cell at or after it, pore bits}
   int W = 0;                    // words per row, ceil(nx / 32)
@@ -617,10 +615,10 @@ void cdi_tune_store(uint64_t key, int variant);
   } while (0)
 
 // Kernel-side entry points used by the API layer.
-cdi_status cdi_flow_build_flags(cdi_domain *d);
+cdi_status cdi_flow_build_flags(cdi_domain *d, void *fflags);
 size_t cdi_lists_work_ints(long long n);
-cdi_status cdi_flow_build_links(cdi_domain *d, int *rank_work);
-cdi_status cdi_build_lists(cdi_domain *d, int *work);
+cdi_status cdi_flow_build_links(cdi_domain *d, const void *fflags, int *rank_work);
+cdi_status cdi_build_lists(cdi_domain *d, const void *fflags, int *work);
 cdi_status cdi_flow_run(cdi_domain *d, const cdi_flow_params *p, int64_t *steps,
                         double *res);
 cdi_status cdi_flow_export(cdi_domain *d, double U_target);

@@ -101,12 +101,12 @@ cdi_status compact(cdi_domain *d, const F *fl, long long n, int *list, int *work
 
 size_t cdi_lists_work_ints(long long n) { return 2 * (size_t)((n + kChunk - 1) / kChunk); }
 
-cdi_status cdi_build_lists(cdi_domain *d, int *work) {
+cdi_status cdi_build_lists(cdi_domain *d, const void *fflags, int *work) {
   cdi_status s;
   if (d->dim == 2)
-    s = compact(d, (const FlowFlag<2>::type *)d->d_fflags, d->Nf, d->d_flow_list, work);
+    s = compact(d, (const FlowFlag<2>::type *)fflags, d->Nf, d->d_flow_list, work);
   else
-    s = compact(d, (const FlowFlag<3>::type *)d->d_fflags, d->Nf, d->d_flow_list, work);
+    s = compact(d, (const FlowFlag<3>::type *)fflags, d->Nf, d->d_flow_list, work);
   if (s != CDI_OK) return s;
   return compact(d, d->d_nflags, d->N, d->d_cell_list, work);
 }

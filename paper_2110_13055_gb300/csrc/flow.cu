@@ -1342,11 +1342,11 @@ cdi_status flow_export(cdi_domain *d, double U_target) {
 }
 
 template <int DIM>
-cdi_status build_flags(cdi_domain *d) {
+cdi_status build_flags(cdi_domain *d, void *fflags) {
   using FT = typename FlowFlag<DIM>::type;
   dim3 grid((d->NX + kRowBlock - 1) / kRowBlock, d->ny, d->nz);
-  k_flow_flags<DIM><<<grid, kRowBlock, 0, d->stream>>>(d->d_mask, (FT *)d->d_fflags, d->nx,
-                                                       d->NX, d->ny, d->nz, d->walls);
+  k_flow_flags<DIM><<<grid, kRowBlock, 0, d->stream>>>(d->d_mask, (FT *)fflags, d->nx, d->NX,
+                                                       d->ny, d->nz, d->walls);
   d->timing.kernel_launches++;
   CDI_TRY(d, cudaGetLastError(), "flow flags");
   return CDI_OK;
@@ -1356,15 +1356,16 @@ cdi_status build_flags(cdi_domain *d) {
 
 int cdi_lbm_shape_block(int v) { return v >= 0 && v < 6 ? kLbmVariantBlock[v] : 0; }
 
-cdi_status cdi_flow_build_flags(cdi_domain *d) {
-  return d->dim == 2 ? build_flags<2>(d) : build_flags<3>(d);
+// The flow flags (Nf words of FlowFlag): read while the domain is built.
+cdi_status cdi_flow_build_flags(cdi_domain *d, void *fflags) {
+  return d->dim == 2 ? build_flags<2>(d, fflags) : build_flags<3>(d, fflags);
 }
 
 // Neighbour data of the compact population layout (after the pore lists):
 // rank[site] scattered from the list (rank_work: Nf ints, -1 for solid), then
 // the flag words, row-base bytes and tile bases of every pore rank; then the
 // overflow table, sized by the sites that need it, is taken and filled.
-cdi_status cdi_flow_build_links(cdi_domain *d, int *rank_work) {
+cdi_status cdi_flow_build_links(cdi_domain *d, const void *fflags, int *rank_work) {
   const int n = (int)d->n_flow_pore;
   const int Q = d->dim == 2 ? 9 : 19;
   unsigned *n_extra = d->d_counter + C_LINK;
@@ -1374,11 +1375,11 @@ cdi_status cdi_flow_build_links(cdi_domain *d, int *rank_work) {
   k_rank_scatter<<<kRedBlocks, kRedThreads, 0, d->stream>>>(d->d_flow_list, n, rank_work);
   if (d->dim == 2)
     k_links<2><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        (const FlowFlag<2>::type *)d->d_fflags, d->d_flow_list, n, rank_work, d->d_lf, d->d_ld,
+        (const FlowFlag<2>::type *)fflags, d->d_flow_list, n, rank_work, d->d_lf, d->d_ld,
         d->d_lb, d->n_ltiles, n_extra, d->NX, d->ny, d->nz, d->walls);
   else
     k_links<3><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        (const FlowFlag<3>::type *)d->d_fflags, d->d_flow_list, n, rank_work, d->d_lf, d->d_ld,
+        (const FlowFlag<3>::type *)fflags, d->d_flow_list, n, rank_work, d->d_lf, d->d_ld,
         d->d_lb, d->n_ltiles, n_extra, d->NX, d->ny, d->nz, d->walls);
   CDI_TRY(d, cudaGetLastError(), "neighbour data");
   unsigned extra = 0;
@@ -1392,11 +1393,11 @@ cdi_status cdi_flow_build_links(cdi_domain *d, int *rank_work) {
                              d->stream), "overflow reset");
   if (d->dim == 2)
     k_links_ovf<2><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        (const FlowFlag<2>::type *)d->d_fflags, d->d_flow_list, n, rank_work, d->d_lf, d->d_ld,
+        (const FlowFlag<2>::type *)fflags, d->d_flow_list, n, rank_work, d->d_lf, d->d_ld,
         d->d_lovf, d->n_lovf, d->NX, d->ny, d->nz);
   else
     k_links_ovf<3><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        (const FlowFlag<3>::type *)d->d_fflags, d->d_flow_list, n, rank_work, d->d_lf, d->d_ld,
+        (const FlowFlag<3>::type *)fflags, d->d_flow_list, n, rank_work, d->d_lf, d->d_ld,
         d->d_lovf, d->n_lovf, d->NX, d->ny, d->nz);
   d->timing.kernel_launches += 3;
   CDI_TRY(d, cudaGetLastError(), "neighbour overflow table");

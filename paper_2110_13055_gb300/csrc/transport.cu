@@ -1123,7 +1123,7 @@ __global__ void k_np_init(CViews<T> C, int n, int ns, T c0, T c0lo) {
 // sum of C at the outlet, 13 pore cells in the outlet column.
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads)
-    k_np_sums(const uint2 *__restrict__ meta, CViews<T> C, const T *__restrict__ u, int n,
+    k_np_sums(const NFlag *__restrict__ fl, CViews<T> C, const T *__restrict__ u, int n,
               int ns, double cell_vol, double *__restrict__ part, unsigned int *counter, double *scal) {
   constexpr int NV = 14;
   __shared__ double sm[NV * 32];
@@ -1131,7 +1131,7 @@ __global__ void __launch_bounds__(kRedThreads)
 #pragma unroll
   for (int j = 0; j < NV; j++) v[j] = 0.0;
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
-    const bool outlet = (meta[r].x >> kEdgeBit) & 1u;
+    const bool outlet = ((unsigned)fl[r] >> kEdgeBit) & 1u;
     const double ux = (double)u[r];
 #pragma unroll
     for (int k = 0; k < kMaxSpecies; k++) {
@@ -1172,14 +1172,14 @@ __global__ void __launch_bounds__(kRedThreads)
 // sum of the x velocity over them (the numerator of Sec. 4's pore mean U).
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads)
-    k_geometry(const uint2 *__restrict__ meta, const T *__restrict__ ux, int n, int faces,
+    k_geometry(const NFlag *__restrict__ fl, const T *__restrict__ ux, int n, int faces,
                double *__restrict__ part, unsigned int *counter, double *scal) {
   __shared__ double sm[3 * 32];
   double v[3] = {0.0, 0.0, 0.0};
   const unsigned face_bits = ((1u << faces) - 1u) << kFaceBit;
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
     v[0] += 1.0;
-    v[1] += (double)__popc(meta[r].x & face_bits);
+    v[1] += (double)__popc((unsigned)fl[r] & face_bits);
     v[2] += (double)ux[r];
   }
   block_reduce<3>(v, sm, OpSum(), 0.0);
@@ -1249,13 +1249,12 @@ __global__ void __launch_bounds__(kRedThreads)
 // neighbour across it (rows wrap periodically), or -1 across a solid face or
 // a lateral wall.  The step kernels read it instead of the row words, which
 // saves them a dependent load and the rank arithmetic.
-__global__ void k_lat_nbr(const uint2 *__restrict__ meta, const uint2 *__restrict__ words,
-                          int n, int W, int ny, int nz, int walls, int faces,
-                          int *__restrict__ lat) {
+__global__ void k_lat_nbr(const NFlag *__restrict__ fl, const int *__restrict__ cells,
+                          const uint2 *__restrict__ words, int n, int nx, int W, int ny, int nz,
+                          int walls, int faces, int *__restrict__ lat) {
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
-    const uint2 m = meta[r];
-    const unsigned f = m.x & 0xffffu;
-    const int x = (int)(m.x >> 16), row = (int)m.y;
+    const unsigned f = fl[r];
+    const int P = cells[r], row = P / nx, x = P - row * nx;
     for (int fc = 2; fc < faces; fc++) {
       const bool solid = (f >> (kFaceBit + fc)) & 1u;
       const bool wall = ((f >> (kEdgeBit + fc)) & 1u) && walls;
@@ -1265,15 +1264,11 @@ __global__ void k_lat_nbr(const uint2 *__restrict__ meta, const uint2 *__restric
   }
 }
 
-// Per pore rank: its face flags, x and row.
-__global__ void k_cmeta(const NFlag *__restrict__ fl, const int *__restrict__ cells, int n,
-                        int nx, uint2 *__restrict__ meta, NFlag *__restrict__ cfl) {
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
-    const int P = cells[r];
-    const int row = P / nx, x = P - row * nx;
-    meta[r] = make_uint2((unsigned)fl[P] | ((unsigned)x << 16), (unsigned)row);
-    cfl[r] = fl[P];
-  }
+// Per pore rank: its face flags.
+__global__ void k_cfl(const NFlag *__restrict__ fl, const int *__restrict__ cells, int n,
+                      NFlag *__restrict__ cfl) {
+  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x)
+    cfl[r] = fl[cells[r]];
 }
 
 // Per 32 cells of a row: the pore bits and the rank of the first pore cell at
@@ -1780,7 +1775,7 @@ cdi_status sweep_run(cdi_domain *d, int n, const double *scale, const int *group
   const double vol = d->dim == 2 ? d->dx * d->dx : d->dx * d->dx * d->dx;
   for (int m = 0; m < n && s == CDI_OK; m++) {
     k_np_sums<T><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        d->d_cmeta, c_views<T>(d, hm[m].C[cur]), hm[m].u, (int)d->n_pore, ns, vol, d->d_part,
+        d->d_cfl, c_views<T>(d, hm[m].C[cur]), hm[m].u, (int)d->n_pore, ns, vol, d->d_part,
         d->d_counter + C_MASS, d->d_scal);
     acc_total(d, hm[m].acc, d->stream, d->d_scal);
     d->timing.kernel_launches += 2;
@@ -1984,7 +1979,7 @@ cdi_status batch_run(cdi_domain *const *doms, int n_doms, int n_combos, int m0, 
     const double area = d->dim == 2 ? d->dx : d->dx * d->dx;
     const double vol = d->dim == 2 ? d->dx * d->dx : d->dx * d->dx * d->dx;
     k_np_sums<T><<<kRedBlocks, kRedThreads, 0, L->stream>>>(
-        d->d_cmeta, c_views<T>(d, hm[m].s.C[cur]), hm[m].s.u, (int)d->n_pore, ns, vol,
+        d->d_cfl, c_views<T>(d, hm[m].s.C[cur]), hm[m].s.u, (int)d->n_pore, ns, vol,
         L->d_part, L->d_counter + C_MASS, L->d_scal);
     acc_total(d, hm[m].s.acc, L->stream, L->d_scal);
     L->timing.kernel_launches += 2;
@@ -2129,11 +2124,11 @@ cdi_status cdi_np_reduce(cdi_domain *d) {
   const double vol = d->dim == 2 ? d->dx * d->dx : d->dx * d->dx * d->dx;
   if (d->prec == CDI_FP64)
     k_np_sums<double><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        d->d_cmeta, c_views<double>(d, d->d_C[d->cur]), (const double *)d->d_u,
+        d->d_cfl, c_views<double>(d, d->d_C[d->cur]), (const double *)d->d_u,
         (int)d->n_pore, d->ns, vol, d->d_part, d->d_counter + C_MASS, d->d_scal);
   else
     k_np_sums<float><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        d->d_cmeta, c_views<float>(d, d->d_C[d->cur]), (const float *)d->d_u,
+        d->d_cfl, c_views<float>(d, d->d_C[d->cur]), (const float *)d->d_u,
         (int)d->n_pore, d->ns, vol, d->d_part, d->d_counter + C_MASS, d->d_scal);
   acc_total(d, d->d_acc, d->stream, d->d_scal);
   d->timing.kernel_launches += 2;
@@ -2150,11 +2145,11 @@ cdi_status cdi_np_reduce(cdi_domain *d) {
 cdi_status cdi_np_geometry(cdi_domain *d, double *pores, double *faces, double *sum_ux) {
   if (d->prec == CDI_FP64)
     k_geometry<double><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        d->d_cmeta, (const double *)d->d_u, (int)d->n_pore, 2 * d->dim, d->d_part,
+        d->d_cfl, (const double *)d->d_u, (int)d->n_pore, 2 * d->dim, d->d_part,
         d->d_counter + C_GEOM, d->d_scal);
   else
     k_geometry<float><<<kRedBlocks, kRedThreads, 0, d->stream>>>(
-        d->d_cmeta, (const float *)d->d_u, (int)d->n_pore, 2 * d->dim, d->d_part,
+        d->d_cfl, (const float *)d->d_u, (int)d->n_pore, 2 * d->dim, d->d_part,
         d->d_counter + C_GEOM, d->d_scal);
   d->timing.kernel_launches++;
   CDI_TRY(d, cudaGetLastError(), "geometry");
@@ -2181,17 +2176,17 @@ cdi_status cdi_np_column_means(cdi_domain *d, int k) {
   return CDI_OK;
 }
 
-// Rank metadata and row words of the compact transport layout (after the
+// Face flags, row words and lateral links of the compact transport layout (after the
 // pore lists and the face flags).
 cdi_status cdi_np_build_compact(cdi_domain *d) {
   const int n = (int)d->n_pore;
   const long long n_words = (long long)d->ny * d->nz * d->W;
-  k_cmeta<<<kRedBlocks, kRedThreads, 0, d->stream>>>(d->d_nflags, d->d_cell_list, n, d->nx,
-                                                     d->d_cmeta, d->d_cfl);
+  k_cfl<<<kRedBlocks, kRedThreads, 0, d->stream>>>(d->d_nflags, d->d_cell_list, n, d->d_cfl);
   k_words<<<kRedBlocks, kRedThreads, 0, d->stream>>>(d->d_nflags, d->d_cell_list, n, d->nx, d->W,
                                                      n_words, d->d_words);
-  k_lat_nbr<<<kRedBlocks, kRedThreads, 0, d->stream>>>(d->d_cmeta, d->d_words, n, d->W, d->ny,
-                                                       d->nz, d->walls, 2 * d->dim, d->d_latnb);
+  k_lat_nbr<<<kRedBlocks, kRedThreads, 0, d->stream>>>(d->d_cfl, d->d_cell_list, d->d_words, n,
+                                                       d->nx, d->W, d->ny, d->nz, d->walls,
+                                                       2 * d->dim, d->d_latnb);
   if (d->dim == 2)
     k_lat_pack<2><<<kRedBlocks, kRedThreads, 0, d->stream>>>(d->d_latnb, n, d->d_latd, d->d_latb);
   else

@@ -290,3 +290,29 @@ def test_allocator_of_looser_alignment(prec):
 
     for x, y in zip(run(Loose()), run(Allocator())):
         assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("prec", [cdi.FP64, cdi.FP32, cdi.FP32_CPAIR])
+@pytest.mark.parametrize("shape", [(301, 403), (48, 51, 55)], ids=str)
+def test_domain_memory(shape, prec):
+    """The most that creating a domain holds, bytes: 2D and 3D packs of
+    porosity 0.6 fit where they fitted before the transport step had face data
+    and 16-bit links of its own (flow flags, ranks and rank metadata then stood
+    beside the fields)."""
+    m = pack(shape)
+    dim, N, n = m.ndim, m.size, int((m == 0).sum())
+    w = 8 if prec == cdi.FP64 else 4
+    flow = 2 * n * (9 * w + 4 + 4 + 4) if dim == 2 else 2 * n * (19 * w + 4 + 4 + 8)
+    flow += 2 * N * ((2 if dim == 2 else 4) + 4 + 8 * dim)        # flags, ranks, velocity
+    transport = n * (4 + 8 + 2 + 8 * (dim - 1) + dim * w + 8)     # lists, links, u, phi
+    transport += n * 2 * 4 * w * (2 if prec == cdi.FP32_CPAIR else 1)
+    accounts = 3 * 4 * 8 * (((n + 30) // 31 + 7) // 8 * 8)
+    before = flow + transport + accounts + N * (1 + 2 + 8 + 32)
+    # tile bases, row words, links of the x edges; partials and the rest
+    rows = N // m.shape[-1]
+    tables = (2 if dim == 2 else 8) * n // 4 + rows * 8 * (-(-m.shape[-1] // 32))
+    tables += (8 if dim == 2 else 18) * 4 * 2 * rows + (1 << 18)
+    a, peak = Allocator(), []
+    a.refuse = lambda nbytes: peak.append(a.total() + nbytes)
+    with cdi.Domain(m, precision=prec, torch_resources=a):
+        assert max(peak) <= before + tables
