@@ -54,10 +54,9 @@ class Request:
     error: str = ""
 
 
-def footprint_bytes(mask: np.ndarray, precision: int, mirror: bool = True) -> int:
-    """Peak device memory a domain for this mask allocates (the allocations of
-    cdi_create_domain, including its create-time work arrays), with one
-    transport state."""
+def required_bytes(mask: np.ndarray, precision: int, mirror: bool = True) -> int:
+    """Device memory that a domain for this mask cannot do without (the
+    allocations of cdi_create_domain), with one transport state."""
     dim = mask.ndim
     N = int(mask.size)
     n_pore = int((mask == 0).sum())
@@ -77,15 +76,22 @@ def footprint_bytes(mask: np.ndarray, precision: int, mirror: bool = True) -> in
     links = (4 + (4 if dim == 2 else 8)) * n_fp + n_off * 4 * ((n_fp + 31) // 32)
     flow = (Q * Tpop * n_fp + links + (Q - 1) * 4 * n_ovf
             + Nf * (2 if dim == 2 else 4) + dim * Nf * 8)
-    # with the lateral differences and, for two species, the face coefficients
-    # (FP64) or the face data and the Bernoulli pairs a resolved double layer needs
-    faces = (dim + 1) * 32 if precision == cdi.FP64 else dim * 8 + (dim + 1) * 16
-    transport = (n_pore * (4 + 8 + 2 + 2 * (dim - 1) * (4 + 2 + 1) + dim * T + 8 + 2 * 4 * Tc
-                           + faces)
+    # face data and lateral differences (about 33 B a pore cell in 3D FP32)
+    # take no more than the flow flags and work arrays counted here, which
+    # stand in the CG vectors while a domain is created
+    transport = (n_pore * (4 + 8 + 2 + 2 * (dim - 1) * 4 + dim * T + 8 + 2 * 4 * Tc)
                  + rows * ((nx + 31) // 32) * 8)
     lattice = N * (1 + 2 + 8 + 4 * 8)                 # mask, face flags, psi, CG vectors
     work = Nf * 4 + 2 * ((Nf + 2047) // 2048) * 4     # create-time rank and list work
     return flow + transport + lattice + work + (4 << 20)
+
+
+def footprint_bytes(mask: np.ndarray, precision: int, mirror: bool = True) -> int:
+    """Peak device memory of a domain for this mask where there is as much: with
+    what explicit steps of two species keep to be faster, the face coefficients
+    (FP64) or the Bernoulli pairs of a resolved double layer (FP32)."""
+    faces = (mask.ndim + 1) * (32 if precision == cdi.FP64 else 16)
+    return required_bytes(mask, precision, mirror) + faces * int((mask == 0).sum())
 
 
 def size_priority(need: int) -> int:
@@ -105,7 +111,8 @@ class Server:
     queue behind a large one that does not fit yet.  To keep a large request
     from waiting for ever, a waiting request that has been passed over
     ``max_bypass`` times is served next: nothing younger is admitted until it
-    fits."""
+    fits.  A request whose footprint is beyond the whole budget, but not what it
+    requires, is given all of the budget and runs alone."""
 
     def __init__(self, slots: int = 4, memory_budget: int = 16 << 30, device: int = 0,
                  solver=None, max_bypass: int | None = None, prioritise_large: bool = True):
@@ -129,6 +136,8 @@ class Server:
     def submit(self, req: Request) -> None:
         req.t_arrival = time.perf_counter()
         need = footprint_bytes(req.mask, req.precision)
+        if need > self.budget:
+            need = max(self.budget, required_bytes(req.mask, req.precision))
         with self._lock:
             self._waiting.append((req, need, [0]))
             self._lock.notify_all()

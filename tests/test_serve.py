@@ -181,3 +181,22 @@ def test_larger_requests_get_higher_stream_priority():
         want = serve.size_priority(serve.footprint_bytes(big, cdi.FP32)) if flag else 0
         assert seen == {"small": 0, "big": want}
         assert not flag or want < 0
+
+
+@pytest.mark.parametrize("precision", [cdi.FP64, cdi.FP32])
+def test_optional_memory_does_not_refuse_a_request(precision):
+    """A request that fits the budget without the memory that only makes it
+    faster is served, by itself; one that does not, is refused."""
+    m = np.zeros((32, 64), np.uint8)
+    least = serve.required_bytes(m, precision)
+    assert least < serve.footprint_bytes(m, precision)
+    lock = threading.Lock()
+    for budget, served in ((least, True), (least - 1, False)):
+        solver, state = _fake_solver([], lock)
+        srv = serve.Server(slots=2, memory_budget=budget, solver=solver)
+        for i in range(3):
+            srv.submit(serve.Request(m, 1.0, 1e-4, 1, precision=precision, tag=i))
+        done = srv.drain(3, timeout=60)
+        srv.close()
+        assert [not r.error for r in done] == [served] * 3
+        assert state["max"] == (1 if served else 0) and srv.max_in_use <= budget
