@@ -168,9 +168,10 @@ __device__ __forceinline__ void combine_partials(const double *partials, int nbl
 // before it only data that no kernel of the sequence writes may be read, and
 // nothing written.  Data that the sequence writes is read by plain loads (not
 // through the non-coherent path, whose loads may be moved).  It takes the gap
-// between short steps: 128x64 FP64 flow 3.4 -> 2.9 us a step and transport 4.1
-// -> 3.2, 1024x512 transport 6.7 -> 6.0, a resolved 101x87x93 pack 17.6 ->
-// 16.0; a 256^3 step (141 us) does not notice.
+// between steps, 0.5 to 2 us: device time of a step without and with it, 128x64
+// FP64 flow 3.3 and 2.6 us, transport 4.1 and 3.2; 1024x512 pair flow 11.9 and
+// 11.4, transport 6.0 and 5.1; transport of a resolved 101x87x93 pack 13.9 and
+// 13.0; 256^3 flow 438.4 and 437.4, transport 140.5 and 138.1.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() {

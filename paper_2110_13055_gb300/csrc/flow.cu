@@ -447,7 +447,7 @@ __global__ void k_links_ovf(const typename FlowFlag<DIM>::type *__restrict__ fl,
 // What bounds it on a large image is L2: even and odd step both move 11.7 TB/s
 // of 32-byte sectors, the odd one 1.46 times as many (its gathers and scatters
 // of 32 consecutive ranks break where a grain ends a row), in 1.43 times the
-// time; 256^3 pack 440 us a launch on average.  Registers are bounded per
+// time; 256^3 pack 437 us a launch on average.  Registers are bounded per
 // variant so that enough blocks are resident and nothing spills.
 // (lbm_collide: FP32 and BF16 storage; gi the values read.)
 template <typename S, int DIM, bool ODD, typename PL>
@@ -504,7 +504,7 @@ __device__ __forceinline__ void lbm_collide(const PL &g, const int (&nb)[Lat<DIM
 // class.  With tau = 1 the first term is zero and left out.  At 2 FP64
 // operations a clock and SM the arithmetic is what bounds a small image:
 // D2Q9 34 operations a site (43 with tau != 1) instead of about 75 term by
-// term; 128x64 image 4.9 -> 3.4 us a step.  (FP32 storage keeps the terms of
+// term; 128x64 image 4.5 -> 3.3 us a step.  (FP32 storage keeps the terms of
 // lbm_collide: there the rounded class constants cost accuracy, 2.5e-7 -> 1.1e-6
 // of the velocity in 600 steps on a 256^3 pack.)
 template <int DIM, bool ODD, typename PL>

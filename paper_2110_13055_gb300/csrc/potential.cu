@@ -605,13 +605,14 @@ static cdi_status cg_iterate(cdi_domain *d, const Geo &g, double *r, double *p, 
 static cdi_status finish_potential(cdi_domain *d, cudaEvent_t ev, bool done, int *iters,
                                    double *relres);
 
-// Screened systems stay with the FP64 iteration and keep their bits.  They
-// need fewer iterations (the condition number is below (12 + kdx2) / kdx2),
-// and they are the fields that transport runs on: its FP32 face data rounds
-// them, and a rounding that a change in their 13th digit turns moves a
-// concentration of a resolved double layer by 2e-7.  (96^3: 75 iterations and
-// 5.5 ms at kdx2 = 0.44, where refinement takes 1.9 ms; 158 and 11.4 ms, 3.7
-// ms at 0.06; 5 and 0.6 ms, 0.4 ms at the default screening.)
+// Screened systems stay with the FP64 iteration and keep their bits, in every
+// storage type.  They need fewer iterations (the condition number is below (12 +
+// kdx2) / kdx2), and they are the fields that transport runs on: the face data
+// of FP32 storage rounds them, and a rounding that a change in their 13th digit
+// turns moves a concentration of a resolved double layer by 2e-7.  It costs
+// time: 96^3, 75 iterations and 5.5 ms at kdx2 = 0.44, where refinement takes
+// 1.9 ms; 158 and 11.4 ms, 3.7 ms at 0.06; 5 and 0.6 ms, 0.4 ms at the default
+// screening.
 constexpr double kRefineBelow = 0.05;
 
 // The refinement above; *done says whether it reached tol.  Where it does not

@@ -208,7 +208,7 @@ __host__ __device__ constexpr long long np_warps(long long n) { return (n + kHom
 // co[a * n + r], and of the feed face at a = DIM (k_np_coef64); a - face is
 // the + face of the cell across it with the two exchanged.  They take the
 // exponentials and divisions (about 60 FP64 operations a face) out of the
-// step: 128x64 image, two species: 16.4 -> 4.0 us a step.  co null (no memory
+// step: 128x64 image, two species: 17.0 -> 4.1 us a step.  co null (no memory
 // for them): every face is evaluated from the velocity and the potential.
 template <int DIM, bool EARLY>
 __device__ __forceinline__ bool np_cell(const double *Cin, double *Cout,
@@ -557,8 +557,8 @@ template <int DIM, int NS> struct NPLane {
 // evaluated once per face and handed to the next lane as its -x flux; per
 // home cell the faces are summed in the order adsorption, +x, -x, +y,
 // -y, +z, -z.  SMALL: every face of the warp has |P| < 1/2, so the
-// arithmetic has no branch and its faces overlap.  EVAL: the Bernoulli pairs are not stored (no memory for
-// them) and are evaluated at every step.
+// arithmetic has no branch and its faces overlap.  EVAL: the Bernoulli pairs
+// are not stored (no memory for them) and are evaluated at every step.
 template <int DIM, int NS, bool PAIR, bool SMALL, bool EVAL>
 __device__ __forceinline__ void np_update(const NPFields &F, int n_cells, int naccs,
                                           const NPConst<float> &c, int w, int r, bool home,
@@ -959,8 +959,9 @@ __device__ __forceinline__ void np_prefetch(const NPFields &F, int n, int naccs,
 }
 
 // FP32 storage: warps of 31 home cells (np_warp31); ahead > 0: np_prefetch.
-// 256^3 pack, pair concentrations: 235 us a step -> 139 us (1.6 -> 2.7 TB/s of
-// the method's 49 bytes a cell); 1024x512: 6.9 -> 5.8 us.
+// 256^3 pack, pair concentrations: 231 -> 141 us a step (1.6 -> 2.6 TB/s of the
+// method's 49 bytes a cell), 1024x512: 6.7 -> 6.0, before early launches
+// (launch_pdl: 138 and 5.1 us).
 template <int DIM, int NS, int BS, bool PAIR, int MODE>
 __global__ void __launch_bounds__(BS)
     k_np_step32(const __grid_constant__ NPFields F, int n, int naccs,
@@ -1467,10 +1468,11 @@ constexpr int kGraphSteps = 64;  // steps per captured transport graph (even)
 
 // Launch shapes: 64, 128 or 256 threads per block (0-2); 3-9 name the default
 // again.  128 is taken unless a shape is fixed: it is the fastest or within
-// 4 % of it on every size measured (256^3: 155 / 139 / 154 us for 64 / 128 /
-// 256; 1024x512: 5.8 / 5.8 / 5.9; 96^3: 11.3 / 10.6 / 11.1), so no launch is
-// spent on timing candidates (FP64, 128x64: 4.0 / 4.0 / 4.9).  Accounts are
-// kept per warp whatever the shape, so every choice computes the same bits.
+// 4 % of it on every size measured (before early launches, us a step for 64 /
+// 128 / 256: 256^3 155 / 139 / 154; 1024x512 5.8 / 5.8 / 5.9; 96^3 11.3 / 10.6 /
+// 11.1; FP64 128x64 4.0 / 4.0 / 4.9), so no launch is spent on timing
+// candidates.  Accounts are kept per warp whatever the shape, so every choice
+// computes the same bits.
 constexpr int kNpDefaultShape = 1;
 constexpr int kNpVariantBlock[10] = {64, 128, 256, 128, 128, 128, 128, 128, 128, 128};
 
