@@ -444,10 +444,12 @@ __global__ void k_links_ovf(const typename FlowFlag<DIM>::type *__restrict__ fl,
 // FP64, FP32 or BF16 storage (S), arithmetic in T = Arith<S>.  Collision (Eq. 8) with the Stokes-linear
 // equilibrium g_eq_i = w_i (drho + 3 e_i.j), j = sum e_i g_i + F/2, and the
 // force source (1 - 1/(2 tau)) 3 w_i e_i.F; omega = 1/tau.
-// What bounds it on a large image is L2: even and odd step both move 11.7 TB/s
-// of 32-byte sectors, the odd one 1.46 times as many (its gathers and scatters
-// of 32 consecutive ranks break where a grain ends a row), in 1.43 times the
-// time; 256^3 pack 437 us a launch on average.  Registers are bounded per
+// What bounds it on a large image: the even step memory (256^3: 6.5 TB/s of
+// DRAM, 0.97 of the copy rate).  The odd step moves 1.46 times the L2 sectors
+// (its gathers and scatters of 32 consecutive ranks break where a grain ends a
+// row) in 1.5 times the time, with no unit near its limit (160^3: L2 44 %, L1 51
+// %, issue 54 %, DRAM 56 %): it waits for link data, then gathers, with 40 % of
+// the warps.  256^3 pack 437 us a launch on average.  Registers are bounded per
 // variant so that enough blocks are resident and nothing spills.
 // (lbm_collide: FP32 and BF16 storage; gi the values read.)
 template <typename S, int DIM, bool ODD, typename PL>
