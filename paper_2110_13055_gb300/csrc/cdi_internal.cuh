@@ -169,7 +169,7 @@ __device__ __forceinline__ void combine_partials(const double *partials, int nbl
 // nothing written.  Data that the sequence writes is read by plain loads (not
 // through the non-coherent path, whose loads may be moved).  It takes the gap
 // between steps, 0.5 to 2 us: device time of a step without and with it, 128x64
-// FP64 flow 3.3 and 2.6 us, transport 4.1 and 3.2; 1024x512 pair flow 11.9 and
+// FP64 flow 3.4 and 2.8 us, transport 4.1 and 3.2; 1024x512 pair flow 11.9 and
 // 11.4, transport 6.0 and 5.1; transport of a resolved 101x87x93 pack 13.9 and
 // 13.0; 256^3 flow 438.4 and 437.4, transport 140.5 and 138.1.
 // ---------------------------------------------------------------------------

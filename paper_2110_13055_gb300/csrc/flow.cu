@@ -499,69 +499,55 @@ __device__ __forceinline__ void lbm_collide(const PL &g, const int (&nb)[Lat<DIM
   *slot_ptr<DIM, ODD, false>(g, nb, k0, 0) = narrow<S>(go0);
 }
 
-// The FP64 collision by opposite pairs (i, o): with s = g_i + g_o and d = g_i -
-// g_o, drho = g_0 + sum s and j = F/2 + sum e d, and both post-collision values
-// are (1 - omega) g + (A_w +- E), A_w = omega w drho by weight class, E = e.(3
-// omega w j + w (1 - 1/(2 tau)) 3 F) with its components formed once per
-// class.  With tau = 1 the first term is zero and left out.  At 2 FP64
-// operations a clock and SM the arithmetic is what bounds a small image:
-// D2Q9 34 operations a site (43 with tau != 1) instead of about 75 term by
-// term; 128x64 image 4.5 -> 3.3 us a step.  (FP32 storage keeps the terms of
-// lbm_collide: there the rounded class constants cost accuracy, 2.5e-7 -> 1.1e-6
-// of the velocity in 600 steps on a 256^3 pack.)
+// The FP64 collision: the operations of lbm_collide in their order, without
+// those that change nothing.  Terms of zero components are left out, e.j is
+// formed once for a direction and its opposite, and at tau = 1 the relaxation
+// g - (g - g_eq), which is g_eq, is not carried out.  At 2 FP64 operations a
+// clock and SM the arithmetic is what bounds a small image: D2Q9 45 operations
+// a site (63 with tau != 1) instead of about 75; 128x64 image 4.5 -> 3.4 us a
+// step, 2.8 with early launches.  (Fewer operations, 34 and 43, come from sums
+// and differences of opposite pairs with (1 - omega) g + omega w (...) formed
+// from a rounded omega w; then the weights and 1 - omega no longer add up to 1,
+// and the mass that a step makes or loses fills dead ends: at tau = 0.8, 2,000
+// steps of a 128x64 pack, the error is 5e-15 to 2e-12 instead of 1e-15 to 2e-14.)
 template <int DIM, bool ODD, typename PL>
 __device__ __forceinline__ void lbm_collide_f64(const PL &g, const int (&nb)[Lat<DIM>::Q], int k0,
                                                 const double (&gi)[Lat<DIM>::Q], double omega,
                                                 double fx_half, double fsrc) {
   using L = Lat<DIM>;
-  constexpr int H = L::H;
+  constexpr int Q = L::Q, H = L::H;
   double drho = gi[0], j[3] = {fx_half, 0.0, 0.0};
 #pragma unroll
-  for (int i = 1; i <= H; i++) {
-    const double d = r_sub(gi[i], gi[i + H]);
-    drho = r_add(drho, r_add(gi[i], gi[i + H]));
+  for (int i = 1; i < Q; i++) {
+    drho = r_add(drho, gi[i]);
     const int e[3] = {L::ex(i), L::ey(i), L::ez(i)};
 #pragma unroll
     for (int a = 0; a < DIM; a++) {
-      if (e[a] > 0) j[a] = r_add(j[a], d);
-      if (e[a] < 0) j[a] = r_sub(j[a], d);
+      if (e[a] > 0) j[a] = r_add(j[a], gi[i]);
+      if (e[a] < 0) j[a] = r_sub(j[a], gi[i]);
     }
   }
-  constexpr double wa = L::w(1), wd = L::w(H);
   auto collide = [&](auto tau1) {
-    constexpr bool T1 = decltype(tau1)::value;
-    auto scaled = [&](double w) { return T1 ? w : r_mul(omega, w); };
-    const double om1 = T1 ? 0.0 : r_sub(1.0, omega);
-    const double A0 = r_mul(scaled(L::w(0)), drho), Aa = r_mul(scaled(wa), drho),
-                 Ad = r_mul(scaled(wd), drho);
-    double Ja[DIM], Jd[DIM];
-#pragma unroll
-    for (int a = 0; a < DIM; a++) {
-      Ja[a] = r_mul(scaled(3.0 * wa), j[a]);
-      Jd[a] = r_mul(scaled(3.0 * wd), j[a]);
-    }
-    Ja[0] = r_fma(wa, fsrc, Ja[0]);
-    Jd[0] = r_fma(wd, fsrc, Jd[0]);
-    auto out = [&](int i, double eq) {
-      *slot_ptr<DIM, ODD, false>(g, nb, k0, i) = T1 ? eq : r_fma(om1, gi[i], eq);
+    auto out = [&](int i, double geq) {  // geq = w (drho + 3 e.j)
+      double v = decltype(tau1)::value ? geq : r_fma(-omega, r_sub(gi[i], geq), gi[i]);
+      if (L::ex(i) != 0) v = r_fma(L::w(i) * L::ex(i), fsrc, v);
+      *slot_ptr<DIM, ODD, false>(g, nb, k0, i) = v;
     };
 #pragma unroll
     for (int i = 1; i <= H; i++) {
       const int e[3] = {L::ex(i), L::ey(i), L::ez(i)};
-      const bool axis = e[0] * e[0] + e[1] * e[1] + e[2] * e[2] == 1;
-      double E = 0.0;
+      double ej = 0.0;
       bool some = false;
 #pragma unroll
       for (int a = 0; a < DIM; a++) {
         if (e[a] == 0) continue;
-        const double c = axis ? Ja[a] : Jd[a];
-        E = some ? (e[a] > 0 ? r_add(E, c) : r_sub(E, c)) : (e[a] > 0 ? c : -c);
+        ej = some ? (e[a] > 0 ? r_add(ej, j[a]) : r_sub(ej, j[a])) : (e[a] > 0 ? j[a] : -j[a]);
         some = true;
       }
-      out(i, r_add(axis ? Aa : Ad, E));
-      out(i + H, r_sub(axis ? Aa : Ad, E));
+      out(i, r_mul(L::w(i), r_fma(3.0, ej, drho)));
+      out(i + H, r_mul(L::w(i), r_fma(-3.0, ej, drho)));
     }
-    out(0, A0);
+    out(0, r_mul(L::w(0), drho));
   };
   // (an integer test: an FP64 comparison would take the FP64 pipe)
   if (__double_as_longlong(omega) == __double_as_longlong(1.0)) collide(std::true_type());
