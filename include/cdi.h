@@ -321,8 +321,10 @@ typedef struct {
  * memory for the members is taken from the domain's allocator for the call
  * only: about n_combos * (3 dim + 2 n_species) * 4 bytes per pore cell in FP32
  * (twice the concentrations' part with pair storage; where a face Peclet
- * number reaches 1/2, (dim + 1) * n_species * 8 more where there is as much).
- * Members that do not fit at once are run in parts, with the same results. */
+ * number reaches 1/2, (dim + 1) * n_species * 8 more where there is as much),
+ * (dim + 2 n_species) * 8 in FP64 with (dim + 1) * n_species * 16 more where
+ * there is as much.  Members that do not fit at once are run in parts, with the
+ * same results. */
 cdi_status cdi_sweep_transport(cdi_domain *dom, const cdi_combo *combos, int n_combos,
                                const cdi_elec_params *p, const cdi_species *sp,
                                int n_species, double c0_molm3, double Ka_mps,
